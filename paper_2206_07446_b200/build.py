@@ -7,7 +7,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libnnv.so")
-SOURCES = ["plan.cpp", "scheduler.cpp", "cachefile.cpp", "transform.cu", "exec_kernels.cu", "gemm_tc.cu", "exec.cu", "pipeline.cu", "noalloc.cu"]
+SOURCES = ["plan.cpp", "scheduler.cpp", "cachefile.cpp", "transform.cu", "exec_kernels.cu", "direct_conv.cu", "gemm_tc.cu", "exec.cu", "pipeline.cu", "noalloc.cu"]
 
 
 def sources():
@@ -27,7 +27,7 @@ def build(force=False, verbose=False):
     if not force and not needs_build():
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
-    cmd = [nvcc, "-std=c++17", "-O3", "-lineinfo", "-shared", "-Xcompiler", "-fPIC",
+    cmd = [nvcc, "-std=c++17", "-O3", "-lineinfo", "-shared", "-Xcompiler", "-fPIC", "--threads", "0",
            "-gencode", "arch=compute_100a,code=sm_100a",
            "-I", os.path.join(ROOT, "include"), "-I", CSRC,
            "-o", LIB] + sources()

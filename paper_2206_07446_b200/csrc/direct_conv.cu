@@ -1,0 +1,271 @@
+// fp32 direct convolution: an implicit GEMM on the FP32 pipes straight from the raw OIHW weights (no weight transform).
+//
+// Bound: the L1 / shared-memory data path (4 x 4 outputs a thread: ~6.5 cycles of shared-memory reads for 4 cycles of
+// FMAs), and on the small layers a cold run picks this kernel for, latency.  A block owns 32 pixels x 32 channels and
+// walks the reduction in chunks of JC (channel, tap) pairs in raw weight order; the next chunk's global loads are in
+// flight while this one is multiplied out of shared memory.
+//   - Eight lanes read 128 contiguous bytes (32 channels of one pixel and tap; 32 weights of one row), so a warp's
+//     gather touches four lines; with 32-byte pieces of 16 lines the gathers alone cost as much L1 time as the
+//     multiplication.  The pairs are stored transposed, [pair][pixel] and [pair][channel], with the 16-byte words of a
+//     row permuted by the pair's index / 4, which makes the stores and the reads free of bank conflicts.
+//   - The block's threads form four groups of 8 x 8 that take a quarter of every chunk each and are summed at the end.
+//   - `splits` blocks of a cluster share the chunks of one tile and add their partial tiles through distributed shared
+//     memory in rank order (the result does not depend on timing).
+// Measured (back to back calls, us; the former 64 x 64 tile with 4-byte gathers -> this kernel): 64 -> 128 3x3 / 2 @56
+// 71 -> 11.3, 64 -> 64 3x3 @56 71 -> 15, 256 -> 256 3x3 @14 274 -> 18, 512 -> 512 3x3 @7 538 -> 23, 1024 -> 256 1x1 @14
+// 140 -> 9.8, 3 -> 32 3x3 / 2 @224 7.7 -> 7.1.
+#include <algorithm>
+#include <type_traits>
+
+#include "nnv_internal.h"
+
+namespace nnv {
+namespace {
+
+constexpr int DC_T = 32;                                      // pixels and channels of a tile
+constexpr int DC_THREADS = 256;
+constexpr int DC_GROUPS = 4;
+
+struct DirectDev {
+    const float* x; const float* w; const float* bias; const float* add; float* y;
+    int act, C, H, W, K, R, S, stride, pad, OH, OW, splits;
+};
+
+__device__ __forceinline__ float direct_act(float v, int act) {
+    if (act == 1) return fmaxf(v, 0.f);
+    if (act == 2) return fminf(fmaxf(v, 0.f), 6.f);
+    return v;
+}
+
+// Reduction pairs per chunk: 32 channels x 9 taps, 64 channels x 1 tap, or 64 flat (c, r, s) positions (TAPS = 0: any filter).
+template <int TAPS> struct DcChunk {
+    static constexpr int CB = TAPS == 9 ? 32 : 64;
+    static constexpr int JC = TAPS == 9 ? 288 : 64;
+};
+
+// Shared memory of a block: both staged operands, at least the four groups' partial tiles.
+__host__ __device__ constexpr int dc_smem_floats(int jc) {
+    return 2 * jc * DC_T > DC_GROUPS * DC_T * (DC_T + 4) ? 2 * jc * DC_T : DC_GROUPS * DC_T * (DC_T + 4);
+}
+
+// Word of (pair j, element e) in a staged operand.
+__device__ __forceinline__ int dc_word(int j, int e) { return j * DC_T + (e ^ (((j >> 2) & 7) << 2)); }
+
+template <int TAPS>
+__global__ void __launch_bounds__(DC_THREADS, 2)
+direct_conv_kernel(const DirectDev g) {
+    pdl_wait();
+    constexpr int JC = DcChunk<TAPS>::JC, CB = DcChunk<TAPS>::CB, T = DC_T, G = DC_GROUPS, GT = DC_THREADS / G;
+    extern __shared__ __align__(16) float sm[];
+    float* const As = sm;
+    float* const Bs = sm + JC * T;
+
+    const int tid = threadIdx.x;
+    const int RS = g.R * g.S, Q = g.C * RS, P = g.OH * g.OW;
+    const int p0 = blockIdx.x * T, k0 = blockIdx.y * T;
+    const int sp = blockIdx.z;
+    const int chunks_all = (Q + JC - 1) / JC;
+    const int ch0 = chunks_all * sp / g.splits, ch1 = chunks_all * (sp + 1) / g.splits;
+
+    // Loader role: element e (pixel of A, channel of B) and word l8 of its eight.  Word loads move four channels / weights;
+    // the flat form moves single positions.
+    constexpr int VW = TAPS ? 4 : 1;
+    constexpr int N = JC / (8 * VW);                           // words a thread fetches per operand and chunk
+    using Word = typename std::conditional<TAPS != 0, float4, float>::type;
+    const int e = tid >> 3, l8 = tid & 7;
+    const int pa = p0 + e, kb = k0 + e;
+    const int oh = pa / g.OW, ow = pa - oh * g.OW;
+    const int ih0 = pa < P ? oh * g.stride - g.pad : -(1 << 20), iw0 = ow * g.stride - g.pad;   // a pixel beyond the grid is outside the image
+    const float* const wrow = g.w + (long long)kb * Q;
+    Word ra[N], rb[N];
+    // Positions outside the image, the filter bank or the reduction are fetched from a valid address and zeroed on
+    // their way into shared memory, so that all loads of a chunk leave back to back.
+    uint32_t live_a = 0, live_b = 0;
+    auto fetch = [&](int ch) {
+        live_a = live_b = 0;
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            int c, r, s;
+            if constexpr (TAPS != 0) {
+                r = TAPS == 9 ? i / 3 : 0;
+                s = TAPS == 9 ? i % 3 : 0;
+                c = ch * CB + (TAPS == 9 ? 0 : 32 * i) + 4 * l8;
+            } else {
+                const int q = ch * JC + 8 * i + l8;
+                if (ch * JC + 8 * i >= Q) break;
+                c = q / RS;
+                const int rs = q - c * RS;
+                r = rs / g.S;
+                s = rs - r * g.S;
+            }
+            const int ih = ih0 + r, iw = iw0 + s;
+            const bool ok = c < g.C && ih >= 0 && ih < g.H && iw >= 0 && iw < g.W;
+            ra[i] = __ldg(reinterpret_cast<const Word*>(ok ? g.x + ((long long)ih * g.W + iw) * g.C + c : g.x));
+            live_a |= ok ? 1u << i : 0u;
+        }
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            const int q = ch * JC + (8 * i + l8) * VW;
+            const bool ok = kb < g.K && q < Q;
+            rb[i] = __ldg(reinterpret_cast<const Word*>(ok ? wrow + q : g.w));
+            live_b |= ok ? 1u << i : 0u;
+        }
+    };
+    auto stash = [&](int ch) {
+        const int left = (Q - ch * JC + 3) & ~3;               // pairs from here on are never read
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            if ((TAPS == 9 ? 36 * l8 : (8 * i + l8) * VW) >= left) break;
+            const float* v = reinterpret_cast<const float*>(&ra[i]);
+#pragma unroll
+            for (int u = 0; u < VW; ++u) {
+                const int j = TAPS == 9 ? (4 * l8 + u) * 9 + i : (8 * i + l8) * VW + u;      // raw weight order: channel-major
+                As[dc_word(j, e)] = (live_a >> i) & 1u ? v[u] : 0.f;
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            const float* v = reinterpret_cast<const float*>(&rb[i]);
+            if ((8 * i + l8) * VW >= left) break;
+#pragma unroll
+            for (int u = 0; u < VW; ++u) Bs[dc_word((8 * i + l8) * VW + u, e)] = (live_b >> i) & 1u ? v[u] : 0.f;
+        }
+    };
+
+    const int grp = tid / GT, gt = tid - grp * GT;
+    const int tx = gt & 7, ty = gt >> 3;                       // tx -> channels, ty -> pixels
+    float acc[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+
+    fetch(ch0);
+    for (int ch = ch0; ch < ch1; ++ch) {
+        if (ch > ch0) __syncthreads();                         // the previous chunk has been multiplied
+        stash(ch);
+        __syncthreads();
+        if (ch + 1 < ch1) fetch(ch + 1);
+        const int words = (min(JC, Q - ch * JC) + 3) >> 2;     // groups of four pairs that exist
+        const int w1 = words * (grp + 1) / G;
+#pragma unroll 1
+        for (int wd = words * grp / G; wd < w1; ++wd) {
+            const float* a = As + wd * 4 * T + ((ty ^ (wd & 7)) << 2);
+            const float* b = Bs + wd * 4 * T + ((tx ^ (wd & 7)) << 2);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float4 av = *reinterpret_cast<const float4*>(a + j * T);
+                const float4 bv = *reinterpret_cast<const float4*>(b + j * T);
+                const float aa[4] = {av.x, av.y, av.z, av.w}, bb[4] = {bv.x, bv.y, bv.z, bv.w};
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int jj = 0; jj < 4; ++jj) acc[i][jj] = fmaf(aa[i], bb[jj], acc[i][jj]);
+            }
+        }
+    }
+    // The next kernel's blocks are let in only now: released at the start they would pile up on the SMs this grid leaves
+    // idle and run there several to an SM (22.5 us a call back to back where one call takes 14, 64 -> 128 3x3 / 2 @56).
+    pdl_trigger();
+    __syncthreads();
+
+    // Partial tiles of the groups, then of the cluster, each summed in index order.
+    constexpr int RP = T + 4;
+    float* red = sm;
+    static_assert(G * T * RP <= dc_smem_floats(JC), "the partial tiles reuse the staging buffers");
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        *reinterpret_cast<float4*>(red + (grp * T + ty * 4 + i) * RP + tx * 4) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+    __syncthreads();
+    auto group_sum = [&](int row, int c4) {
+        float4 s = *reinterpret_cast<const float4*>(red + row * RP + c4);
+#pragma unroll
+        for (int q = 1; q < G; ++q) {
+            const float4 v = *reinterpret_cast<const float4*>(red + (q * T + row) * RP + c4);
+            s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+        }
+        return s;
+    };
+    if (g.splits > 1) {
+        for (int idx = tid; idx < T * (T / 4); idx += DC_THREADS) {      // into group 0's place: every thread its own words
+            const int row = idx / (T / 4), c4 = (idx % (T / 4)) * 4;
+            *reinterpret_cast<float4*>(red + row * RP + c4) = group_sum(row, c4);
+        }
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
+    const bool vec = (g.K & 3) == 0;
+    const int rows = T / g.splits;                             // splits is a power of two up to 8
+    for (int idx = tid; idx < rows * (T / 4); idx += DC_THREADS) {
+        const int row = sp * rows + idx / (T / 4), c4 = (idx % (T / 4)) * 4;
+        float4 s;
+        if (g.splits == 1) {
+            s = group_sum(row, c4);
+        } else {
+            const uint32_t local = (uint32_t)__cvta_generic_to_shared(red + row * RP + c4);
+            float4 part[8];                                    // all remote loads leave before the first is used
+#pragma unroll
+            for (int rk = 0; rk < 8; ++rk)
+                if (rk < g.splits) {
+                    uint32_t remote;
+                    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(rk));
+                    asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];"
+                                 : "=f"(part[rk].x), "=f"(part[rk].y), "=f"(part[rk].z), "=f"(part[rk].w) : "r"(remote));
+                }
+            s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int rk = 0; rk < 8; ++rk)
+                if (rk < g.splits) { s.x += part[rk].x; s.y += part[rk].y; s.z += part[rk].z; s.w += part[rk].w; }
+        }
+        const int p = p0 + row, k = k0 + c4;
+        if (p >= P || k >= g.K) continue;
+        const long long o = (long long)p * g.K + k;
+        float v[4] = {s.x, s.y, s.z, s.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (k + j >= g.K) break;
+            if (g.bias) v[j] += __ldg(g.bias + k + j);
+            if (g.add) v[j] += __ldg(g.add + o + j);
+            v[j] = direct_act(v[j], g.act);
+            if (!vec) g.y[o + j] = v[j];
+        }
+        if (vec) *reinterpret_cast<float4*>(g.y + o) = make_float4(v[0], v[1], v[2], v[3]);
+    }
+    if (g.splits > 1) {                                        // nobody leaves while its partial tile may still be read
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
+}
+
+template <int TAPS>
+nnv_status_t launch_dc(const DirectDev& g, cudaStream_t st) {
+    constexpr size_t smem = sizeof(float) * dc_smem_floats(DcChunk<TAPS>::JC);
+    static const cudaError_t attr = cudaFuncSetAttribute(direct_conv_kernel<TAPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    NNV_CUDA(attr);
+    const dim3 grid(ceil_div(g.OH * g.OW, DC_T), ceil_div(g.K, DC_T), g.splits);
+    NNV_REQUIRE(grid.y <= 65535, NNV_ERR_UNSUPPORTED, "too many output channels for the direct kernel");
+    NNV_CUDA(launch_pdl_cluster(direct_conv_kernel<TAPS>, grid, dim3(DC_THREADS), smem, st, g.splits, g));
+    return NNV_OK;
+}
+
+}  // namespace
+
+nnv_status_t launch_direct(const float* x, const float* w, const float* bias, const float* add, float* y, int act,
+                           int C, int H, int W, int K, int R, int S, int stride, int pad, int OH, int OW,
+                           cudaStream_t st) {
+    DirectDev g{x, w, bias, add, y, act, C, H, W, K, R, S, stride, pad, OH, OW, 1};
+    const bool al16 = ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(w) | reinterpret_cast<uintptr_t>(y)) & 15) == 0;
+    const int taps = (C % 4) == 0 && al16 ? ((R == 3 && S == 3) ? 9 : (R == 1 && S == 1) ? 1 : 0) : 0;
+    const int jc = taps == 9 ? 288 : 64, chunks = ceil_div(C * R * S, jc);
+    // The split with the least estimated time, in cycles: an SM's blocks share its L1, so a chunk costs blocks per SM x ~16
+    // cycles a pair; a split adds two cluster barriers and the remote reads.
+    const long long tiles = (long long)ceil_div(OH * OW, DC_T) * ceil_div(K, DC_T);
+    double best = 1e30;
+    for (int s = 1; s <= 8 && s <= chunks; s *= 2) {
+        const double t = (double)((tiles * s + 147) / 148) * ceil_div(chunks, s) * jc * 16.0 + (s > 1 ? 3000.0 : 0.0);
+        if (t < best - 1e-9) { best = t; g.splits = s; }
+    }
+    return taps == 9 ? launch_dc<9>(g, st) : taps == 1 ? launch_dc<1>(g, st) : launch_dc<0>(g, st);
+}
+
+}  // namespace nnv

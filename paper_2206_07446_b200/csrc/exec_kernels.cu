@@ -311,91 +311,6 @@ nnv_status_t launch_wino_output(int m, const float* Mt, float* y, const float* b
     return NNV_OK;
 }
 
-// ---- fp32 direct convolution ----------------------------------------------------------------
-// Implicit GEMM on the FP32 pipes straight from the raw OIHW weights: the reduction index is
-// q = c*R*S + r*S + s, which is exactly the raw row W[k][:], so no weight transform is needed.
-// Tile: 64 pixels x 64 output channels per block, 16 reduction steps per stage, 4x4 per thread.
-constexpr int DC_BM = 64, DC_BN = 64, DC_BK = 16;
-__global__ void __launch_bounds__(256)
-direct_conv_kernel(const float* __restrict__ x, const float* __restrict__ w, const float* __restrict__ bias,
-                   const float* __restrict__ add, float* __restrict__ y, int act, int C, int H, int W, int K, int R,
-                   int S, int stride, int pad, int OH, int OW) {
-    pdl_enter();
-    __shared__ float As[DC_BK][DC_BM + 4];
-    __shared__ float Bs[DC_BK][DC_BN + 4];
-    const int P = OH * OW, RS = R * S, Q = C * RS;
-    const int p0 = blockIdx.x * DC_BM, k0 = blockIdx.y * DC_BN;
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;      // tx -> channels, ty -> pixels
-    float acc[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-
-    for (int q0 = 0; q0 < Q; q0 += DC_BK) {
-#pragma unroll
-        for (int it = 0; it < 4; ++it) {                          // A: 64 x 16 gathered input
-            const int e = threadIdx.x + it * 256;
-            const int pm = e % DC_BM, kk = e / DC_BM;
-            const int p = p0 + pm, q = q0 + kk;
-            float v = 0.f;
-            if (p < P && q < Q) {
-                const int c = q / RS, rs = q - c * RS;
-                const int r = rs / S, s = rs - r * S;
-                const int oh = p / OW, ow = p - oh * OW;
-                const int ih = oh * stride + r - pad, iw = ow * stride + s - pad;
-                if (ih >= 0 && ih < H && iw >= 0 && iw < W) v = __ldg(x + ((long long)ih * W + iw) * C + c);
-            }
-            As[kk][pm] = v;
-        }
-#pragma unroll
-        for (int it = 0; it < 4; ++it) {                          // B: 64 x 16 raw weights
-            const int e = threadIdx.x + it * 256;
-            const int kk = e % DC_BK, n = e / DC_BK;
-            const int k = k0 + n, q = q0 + kk;
-            Bs[kk][n] = (k < K && q < Q) ? __ldg(w + (long long)k * Q + q) : 0.f;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < DC_BK; ++kk) {
-            float a[4], b[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx * 4 + j];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int p = p0 + ty * 4 + i;
-        if (p >= P) continue;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int k = k0 + tx * 4 + j;
-            if (k >= K) continue;
-            const long long o = (long long)p * K + k;
-            float v = acc[i][j];
-            if (bias) v += __ldg(bias + k);
-            if (add) v += __ldg(add + o);
-            y[o] = apply_act(v, act);
-        }
-    }
-}
-
-nnv_status_t launch_direct(const float* x, const float* w, const float* bias, const float* add, float* y, int act,
-                           int C, int H, int W, int K, int R, int S, int stride, int pad, int OH, int OW,
-                           cudaStream_t st) {
-    dim3 grid(ceil_div(OH * OW, DC_BM), ceil_div(K, DC_BN));
-    NNV_LAUNCH((direct_conv_kernel), grid, 256, 0, st, x, w, bias, add, y, act, C, H, W, K, R, S, stride, pad, OH, OW);
-    NNV_CUDA(cudaGetLastError());
-    return NNV_OK;
-}
-
 // ---- fp32 depthwise convolution -------------------------------------------------------------
 // One thread per (output pixel, channel), channel fastest; raw weights W[c][r][s] are read as is.
 __global__ void __launch_bounds__(256)
