@@ -153,8 +153,8 @@ nnv_status_t nnv_plan_destroy(nnv_plan_t* plan);
  * candidate kernels, Section 3.3; this lets a harness also profile candidate TILINGS of one
  * kernel).  Process-wide; read whenever a launch is planned; a recorded graph is tied to the
  * settings it was recorded under.  spec: "key=value;key=value", NULL or "" = all defaults.
- *   gemm_tile=BN,splits   column tile (16..128, multiple of 16) and K splits (1,2,4,8) of the GEMM
- *   gemm_ring=N           shared-memory ring depth 2..8        gemm_prefill=0|1
+ *   gemm_tile=BN,splits   column tile (16..128, multiple of 16) and K splits (1,2,4,8,16) of the GEMM
+ *   gemm_ring=N           shared-memory ring depth 2..8        gemm_prefill=0|1 (no effect)
  *   conv3x3=off|auto|MT,BN,splits[,boxes,weight_tiles]          the halo-resident 3x3 kernel
  *   conv3x3p=off|BN,ctas_per_sm[,boxes,weight_tiles]           the persistent form of the 3x3 kernel (off unless asked for)
  *   conv3x3w=off|auto|on  the weights-stationary form of the 3x3 kernel (layers whose weight slice fits shared memory):

@@ -37,7 +37,6 @@ __global__ void __launch_bounds__(GEMM_THREADS)
 conv3x3_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                   const __grid_constant__ CUtensorMap tmD, const ConvDev g) {
     extern __shared__ uint8_t smem_raw[];
-    pdl_trigger();
     const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const int BN = g.BN, MT = g.MT, NA = g.na, NB = g.nb;
     // BF16 math: a box slot holds the fp32 box as the TMA delivers it (128-byte rows, swizzled) and, behind it, the same
@@ -85,6 +84,7 @@ conv3x3_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     tc_fence_after();
     const uint32_t tmem_base = *holder_ptr;
     pdl_wait();                                               // set-up above overlaps the previous kernel's tail
+    pdl_trigger();
     if (threadIdx.x == 32) stamp_start(g.stamp);
 
     // One weight tile into ring slot `sb`: a 128-byte-swizzled fp32 tile, or a box of four 8-element bf16 chunks x BN rows
@@ -423,7 +423,6 @@ struct ConvPDev {
 __global__ void __launch_bounds__(GEMM_THREADS)
 conv3x3_tc_persistent_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const ConvPDev g) {
     extern __shared__ uint8_t smem_raw[];
-    pdl_trigger();
     const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const int BN = g.BN, NA = g.na, NB = g.nb;
     constexpr uint32_t a_slot_bytes = 18u * 1024u;                 // (16 + 2) rows of 8 pixels x 128 bytes
@@ -458,6 +457,7 @@ conv3x3_tc_persistent_kernel(const __grid_constant__ CUtensorMap tmA, const __gr
     tc_fence_after();
     const uint32_t tmem_base = *holder_ptr;
     pdl_wait();                                               // set-up above overlaps the previous kernel's tail
+    pdl_trigger();
     if (threadIdx.x == 32) stamp_start(g.stamp);
 
     if (warp == 0) {
@@ -636,7 +636,6 @@ __global__ void __launch_bounds__(GEMM_THREADS)
 conv3x3_tc_ws_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                      const __grid_constant__ CUtensorMap tmD, const ConvWDev g) {
     extern __shared__ uint8_t smem_raw[];
-    pdl_trigger();
     const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const int BN = g.BN, NWT = 9 * g.cblk;
     constexpr uint32_t a_slot_bytes = 18u * 1024u;                 // (16 + 2) rows of 8 pixels x 128 bytes
@@ -672,6 +671,7 @@ conv3x3_tc_ws_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
     tc_fence_after();
     const uint32_t tmem_base = *holder_ptr;
     pdl_wait();                                               // set-up above overlaps the previous kernel's tail
+    pdl_trigger();
     if (threadIdx.x == 32) stamp_start(g.stamp);
 
     if (warp == 0) {

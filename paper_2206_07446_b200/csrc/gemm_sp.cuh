@@ -31,7 +31,6 @@ constexpr int SP_MAX_STAGES = 8;
 __global__ void __launch_bounds__(GEMM_THREADS)
 gemm_sp_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX, const SpDev g) {
     extern __shared__ uint8_t smem_raw[];
-    pdl_trigger();
     const int STAGES = g.stages;
     const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t stage_bytes = A_STAGE_BYTES + g.b_slot_bytes;
@@ -82,6 +81,7 @@ gemm_sp_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     tc_fence_after();
     const uint32_t tmem_base = *holder_ptr;
     pdl_wait();
+    pdl_trigger();
     if (threadIdx.x == 32) stamp_start(g.stamp);
 
     if (warp == 0) {

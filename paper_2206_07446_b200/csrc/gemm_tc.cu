@@ -5,13 +5,19 @@
 // and the 1x1 GEMM (X[P][C] x W[K][C]) all present themselves.  Pixels / tiles sit on the MMA's
 // M dimension (128 TMEM lanes), output channels on N.
 //
-// Structure of one CTA (one 128 x BN output tile, 192 threads):
-//   warp 0   TMA producer: cp.async.bulk.tensor loads of 128-byte-wide K slices of A and B into a
-//            ring of shared-memory stages (128B swizzle), completion on "full" mbarriers
-//   warp 1   allocates TMEM, issues tcgen05.mma (one lane) from shared-memory descriptors into
-//            the fp32 accumulator in TMEM, releases stages with tcgen05.commit on "empty" mbarriers
-//   warps 2-5  epilogue: tcgen05.ld the accumulator (each warp its own 32 TMEM lanes), apply
+// Structure of one CTA (one 128 x BN output tile, 256 threads):
+//   warps 0, 7  TMA producers of A and B: cp.async.bulk.tensor loads of 128-byte-wide K slices into a ring of
+//            shared-memory stages (128B swizzle), completion on "full" mbarriers
+//   warps 1, 6  issue tcgen05.mma (one lane each) from shared-memory descriptors for alternate K blocks, each into its own
+//            fp32 accumulator in TMEM, and release stages with tcgen05.commit on "empty" mbarriers; warp 1 allocates TMEM
+//   warps 2-5  epilogue: tcgen05.ld the accumulators (each warp its own 32 TMEM lanes), apply
 //            bias / residual / activation, store fp32 rows
+// These layers are latency-bound (5 - 10 dependent phases of ~0.1 - 0.5 us each); what bounds each phase was read from
+// device-clock probes.  Two producers and two issuers: one thread pays 157 cycles per load and ~560 per K block of waiting,
+// issuing four MMAs and committing, more than the fill (~320 cycles of 24 KB) or the tensor pipe need.  Their loops run under
+// elect.sync, not "lane == 0": the operands then stay in uniform registers (a K block 340 -> 260 cycles).
+// 1024 -> 256 1x1 @14 (64 CTAs, 8 splits) went from 9900 to 6200 cycles from the previous kernel's end, chained calls of
+// 64 -> 64 3x3 @56 from 8.2 to 5.2 us, 256 -> 256 3x3 @14 from 9.1 to 5.6 us, 512 -> 2048 1x1 @7 from 6.2 to 4.3 us.
 // Every mbarrier wait is bounded; a wait that gives up records NNV_ERR_TIMEOUT in a device status
 // word and the CTA drains and exits instead of hanging.
 #include <cuda.h>
@@ -22,6 +28,7 @@
 #include <cmath>
 #include <cstdio>
 #include <mutex>
+#include <type_traits>
 
 #include "nnv_internal.h"
 
@@ -66,6 +73,8 @@ constexpr int BM = 128;                 // rows of A per tile = TMEM lanes
 constexpr int BK_BYTES = 128;           // bytes of K per stage row = one 128B swizzle atom
 constexpr int A_STAGE_BYTES = BM * BK_BYTES;
 constexpr int GEMM_THREADS = 192;
+constexpr int GEMM_TC_THREADS = 256;                          // gemm_tc_kernel: a second MMA issuer and a second producer
+constexpr int GEMM_BAR_BYTES = 8 * (3 * 8 + 4) + 512;         // barriers, TMEM address, bias of the tile's columns
 constexpr uint32_t WAIT_LIMIT = 1u << 20;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -122,10 +131,23 @@ __device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk
 // All of this thread's tile stores have finished READING shared memory (the global writes complete with the grid).
 __device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 
-// Barrier over every thread of every CTA in the cluster (release / acquire).
+// Barrier over every thread of every CTA in the cluster (release / acquire), in one piece or as its two halves.
+__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync_all() {
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    cluster_arrive();
+    cluster_wait();
+}
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t local, int rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local), "r"(rank));
+    return r;
+}
+// Bulk copy of `bytes` (a multiple of 16) from this CTA's shared memory into a cluster CTA's, counted on the barrier there.
+__device__ __forceinline__ void bulk_push(uint32_t remote_dst, uint32_t src, uint32_t bytes, uint32_t remote_bar) {
+    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(remote_dst), "r"(src), "r"(bytes), "r"(remote_bar) : "memory");
 }
 
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -174,14 +196,35 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+__device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, uint32_t (&r)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr)
+        : "memory");
+}
+__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
+// One lane of a converged warp, picked by the hardware: code under this predicate may keep its operands in uniform registers.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
+
 struct GemmDev {
     unsigned long long* stamp;        // device-clock stamps of this launch, or null
     float* D;
     const float* bias;
     const float* addend;
     long long ldd, strideD;
-    int M, N, Kd, BN, act, tmem_cols, splits, stages, prefill;
+    int M, N, Kd, BN, act, tmem_cols, splits, stages, issuers;
+    int rows;                         // rows of A per tile, at most 128
+    int z_tiles;                      // output map: 0 = {N, M, batch}; else {N, rows, tiles} with this many tiles per batch entry
+    uint32_t bar_off;                 // byte offset (from the aligned base) of the barriers
     int tma_out;                      // 0: plain stores; else the column width (16 or 32) of the staged tiles stored by TMA
+    uint32_t recv_off;                // splits > 1: byte offset (from the aligned base) of the received partial rows
     uint32_t stage_off;               // byte offset (from the aligned base) of the dedicated staging tile; 0 = the idle ring
     // implicit im2col (A is the NHWC activation itself): 0 = off
     int ic_on, ic_C, ic_cblk, ic_S, ic_OW, ic_stride, ic_pad;
@@ -273,33 +316,42 @@ template <int MODE> struct ModeTraits {
 };
 
 template <int MODE>
-__host__ __device__ constexpr uint32_t stage_bytes_of(int BN) {
+__host__ __device__ constexpr uint32_t stage_bytes_of(int BN, int rows = 128) {
     // staged TMA tiles (A: 128 rows x 128 B, B: BN rows x 128 B); mode 2 adds hi and lo bf16 tiles
     if (MODE == 3) return (uint32_t)(A_STAGE_BYTES + A_STAGE_BYTES / 2 + BN * 64);   // fp32 A, bf16 A, bf16 B (32 elements per row)
-    return (uint32_t)(A_STAGE_BYTES + BN * BK_BYTES) * (MODE == 2 ? 2u : 1u);
+    if (MODE == 2) return 2u * (uint32_t)(A_STAGE_BYTES + BN * BK_BYTES);
+    return (((uint32_t)rows * BK_BYTES + 1023u) & ~1023u) + (uint32_t)(BN * BK_BYTES);
+}
+// Modes 0 and 1 keep only the `rows` rows of A that are loaded (the MMA's other rows read whatever follows and are never
+// written out); the conversion modes keep room for all 128.
+template <int MODE>
+__host__ __device__ constexpr uint32_t a_stage_of(int rows) {
+    return MODE >= 2 ? (uint32_t)A_STAGE_BYTES : ((uint32_t)rows * BK_BYTES + 1023u) & ~1023u;
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(GEMM_THREADS)
+__global__ void __launch_bounds__(GEMM_TC_THREADS, 3)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmD, const __grid_constant__ CUtensorMap tmAdd, const GemmDev g) {
     extern __shared__ uint8_t smem_raw[];
-    pdl_trigger();
     const int STAGES = g.stages;                              // depth of the shared-memory ring (2..8)
     constexpr int MAXS = 8;
     constexpr int BKE = ModeTraits<MODE>::BKE;
     const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const int BN = g.BN;
     const uint32_t b_stage_bytes = (uint32_t)BN * BK_BYTES;
-    const uint32_t tma_bytes = A_STAGE_BYTES + (MODE == 3 ? (uint32_t)BN * 64u : b_stage_bytes);
-    const uint32_t stage_bytes = stage_bytes_of<MODE>(BN);
-    const uint32_t bars = sbase + STAGES * stage_bytes;       // full[S], empty[S], conv[S], tmem_full, holder
+    const uint32_t b_bytes = MODE == 3 ? (uint32_t)BN * 64u : b_stage_bytes, a_bytes = (uint32_t)g.rows * BK_BYTES;
+    const uint32_t a_stage = a_stage_of<MODE>(g.rows);
+    const uint32_t stage_bytes = stage_bytes_of<MODE>(BN, g.rows);
+    const uint32_t bars = sbase + g.bar_off;                  // behind the ring       // full[S], empty[S], conv[S], tmem_full, holder
     auto full_bar = [&](int s) { return bars + 8u * s; };
     auto empty_bar = [&](int s) { return bars + 8u * (MAXS + s); };
     auto conv_bar = [&](int s) { return bars + 8u * (2 * MAXS + s); };
     const uint32_t tmem_full_bar = bars + 8u * (3 * MAXS);
     const uint32_t holder = bars + 8u * (3 * MAXS + 1);
     const uint32_t addend_bar = bars + 8u * (3 * MAXS + 2);
+    const uint32_t recv_bar = bars + 8u * (3 * MAXS + 3);
+    const uint32_t sbias = bars + 8u * (3 * MAXS + 4);        // the tile's BN bias values (zeros without a bias)
     // Write-out through shared memory (g.tma_out): the tile is staged as [column chunk][warp quarter] sub-tiles of
     // 32 rows x CW columns in the swizzled layout of the output tensor map and stored by TMA.  With a residual
     // addend the sub-tiles live in their own region and the addend is loaded INTO them while the K loop runs, so
@@ -307,28 +359,36 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const int CW = g.tma_out;
     const uint32_t chunk_bytes = 32u * (uint32_t)CW * 4u;
     const uint32_t stg0 = sbase + g.stage_off;
+    const int quarters = (g.rows + 31) >> 5;                  // 32-row sub-tiles of the tile
+    const int y0 = g.z_tiles ? 0 : (int)blockIdx.x * g.rows;  // output map: first row and third coordinate of the tile
     volatile uint32_t* holder_ptr = reinterpret_cast<volatile uint32_t*>(smem_raw + (holder - smem_u32(smem_raw)));
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     // blockIdx.z = batch * splits + split; the `splits` CTAs of one output tile form a thread-block
     // cluster, each reducing its own contiguous range of K blocks.
     const int splits = g.splits;
     const int sp = (int)blockIdx.z % splits, b = (int)blockIdx.z / splits;
-    const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
+    const int zd = g.z_tiles ? b * g.z_tiles + (int)blockIdx.x : b;
+    const int m0 = blockIdx.x * g.rows, n0 = blockIdx.y * BN;
     const int nkb_all = g.ic_on ? g.Kd : (g.Kd + BKE - 1) / BKE;  // implicit mode: Kd already counts K blocks
     const int kb0 = (nkb_all * sp) / splits;                  // K blocks number a few thousand at most: 32-bit is enough
     const int nkb = (nkb_all * (sp + 1)) / splits - kb0;
+    // Split K: rank `sp` of the cluster owns the tile's rows [sp * rows_per, ...); only rows that exist are reduced.
+    const int live = min(g.rows, g.M - m0);
+    const int rows_per = (live + splits - 1) / splits;
+    const int my_rows = max(0, min(rows_per, live - sp * rows_per));
 
     if (warp == 0 && lane == 0) {
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmB)) : "memory");
         for (int s = 0; s < STAGES; ++s) {
-            mbar_init(full_bar(s), 1);
+            mbar_init(full_bar(s), 2);
             mbar_init(empty_bar(s), 1);
             mbar_init(conv_bar(s), 128);
         }
-        mbar_init(tmem_full_bar, 1);
+        mbar_init(tmem_full_bar, (uint32_t)g.issuers);
         mbar_init(addend_bar, 1);
+        mbar_init(recv_bar, 1);
         if (CW) {
             asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmD)) : "memory");
             if (g.addend) asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmAdd)) : "memory");
@@ -355,63 +415,70 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         ic_fr = ic_tap / g.ic_S;
         ic_fs = ic_tap - ic_fr * g.ic_S;
     }
-    auto issue_stage = [&](int it, int s) {
-        const int kb = kb0 + it;
-        mbar_expect_tx(full_bar(s), tma_bytes);
+    auto issue_a = [&](int it, int s) {
+        mbar_expect_tx(full_bar(s), a_bytes);
         const uint32_t a_dst = sbase + s * stage_bytes;
         if (g.ic_on) {
-            // A comes straight from the activation: block `kb` is channel block ic_cb of tap (ic_fr, ic_fs)
+            // A comes straight from the activation: the block is channel block ic_cb of tap (ic_fr, ic_fs)
             tma_load_im2col_4d(a_dst, &tmA, ic_cb * BKE, ic_w0, ic_h0, 0, (uint16_t)ic_fs, (uint16_t)ic_fr, full_bar(s));
-            if constexpr (MODE == 3) {   // B: one box of four 8-element chunks x BN rows, staged after the fp32 and the bf16 A tile
-                tma_load_3d(a_dst + A_STAGE_BYTES + A_STAGE_BYTES / 2, &tmB, 0, n0, (ic_tap * g.ic_C + ic_cb * BKE) >> 3, full_bar(s));
-            } else {
-                tma_load_3d(a_dst + A_STAGE_BYTES, &tmB, ic_tap * g.ic_C + ic_cb * BKE, n0, b, full_bar(s));
-            }
             if (++ic_cb == g.ic_cblk) {
-                ic_cb = 0; ++ic_tap;
+                ic_cb = 0;
                 if (++ic_fs == g.ic_S) { ic_fs = 0; ++ic_fr; }
             }
         } else {
-            tma_load_3d(a_dst, &tmA, kb * BKE, m0, b, full_bar(s));
-            if constexpr (MODE == 3) {
-                tma_load_3d(a_dst + A_STAGE_BYTES + A_STAGE_BYTES / 2, &tmB, 0, n0, (kb * BKE) >> 3, full_bar(s));
-            } else {
-                tma_load_3d(a_dst + A_STAGE_BYTES, &tmB, kb * BKE, n0, b, full_bar(s));
-            }
+            tma_load_3d(a_dst, &tmA, (kb0 + it) * BKE, m0, b, full_bar(s));
         }
     };
-    // The producer fills the whole ring before the CTA-wide barrier: the first loads fly while
-    // TMEM is being allocated.  It only needs its own barrier initialisation and the previous
-    // kernel's results (pdl_wait).
-    const int prefill = g.prefill ? (nkb < STAGES ? nkb : STAGES) : 0;
-    if (warp == 0 && lane == 0) {
-        pdl_wait();
-        for (int it = 0; it < prefill; ++it) issue_stage(it, it);
-        if (CW && g.addend) {                                 // the residual tile, straight into the staging sub-tiles
-            const int nch = BN / CW;
-            mbar_expect_tx(addend_bar, (uint32_t)nch * 4u * chunk_bytes);
-            for (int j = 0; j < nch; ++j)
-                for (int q = 0; q < 4; ++q)
-                    tma_load_3d(stg0 + (uint32_t)(j * 4 + q) * chunk_bytes, &tmAdd, n0 + j * CW, m0 + q * 32, 0, addend_bar);
+    auto issue_b = [&](int it, int s) {
+        int q = (kb0 + it) * BKE;                             // the block's first position in the packed weight rows
+        if (g.ic_on) {
+            q = ic_tap * g.ic_C + ic_cb * BKE;
+            if (++ic_cb == g.ic_cblk) { ic_cb = 0; ++ic_tap; }
         }
-    }
+        mbar_expect_tx(full_bar(s), b_bytes);
+        const uint32_t b_dst = sbase + s * stage_bytes + a_stage;
+        // MODE 3: one box of four 8-element chunks x BN rows, staged after the fp32 and the bf16 A tile
+        if constexpr (MODE == 3) tma_load_3d(b_dst + A_STAGE_BYTES / 2, &tmB, 0, n0, q >> 3, full_bar(s));
+        else tma_load_3d(b_dst, &tmB, q, n0, b, full_bar(s));
+    };
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    if (splits > 1) {
+        if (threadIdx.x == 64 && my_rows) mbar_expect_tx(recv_bar, (uint32_t)(splits * my_rows * BN) * 4u);
+        __syncwarp();
+        cluster_arrive_relaxed();                             // this CTA's (fenced) barriers may be signalled from here on
+    }
     const uint32_t tmem_base = *holder_ptr;
     pdl_wait();                                               // set-up above overlaps the previous kernel's tail
+    pdl_trigger();
     if (threadIdx.x == 32) stamp_start(g.stamp);
 
-    bool epi_ok = false;
-    if (warp == 0) {
-        if (lane == 0) {
+    bool cluster_arrived = false;                             // the epilogue warps arrive early, in their own code
+    if (warp == 0 || warp == 7) {
+        // Producers.  A load costs the thread that issues it ~157 cycles whatever its size, which for one thread issuing both
+        // operands (314 cycles a K block) is more than the MMAs take: the activation's and the weights' loads come from a
+        // warp each, the residual tile from the weights' one (it has fewer bytes to wait for).
+        if (elect_one()) {
             bool ok = true;
-            int s = prefill == STAGES ? 0 : prefill;
-            uint32_t ph = prefill == STAGES ? 1u : 0u;
-            for (int it = prefill; it < nkb && ok; ++it) {
-                ok = mbar_wait(empty_bar(s), ph ^ 1u);
+            int s = 0;
+            uint32_t ph = 0;
+            const int first = min(nkb, STAGES);
+            for (int it = 0; it < nkb; ++it) {
+                if (it >= STAGES) ok = mbar_wait(empty_bar(s), ph ^ 1u);
                 if (!ok) break;
-                issue_stage(it, s);
+                if (warp == 0) {
+                    issue_a(it, s);
+                } else {
+                    issue_b(it, s);
+                    if (it == first - 1 && CW && g.addend) {  // straight into the staging sub-tiles
+                        const int nch = BN / CW;
+                        mbar_expect_tx(addend_bar, (uint32_t)(nch * quarters) * chunk_bytes);
+                        for (int j = 0; j < nch; ++j)
+                            for (int q = 0; q < quarters; ++q)
+                                tma_load_3d(stg0 + (uint32_t)(j * quarters + q) * chunk_bytes, &tmAdd, n0 + j * CW, y0 + q * 32, zd, addend_bar);
+                    }
+                }
                 if (++s == STAGES) { s = 0; ph ^= 1u; }
             }
             if (!ok) {
@@ -419,22 +486,30 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 for (int i = 0; i < 1000; ++i) __nanosleep(1000);   // let loads already in flight land
             }
         }
-    } else if (warp == 1) {
-        if (lane == 0) {
+        __syncwarp();
+        if (splits > 1) cluster_wait();
+    } else if (warp == 1 || warp == 6) {
+        // MMA issuers.  One thread that waits for a stage, issues its four MMAs into one accumulator and commits takes
+        // ~560 cycles a K block (device-clock probes), several times what the tensor pipe needs at these tile widths, so
+        // `g.issuers` warps take the K blocks in turn, each into an accumulator of its own; the epilogue adds them.
+        const int iss = warp == 1 ? 0 : warp - 5;
+        if (iss < g.issuers && elect_one()) {
             // instruction descriptor: fp32 accumulate, A/B format, both K-major, N, M = 128
             const uint32_t fmt = (MODE == 0) ? 2u : 1u;
             const uint32_t idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+            const uint32_t acc = tmem_base + (uint32_t)(iss * BN);
             bool ok = true;
-            int s = 0;
-            uint32_t ph = 0;
-            for (int it = 0; it < nkb; ++it, s = (s + 1 == STAGES ? 0 : s + 1), ph ^= (s == 0 ? 1u : 0u)) {
+            int s = iss % STAGES;
+            uint32_t ph = (uint32_t)(iss / STAGES) & 1u;
+            for (int it = iss; it < nkb; it += g.issuers) {
                 ok = mbar_wait((MODE == 2 || MODE == 3) ? conv_bar(s) : full_bar(s), ph);
                 if (!ok) break;
                 tc_fence_after();
+                const uint32_t first = it != iss ? 1u : 0u;     // 0: the accumulator's first MMA overwrites it
                 const uint32_t a_src = sbase + s * stage_bytes;
                 if constexpr (MODE == 2) {
                     // converted tiles follow the staged ones: A_hi, A_lo (8 KB each), B_hi, B_lo
-                    const uint32_t a_hi = a_src + tma_bytes, a_lo = a_hi + A_STAGE_BYTES / 2;
+                    const uint32_t a_hi = a_src + A_STAGE_BYTES + b_stage_bytes, a_lo = a_hi + A_STAGE_BYTES / 2;
                     const uint32_t b_hi = a_lo + A_STAGE_BYTES / 2, b_lo = b_hi + b_stage_bytes / 2;
                     const uint32_t lbo_a = BM * 16u, lbo_b = (uint32_t)BN * 16u;
 #pragma unroll
@@ -443,242 +518,265 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                         const uint64_t al = make_smem_desc_plain(a_lo + kk * 2 * lbo_a, lbo_a, 128);
                         const uint64_t bh = make_smem_desc_plain(b_hi + kk * 2 * lbo_b, lbo_b, 128);
                         const uint64_t bl = make_smem_desc_plain(b_lo + kk * 2 * lbo_b, lbo_b, 128);
-                        umma<true>(tmem_base, al, bh, idesc, (it | kk) ? 1u : 0u);   // small terms first
-                        umma<true>(tmem_base, ah, bl, idesc, 1u);
-                        umma<true>(tmem_base, ah, bh, idesc, 1u);
+                        umma<true>(acc, al, bh, idesc, kk ? 1u : first);   // small terms first
+                        umma<true>(acc, ah, bl, idesc, 1u);
+                        umma<true>(acc, ah, bh, idesc, 1u);
                     }
                 } else if constexpr (MODE == 3) {
                     const uint32_t a_bf = a_src + A_STAGE_BYTES, b_bf = a_bf + A_STAGE_BYTES / 2;
                     const uint32_t lbo_a = BM * 16u, lbo_b = (uint32_t)BN * 16u;
 #pragma unroll
                     for (int kk = 0; kk < 2; ++kk)             // 2 K-steps of 16 bf16 = 2 core matrices each
-                        umma<true>(tmem_base, make_smem_desc_plain(a_bf + kk * 2 * lbo_a, lbo_a, 128),
-                                   make_smem_desc_plain(b_bf + kk * 2 * lbo_b, lbo_b, 128), idesc, (it | kk) ? 1u : 0u);
+                        umma<true>(acc, make_smem_desc_plain(a_bf + kk * 2 * lbo_a, lbo_a, 128),
+                                   make_smem_desc_plain(b_bf + kk * 2 * lbo_b, lbo_b, 128), idesc, kk ? 1u : first);
                 } else {
                     const uint64_t adesc = make_smem_desc(a_src);
-                    const uint64_t bdesc = make_smem_desc(a_src + A_STAGE_BYTES);
+                    const uint64_t bdesc = make_smem_desc(a_src + a_stage);
 #pragma unroll
                     for (int kk = 0; kk < 4; ++kk)             // 4 MMAs of 32 bytes of K each
-                        umma<MODE == 1>(tmem_base, adesc + (uint64_t)(kk * 2), bdesc + (uint64_t)(kk * 2), idesc, (it | kk) ? 1u : 0u);
+                        umma<MODE == 1>(acc, adesc + (uint64_t)(kk * 2), bdesc + (uint64_t)(kk * 2), idesc, kk ? 1u : first);
                 }
                 umma_commit(empty_bar(s));
+                s += g.issuers;
+                while (s >= STAGES) { s -= STAGES; ph ^= 1u; }
             }
             if (ok) umma_commit(tmem_full_bar);
             else atomicExch(&g_device_status, (int)NNV_ERR_TIMEOUT);
         }
+        __syncwarp();
+        if (splits > 1) cluster_wait();
     } else {
-        bool ok = true;
-        if constexpr (MODE == 3) {
-            // warps 2-5 first round every staged fp32 A tile to bf16 (the weights arrive as bf16)
-            const int idx = (int)threadIdx.x - 64;              // 0..127: one row of A each
-            int s = 0;
-            uint32_t ph = 0;
-            for (int it = 0; it < nkb; ++it, s = (s + 1 == STAGES ? 0 : s + 1), ph ^= (s == 0 ? 1u : 0u)) {
-                ok = mbar_wait(full_bar(s), ph);
-                if (!ok) break;
-                const uint32_t a_src = sbase + s * stage_bytes;
-                convert_row_bf16(a_src, a_src + A_STAGE_BYTES, idx, BM);
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> visible to the MMA's reads
-                mbar_arrive(conv_bar(s));
+        // Epilogue warps.  A warp that has its scheduler to itself pays 5 - 30 cycles for every dependent instruction, so
+        // whatever does not need the accumulator -- indices, addresses, the bias -- is worked out before the wait for it.
+        const int quarter = warp & 3;                         // the TMEM lanes this warp may read
+        const int t = (int)threadIdx.x - 64;
+        uint8_t* const sm = smem_raw + (sbase - smem_u32(smem_raw));
+        const float bias = (g.bias && t < BN && n0 + t < g.N) ? __ldg(g.bias + n0 + t) : 0.f;
+        const int naccs = min(g.issuers, nkb);
+        const uint32_t tacc = tmem_base + ((uint32_t)(quarter * 32) << 16);
+        const float hi = g.act == 2 ? 6.f : INFINITY;
+        auto act4 = [&](float4& v) {
+            if (g.act) {
+                v.x = fminf(fmaxf(v.x, 0.f), hi); v.y = fminf(fmaxf(v.y, 0.f), hi);
+                v.z = fminf(fmaxf(v.z, 0.f), hi); v.w = fminf(fmaxf(v.w, 0.f), hi);
             }
-        }
-        if constexpr (MODE == 2) {
-            // warps 2-5 first convert every staged fp32 tile into its bf16 hi / lo tiles
-            const int idx = (int)threadIdx.x - 64;              // 0..127: one row of A (and of B) each
-            int s = 0;
-            uint32_t ph = 0;
-            for (int it = 0; it < nkb; ++it, s = (s + 1 == STAGES ? 0 : s + 1), ph ^= (s == 0 ? 1u : 0u)) {
-                ok = mbar_wait(full_bar(s), ph);
-                if (!ok) break;
-                const uint32_t a_src = sbase + s * stage_bytes;
-                const uint32_t a_hi = a_src + tma_bytes, a_lo = a_hi + A_STAGE_BYTES / 2;
-                const uint32_t b_hi = a_lo + A_STAGE_BYTES / 2, b_lo = b_hi + b_stage_bytes / 2;
-                convert_row(a_src, a_hi, a_lo, idx, BM);
-                if (idx < BN) convert_row(a_src + A_STAGE_BYTES, b_hi, b_lo, idx, BN);
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> visible to the MMA's reads
-                mbar_arrive(conv_bar(s));
-            }
-        }
-        ok = ok && mbar_wait(tmem_full_bar, 0);
-        tc_fence_after();
-        if (!ok) {
-            if (lane == 0) atomicExch(&g_device_status, (int)NNV_ERR_TIMEOUT);
-        } else if (splits == 1 && CW) {
-            // lane = one accumulator row; per column chunk: TMEM -> registers -> (+ bias, + addend from the staging
-            // sub-tile, activation) -> staging sub-tile -> one TMA store per warp and chunk
-            const int quarter = warp & 3;
-            const int nch = BN / CW;
-            bool aok = true;
-            if (g.addend) aok = mbar_wait(addend_bar, 0);
-            if (!aok) {
-                if (lane == 0) atomicExch(&g_device_status, (int)NNV_ERR_TIMEOUT);
+        };
+        // 16 accumulator columns of this lane's row, the issuers' accumulators added in order
+        auto acc16 = [&](int c0, float (&v)[16]) {
+            uint32_t r[16];
+            tmem_ld16_nowait(tacc + (uint32_t)c0, r);
+            if (naccs > 1) {
+                uint32_t q[16];
+                tmem_ld16_nowait(tacc + (uint32_t)(BN + c0), q);
+                tmem_wait_ld();
+#pragma unroll
+                for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]) + __uint_as_float(q[i]);
             } else {
-                const bool row_live = m0 + quarter * 32 < g.M;
-                for (int j = 0; j < nch; ++j) {
-                    const uint32_t buf = stg0 + (uint32_t)(j * 4 + quarter) * chunk_bytes;
-                    const uint32_t rowa = buf + (uint32_t)lane * (uint32_t)CW * 4u;
-                    const int nbase = n0 + j * CW;
+                tmem_wait_ld();
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        if (h * 16 >= CW) break;
-                        uint32_t r[16];
-                        tmem_ld16(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(j * CW + h * 16), r);
+                for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+            }
+        };
+        bool ok = true;
+        if constexpr (MODE == 2 || MODE == 3) {
+            // round every staged fp32 tile first: MODE 3 A to bf16 (the weights arrive as bf16), MODE 2 both
+            // operands into their bf16 hi / lo tiles
+            int s = 0;
+            uint32_t ph = 0;
+            for (int it = 0; it < nkb; ++it, s = (s + 1 == STAGES ? 0 : s + 1), ph ^= (s == 0 ? 1u : 0u)) {
+                ok = mbar_wait(full_bar(s), ph);
+                if (!ok) break;
+                const uint32_t a_src = sbase + s * stage_bytes;
+                if constexpr (MODE == 3) {
+                    if (t < g.rows) convert_row_bf16(a_src, a_src + A_STAGE_BYTES, t, BM);
+                } else {
+                    const uint32_t a_hi = a_src + A_STAGE_BYTES + b_stage_bytes, a_lo = a_hi + A_STAGE_BYTES / 2;
+                    const uint32_t b_hi = a_lo + A_STAGE_BYTES / 2, b_lo = b_hi + b_stage_bytes / 2;
+                    if (t < g.rows) convert_row(a_src, a_hi, a_lo, t, BM);
+                    if (t < BN) convert_row(a_src + A_STAGE_BYTES, b_hi, b_lo, t, BN);
+                }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> visible to the MMA's reads
+                mbar_arrive(conv_bar(s));
+            }
+        }
+        float* const s_bias = reinterpret_cast<float*>(sm + (sbias - sbase));
+        if (t < BN) s_bias[t] = bias;
+        asm volatile("barrier.sync 1, 128;" ::: "memory");
+        auto wait_acc = [&]() {
+            ok = ok && mbar_wait(tmem_full_bar, 0);
+            tc_fence_after();
+            if (!ok && lane == 0) atomicExch(&g_device_status, (int)NNV_ERR_TIMEOUT);
+            ok = __all_sync(0xffffffffu, ok);
+        };
+        if (splits == 1 && CW) {
+            // lane = one accumulator row; per 16 columns: TMEM -> registers -> (+ bias, + addend from the staging sub-tile,
+            // activation) -> staging sub-tile, and per sub-tile one TMA store per warp
+            const uint32_t swz = CW == 32 ? (uint32_t)(lane & 7) : (uint32_t)((lane >> 1) & 3);
+            const bool row_live = quarter * 32 < live;
+            uint8_t* row0 = sm + g.stage_off + (uint32_t)quarter * chunk_bytes + (uint32_t)lane * (uint32_t)CW * 4u;
+            wait_acc();
+            if (ok && g.addend) ok = mbar_wait(addend_bar, 0);
+            ok = __all_sync(0xffffffffu, ok);
+            if (ok && row_live) {
+#pragma unroll 1
+                for (int c0 = 0; c0 < BN; c0 += 16) {
+                    float v[16];
+                    acc16(c0, v);
+                    const uint32_t half = CW == 32 ? (uint32_t)(c0 >> 2) & 4u : 0u;      // 16-byte word of the sub-tile's row
+                    float4 o[4];
 #pragma unroll
-                        for (int c4 = 0; c4 < 4; ++c4) {
-                            const int c = h * 4 + c4;                       // 16-byte chunk of the row
-                            const int n = nbase + c * 4;
-                            const uint32_t sw = (CW == 32) ? (uint32_t)(c ^ (lane & 7)) : (uint32_t)(c ^ ((lane >> 1) & 3));
-                            const uint32_t addr = rowa + sw * 16u;
-                            float4 v = make_float4(__uint_as_float(r[c4 * 4]), __uint_as_float(r[c4 * 4 + 1]),
-                                                   __uint_as_float(r[c4 * 4 + 2]), __uint_as_float(r[c4 * 4 + 3]));
-                            if (g.bias && n < g.N) {
-                                const float4 bb = __ldg(reinterpret_cast<const float4*>(g.bias + n));
-                                v.x += bb.x; v.y += bb.y; v.z += bb.z; v.w += bb.w;
-                            }
-                            if (g.addend) {
-                                float4 aa;
-                                asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(aa.x), "=f"(aa.y), "=f"(aa.z), "=f"(aa.w) : "r"(addr));
-                                v.x += aa.x; v.y += aa.y; v.z += aa.z; v.w += aa.w;
-                            }
-                            v.x = act_fn(v.x, g.act); v.y = act_fn(v.y, g.act); v.z = act_fn(v.z, g.act); v.w = act_fn(v.w, g.act);
-                            asm volatile("st.shared.v4.f32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+                    for (int c = 0; c < 4; ++c) {
+                        const float4 bb = *reinterpret_cast<const float4*>(s_bias + c0 + c * 4);
+                        o[c] = make_float4(v[c * 4] + bb.x, v[c * 4 + 1] + bb.y, v[c * 4 + 2] + bb.z, v[c * 4 + 3] + bb.w);
+                    }
+                    if (g.addend) {
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) {
+                            const float4 aa = *reinterpret_cast<const float4*>(row0 + (((half + (uint32_t)c) ^ swz) << 4));
+                            o[c].x += aa.x; o[c].y += aa.y; o[c].z += aa.z; o[c].w += aa.w;
                         }
                     }
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> visible to the TMA's reads
-                    __syncwarp();
-                    if (lane == 0 && row_live && nbase < g.N) {
-                        tma_store_3d(&tmD, buf, nbase, m0 + quarter * 32, b);
-                        tma_store_commit();
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        act4(o[c]);
+                        *reinterpret_cast<float4*>(row0 + (((half + (uint32_t)c) ^ swz) << 4)) = o[c];
+                    }
+                    if (CW == 16 || half) {                   // the sub-tile is complete
+                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> visible to the TMA's reads
+                        __syncwarp();
+                        if (lane == 0 && row_live && n0 + c0 + 16 - CW < g.N) {
+                            tma_store_3d(&tmD, smem_u32(row0), n0 + c0 + 16 - CW, y0 + quarter * 32, zd);
+                            tma_store_commit();
+                        }
+                        row0 += (uint32_t)quarters * chunk_bytes;
                     }
                 }
                 if (lane == 0) tma_store_wait_read();
             }
         } else if (splits == 1) {
-            const int quarter = warp & 3;                     // TMEM lanes this warp may read
-            const int m = m0 + quarter * 32 + lane;
-            float* drow = g.D + (long long)b * g.strideD + (long long)m * g.ldd;
-            const float* arow = g.addend ? g.addend + (long long)m * g.ldd : nullptr;
-            const bool vec = ((g.ldd & 3) == 0) && ((g.N & 3) == 0) && ((reinterpret_cast<uintptr_t>(g.D) & 15) == 0) &&
-                             (!g.addend || (reinterpret_cast<uintptr_t>(g.addend) & 15) == 0) &&
-                             (!g.bias || (reinterpret_cast<uintptr_t>(g.bias) & 15) == 0);
-            for (int c0 = 0; c0 < BN; c0 += 16) {
-                uint32_t r[16];
-                tmem_ld16(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c0, r);
-                if (m >= g.M) continue;
-                const int n = n0 + c0;
-                if (vec) {
-#pragma unroll
-                    for (int j = 0; j < 16; j += 4) {
-                        if (n + j >= g.N) break;
-                        float4 v = make_float4(__uint_as_float(r[j]), __uint_as_float(r[j + 1]), __uint_as_float(r[j + 2]),
-                                               __uint_as_float(r[j + 3]));
-                        if (g.bias) {
-                            const float4 bb = __ldg(reinterpret_cast<const float4*>(g.bias + n + j));
-                            v.x += bb.x; v.y += bb.y; v.z += bb.z; v.w += bb.w;
-                        }
-                        if (arow) {
-                            const float4 aa = __ldg(reinterpret_cast<const float4*>(arow + n + j));
-                            v.x += aa.x; v.y += aa.y; v.z += aa.z; v.w += aa.w;
-                        }
-                        v.x = act_fn(v.x, g.act); v.y = act_fn(v.y, g.act); v.z = act_fn(v.z, g.act); v.w = act_fn(v.w, g.act);
-                        *reinterpret_cast<float4*>(drow + n + j) = v;
-                    }
-                } else {
+            wait_acc();
+            if (ok) {
+                const int m = m0 + quarter * 32 + lane;
+                float* drow = g.D + (long long)b * g.strideD + (long long)m * g.ldd;
+                const float* arow = g.addend ? g.addend + (long long)m * g.ldd : nullptr;
+                for (int c0 = 0; c0 < BN; c0 += 16) {
+                    float v[16];
+                    acc16(c0, v);
+                    if (quarter * 32 + lane >= live) continue;
 #pragma unroll
                     for (int j = 0; j < 16; ++j) {
-                        if (n + j < g.N) {
-                            float v = __uint_as_float(r[j]);
-                            if (g.bias) v += __ldg(g.bias + n + j);
-                            if (arow) v += __ldg(arow + n + j);
-                            drow[n + j] = act_fn(v, g.act);
+                        const int n = n0 + c0 + j;
+                        if (n < g.N) {
+                            float o = v[j] + s_bias[c0 + j];
+                            if (arow) o += __ldg(arow + n);
+                            drow[n] = act_fn(o, g.act);
                         }
                     }
                 }
             }
         } else {
-            epi_ok = true;
-            // park this CTA's (partial) tile in its own shared memory (the stage ring is idle by now):
-            // P[row][col], row pitch BN + 4 words
-            const int quarter = warp & 3;
-            const int row = quarter * 32 + lane;
-            const uint32_t prow = sbase + (uint32_t)row * (uint32_t)(BN + 4) * 4u;
-            for (int c0 = 0; c0 < BN; c0 += 16) {
-                uint32_t r[16];
-                tmem_ld16(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c0, r);
-#pragma unroll
-                for (int j = 0; j < 16; j += 4)
-                    asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(prow + (uint32_t)(c0 + j) * 4u), "r"(r[j]),
-                                 "r"(r[j + 1]), "r"(r[j + 2]), "r"(r[j + 3]) : "memory");
+            // Split K, sender: park the partial tile in the stage ring (idle by then) as rows of BN words, the 16-byte words
+            // of a row rotated by its index so that the lanes' stores meet different banks, and let the copy engine push
+            // every owner its rows of this warp's 32.  Owner: the rows arrive from every CTA of the cluster (its own
+            // included); they are added in rank order (a fixed order: the result does not depend on timing), bias /
+            // residual / activation are applied and row-contiguous 128-bit words are stored.
+            const int nch = BN / 4, r0 = sp * rows_per, q0 = quarter * 32;
+            uint8_t* const prow = sm + (uint32_t)(q0 + lane) * (uint32_t)BN * 4u;
+            int pos = (q0 + lane) % nch;
+            const int a0 = max(q0, lane * rows_per), a1 = min(min(q0 + 32, live), (lane + 1) * rows_per);
+            const bool sends = lane < splits && a1 > a0;
+            uint32_t push_dst = 0, push_bar = 0;
+            if (sends) {
+                push_dst = cluster_addr(sbase + g.recv_off + (uint32_t)((r0 + a0 - lane * rows_per) * BN) * 4u, lane);
+                push_bar = cluster_addr(recv_bar, lane);
             }
+            const bool vec = ((g.ldd & 3) == 0) && ((g.N & 3) == 0) && ((reinterpret_cast<uintptr_t>(g.D) & 15) == 0) &&
+                             (!g.addend || (reinterpret_cast<uintptr_t>(g.addend) & 15) == 0);
+            // thread t walks the (row, 4-column group) grid of its CTA's rows in steps of 128
+            const int qstep = 128 / nch, rstep = 128 - qstep * nch;
+            int rr = t / nch, cc = t - rr * nch, rot = (r0 + rr) % nch;
+            const int rot_step = qstep % nch;
+            const uint8_t* const recv = sm + g.recv_off;
+            const uint32_t part_stride = (uint32_t)(rows_per * BN) * 4u;
+            float* const dbase = g.D + (long long)b * g.strideD + (long long)(m0 + r0) * g.ldd + n0;
+            const float* const abase = g.addend ? g.addend + (long long)(m0 + r0) * g.ldd + n0 : nullptr;
+            cluster_wait();                                   // every CTA's barriers are initialised
+            wait_acc();
+            if (ok && q0 < live) {
+#pragma unroll 1
+                for (int c0 = 0; c0 < BN; c0 += 16) {
+                    float v[16];
+                    acc16(c0, v);
+#pragma unroll
+                    for (int j = 0; j < 16; j += 4) {
+                        if (q0 + lane < live) *reinterpret_cast<float4*>(prow + pos * 16) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+                        pos = pos + 1 == nch ? 0 : pos + 1;
+                    }
+                }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> visible to the bulk copies
+                __syncwarp();
+                if (sends) bulk_push(push_dst, sbase + (uint32_t)(a0 * BN) * 4u, (uint32_t)((a1 - a0) * BN) * 4u, push_bar);
+            }
+            int total = my_rows * nch;
+            if (my_rows && !mbar_wait(recv_bar, 0)) {
+                if (lane == 0) atomicExch(&g_device_status, (int)NNV_ERR_TIMEOUT);
+                total = 0;
+            }
+            __syncwarp();
+            cluster_arrive_relaxed();                         // this CTA's rows have arrived: their senders may leave
+            cluster_arrived = true;
+            auto reduce = [&](auto nsplits) {
+                constexpr int NS = decltype(nsplits)::value;
+#pragma unroll 2
+                for (int idx = t; idx < total; idx += 128) {
+                    const int p = cc + rot >= nch ? cc + rot - nch : cc + rot;
+                    const uint8_t* src = recv + (uint32_t)(rr * BN) * 4u + (uint32_t)p * 16u;
+                    constexpr int NB = NS < 8 ? NS : 8;       // loads in flight
+                    float4 v[NB];
+#pragma unroll
+                    for (int rk = 0; rk < NB; ++rk) v[rk] = *reinterpret_cast<const float4*>(src + rk * part_stride);
+                    float4 o = *reinterpret_cast<const float4*>(s_bias + cc * 4);
+                    const int n = cc * 4;
+                    const long long off = (long long)rr * g.ldd + n;
+                    float4 a = v[0];
+#pragma unroll
+                    for (int rk = 1; rk < NB; ++rk) { a.x += v[rk].x; a.y += v[rk].y; a.z += v[rk].z; a.w += v[rk].w; }
+                    if constexpr (NS > 8) {
+#pragma unroll
+                        for (int rk = 0; rk < 8; ++rk) v[rk] = *reinterpret_cast<const float4*>(src + (rk + 8) * part_stride);
+#pragma unroll
+                        for (int rk = 0; rk < 8; ++rk) { a.x += v[rk].x; a.y += v[rk].y; a.z += v[rk].z; a.w += v[rk].w; }
+                    }
+                    o.x += a.x; o.y += a.y; o.z += a.z; o.w += a.w;
+                    if (n0 + n < g.N) {
+                        if (vec) {
+                            if (abase) {
+                                const float4 aa = __ldg(reinterpret_cast<const float4*>(abase + off));
+                                o.x += aa.x; o.y += aa.y; o.z += aa.z; o.w += aa.w;
+                            }
+                            act4(o);
+                            *reinterpret_cast<float4*>(dbase + off) = o;
+                        } else {
+                            const float vv[4] = {o.x, o.y, o.z, o.w};
+                            for (int j = 0; j < 4 && n0 + n + j < g.N; ++j)
+                                dbase[off + j] = act_fn(abase ? vv[j] + __ldg(abase + off + j) : vv[j], g.act);
+                        }
+                    }
+                    rr += qstep; cc += rstep; rot += rot_step;
+                    if (cc >= nch) { cc -= nch; ++rr; ++rot; }
+                    if (rot >= nch) rot -= nch;
+                }
+            };
+            if (splits == 16) reduce(std::integral_constant<int, 16>());
+            else if (splits == 8) reduce(std::integral_constant<int, 8>());
+            else if (splits == 4) reduce(std::integral_constant<int, 4>());
+            else reduce(std::integral_constant<int, 2>());
         }
     }
     __syncwarp();
-    {
-        // Split-K write-out.  Every CTA of the cluster has parked its partial tile in shared memory;
-        // CTA `sp` sums rows [sp*128/splits, (sp+1)*128/splits) over the cluster through distributed
-        // shared memory in rank order (a fixed order: the result does not depend on timing), then
-        // applies bias / residual / activation and stores row-contiguous 128-bit words.  The
-        // cluster barriers are reached by every thread on every path.
-        if (splits > 1) cluster_sync_all();
-        if (splits > 1 && warp >= 2 && g_device_status == 0) {
-            const int t = (int)threadIdx.x - 64;
-            // only the rows of the tile that exist are reduced, shared evenly by the cluster's CTAs
-            const int live = min(BM, g.M - m0);
-            const int rows_per = (live + splits - 1) / splits, r0 = sp * rows_per;
-            const int c4n = BN / 4;
-            const bool vec = ((g.ldd & 3) == 0) && ((g.N & 3) == 0) && ((reinterpret_cast<uintptr_t>(g.D) & 15) == 0) &&
-                             (!g.addend || (reinterpret_cast<uintptr_t>(g.addend) & 15) == 0) &&
-                             (!g.bias || (reinterpret_cast<uintptr_t>(g.bias) & 15) == 0);
-            // Thread t walks the (row, 4-column group) grid in steps of 128 without divisions.  The loop
-            // is kept small on purpose (no unrolling): each CTA runs it once, and instruction fetch of
-            // cold code costs more here than the arithmetic.
-            const int total = max(0, min(rows_per, live - r0)) * c4n;
-            const int qstep = 128 / c4n, rstep = 128 - qstep * c4n;
-            int row = r0 + t / c4n, col4 = t % c4n;
-            float* const dbase = g.D + (long long)b * g.strideD;
-#pragma unroll 1
-            for (int idx = t; idx < total; idx += 128) {
-                const int rr = row, cc = col4 * 4;
-                row += qstep; col4 += rstep;
-                if (col4 >= c4n) { col4 -= c4n; ++row; }
-                const uint32_t local = sbase + ((uint32_t)rr * (uint32_t)(BN + 4) + (uint32_t)cc) * 4u;
-                // all remote loads are issued before the first is consumed, so their latencies overlap
-                float4 v[8];
-#pragma unroll
-                for (int rk = 0; rk < 8; ++rk) {
-                    if (rk < splits) {
-                        uint32_t remote;
-                        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(rk));
-                        asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v[rk].x), "=f"(v[rk].y), "=f"(v[rk].z), "=f"(v[rk].w) : "r"(remote));
-                    }
-                }
-                float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-                for (int rk = 0; rk < 8; ++rk)
-                    if (rk < splits) { acc.x += v[rk].x; acc.y += v[rk].y; acc.z += v[rk].z; acc.w += v[rk].w; }
-                const int m = m0 + rr, n = n0 + cc;
-                if (m >= g.M || n >= g.N) continue;
-                float* drow = dbase + (long long)m * g.ldd;
-                const float* arow = g.addend ? g.addend + (long long)m * g.ldd : nullptr;
-                float vv[4] = {acc.x, acc.y, acc.z, acc.w};
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    if (vec || n + j < g.N) {
-                        if (g.bias) vv[j] += __ldg(g.bias + n + j);
-                        if (arow) vv[j] += __ldg(arow + n + j);
-                        vv[j] = act_fn(vv[j], g.act);
-                    }
-                }
-                if (vec) {
-                    *reinterpret_cast<float4*>(drow + n) = make_float4(vv[0], vv[1], vv[2], vv[3]);
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        if (n + j < g.N) drow[n + j] = vv[j];
-                }
-            }
-        }
-        if (splits > 1) cluster_sync_all();                   // nobody leaves while its tile may still be read
+    if (splits > 1) {
+        if (!cluster_arrived) cluster_arrive_relaxed();
+        cluster_wait();                                       // nobody leaves while its rows may still be on their way
     }
     tc_fence_before();
     __syncthreads();
@@ -736,7 +834,7 @@ nnv_status_t encode_operand(CUtensorMap* map, const void* base, bool bf16, int K
 // 3-D map over the fp32 output (or the residual addend, same geometry): dims {N, M, batch}, boxes of
 // `cw` columns (32 with the 128-byte swizzle, 16 with the 64-byte one) x 32 rows.
 nnv_status_t encode_output(CUtensorMap* map, const void* base, int N, int M, int batch, int64_t ld, int64_t batch_stride, int cw) {
-    cuuint64_t dims[3] = {(cuuint64_t)N, (cuuint64_t)M, (cuuint64_t)batch};
+    cuuint64_t dims[3] = {(cuuint64_t)N, (cuuint64_t)M, (cuuint64_t)batch};    // or {N, rows of a tile, tiles}
     cuuint64_t strides[2] = {(cuuint64_t)(ld * 4), (cuuint64_t)(batch_stride * 4)};
     cuuint32_t box[3] = {(cuuint32_t)cw, 32, 1};
     cuuint32_t estr[3] = {1, 1, 1};
@@ -747,9 +845,9 @@ nnv_status_t encode_output(CUtensorMap* map, const void* base, int N, int M, int
     return NNV_OK;
 }
 
-// 4-D im2col map over an NHWC fp32 activation {C, W, H, 1}: 32 channels x 128 output pixels per load.
+// 4-D im2col map over an NHWC fp32 activation {C, W, H, 1}: 32 channels x `pixels` output pixels per load.
 nnv_status_t encode_im2col_operand(CUtensorMap* map, const void* base, int C, int H, int W, int R, int S, int stride,
-                                   int pad) {
+                                   int pad, int pixels) {
     NNV_REQUIRE(g_encode_im2col != nullptr, NNV_ERR_CUDA, "cuTensorMapEncodeIm2col is not available from this driver");
     NNV_REQUIRE((reinterpret_cast<uintptr_t>(base) & 15) == 0 && (C % 4) == 0, NNV_ERR_INVALID_ARG,
                 "implicit-GEMM activation must be 16-byte aligned with C a multiple of 4");
@@ -759,7 +857,7 @@ nnv_status_t encode_im2col_operand(CUtensorMap* map, const void* base, int C, in
     int upper[2] = {pad - (S - 1), pad - (R - 1)};
     cuuint32_t estr[4] = {1, (cuuint32_t)stride, (cuuint32_t)stride, 1};
     CUresult r = g_encode_im2col(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<void*>(base), dims, strides, lower,
-                                 upper, 32, BM, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                                 upper, 32, pixels, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                                  CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     NNV_REQUIRE(r == CUDA_SUCCESS, NNV_ERR_CUDA, "cuTensorMapEncodeIm2col failed with code %d", (int)r);
     return NNV_OK;
@@ -849,6 +947,59 @@ bool pick_conv_tiling(int C, int H, int W, int N, int bf16, ConvTiling* out) {
     return found;
 }
 
+uint32_t gemm_stage_bytes(int mode, int bn, int rows) {
+    return mode == GEMM_X3 ? stage_bytes_of<2>(bn) : mode == GEMM_BF16_CVT ? stage_bytes_of<3>(bn) : stage_bytes_of<0>(bn, rows);
+}
+
+// Rows of A per tile.  As few 128-row tiles as hold M, of equal height when they divide M (7 x 7 and 14 x 14 grids: one
+// tile of 49, two of 98): rows that do not exist would fill shared memory all the same.
+int gemm_rows(int M) {
+    const int tiles = ceil_div(M, BM);
+    return M % tiles == 0 ? M / tiles : BM;
+}
+
+// Ring depth: 8 stages when every CTA has an SM to itself (a lone CTA needs that many loads in flight on weights that come
+// cold from HBM), 4 when several share one, and no more than the K blocks a CTA walks: the shared memory left over lets
+// the next kernel's CTAs in early (warm ResNet-50-shaped inference 426 -> 415 us).
+int gemm_ring(int mode, int bn, int rows, long long ctas, int nkb) {
+    const int most = mode == GEMM_X3 ? 3 : (ctas <= 148 && 8u * gemm_stage_bytes(mode, bn, rows) <= 200u * 1024u) ? 8 : 4;
+    return std::max(2, std::min(most, nkb));
+}
+
+// Tiling of gemm_tc_kernel: fixed cost + waves x (K blocks per CTA x time per block + write-out).  A K block costs a CTA four
+// MMAs of ~82 cycles whatever BN <= 128 is, or the fill of its shared memory (per SM, and from L2 over all SMs); a split
+// adds the pushes of the partial rows.  Constants (microseconds) fitted to a sweep of every BN and split over the 101 GEMM
+// layer shapes of the ResNet / MobileNetV2 / VGG configurations at several resolutions, chained launches: the chosen
+// tilings are 0.05 us a launch above the best measured ones on average.
+struct GemmTiling { int BN, splits; };
+GemmTiling pick_gemm_tiling(int mode, int M, int N, int batch, int nkb) {
+    const int m_tiles = ceil_div(M, BM), rows = gemm_rows(M);
+    GemmTiling best{16, 1};
+    double best_t = 1e30;
+    for (int bn = 16; bn <= std::min(128, ceil_div(N, 16) * 16); bn += bn < 64 ? 16 : 32) {
+        const double kb_bytes = (double)(rows * BK_BYTES + bn * BK_BYTES);
+        for (int sp = 1; sp <= 16 && sp <= nkb; sp *= 2) {
+            const long long ctas = (long long)m_tiles * ceil_div(N, bn) * batch * sp;
+            const int nk = ceil_div(nkb, sp), ring = gemm_ring(mode, bn, rows, ctas, nk);
+            int tmem = 32;
+            while (tmem < 2 * bn) tmem *= 2;
+            const double smem = 2048.0 + (double)ring * gemm_stage_bytes(mode, bn, rows) + (sp > 1 ? 4.0 * rows * bn : 0.0);
+            const int occ = std::max(1, std::min({3, (int)(226.0 * 1024.0 / smem), 512 / tmem}));
+            // whole clusters must find free SMs inside one GPC: how many CTAs fit with one, two and three to an SM (as
+            // cudaOccupancyMaxActiveClusters reports)
+            static const int cap[5][3] = {{148, 296, 444}, {148, 296, 444}, {132, 284, 416}, {120, 264, 384}, {112, 224, 336}};
+            const long long slots = cap[sp == 16 ? 4 : sp == 8 ? 3 : sp == 4 ? 2 : sp - 1][occ - 1];
+            const double waves = (double)((ctas + slots - 1) / slots);
+            const double res = (double)std::min<long long>(occ, (ctas + 147) / 148);
+            const double kb = std::max({0.146 * res, kb_bytes * res / 108e3, kb_bytes * (double)std::min(ctas, slots) / 10.9e6});
+            const double split = sp > 1 ? 0.26 + 0.021 * std::log2((double)sp) + 1.22e-4 * bn * rows * res : 0.0;
+            const double t = 1.87 + waves * (nk * kb + 0.40 + 0.0093 * bn + split);
+            if (t < best_t - 1e-9) { best_t = t; best = GemmTiling{bn, sp}; }
+        }
+    }
+    return best;
+}
+
 std::once_flag g_attr_once;
 
 }  // namespace
@@ -856,10 +1007,14 @@ std::once_flag g_attr_once;
 nnv_status_t gemm_tc_init() {
     NNV_TRY(get_encoder());
     std::call_once(g_attr_once, [] {
-        cudaFuncSetAttribute(gemm_tc_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
-        cudaFuncSetAttribute(gemm_tc_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
-        cudaFuncSetAttribute(gemm_tc_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
-        cudaFuncSetAttribute(gemm_tc_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
+        cudaFuncSetAttribute(gemm_tc_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
+        cudaFuncSetAttribute(gemm_tc_kernel<0>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        cudaFuncSetAttribute(gemm_tc_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
+        cudaFuncSetAttribute(gemm_tc_kernel<1>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        cudaFuncSetAttribute(gemm_tc_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
+        cudaFuncSetAttribute(gemm_tc_kernel<2>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        cudaFuncSetAttribute(gemm_tc_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
+        cudaFuncSetAttribute(gemm_tc_kernel<3>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         cudaFuncSetAttribute(conv3x3_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
         cudaFuncSetAttribute(gemm_sp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
         cudaFuncSetAttribute(conv3x3_tc_persistent_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
@@ -932,13 +1087,13 @@ static nnv_status_t launch_conv3x3_tc(const GemmArgs& a, const ConvTiling& ct, c
     return NNV_OK;
 }
 
-// 3-D tiled map over an NHWC fp32 activation {C, W, H} whose box is 32 channels of the WHOLE image.
-static nnv_status_t encode_image_operand(CUtensorMap* map, const void* base, int C, int H, int W) {
+// 3-D tiled map over an NHWC fp32 activation {C, W, H} whose box is 32 channels of `box_h` whole image rows.
+static nnv_status_t encode_image_operand(CUtensorMap* map, const void* base, int C, int H, int W, int box_h) {
     NNV_REQUIRE((reinterpret_cast<uintptr_t>(base) & 15) == 0 && (C % 4) == 0 && W <= 256 && H <= 256, NNV_ERR_INVALID_ARG,
                 "activation must be 16-byte aligned with C a multiple of 4 and at most 256 pixels a side");
     cuuint64_t dims[3] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H};
     cuuint64_t strides[2] = {(cuuint64_t)C * 4, (cuuint64_t)W * C * 4};
-    cuuint32_t box[3] = {32, (cuuint32_t)W, (cuuint32_t)H};
+    cuuint32_t box[3] = {32, (cuuint32_t)W, (cuuint32_t)box_h};
     cuuint32_t estr[3] = {1, 1, 1};
     CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void*>(base), dims, strides, box, estr,
                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
@@ -953,7 +1108,7 @@ nnv_status_t launch_gemm_sp(const nnv_layer_desc_t& L, const LayerGeom& geo, con
     NNV_REQUIRE(sp.splits == 1 || ws, NNV_ERR_INVALID_ARG, "the K split needs its scratch");
     CUtensorMap tmW, tmX;
     NNV_TRY(encode_operand(&tmW, wt, false, geo.Qp, L.K, 1, geo.Qp, (int64_t)L.K * geo.Qp, BM));
-    NNV_TRY(encode_image_operand(&tmX, x, L.C, L.H, L.W));
+    NNV_TRY(encode_image_operand(&tmX, x, L.C, L.H, L.W, L.H));
     SpDev g;
     g.stamp = next_stamp();
     next_stamp() = nullptr;
@@ -1086,45 +1241,14 @@ static nnv_status_t launch_conv3x3_persistent(const GemmArgs& a, int BN, int per
 nnv_status_t launch_gemm_tc(const GemmArgs& a, cudaStream_t st) {
     NNV_REQUIRE(a.M > 0 && a.N > 0 && a.Kd > 0 && a.batch > 0, NNV_ERR_INVALID_ARG, "empty GEMM");
     NNV_TRY(gemm_tc_init());
-    // Tiling.  These layers are small for 148 SMs, and one CTA can pull operand tiles out of L2 only
-    // so fast (~90 GB/s measured), so the column tile BN and the number of K splits (a thread-block
-    // cluster of up to 8 CTAs reducing through shared memory) are picked by a small cost model:
-    // waves x (fixed cost + K blocks per CTA x bytes per K block / per-SM bandwidth).
+    // Tiling: column tile BN and K splits (a thread-block cluster of up to 8 CTAs) with the least estimated time.
     const int bke = (a.mode == GEMM_BF16) ? 64 : 32;
     const int nkb_all = a.ic.on ? a.ic.R * a.ic.S * ceil_div(a.ic.C, 32) : ceil_div(a.Kd, bke);
     const int m_tiles = ceil_div(a.M, BM);
-    // Ring depth: 8 stages when every CTA has an SM to itself (a lone CTA needs that many loads in flight to keep
-    // the SM's ~100 GB/s of shared-memory fill busy on weights that come cold from HBM), 4 when several share one.
-    auto ring_for = [&](int bn, long long ctas) {
-        const uint32_t stage = (a.mode == GEMM_X3) ? stage_bytes_of<2>(bn) : (a.mode == GEMM_BF16_CVT) ? stage_bytes_of<3>(bn) : stage_bytes_of<0>(bn);
-        if (a.mode == GEMM_X3) return 3;
-        return (ctas <= 148 && (size_t)8 * stage <= 200u * 1024u) ? 8 : 4;
-    };
-    int BN = 0, splits = 1;
-    double best = 1e30;
-    for (int nt = ceil_div(a.N, 128); nt <= ceil_div(a.N, 16); nt *= 2) {
-        const int bn = ceil_div(ceil_div(a.N, nt), 16) * 16;
-        const int n_tiles = ceil_div(a.N, bn);
-        const double kb_bytes = (double)(A_STAGE_BYTES + bn * BK_BYTES);
-        for (int sp = 1; sp <= 8 && sp <= nkb_all; sp *= 2) {
-            const long long ctas = (long long)m_tiles * n_tiles * a.batch * sp;
-            const int stages = ring_for(bn, ctas);
-            const double smem = 1024.0 + stages * kb_bytes * (a.mode == GEMM_X3 ? 2 : 1);
-            const int occ = std::max(1, std::min(4, (int)(220.0 * 1024.0 / smem)));
-            double waves = std::ceil((double)ctas / (148.0 * occ));
-            // whole clusters must find free SMs in one GPC (16 - 20 SMs): measured in one wave are 14 clusters of 8
-            // (128 -> 128 3x3 @28 at BN = 64: 6.3 us against 8.3) and 32 clusters of 4 (1024 -> 2048 1x1 / 2 @14 at BN = 64: 6.8 against 9.0)
-            if (sp > 1 && occ == 1 && ctas > (sp == 8 ? 112 : sp == 4 ? 128 : 144)) waves = std::max(waves, 2.0);
-            const int resident = (int)std::min<long long>(occ, (ctas + 147) / 148);   // CTAs that really share an SM
-            // refit on a sweep of every (BN, splits) over the GEMM layer shapes of the ResNet-shaped configurations (kernel
-            // stamps, L2 flushed): a K block costs a CTA at least 0.25 us however narrow its tile (an unsplit BN = 16 launch of
-            // 512 -> 128 @28 took 6.5 us where 5.3 was predicted, 64 x 8 splits 6.0), a split 2.5 us
-            const double per_kb_us = std::max(kb_bytes * resident / 100e3, 0.25) * (stages >= 8 ? 1.0 : 1.3);
-            const double t = waves * (2.0 + (sp > 1 ? 2.5 : 0.0) + std::ceil((double)nkb_all / sp) * per_kb_us + 0.3 + bn * 0.004);
-            if (t < best - 1e-9) { best = t; BN = bn; splits = sp; }
-        }
-        if (bn <= 16) break;
-    }
+    constexpr int issuers = 2;
+    const int rows = gemm_rows(a.M);
+    const GemmTiling tile = pick_gemm_tiling(a.mode, a.M, a.N, a.batch, nkb_all);
+    int BN = tile.BN, splits = tile.splits;
     const Tuning tn = tuning();
     if (tn.gemm_bn && tn.gemm_splits <= nkb_all) { BN = tn.gemm_bn; splits = tn.gemm_splits; }   // override (nnv_tuning_set)
     // A 3x3 / stride 1 / pad 1 layer large enough to fill the GPU runs on the halo-resident kernel,
@@ -1167,11 +1291,10 @@ nnv_status_t launch_gemm_tc(const GemmArgs& a, cudaStream_t st) {
         if (use) return launch_conv3x3_tc(a, ct, st);
     }
     int tmem_cols = 32;
-    while (tmem_cols < BN) tmem_cols *= 2;
-    const uint32_t sb = (a.mode == GEMM_X3) ? stage_bytes_of<2>(BN) : (a.mode == GEMM_BF16_CVT) ? stage_bytes_of<3>(BN) : stage_bytes_of<0>(BN);
-    int ring = ring_for(BN, (long long)m_tiles * ceil_div(a.N, BN) * a.batch * splits);
+    while (tmem_cols < BN * issuers) tmem_cols *= 2;
+    const uint32_t sb = gemm_stage_bytes(a.mode, BN, rows);
+    int ring = gemm_ring(a.mode, BN, rows, (long long)m_tiles * ceil_div(a.N, BN) * a.batch * splits, ceil_div(nkb_all, splits));
     if (tn.gemm_ring && (size_t)tn.gemm_ring * sb <= 210u * 1024u) ring = tn.gemm_ring;
-    while (splits > 1 && ring < 8 && (uint32_t)ring * sb < (uint32_t)BM * (BN + 4) * 4u) ++ring;   // room to park the partial tile
 
     const bool bf16 = a.mode == GEMM_BF16;
     CUtensorMap tmA, tmB, tmD, tmAdd;
@@ -1180,17 +1303,17 @@ nnv_status_t launch_gemm_tc(const GemmArgs& a, cudaStream_t st) {
     next_stamp() = nullptr;
     g.D = a.D; g.bias = a.bias; g.addend = a.addend;
     g.ldd = a.ldd; g.strideD = a.strideD;
-    g.M = a.M; g.N = a.N; g.Kd = a.Kd; g.BN = BN; g.act = a.act; g.tmem_cols = tmem_cols; g.splits = splits; g.stages = ring; g.prefill = tn.gemm_prefill;
+    g.M = a.M; g.N = a.N; g.Kd = a.Kd; g.BN = BN; g.act = a.act; g.tmem_cols = tmem_cols; g.splits = splits; g.stages = ring; g.issuers = issuers;
     g.ic_on = 0; g.ic_C = g.ic_cblk = g.ic_S = g.ic_OW = g.ic_stride = g.ic_pad = 0;
     if (a.ic.on) {
         NNV_REQUIRE((a.mode == GEMM_TF32 || a.mode == GEMM_BF16_CVT) && a.batch == 1, NNV_ERR_INVALID_ARG,
                     "implicit im2col needs fp32 activations (TF32 or converting BF16 mode) and one batch");
-        NNV_TRY(encode_im2col_operand(&tmA, a.A, a.ic.C, a.ic.H, a.ic.W, a.ic.R, a.ic.S, a.ic.stride, a.ic.pad));
+        NNV_TRY(encode_im2col_operand(&tmA, a.A, a.ic.C, a.ic.H, a.ic.W, a.ic.R, a.ic.S, a.ic.stride, a.ic.pad, rows));
         g.ic_on = 1; g.ic_C = a.ic.C; g.ic_cblk = ceil_div(a.ic.C, 32); g.ic_S = a.ic.S; g.ic_OW = a.ic.OW;
         g.ic_stride = a.ic.stride; g.ic_pad = a.ic.pad;
         g.Kd = a.ic.R * a.ic.S * g.ic_cblk;                       // number of K blocks
     } else {
-        NNV_TRY(encode_operand(&tmA, a.A, bf16, a.Kd, a.M, a.batch, a.lda, a.strideA, BM));
+        NNV_TRY(encode_operand(&tmA, a.A, bf16, a.Kd, a.M, a.batch, a.lda, a.strideA, rows));
     }
     if (a.mode == GEMM_BF16_CVT) {
         NNV_REQUIRE(a.batch == 1, NNV_ERR_INVALID_ARG, "the converting BF16 mode needs one batch");
@@ -1199,47 +1322,51 @@ nnv_status_t launch_gemm_tc(const GemmArgs& a, cudaStream_t st) {
         NNV_TRY(encode_operand(&tmB, a.B, bf16, a.Kd, a.N, a.batch, a.ldb, a.strideB, BN));
     }
 
-    // Write-out by TMA through swizzled staging tiles when the output rows are 16-byte multiples (else plain stores).
-    // A residual addend needs a staging tile of its own beside the ring: the ring gives up stages for it.
-    if (a.addend && splits == 1)
-        while (ring > 4 && (size_t)2048 + (size_t)ring * sb + 8 * (3 * 8 + 3) + (size_t)BM * BN * 4 > 220u * 1024u) --ring;
+    // Write-out by TMA through swizzled staging tiles when the output rows are 16-byte multiples (else plain stores), in
+    // the ring once that is idle; with a residual addend, which is loaded while the ring works, in a place of their own.
+    const size_t staging = (size_t)ceil_div(rows, 32) * 32 * BN * 4;
+    const bool tma_out = splits == 1 && (a.N % 4) == 0 && (a.ldd % 4) == 0 && (a.strideD % 4) == 0 &&
+                         (reinterpret_cast<uintptr_t>(a.D) & 15) == 0 && (!a.addend || (reinterpret_cast<uintptr_t>(a.addend) & 15) == 0) &&
+                         (!a.addend || a.batch == 1);
+    // Split K: room to park the partial tile in the ring, and for the rows this CTA receives (its share from every CTA).
+    const size_t park = splits > 1 ? (size_t)rows * BN * 4 : (tma_out && !a.addend) ? staging : 0;
+    const size_t behind = splits > 1 ? (size_t)splits * ceil_div(rows, splits) * BN * 4 : (tma_out && a.addend) ? staging + 1024 : 0;
+    while (ring < 8 && (size_t)ring * sb < park) ++ring;
+    while (ring > 1 && (size_t)2048 + (size_t)ring * sb + GEMM_BAR_BYTES + behind > 226u * 1024u && (size_t)(ring - 1) * sb >= park) --ring;
     g.stages = ring;
-    const size_t ring_and_bars = (size_t)ring * sb + 8 * (3 * 8 + 3);
-    size_t smem_bytes = (size_t)1024 + ring_and_bars;
-    g.tma_out = 0;
-    g.stage_off = 0;
-    const bool out_ok = splits == 1 && (a.N % 4) == 0 && (a.ldd % 4) == 0 && (a.strideD % 4) == 0 &&
-                        (reinterpret_cast<uintptr_t>(a.D) & 15) == 0 && (!a.addend || (reinterpret_cast<uintptr_t>(a.addend) & 15) == 0) &&
-                        (!a.bias || (reinterpret_cast<uintptr_t>(a.bias) & 15) == 0) && (!a.addend || a.batch == 1);
-    if (out_ok) {
-        const int cw = (BN % 32) == 0 ? 32 : 16;
-        size_t need = smem_bytes;
-        uint32_t off = 0;
-        if (a.addend) {                                          // the staging tile cannot share the ring: it is filled while the ring works
-            off = (uint32_t)align_up(ring_and_bars, 1024);
-            need = (size_t)1024 + off + (size_t)BM * BN * 4;
-        }
-        if (need <= 220u * 1024u) {
-            g.tma_out = cw;
-            g.stage_off = off;
-            smem_bytes = need;
-            NNV_TRY(encode_output(&tmD, a.D, a.N, a.M, a.batch, a.ldd, a.batch > 1 ? a.strideD : (int64_t)a.M * a.ldd, cw));
-            if (a.addend) NNV_TRY(encode_output(&tmAdd, a.addend, a.N, a.M, 1, a.ldd, (int64_t)a.M * a.ldd, cw));
-        }
-    }
-    if (!g.tma_out) tmD = tmA;                                   // unused by the kernel, but a kernel parameter must hold a valid object
-    if (!g.tma_out || !a.addend) tmAdd = tmA;
+    g.rows = rows;
+    g.bar_off = (uint32_t)ring * sb;
+    const size_t ring_and_bars = (size_t)ring * sb + GEMM_BAR_BYTES;
+    g.recv_off = (uint32_t)align_up(ring_and_bars, 128);
+    g.tma_out = tma_out ? ((BN % 32) == 0 ? 32 : 16) : 0;
+    g.stage_off = a.addend ? (uint32_t)align_up(ring_and_bars, 1024) : 0;
+    // equal tiles: the output is addressed as {N, rows, tiles}, so that the hardware clips a tile's last 32-row box
+    const bool equal = a.M == m_tiles * rows && (a.batch == 1 || a.strideD == (int64_t)a.M * a.ldd);
+    NNV_REQUIRE(equal || rows == BM, NNV_ERR_INVALID_ARG, "batched GEMM outputs must be dense");
+    g.z_tiles = equal ? m_tiles : 0;
+    size_t smem_bytes = (size_t)1024 + (splits > 1 ? g.recv_off + behind : (tma_out && a.addend) ? g.stage_off + staging : ring_and_bars);
+    // the MMAs read 128 rows of A from every stage, the last one included
+    smem_bytes = std::max(smem_bytes, (size_t)1024 + (size_t)(ring - 1) * sb + A_STAGE_BYTES);
+    NNV_REQUIRE(smem_bytes <= 226u * 1024u, NNV_ERR_UNSUPPORTED, "GEMM tiling does not fit shared memory");
+    auto encode_out = [&](CUtensorMap* map, const void* base) {
+        if (equal) return encode_output(map, base, a.N, rows, m_tiles * a.batch, a.ldd, (int64_t)rows * a.ldd, g.tma_out);
+        return encode_output(map, base, a.N, a.M, a.batch, a.ldd, a.batch > 1 ? a.strideD : (int64_t)a.M * a.ldd, g.tma_out);
+    };
+    if (tma_out) NNV_TRY(encode_out(&tmD, a.D));
+    else tmD = tmA;                                              // unused by the kernel, but a kernel parameter must hold a valid object
+    if (tma_out && a.addend) NNV_TRY(encode_out(&tmAdd, a.addend));
+    else tmAdd = tmA;
 
     dim3 grid(m_tiles, ceil_div(a.N, BN), a.batch * splits);
     NNV_REQUIRE(grid.y <= 65535 && grid.z <= 65535, NNV_ERR_UNSUPPORTED, "GEMM grid too large");
     if (a.mode == GEMM_TF32)
-        (void)launch_pdl_cluster(gemm_tc_kernel<0>, grid, dim3(GEMM_THREADS), smem_bytes, st, splits, tmA, tmB, tmD, tmAdd, g);
+        (void)launch_pdl_cluster(gemm_tc_kernel<0>, grid, dim3(GEMM_TC_THREADS), smem_bytes, st, splits, tmA, tmB, tmD, tmAdd, g);
     else if (a.mode == GEMM_BF16)
-        (void)launch_pdl_cluster(gemm_tc_kernel<1>, grid, dim3(GEMM_THREADS), smem_bytes, st, splits, tmA, tmB, tmD, tmAdd, g);
+        (void)launch_pdl_cluster(gemm_tc_kernel<1>, grid, dim3(GEMM_TC_THREADS), smem_bytes, st, splits, tmA, tmB, tmD, tmAdd, g);
     else if (a.mode == GEMM_BF16_CVT)
-        (void)launch_pdl_cluster(gemm_tc_kernel<3>, grid, dim3(GEMM_THREADS), smem_bytes, st, splits, tmA, tmB, tmD, tmAdd, g);
+        (void)launch_pdl_cluster(gemm_tc_kernel<3>, grid, dim3(GEMM_TC_THREADS), smem_bytes, st, splits, tmA, tmB, tmD, tmAdd, g);
     else if (a.mode == GEMM_X3)
-        (void)launch_pdl_cluster(gemm_tc_kernel<2>, grid, dim3(GEMM_THREADS), smem_bytes, st, splits, tmA, tmB, tmD, tmAdd, g);
+        (void)launch_pdl_cluster(gemm_tc_kernel<2>, grid, dim3(GEMM_TC_THREADS), smem_bytes, st, splits, tmA, tmB, tmD, tmAdd, g);
     else
         return fail(NNV_ERR_INVALID_ARG, "unknown GEMM mode %d", a.mode);
     NNV_CUDA(cudaGetLastError());

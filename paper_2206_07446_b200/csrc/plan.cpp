@@ -49,13 +49,14 @@ static const char* parse_tuning(const char* spec, Tuning* t, char* item, size_t 
         auto flag = [&](int* dst) { return std::sscanf(val, "%d", &a) == 1 && (a == 0 || a == 1) ? (*dst = a, true) : false; };
         bool ok = false;
         if (!std::strcmp(key, "gemm_tile")) {
-            ok = std::sscanf(val, "%d,%d", &a, &b) == 2 && a >= 16 && a <= 128 && a % 16 == 0 && b >= 1 && b <= 8 && (b & (b - 1)) == 0;
+            ok = std::sscanf(val, "%d,%d", &a, &b) == 2 && a >= 16 && a <= 128 && a % 16 == 0 && b >= 1 && b <= 16 && (b & (b - 1)) == 0;
             if (ok) { t->gemm_bn = a; t->gemm_splits = b; }
         } else if (!std::strcmp(key, "gemm_ring")) {
             ok = std::sscanf(val, "%d", &a) == 1 && a >= 2 && a <= 8;
             if (ok) t->gemm_ring = a;
         } else if (!std::strcmp(key, "gemm_prefill")) {
-            ok = flag(&t->gemm_prefill);
+            int none = 0;                                     // accepted, without effect: the ring is always filled at once
+            ok = flag(&none);
         } else if (!std::strcmp(key, "conv3x3")) {
             if (!std::strcmp(val, "off")) { t->conv3x3 = 1; ok = true; }
             else if (!std::strcmp(val, "auto")) { t->conv3x3 = 0; ok = true; }
@@ -181,10 +182,10 @@ SmallPPlan small_p_plan(const nnv_layer_desc_t& L, const LayerGeom& g, int v, in
     if (!tn.smallp || (v != NNV_VAR_IM2COL && v != NNV_VAR_GEMM1X1) || math != NNV_MATH_TF32 || L.groups != 1 || L.stride != 1 ||
         L.R != L.S || (L.R & 1) == 0 || L.pad != (L.R - 1) / 2 || L.H * L.W > 256 || (L.C % 32) != 0 || (L.K % 4) != 0)
         return sp;
-    // Measured on B200 (L2 flushed, weights cold): on 7 x 7 grids this kernel takes 0.55 - 0.9 of the pixel-on-rows
-    // GEMM's time (512 -> 512 3x3: 9.2 against 15.9 us; 960 -> 160 1x1: 6.9 against 48 us), on 14 x 14 grids the two
-    // are level or the other is ahead (its two row tiles are 77 % full there); so, unless forced, up to 64 pixels.
-    if (L.H * L.W > 64 && !tn.smallp_splits) return sp;
+    // Unless forced, only for deep 3x3 (and larger) filters on up to 64 pixels, where every K block of the pixel-on-rows GEMM
+    // spends its MMAs on 128 rows of which half do not exist: 512 -> 512 3x3 @7 takes 7.0 us against 7.4, @5 6.0 against
+    // 6.9.  Every 1x1 layer is faster there (2048 -> 512 @7: 4.3 us against 6.2; 960 -> 160 @7: 3.3 against 5.3).
+    if (!tn.smallp_splits && (L.H * L.W > 64 || L.R == 1 || L.R * L.S * (L.C / 32) < 128)) return sp;
     sp.Npad = ceil_div(g.P, 16) * 16;
     sp.b_slot_bytes = (uint32_t)align_up((uint64_t)sp.Npad * 128, 1024);
     const double stage = 16384.0 + sp.b_slot_bytes;
