@@ -59,7 +59,7 @@ conv3x3_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     auto a_conv = [&](int s) { return bars + 8u * (2 * CONV_MAX_NA + 2 * CONV_MAX_NB + 2 + s); };   // box s is converted
     volatile uint32_t* holder_ptr = reinterpret_cast<volatile uint32_t*>(smem_raw + (holder - smem_u32(smem_raw)));
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int splits = g.splits, sp = (int)blockIdx.z;       // the cluster spans grid z: one K split per CTA
     const int tile_h = (int)blockIdx.x / g.tiles_w, tile_w = (int)blockIdx.x - tile_h * g.tiles_w;
     const int oh0 = tile_h * 16 * MT, ow0 = tile_w * 8, n0 = blockIdx.y * BN;
@@ -102,7 +102,7 @@ conv3x3_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     // and the (smaller, three times as many) weight tiles are issued by different warps -- warp 2's first lane serves
     // the weight ring before it joins the epilogue.
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             bool ok = true;
             int sa = 0, sb0 = 0;                              // ring slots and their phases, carried along (no divisions:
             uint32_t pa = 0, pb0 = 0;                         // every instruction of this single-thread loop is latency)
@@ -130,7 +130,7 @@ conv3x3_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             // instruction descriptor: fp32 accumulate, TF32 (or bf16) operands, both K-major, N = BN, M = 128
             const uint32_t fmt = bf16 ? 1u : 2u;
             const uint32_t idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
@@ -192,7 +192,7 @@ conv3x3_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                 if (++sa == NA) { sa = 0; pa ^= 1u; }
             }
             ok = __all_sync(0xffffffffu, (int)ok) != 0;
-        } else if (warp == 2 && lane == 0) {                  // the weight-tile producer
+        } else if (warp == 2 && elect_one()) {                  // the weight-tile producer
             int sb = 0;
             uint32_t pb = 0;
             for (int cbi = 0; cbi < ncb && ok; ++cbi) {
@@ -211,7 +211,7 @@ conv3x3_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                 for (int i = 0; i < 1000; ++i) __nanosleep(1000);   // let loads already in flight land
             }
         }
-        ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;       // the whole warp takes the producer's result
+        ok = __all_sync(0xffffffffu, (int)ok) != 0;           // the whole warp takes the producer's result
         ok = mbar_wait(tmem_full_bar, 0) && ok;
         ok = __all_sync(0xffffffffu, (int)ok) != 0;           // (the epilogue's TMEM reads are warp-wide instructions)
         tc_fence_after();

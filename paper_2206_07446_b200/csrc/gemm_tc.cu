@@ -73,7 +73,8 @@ constexpr int BM = 128;                 // rows of A per tile = TMEM lanes
 constexpr int BK_BYTES = 128;           // bytes of K per stage row = one 128B swizzle atom
 constexpr int A_STAGE_BYTES = BM * BK_BYTES;
 constexpr int GEMM_THREADS = 192;
-constexpr int GEMM_TC_THREADS = 256;                          // gemm_tc_kernel: a second MMA issuer and a second producer
+// gemm_tc_kernel: a second MMA issuer and a second producer; splitting both operands (mode 2) takes four more warps
+constexpr int gemm_tc_threads(int mode) { return mode == 2 ? 384 : 256; }
 constexpr int GEMM_BAR_BYTES = 8 * (3 * 8 + 4) + 512;         // barriers, TMEM address, bias of the tile's columns
 constexpr uint32_t WAIT_LIMIT = 1u << 20;
 
@@ -253,36 +254,38 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 
 // Split eight fp32 values into bf16 hi = rn(x) and lo = rn(x - hi), packed as two 16-byte chunks.
 __device__ __forceinline__ void split8(const float4& a, const float4& b, uint4& hi, uint4& lo) {
-    const float x[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-    uint32_t h[4], l[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const __nv_bfloat16 h0 = __float2bfloat16_rn(x[2 * i]), h1 = __float2bfloat16_rn(x[2 * i + 1]);
-        const __nv_bfloat16 l0 = __float2bfloat16_rn(x[2 * i] - __bfloat162float(h0));
-        const __nv_bfloat16 l1 = __float2bfloat16_rn(x[2 * i + 1] - __bfloat162float(h1));
-        h[i] = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
-        l[i] = (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
-    }
-    hi = make_uint4(h[0], h[1], h[2], h[3]);
-    lo = make_uint4(l[0], l[1], l[2], l[3]);
+    auto split2 = [](float x, float y, uint32_t& h, uint32_t& l) {
+        const __nv_bfloat162 p = __floats2bfloat162_rn(x, y);
+        h = *reinterpret_cast<const uint32_t*>(&p);
+        const __nv_bfloat162 q = __floats2bfloat162_rn(x - __uint_as_float(h << 16), y - __uint_as_float(h & 0xFFFF0000u));
+        l = *reinterpret_cast<const uint32_t*>(&q);
+    };
+    split2(a.x, a.y, hi.x, lo.x); split2(a.z, a.w, hi.y, lo.y);
+    split2(b.x, b.y, hi.z, lo.z); split2(b.z, b.w, hi.w, lo.w);
 }
 
-// Converts one row (32 fp32 = 128 bytes, stored by TMA with the 128-byte swizzle) of a staged tile
-// into the hi and lo bf16 tiles (un-swizzled core-matrix layout, `rows` rows tall).
-__device__ __forceinline__ void convert_row(uint32_t src_tile, uint32_t hi_tile, uint32_t lo_tile, int r, int rows) {
-    const uint32_t src = src_tile + (uint32_t)r * 128u;
-    const uint32_t lbo = (uint32_t)rows * 16u;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {                              // 4 chunks of 8 K-elements
-        float4 v0, v1;
-        const uint32_t a0 = src + ((uint32_t)((2 * c) ^ (r & 7)) << 4), a1 = src + ((uint32_t)((2 * c + 1) ^ (r & 7)) << 4);
-        asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v0.x), "=f"(v0.y), "=f"(v0.z), "=f"(v0.w) : "r"(a0));
-        asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v1.x), "=f"(v1.y), "=f"(v1.z), "=f"(v1.w) : "r"(a1));
+__device__ __forceinline__ uint4 pack8_bf16(const float4& a, const float4& b) {
+    const __nv_bfloat162 p0 = __floats2bfloat162_rn(a.x, a.y), p1 = __floats2bfloat162_rn(a.z, a.w);
+    const __nv_bfloat162 p2 = __floats2bfloat162_rn(b.x, b.y), p3 = __floats2bfloat162_rn(b.z, b.w);
+    return make_uint4(*reinterpret_cast<const uint32_t*>(&p0), *reinterpret_cast<const uint32_t*>(&p1),
+                      *reinterpret_cast<const uint32_t*>(&p2), *reinterpret_cast<const uint32_t*>(&p3));
+}
+
+// Converts chunk c (8 of the 32 elements) of row r of a staged fp32 tile (TMA, 128-byte swizzle) into bf16 tiles in the
+// un-swizzled core-matrix layout, `rows` rows tall: hi and lo, or (SPLIT = false) one tile rounded to nearest even.
+template <bool SPLIT>
+__device__ __forceinline__ void convert_chunk(const uint8_t* src_tile, uint8_t* hi_tile, uint8_t* lo_tile, int r, int c, int rows) {
+    const uint8_t* src = src_tile + r * 128;
+    const float4 v0 = *reinterpret_cast<const float4*>(src + (((2 * c) ^ (r & 7)) << 4));
+    const float4 v1 = *reinterpret_cast<const float4*>(src + (((2 * c + 1) ^ (r & 7)) << 4));
+    const int off = (c * rows + r) * 16;
+    if constexpr (SPLIT) {
         uint4 hi, lo;
         split8(v0, v1, hi, lo);
-        const uint32_t off = (uint32_t)c * lbo + (uint32_t)r * 16u;
-        asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(hi_tile + off), "r"(hi.x), "r"(hi.y), "r"(hi.z), "r"(hi.w) : "memory");
-        asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(lo_tile + off), "r"(lo.x), "r"(lo.y), "r"(lo.z), "r"(lo.w) : "memory");
+        *reinterpret_cast<uint4*>(hi_tile + off) = hi;
+        *reinterpret_cast<uint4*>(lo_tile + off) = lo;
+    } else {
+        *reinterpret_cast<uint4*>(hi_tile + off) = pack8_bf16(v0, v1);
     }
 }
 
@@ -315,22 +318,21 @@ template <int MODE> struct ModeTraits {
     static constexpr int BKE = (MODE == 1) ? 64 : 32;          // K elements per stage
 };
 
+// A stage holds the `rows` rows of A that are loaded (the MMA's other rows read whatever follows and are never written out)
+// and BN rows of B, 128 bytes each; the conversion modes add the bf16 tiles, `pad8(rows)` rows tall: A (hi, lo), B (hi, lo) in
+// mode 2; A in mode 3, whose B arrives as bf16.
+__host__ __device__ constexpr int pad8(int rows) { return (rows + 7) & ~7; }
+__host__ __device__ constexpr uint32_t a_stage_of(int rows) { return ((uint32_t)rows * BK_BYTES + 1023u) & ~1023u; }
 template <int MODE>
-__host__ __device__ constexpr uint32_t stage_bytes_of(int BN, int rows = 128) {
-    // staged TMA tiles (A: 128 rows x 128 B, B: BN rows x 128 B); mode 2 adds hi and lo bf16 tiles
-    if (MODE == 3) return (uint32_t)(A_STAGE_BYTES + A_STAGE_BYTES / 2 + BN * 64);   // fp32 A, bf16 A, bf16 B (32 elements per row)
-    if (MODE == 2) return 2u * (uint32_t)(A_STAGE_BYTES + BN * BK_BYTES);
-    return (((uint32_t)rows * BK_BYTES + 1023u) & ~1023u) + (uint32_t)(BN * BK_BYTES);
-}
-// Modes 0 and 1 keep only the `rows` rows of A that are loaded (the MMA's other rows read whatever follows and are never
-// written out); the conversion modes keep room for all 128.
-template <int MODE>
-__host__ __device__ constexpr uint32_t a_stage_of(int rows) {
-    return MODE >= 2 ? (uint32_t)A_STAGE_BYTES : ((uint32_t)rows * BK_BYTES + 1023u) & ~1023u;
+__host__ __device__ constexpr uint32_t stage_bytes_of(int BN, int rows) {
+    const uint32_t a = a_stage_of(rows), b = (uint32_t)(BN * BK_BYTES);
+    if (MODE == 3) return (a + (uint32_t)(pad8(rows) * 64) + b / 2 + 1023u) & ~1023u;
+    if (MODE == 2) return (a + b + (uint32_t)(pad8(rows) * 128) + b + 1023u) & ~1023u;
+    return a + b;
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(GEMM_TC_THREADS, 3)
+__global__ void __launch_bounds__(gemm_tc_threads(MODE), MODE == 2 ? 2 : 3)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmD, const __grid_constant__ CUtensorMap tmAdd, const GemmDev g) {
     extern __shared__ uint8_t smem_raw[];
@@ -341,7 +343,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const int BN = g.BN;
     const uint32_t b_stage_bytes = (uint32_t)BN * BK_BYTES;
     const uint32_t b_bytes = MODE == 3 ? (uint32_t)BN * 64u : b_stage_bytes, a_bytes = (uint32_t)g.rows * BK_BYTES;
-    const uint32_t a_stage = a_stage_of<MODE>(g.rows);
+    const uint32_t a_stage = a_stage_of(g.rows);
+    const int rp = pad8(g.rows);
     const uint32_t stage_bytes = stage_bytes_of<MODE>(BN, g.rows);
     const uint32_t bars = sbase + g.bar_off;                  // behind the ring       // full[S], empty[S], conv[S], tmem_full, holder
     auto full_bar = [&](int s) { return bars + 8u * s; };
@@ -384,7 +387,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(full_bar(s), 2);
             mbar_init(empty_bar(s), 1);
-            mbar_init(conv_bar(s), 128);
+            mbar_init(conv_bar(s), MODE == 2 ? 8 : 4);
         }
         mbar_init(tmem_full_bar, (uint32_t)g.issuers);
         mbar_init(addend_bar, 1);
@@ -438,7 +441,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         mbar_expect_tx(full_bar(s), b_bytes);
         const uint32_t b_dst = sbase + s * stage_bytes + a_stage;
         // MODE 3: one box of four 8-element chunks x BN rows, staged after the fp32 and the bf16 A tile
-        if constexpr (MODE == 3) tma_load_3d(b_dst + A_STAGE_BYTES / 2, &tmB, 0, n0, q >> 3, full_bar(s));
+        if constexpr (MODE == 3) tma_load_3d(b_dst + rp * 64, &tmB, 0, n0, q >> 3, full_bar(s));
         else tma_load_3d(b_dst, &tmB, q, n0, b, full_bar(s));
     };
     tc_fence_before();
@@ -454,6 +457,45 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     pdl_trigger();
     if (threadIdx.x == 32) stamp_start(g.stamp);
 
+    // Operand conversion (modes 2 and 3), by warps 2-5 (and 8-11 in mode 2) together: MODE 3 rounds A to bf16 (the weights arrive as
+    // bf16), MODE 2 splits both operands into bf16 hi / lo tiles.  The work of a stage is dealt to the warps in pieces of
+    // 32 rows x 8 elements: a thread that converted whole rows of A and B alone paid ~3400 cycles a K block in dependent
+    // instructions, most of the kernel's time (512 -> 512 F(4,3) @7, whole layer: 38.7 -> 23.5 us).
+    auto convert_stages = [&](int cw) -> bool {
+        uint8_t* const sm0 = smem_raw + (sbase - smem_u32(smem_raw));
+        const int ga = (g.rows + 31) >> 5, gb = (BN + 31) >> 5;
+        int s = 0;
+        uint32_t ph = 0;
+        for (int it = 0; it < nkb; ++it, s = (s + 1 == STAGES ? 0 : s + 1), ph ^= (s == 0 ? 1u : 0u)) {
+            if (!mbar_wait(full_bar(s), ph)) return false;
+            uint8_t* const st = sm0 + s * stage_bytes;
+            uint8_t* const cv = st + a_stage + (MODE == 2 ? b_stage_bytes : 0u);      // converted tiles: A hi, A lo, B hi, B lo
+            if constexpr (MODE == 3) {
+                const int r = cw * 32 + lane;                 // a row of A per thread
+                if (r < g.rows) {
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) convert_chunk<false>(st, cv, cv, r, c, rp);
+                }
+            } else {
+#pragma unroll 2
+                for (int i = cw; i < 4 * (ga + gb); i += 8) {
+                    const int grp = i >> 2, c = i & 3;
+                    if (grp < ga) {
+                        const int r = grp * 32 + lane;
+                        if (r < g.rows) convert_chunk<true>(st, cv, cv + rp * 64, r, c, rp);
+                    } else {
+                        const int r = (grp - ga) * 32 + lane;
+                        uint8_t* const bh = cv + rp * 128;
+                        if (r < BN) convert_chunk<true>(st + a_stage, bh, bh + b_stage_bytes / 2, r, c, BN);
+                    }
+                }
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> visible to the MMA's reads
+            __syncwarp();
+            if (lane == 0) mbar_arrive(conv_bar(s));
+        }
+        return true;
+    };
     bool cluster_arrived = false;                             // the epilogue warps arrive early, in their own code
     if (warp == 0 || warp == 7) {
         // Producers.  A load costs the thread that issues it ~157 cycles whatever its size, which for one thread issuing both
@@ -488,6 +530,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         }
         __syncwarp();
         if (splits > 1) cluster_wait();
+    } else if (warp >= 8) {
+        if constexpr (MODE == 2) {
+            if (!convert_stages(warp - 4) && lane == 0) atomicExch(&g_device_status, (int)NNV_ERR_TIMEOUT);
+        }
+        __syncwarp();
+        if (splits > 1) cluster_wait();
     } else if (warp == 1 || warp == 6) {
         // MMA issuers.  One thread that waits for a stage, issues its four MMAs into one accumulator and commits takes
         // ~560 cycles a K block (device-clock probes), several times what the tensor pipe needs at these tile widths, so
@@ -509,9 +557,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 const uint32_t a_src = sbase + s * stage_bytes;
                 if constexpr (MODE == 2) {
                     // converted tiles follow the staged ones: A_hi, A_lo (8 KB each), B_hi, B_lo
-                    const uint32_t a_hi = a_src + A_STAGE_BYTES + b_stage_bytes, a_lo = a_hi + A_STAGE_BYTES / 2;
-                    const uint32_t b_hi = a_lo + A_STAGE_BYTES / 2, b_lo = b_hi + b_stage_bytes / 2;
-                    const uint32_t lbo_a = BM * 16u, lbo_b = (uint32_t)BN * 16u;
+                    const uint32_t a_hi = a_src + a_stage + b_stage_bytes, a_lo = a_hi + rp * 64;
+                    const uint32_t b_hi = a_lo + rp * 64, b_lo = b_hi + b_stage_bytes / 2;
+                    const uint32_t lbo_a = (uint32_t)rp * 16u, lbo_b = (uint32_t)BN * 16u;
 #pragma unroll
                     for (int kk = 0; kk < 2; ++kk) {            // 2 K-steps of 16 bf16 = 2 core matrices each
                         const uint64_t ah = make_smem_desc_plain(a_hi + kk * 2 * lbo_a, lbo_a, 128);
@@ -523,8 +571,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                         umma<true>(acc, ah, bh, idesc, 1u);
                     }
                 } else if constexpr (MODE == 3) {
-                    const uint32_t a_bf = a_src + A_STAGE_BYTES, b_bf = a_bf + A_STAGE_BYTES / 2;
-                    const uint32_t lbo_a = BM * 16u, lbo_b = (uint32_t)BN * 16u;
+                    const uint32_t a_bf = a_src + a_stage, b_bf = a_bf + rp * 64;
+                    const uint32_t lbo_a = (uint32_t)rp * 16u, lbo_b = (uint32_t)BN * 16u;
 #pragma unroll
                     for (int kk = 0; kk < 2; ++kk)             // 2 K-steps of 16 bf16 = 2 core matrices each
                         umma<true>(acc, make_smem_desc_plain(a_bf + kk * 2 * lbo_a, lbo_a, 128),
@@ -578,27 +626,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             }
         };
         bool ok = true;
-        if constexpr (MODE == 2 || MODE == 3) {
-            // round every staged fp32 tile first: MODE 3 A to bf16 (the weights arrive as bf16), MODE 2 both
-            // operands into their bf16 hi / lo tiles
-            int s = 0;
-            uint32_t ph = 0;
-            for (int it = 0; it < nkb; ++it, s = (s + 1 == STAGES ? 0 : s + 1), ph ^= (s == 0 ? 1u : 0u)) {
-                ok = mbar_wait(full_bar(s), ph);
-                if (!ok) break;
-                const uint32_t a_src = sbase + s * stage_bytes;
-                if constexpr (MODE == 3) {
-                    if (t < g.rows) convert_row_bf16(a_src, a_src + A_STAGE_BYTES, t, BM);
-                } else {
-                    const uint32_t a_hi = a_src + A_STAGE_BYTES + b_stage_bytes, a_lo = a_hi + A_STAGE_BYTES / 2;
-                    const uint32_t b_hi = a_lo + A_STAGE_BYTES / 2, b_lo = b_hi + b_stage_bytes / 2;
-                    if (t < g.rows) convert_row(a_src, a_hi, a_lo, t, BM);
-                    if (t < BN) convert_row(a_src + A_STAGE_BYTES, b_hi, b_lo, t, BN);
-                }
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> visible to the MMA's reads
-                mbar_arrive(conv_bar(s));
-            }
-        }
+        if constexpr (MODE >= 2) ok = convert_stages(warp - 2);
         float* const s_bias = reinterpret_cast<float*>(sm + (sbias - sbase));
         if (t < BN) s_bias[t] = bias;
         asm volatile("barrier.sync 1, 128;" ::: "memory");
@@ -948,7 +976,7 @@ bool pick_conv_tiling(int C, int H, int W, int N, int bf16, ConvTiling* out) {
 }
 
 uint32_t gemm_stage_bytes(int mode, int bn, int rows) {
-    return mode == GEMM_X3 ? stage_bytes_of<2>(bn) : mode == GEMM_BF16_CVT ? stage_bytes_of<3>(bn) : stage_bytes_of<0>(bn, rows);
+    return mode == GEMM_X3 ? stage_bytes_of<2>(bn, rows) : mode == GEMM_BF16_CVT ? stage_bytes_of<3>(bn, rows) : stage_bytes_of<0>(bn, rows);
 }
 
 // Rows of A per tile.  As few 128-row tiles as hold M, of equal height when they divide M (7 x 7 and 14 x 14 grids: one
@@ -962,7 +990,10 @@ int gemm_rows(int M) {
 // cold from HBM), 4 when several share one, and no more than the K blocks a CTA walks: the shared memory left over lets
 // the next kernel's CTAs in early (warm ResNet-50-shaped inference 426 -> 415 us).
 int gemm_ring(int mode, int bn, int rows, long long ctas, int nkb) {
-    const int most = mode == GEMM_X3 ? 3 : (ctas <= 148 && 8u * gemm_stage_bytes(mode, bn, rows) <= 200u * 1024u) ? 8 : 4;
+    const int sb = (int)gemm_stage_bytes(mode, bn, rows);
+    // (X3 stages are twice as large: as many as fit one CTA, or two CTAs on an SM)
+    if (mode == GEMM_X3) return std::max(2, std::min({4, (ctas <= 148 ? 200 : 104) * 1024 / sb, nkb}));
+    const int most = (ctas <= 148 && 8 * sb <= 200 * 1024) ? 8 : 4;
     return std::max(2, std::min(most, nkb));
 }
 
@@ -1360,13 +1391,13 @@ nnv_status_t launch_gemm_tc(const GemmArgs& a, cudaStream_t st) {
     dim3 grid(m_tiles, ceil_div(a.N, BN), a.batch * splits);
     NNV_REQUIRE(grid.y <= 65535 && grid.z <= 65535, NNV_ERR_UNSUPPORTED, "GEMM grid too large");
     if (a.mode == GEMM_TF32)
-        (void)launch_pdl_cluster(gemm_tc_kernel<0>, grid, dim3(GEMM_TC_THREADS), smem_bytes, st, splits, tmA, tmB, tmD, tmAdd, g);
+        (void)launch_pdl_cluster(gemm_tc_kernel<0>, grid, dim3(gemm_tc_threads(0)), smem_bytes, st, splits, tmA, tmB, tmD, tmAdd, g);
     else if (a.mode == GEMM_BF16)
-        (void)launch_pdl_cluster(gemm_tc_kernel<1>, grid, dim3(GEMM_TC_THREADS), smem_bytes, st, splits, tmA, tmB, tmD, tmAdd, g);
+        (void)launch_pdl_cluster(gemm_tc_kernel<1>, grid, dim3(gemm_tc_threads(1)), smem_bytes, st, splits, tmA, tmB, tmD, tmAdd, g);
     else if (a.mode == GEMM_BF16_CVT)
-        (void)launch_pdl_cluster(gemm_tc_kernel<3>, grid, dim3(GEMM_TC_THREADS), smem_bytes, st, splits, tmA, tmB, tmD, tmAdd, g);
+        (void)launch_pdl_cluster(gemm_tc_kernel<3>, grid, dim3(gemm_tc_threads(3)), smem_bytes, st, splits, tmA, tmB, tmD, tmAdd, g);
     else if (a.mode == GEMM_X3)
-        (void)launch_pdl_cluster(gemm_tc_kernel<2>, grid, dim3(GEMM_TC_THREADS), smem_bytes, st, splits, tmA, tmB, tmD, tmAdd, g);
+        (void)launch_pdl_cluster(gemm_tc_kernel<2>, grid, dim3(gemm_tc_threads(2)), smem_bytes, st, splits, tmA, tmB, tmD, tmAdd, g);
     else
         return fail(NNV_ERR_INVALID_ARG, "unknown GEMM mode %d", a.mode);
     NNV_CUDA(cudaGetLastError());
