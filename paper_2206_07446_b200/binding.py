@@ -1,4 +1,4 @@
-"""ctypes binding of libnnv.so: argument marshalling only.
+"""Binding of libnnv.so (ctypes, and an extension module for the per-layer calls): argument marshalling only.
 
 Every function here has the name of the C entry point it calls (see
 include/nnv.h) and does nothing but convert Python values to C arguments and
@@ -182,6 +182,7 @@ class Plan:
         h = _vp()
         _check(_lib.nnv_plan_create(arr, n, o, ctypes.byref(h)))
         self.handle = h
+        self.address = int(h.value)
         self.n = n
         self.layers = [dict(L) for L in layers]
 
@@ -189,6 +190,7 @@ class Plan:
         if getattr(self, "handle", None):
             _lib.nnv_plan_destroy(self.handle)
             self.handle = None
+            self.address = 0
 
     def __del__(self):
         try:
@@ -632,5 +634,16 @@ def nnv_device_status():
     _check(_lib.nnv_device_status(ctypes.byref(c)))
     return int(c.value)
 
+
+# The calls a program makes once per layer go through the extension module (the functions above, without ctypes' cost per
+# argument); what it does not convert itself it hands back to them.
+try:
+    from . import _nnvcall
+except ImportError as e:
+    raise ImportError("_nnvcall.so is not built (%s). Run `python -m paper_2206_07446_b200.build`." % e)
+_nnvcall.set_fallbacks(nnv_conv_exec, nnv_transform_weights, nnv_transform_all, _check)
+nnv_conv_exec = _nnvcall.nnv_conv_exec
+nnv_transform_weights = _nnvcall.nnv_transform_weights
+nnv_transform_all = _nnvcall.nnv_transform_all
 
 EXPORTED_SYMBOLS = sorted(list(_SIGS.keys()) + ["nnv_last_error", "nnv_version"])

@@ -1,12 +1,15 @@
-"""Build libnnv.so in-tree with nvcc for sm_100a (no other architecture, no fallback)."""
+"""Build libnnv.so in-tree with nvcc for sm_100a (no other architecture, no fallback), and the extension module that
+marshals the per-layer calls for Python."""
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libnnv.so")
+PYCALL = os.path.join(HERE, "_nnvcall.so")
 SOURCES = ["plan.cpp", "scheduler.cpp", "cachefile.cpp", "transform.cu", "exec_kernels.cu", "direct_conv.cu", "gemm_tc.cu", "exec.cu", "pipeline.cu", "noalloc.cu"]
 
 
@@ -15,11 +18,11 @@ def sources():
 
 
 def needs_build():
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(PYCALL):
         return True
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(PYCALL))
     headers = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".h", ".cuh"))]
-    deps = sources() + headers + [os.path.join(ROOT, "include", "nnv.h")]
+    deps = sources() + [os.path.join(CSRC, "pycall.cpp")] + headers + [os.path.join(ROOT, "include", "nnv.h")]
     return any(os.path.getmtime(d) > t for d in deps)
 
 
@@ -35,6 +38,9 @@ def build(force=False, verbose=False):
         cmd.insert(1, "-Xptxas")
         cmd.insert(2, "-v")
     subprocess.check_call(cmd)
+    subprocess.check_call([os.environ.get("CXX", "g++"), "-std=c++17", "-O2", "-shared", "-fPIC", "-Wall",
+                           "-I", sysconfig.get_paths()["include"], "-I", os.path.join(ROOT, "include"),
+                           "-o", PYCALL, os.path.join(CSRC, "pycall.cpp"), "-L", HERE, "-l:libnnv.so", "-Wl,-rpath,$ORIGIN"])
     return LIB
 
 
