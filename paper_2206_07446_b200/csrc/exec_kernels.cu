@@ -459,6 +459,34 @@ maxpool_kernel(const float* __restrict__ x, float* __restrict__ y, int C, int H,
     }
 }
 
+// C % 4 == 0: four channels per thread.  R is 2 or 3 in practice; the window's loads do not depend on one another.
+template <int R>
+__global__ void __launch_bounds__(256)
+maxpool_v4_kernel(const float4* __restrict__ x, float4* __restrict__ y, int C4, int H, int W, int stride, int pad, int OH, int OW) {
+    pdl_enter();
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    if (i >= OH * OW * C4) return;
+    const int p = i / C4, c = i - p * C4;
+    const int oh = p / OW, ow = p - oh * OW;
+    const int h0 = oh * stride - pad, w0 = ow * stride - pad;
+    float4 v[R][R];
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int s = 0; s < R; ++s) {
+            const int h = h0 + r, w = w0 + s;
+            v[r][s] = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+            if (h >= 0 && h < H && w >= 0 && w < W) v[r][s] = __ldg(x + ((long long)h * W + w) * C4 + c);
+        }
+    float4 m = v[0][0];
+#pragma unroll
+    for (int q = 1; q < R * R; ++q) {
+        const float4 t = v[q / R][q % R];
+        m.x = fmaxf(m.x, t.x); m.y = fmaxf(m.y, t.y); m.z = fmaxf(m.z, t.z); m.w = fmaxf(m.w, t.w);
+    }
+    y[i] = m;
+}
+
 __global__ void __launch_bounds__(256)
 gavgpool_kernel(const float* __restrict__ x, float* __restrict__ y, int C, int HW) {
     pdl_enter();
@@ -469,30 +497,68 @@ gavgpool_kernel(const float* __restrict__ x, float* __restrict__ y, int C, int H
     y[c] = s / (float)HW;
 }
 
+// Few channels (a model's image): a thread moves V neighbouring pixels, 4 V bytes from every channel plane, so that a read
+// in place from pinned host memory asks for whole lines once.
+template <int V>
 __global__ void __launch_bounds__(256)
-chw_to_hwc_kernel(const float* __restrict__ in, float* __restrict__ out, int C, int HW) {
+chw_to_hwc_few_kernel(const float* __restrict__ in, float* __restrict__ out, int C, int HW) {
     pdl_enter();
-    const long long n = (long long)C * HW;
-    for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < n; i += (long long)gridDim.x * 256) {
-        const int p = (int)(i / C), c = (int)(i - (long long)p * C);
-        out[i] = __ldg(in + (long long)c * HW + p);
+    const int p = (blockIdx.x * 256 + threadIdx.x) * V;
+    if (p >= HW) return;
+    float v[4][V];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        if (c >= C) break;
+        if constexpr (V == 4) {
+            const float4 q = __ldg(reinterpret_cast<const float4*>(in + (long long)c * HW + p));
+            v[c][0] = q.x; v[c][1] = q.y; v[c][2] = q.z; v[c][3] = q.w;
+        } else {
+            v[c][0] = __ldg(in + (long long)c * HW + p);
+        }
     }
+#pragma unroll
+    for (int j = 0; j < V; ++j)
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            if (c < C) out[(long long)(p + j) * C + c] = v[c][j];
 }
 
+// [R][Cn] -> [Cn][R] in tiles of 32 x 32 through shared memory: reads and writes are both contiguous along a warp.  With a
+// status word given, one thread copies it to the host (the last kernel of a run; a copy of its own would cost more).
 __global__ void __launch_bounds__(256)
-hwc_to_chw_kernel(const float* __restrict__ in, float* __restrict__ out, int C, int HW) {
+transpose_kernel(const float* __restrict__ in, float* __restrict__ out, int R, int Cn, const int* status, int* h_status) {
     pdl_enter();
-    const long long n = (long long)C * HW;
-    for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < n; i += (long long)gridDim.x * 256) {
-        const int c = (int)(i / HW), p = (int)(i - (long long)c * HW);
-        out[i] = __ldg(in + (long long)p * C + c);
+    __shared__ float tile[32][33];
+    const int tiles_c = (Cn + 31) / 32;
+    const int c0 = (int)(blockIdx.x % tiles_c) * 32, r0 = (int)(blockIdx.x / tiles_c) * 32;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int r = r0 + ty + 8 * i;
+        if (r < R && c0 + tx < Cn) tile[ty + 8 * i][tx] = __ldg(in + (long long)r * Cn + c0 + tx);
     }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int c = c0 + ty + 8 * i;
+        if (c < Cn && r0 + tx < R) out[(long long)c * R + r0 + tx] = tile[tx][ty + 8 * i];
+    }
+    if (h_status && blockIdx.x == 0 && threadIdx.x == 0) *h_status = *reinterpret_cast<const volatile int*>(status);
 }
 
 static inline unsigned grid_for(long long n) { return (unsigned)std::min<long long>((n + 255) / 256, 148ll * 32); }
 
 nnv_status_t launch_maxpool(const float* x, float* y, int C, int H, int W, int R, int stride, int pad, int OH,
                             int OW, cudaStream_t st) {
+    if ((R == 2 || R == 3) && (C % 4) == 0 && ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(y)) & 15) == 0 &&
+        (long long)OH * OW * C < (1ll << 31)) {
+        const dim3 grid(ceil_div(OH * OW * (C / 4), 256));
+        const float4* x4 = reinterpret_cast<const float4*>(x);
+        float4* y4 = reinterpret_cast<float4*>(y);
+        if (R == 2) NNV_CUDA(launch_pdl(maxpool_v4_kernel<2>, grid, dim3(256), 0, st, x4, y4, C / 4, H, W, stride, pad, OH, OW));
+        else NNV_CUDA(launch_pdl(maxpool_v4_kernel<3>, grid, dim3(256), 0, st, x4, y4, C / 4, H, W, stride, pad, OH, OW));
+        return NNV_OK;
+    }
     NNV_LAUNCH((maxpool_kernel), grid_for((long long)OH * OW * C), 256, 0, st, x, y, C, H, W, R, stride, pad, OH, OW);
     NNV_CUDA(cudaGetLastError());
     return NNV_OK;
@@ -502,15 +568,25 @@ nnv_status_t launch_gavgpool(const float* x, float* y, int C, int H, int W, cuda
     NNV_CUDA(cudaGetLastError());
     return NNV_OK;
 }
-nnv_status_t launch_chw_to_hwc(const float* in, float* out, int C, int H, int W, cudaStream_t st) {
-    NNV_LAUNCH((chw_to_hwc_kernel), grid_for((long long)C * H * W), 256, 0, st, in, out, C, H * W);
-    NNV_CUDA(cudaGetLastError());
+static nnv_status_t launch_transpose(const float* in, float* out, int R, int Cn, const int* status, int* h_status, cudaStream_t st) {
+    const long long tiles = (long long)ceil_div(Cn, 32) * ceil_div(R, 32);
+    NNV_REQUIRE(tiles < (1ll << 31), NNV_ERR_UNSUPPORTED, "image too large for the layout conversion");
+    const dim3 grid((unsigned)tiles);
+    NNV_CUDA(launch_pdl(transpose_kernel, grid, dim3(256), 0, st, in, out, R, Cn, status, h_status));
     return NNV_OK;
 }
-nnv_status_t launch_hwc_to_chw(const float* in, float* out, int C, int H, int W, cudaStream_t st) {
-    NNV_LAUNCH((hwc_to_chw_kernel), grid_for((long long)C * H * W), 256, 0, st, in, out, C, H * W);
-    NNV_CUDA(cudaGetLastError());
+nnv_status_t launch_chw_to_hwc(const float* in, float* out, int C, int H, int W, cudaStream_t st) {
+    const int HW = H * W;
+    if (C <= 4 && (HW % 4) == 0 && (reinterpret_cast<uintptr_t>(in) & 15) == 0)
+        NNV_CUDA(launch_pdl(chw_to_hwc_few_kernel<4>, dim3(ceil_div(HW, 1024)), dim3(256), 0, st, in, out, C, HW));
+    else if (C <= 4)
+        NNV_CUDA(launch_pdl(chw_to_hwc_few_kernel<1>, dim3(ceil_div(HW, 256)), dim3(256), 0, st, in, out, C, HW));
+    else
+        return launch_transpose(in, out, C, HW, nullptr, nullptr, st);
     return NNV_OK;
+}
+nnv_status_t launch_hwc_to_chw(const float* in, float* out, int C, int H, int W, cudaStream_t st, const int* status, int* h_status) {
+    return launch_transpose(in, out, H * W, C, status, h_status, st);
 }
 
 }  // namespace nnv

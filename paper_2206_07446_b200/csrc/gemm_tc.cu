@@ -62,8 +62,10 @@ nnv_status_t stamps_device_base(unsigned long long** base) {
     return NNV_OK;
 }
 
-nnv_status_t enqueue_status_read(int* h_pinned, cudaStream_t st) {
-    NNV_CUDA(cudaMemcpyFromSymbolAsync(h_pinned, g_device_status, sizeof(int), 0, cudaMemcpyDeviceToHost, st));
+nnv_status_t device_status_address(const int** d) {
+    void* ptr = nullptr;
+    NNV_CUDA(cudaGetSymbolAddress(&ptr, g_device_status));
+    *d = static_cast<const int*>(ptr);
     return NNV_OK;
 }
 

@@ -272,7 +272,9 @@ nnv_status_t launch_maxpool(const float* d_x, float* d_y, int C, int H, int W, i
                             int OH, int OW, cudaStream_t st);
 nnv_status_t launch_gavgpool(const float* d_x, float* d_y, int C, int H, int W, cudaStream_t st);
 nnv_status_t launch_chw_to_hwc(const float* d_in, float* d_out, int C, int H, int W, cudaStream_t st);
-nnv_status_t launch_hwc_to_chw(const float* d_in, float* d_out, int C, int H, int W, cudaStream_t st);
+// status / h_status: the kernel also copies the device status word into host memory (null: not).
+nnv_status_t launch_hwc_to_chw(const float* d_in, float* d_out, int C, int H, int W, cudaStream_t st, const int* status = nullptr,
+                               int* h_status = nullptr);
 
 // Winograd F(2x2,3x3), TF32, as one kernel (wino_fused.cuh): x NHWC, U[16][K][Cp] fp32, y NHWC.  Needs C % 8 == 0 and
 // K % 8 == 0 (wino_fused_applies).
@@ -316,7 +318,7 @@ void cache_geometry(const nnv_cache* c, uint64_t* raw_off, uint64_t* cached_off,
 const nnv_layer_desc_t* cache_layers(const nnv_cache* c);      // the file's layer table (n_layers entries)
 
 nnv_status_t read_device_status(int32_t* code);
-// Enqueue a copy of the device status word into pinned host memory on `st` (no synchronisation).
-nnv_status_t enqueue_status_read(int* h_pinned, cudaStream_t st);
+// Device address of the status word on the current device.
+nnv_status_t device_status_address(const int** d);
 
 }  // namespace nnv

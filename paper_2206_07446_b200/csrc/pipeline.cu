@@ -119,6 +119,8 @@ static nnv_status_t run_model(nnv_plan* p, const nnv_choice_t* choices, const vo
     const bool tm = timings != nullptr;
     if (tm) std::memset(timings, 0, sizeof(nnv_timing_t) * n);
     NNV_TRY(gemm_tc_init());
+    const int* d_status = nullptr;
+    NNV_TRY(device_status_address(&d_status));
 
     // Residual-branch layers (a conv whose output is only ever the addend of a later layer, e.g. the
     // 1x1 downsample of a ResNet block) run on a side stream of the plan's own, beside the main
@@ -144,6 +146,12 @@ static nnv_status_t run_model(nnv_plan* p, const nnv_choice_t* choices, const vo
         NNV_CUDA(cudaStreamCreateWithPriority(&p->s_side, cudaStreamNonBlocking, prio));
     }
     cudaStream_t s_side = p->s_side;
+    // Layers whose completion another stream waits for: consumers on the other execution stream, and with staging slots
+    // every conv layer (its slot is free then).  An event nobody waits for costs the host ~0.5 us of an eager run.
+    std::vector<char> need_done(n, depth > 0 && !queued ? 1 : 0);
+    for (int i = 0; i < n; ++i)
+        for (int prod : {p->layers[i].in0, p->layers[i].in1})
+            if (prod >= 0 && on_side[prod] != on_side[i]) need_done[prod] = 1;
     const cudaEvent_t ev_input = p->ev[3 * n + 6 + NNV_MAX_QUEUES], ev_side_join = p->ev[3 * n + 7 + NNV_MAX_QUEUES];
 
     // A host-to-device copy costs ~4 us on top of its bytes even when it directly follows another one on
@@ -247,7 +255,9 @@ static nnv_status_t run_model(nnv_plan* p, const nnv_choice_t* choices, const vo
     // direction are served in the order they were submitted, whatever their streams)
     const nnv_layer_desc_t& L0 = p->layers[0];
     const float* in_chw = input;
-    if (host_io) {
+    // (with no weights to read the layout conversion takes the image in place from pinned memory: one launch less in front
+    // of the first layer; beside weight copies the copy engine moves it faster)
+    if (host_io && !(resident && host_blob_is_mapped(input))) {
         NNV_CUDA(cudaMemcpyAsync(base + A.in_chw, input, 4ull * L0.C * L0.H * L0.W, cudaMemcpyHostToDevice, s_exec));
         in_chw = (const float*)(base + A.in_chw);
     }
@@ -287,6 +297,7 @@ static nnv_status_t run_model(nnv_plan* p, const nnv_choice_t* choices, const vo
     }
 
     std::vector<int> conv_ids;
+    cudaEvent_t waited[2] = {nullptr, nullptr};               // the latest event s_exec / s_side waited for
     for (int i = 0; i < n; ++i) {
         const nnv_layer_desc_t& L = p->layers[i];
         const void* in = L.in0 < 0 ? base + A.in_hwc : base + A.act_off[L.in0];
@@ -300,7 +311,7 @@ static nnv_status_t run_model(nnv_plan* p, const nnv_choice_t* choices, const vo
             if (tm) NNV_CUDA(cudaEventRecord(TEV(i, 4), s_exec));
             NNV_TRY(do_pool(*p, i, in, out, s_exec));
             if (tm) NNV_CUDA(cudaEventRecord(TEV(i, 5), s_exec));
-            NNV_CUDA(cudaEventRecord(EV(i, 2), s_exec));
+            if (need_done[i]) NNV_CUDA(cudaEventRecord(EV(i, 2), s_exec));
             continue;
         }
         const nnv_choice_t ch = choices[i];
@@ -445,7 +456,11 @@ static nnv_status_t run_model(nnv_plan* p, const nnv_choice_t* choices, const vo
         }
 
         // execute
-        if (ready) NNV_CUDA(cudaStreamWaitEvent(se, ready, 0));
+        // (one wait serves all layers of a chunk on a stream: the event is the chunk's)
+        if (ready && ready != waited[on_side[i]]) {
+            NNV_CUDA(cudaStreamWaitEvent(se, ready, 0));
+            waited[on_side[i]] = ready;
+        }
         if (wait_warm && i < (int)p->warm_ev.size() && p->warm_ev[i]) NNV_CUDA(cudaStreamWaitEvent(se, p->warm_ev[i], 0));
         if (tm) NNV_CUDA(cudaEventRecord(TEV(i, 4), se));
         const void* add = L.in1 >= 0 ? base + A.act_off[L.in1] : nullptr;
@@ -454,7 +469,7 @@ static nnv_status_t run_model(nnv_plan* p, const nnv_choice_t* choices, const vo
                         base + A.ws_off, A.ws_bytes, se));
         next_stamp() = nullptr;
         if (tm) NNV_CUDA(cudaEventRecord(TEV(i, 5), se));
-        NNV_CUDA(cudaEventRecord(EV(i, 2), se));
+        if (need_done[i]) NNV_CUDA(cudaEventRecord(EV(i, 2), se));
         if (tm) {
             timings[i].h2d_bytes = copied;
             timings[i].xform_bytes = (has_xf && !cached) ? rbytes + tbytes : 0;
@@ -470,9 +485,12 @@ static nnv_status_t run_model(nnv_plan* p, const nnv_choice_t* choices, const vo
     // last layer's output: device NHWC -> NCHW
     const nnv_layer_desc_t& Ln = p->layers[n - 1];
     const LayerGeom& gn = p->geom[n - 1];
-    float* out_chw = host_io ? (float*)(base + A.out_chw) : output;
-    NNV_TRY(launch_hwc_to_chw((const float*)(base + A.act_off[n - 1]), out_chw, Ln.K, gn.OH, gn.OW, s_exec));
-    if (host_io) NNV_CUDA(cudaMemcpyAsync(output, out_chw, 4ull * gn.P * Ln.K, cudaMemcpyDeviceToHost, s_exec));
+    // Straight into the caller's buffer, also when that is pinned host memory, and the status word with it: the two copies
+    // this replaces cost ~5 us at the end of every run.
+    const bool out_direct = !host_io || host_blob_is_mapped(output);
+    float* out_chw = out_direct ? output : (float*)(base + A.out_chw);
+    NNV_TRY(launch_hwc_to_chw((const float*)(base + A.act_off[n - 1]), out_chw, Ln.K, gn.OH, gn.OW, s_exec, d_status, p->h_status));
+    if (!out_direct) NNV_CUDA(cudaMemcpyAsync(output, out_chw, 4ull * gn.P * Ln.K, cudaMemcpyDeviceToHost, s_exec));
     if (queued) {
         for (int j = 0; j < n_little; ++j) {
             NNV_CUDA(cudaEventRecord(p->ev[3 * n + 6 + j], s_prep[j]));
@@ -486,7 +504,6 @@ static nnv_status_t run_model(nnv_plan* p, const nnv_choice_t* choices, const vo
         NNV_CUDA(cudaEventRecord(p->ev[3 * n + 2], s_xform));
         NNV_CUDA(cudaStreamWaitEvent(s_exec, p->ev[3 * n + 2], 0));
     }
-    NNV_TRY(enqueue_status_read(p->h_status, s_exec));
     if (wc) {
         // K_warm - K_cold: behind everything the cold inference needs (the streams are idle from here
         // on, and s_exec no longer waits for them), read what was not read yet and transform it with
