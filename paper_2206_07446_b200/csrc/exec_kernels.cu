@@ -349,70 +349,66 @@ depthwise_kernel(const float* __restrict__ x, const float* __restrict__ w, const
     }
 }
 
-// 3x3 depthwise, stride 1 or 2, C % 4 == 0: one thread = four channels x four neighbouring output pixels of a row.
-// Every access is 16 bytes and a warp's accesses are 512 contiguous bytes (channel groups are the fastest index); the
-// (3 STRIDE + 3) x 3 input window is loaded once for the four outputs (18 loads instead of 36 at stride 1), and the
-// thread's 36 weights are nine 16-byte loads of the raw W[c][r][s] rows, rearranged in registers.
-template <int STRIDE>
+// 3x3 depthwise, stride 1 or 2, C % 4 == 0: one thread = four channels x PX neighbouring output pixels of a row (the input
+// window is loaded once for them).  A block takes `cg` channel quads (consecutive threads: contiguous 16-byte accesses) and as
+// many pixel groups as fill it; its raw weights W[c][r][s], one contiguous range, come through shared memory -- read by each
+// thread for itself, nine loads 144 bytes apart, they cost more cache lines than the activation.
+constexpr int DW_MAX_CG = 32;
+template <int STRIDE, int PX>
 __global__ void __launch_bounds__(256)
 depthwise3x3_v4_kernel(const float* __restrict__ x, const float* __restrict__ w, const float* __restrict__ bias,
-                       const float* __restrict__ add, float* __restrict__ y, int act, int C, int H, int W, int pad, int OH, int OW) {
+                       const float* __restrict__ add, float* __restrict__ y, int act, int C, int H, int W, int pad, int OH, int OW, int cg) {
     pdl_enter();
-    constexpr int NCOL = 3 * STRIDE + 3;
-    const int C4 = C >> 2, OW4 = (OW + 3) >> 2;
-    const long long n = (long long)OH * OW4 * C4;
-    for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < n; i += (long long)gridDim.x * 256) {
-        const int c4 = (int)(i % C4);
-        const long long pq = i / C4;
-        const int oq = (int)(pq % OW4), oh = (int)(pq / OW4);
-        const int c = c4 * 4, ow0 = oq * 4;
-        float wv[36];                                         // [channel 0..3][tap 0..8]
+    constexpr int NCOL = (PX - 1) * STRIDE + 3;
+    __shared__ __align__(16) float sw[DW_MAX_CG * 36];
+    const int C4 = C >> 2, OWP = (OW + PX - 1) / PX;
+    const int q0 = blockIdx.y * cg, nq = min(cg, C4 - q0);     // this block's channel quads
+    const int ppb = 256 / cg, lc = threadIdx.x % cg, lp = threadIdx.x / cg;
+    const int pg = blockIdx.x * ppb + lp;                      // pixel group
+    const bool live = lp < ppb && lc < nq && pg < OH * OWP;
+    const int oh = pg / OWP, ow0 = (pg - oh * OWP) * PX;
+    const int c = (q0 + lc) * 4;
+    const int ih0 = oh * STRIDE - pad, iw0 = ow0 * STRIDE - pad;
+    float4 v[3][NCOL];
 #pragma unroll
-        for (int j = 0; j < 9; ++j) {
-            const float4 t = __ldg(reinterpret_cast<const float4*>(w + (long long)c * 9) + j);
-            wv[4 * j] = t.x; wv[4 * j + 1] = t.y; wv[4 * j + 2] = t.z; wv[4 * j + 3] = t.w;
+    for (int r = 0; r < 3; ++r)
+#pragma unroll
+        for (int col = 0; col < NCOL; ++col) {
+            const int ih = ih0 + r, iw = iw0 + col;
+            v[r][col] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (live && ih >= 0 && ih < H && iw >= 0 && iw < W) v[r][col] = __ldg(reinterpret_cast<const float4*>(x + ((long long)ih * W + iw) * C + c));
         }
-        float4 acc[4];
-        const float4 b4 = bias ? __ldg(reinterpret_cast<const float4*>(bias + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int i = threadIdx.x; i < nq * 9; i += 256) reinterpret_cast<float4*>(sw)[i] = __ldg(reinterpret_cast<const float4*>(w + (long long)q0 * 36) + i);
+    __syncthreads();
+    if (!live) return;
+    float wv[36];                                             // [channel 0..3][tap 0..8]
 #pragma unroll
-        for (int p = 0; p < 4; ++p) acc[p] = b4;
-        const int iw0 = ow0 * STRIDE - pad;
+    for (int j = 0; j < 9; ++j) {
+        const float4 t = *reinterpret_cast<const float4*>(sw + lc * 36 + 4 * j);
+        wv[4 * j] = t.x; wv[4 * j + 1] = t.y; wv[4 * j + 2] = t.z; wv[4 * j + 3] = t.w;
+    }
+    const float4 b4 = bias ? __ldg(reinterpret_cast<const float4*>(bias + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int r = 0; r < 3; ++r) {
-            const int ih = oh * STRIDE + r - pad;
-            if (ih < 0 || ih >= H) continue;
-            const float* row = x + ((long long)ih * W) * C + c;
+    for (int p = 0; p < PX; ++p) {
+        const int ow = ow0 + p;
+        if (ow >= OW) break;
+        float4 o = b4;
 #pragma unroll
-            for (int col = 0; col < NCOL; ++col) {
-                const int iw = iw0 + col;
-                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (iw >= 0 && iw < W) v = __ldg(reinterpret_cast<const float4*>(row + (long long)iw * C));
+        for (int r = 0; r < 3; ++r)
 #pragma unroll
-                for (int p = 0; p < 4; ++p) {
-                    const int sft = col - p * STRIDE;         // the tap column this input column is for output p
-                    if (sft >= 0 && sft < 3) {
-                        const int t = r * 3 + sft;
-                        acc[p].x = fmaf(v.x, wv[t], acc[p].x);
-                        acc[p].y = fmaf(v.y, wv[9 + t], acc[p].y);
-                        acc[p].z = fmaf(v.z, wv[18 + t], acc[p].z);
-                        acc[p].w = fmaf(v.w, wv[27 + t], acc[p].w);
-                    }
-                }
+            for (int sx = 0; sx < 3; ++sx) {
+                const float4 t = v[r][p * STRIDE + sx];
+                const int k = r * 3 + sx;
+                o.x = fmaf(t.x, wv[k], o.x); o.y = fmaf(t.y, wv[9 + k], o.y);
+                o.z = fmaf(t.z, wv[18 + k], o.z); o.w = fmaf(t.w, wv[27 + k], o.w);
             }
+        const long long off = ((long long)oh * OW + ow) * C + c;
+        if (add) {
+            const float4 a4 = __ldg(reinterpret_cast<const float4*>(add + off));
+            o.x += a4.x; o.y += a4.y; o.z += a4.z; o.w += a4.w;
         }
-#pragma unroll
-        for (int p = 0; p < 4; ++p) {
-            const int ow = ow0 + p;
-            if (ow >= OW) break;
-            const long long o = ((long long)oh * OW + ow) * C + c;
-            float4 v = acc[p];
-            if (add) {
-                const float4 a4 = __ldg(reinterpret_cast<const float4*>(add + o));
-                v.x += a4.x; v.y += a4.y; v.z += a4.z; v.w += a4.w;
-            }
-            v.x = apply_act(v.x, act); v.y = apply_act(v.y, act); v.z = apply_act(v.z, act); v.w = apply_act(v.w, act);
-            *reinterpret_cast<float4*>(y + o) = v;
-        }
+        o.x = apply_act(o.x, act); o.y = apply_act(o.y, act); o.z = apply_act(o.z, act); o.w = apply_act(o.w, act);
+        *reinterpret_cast<float4*>(y + off) = o;
     }
 }
 
@@ -421,12 +417,17 @@ nnv_status_t launch_depthwise(const float* x, const float* w, const float* bias,
                               cudaStream_t st) {
     const bool al16 = ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(w) | reinterpret_cast<uintptr_t>(y) |
                         reinterpret_cast<uintptr_t>(bias) | reinterpret_cast<uintptr_t>(add)) & 15) == 0;
-    if (R == 3 && S == 3 && (stride == 1 || stride == 2) && (C % 4) == 0 && al16) {
-        const long long n4 = (long long)OH * ((OW + 3) / 4) * (C / 4);
-        const unsigned grid4 = (unsigned)std::min<long long>((n4 + 255) / 256, 148ll * 32);
-        if (stride == 1) NNV_LAUNCH((depthwise3x3_v4_kernel<1>), grid4, 256, 0, st, x, w, bias, add, y, act, C, H, W, pad, OH, OW);
-        else NNV_LAUNCH((depthwise3x3_v4_kernel<2>), grid4, 256, 0, st, x, w, bias, add, y, act, C, H, W, pad, OH, OW);
-        NNV_CUDA(cudaGetLastError());
+    if (R == 3 && S == 3 && (stride == 1 || stride == 2) && (C % 4) == 0 && al16 && (long long)OH * OW < (1 << 24) && C <= (1 << 22)) {
+        // Channel quads per block: even shares of at most 32.  Pixels per thread: four, fewer where that leaves SMs without a
+        // block (10 x 10 x 384: 12 blocks of 256 threads with four, 39 with one).
+        const int C4 = C / 4, cg = ceil_div(C4, ceil_div(C4, DW_MAX_CG)), ppb = 256 / cg;
+        auto grid_of = [&](int px) { return dim3(ceil_div(OH * ceil_div(OW, px), ppb), ceil_div(C4, cg)); };
+        int px = 4;
+        while (px > 1 && (long long)grid_of(px).x * grid_of(px).y < 148) px /= 2;
+        const dim3 grid = grid_of(px);
+        auto go = [&](auto kernel) { return launch_pdl(kernel, grid, dim3(256), 0, st, x, w, bias, add, y, act, C, H, W, pad, OH, OW, cg); };
+        if (stride == 1) NNV_CUDA(px == 4 ? go(depthwise3x3_v4_kernel<1, 4>) : px == 2 ? go(depthwise3x3_v4_kernel<1, 2>) : go(depthwise3x3_v4_kernel<1, 1>));
+        else NNV_CUDA(px == 4 ? go(depthwise3x3_v4_kernel<2, 4>) : px == 2 ? go(depthwise3x3_v4_kernel<2, 2>) : go(depthwise3x3_v4_kernel<2, 1>));
         return NNV_OK;
     }
     const long long n = (long long)OH * OW * C;
