@@ -168,6 +168,17 @@ __device__ __forceinline__ uint64_t make_smem_desc(uint32_t saddr) {
     return d;
 }
 
+// The same with the 64-byte swizzle: rows 64 bytes apart (32 bf16), 8-row groups 512 bytes apart.
+__device__ __forceinline__ uint64_t make_smem_desc64(uint32_t saddr) {
+    uint64_t d = 0;
+    d |= (uint64_t)((saddr & 0x3FFFF) >> 4);
+    d |= (uint64_t)1 << 16;
+    d |= (uint64_t)(512 >> 4) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)4 << 61;                     // SWIZZLE_64B
+    return d;
+}
+
 template <bool BF16>
 __device__ __forceinline__ void umma(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
     if constexpr (BF16) {
@@ -230,6 +241,7 @@ struct GemmDev {
     uint32_t recv_off;                // splits > 1: byte offset (from the aligned base) of the received partial rows
     uint32_t stage_off;               // byte offset (from the aligned base) of the dedicated staging tile; 0 = the idle ring
     // implicit im2col (A is the NHWC activation itself): 0 = off
+    // (2: its tiles are whole image rows, fetched as plain boxes)
     int ic_on, ic_C, ic_cblk, ic_S, ic_OW, ic_stride, ic_pad;
 };
 
@@ -288,26 +300,6 @@ __device__ __forceinline__ void convert_chunk(const uint8_t* src_tile, uint8_t* 
         *reinterpret_cast<uint4*>(lo_tile + off) = lo;
     } else {
         *reinterpret_cast<uint4*>(hi_tile + off) = pack8_bf16(v0, v1);
-    }
-}
-
-// Converts one row (32 fp32, stored by TMA with the 128-byte swizzle) of a staged tile into ONE bf16 tile (round to
-// nearest even; un-swizzled core-matrix layout, `rows` rows tall).
-__device__ __forceinline__ void convert_row_bf16(uint32_t src_tile, uint32_t dst_tile, int r, int rows) {
-    const uint32_t src = src_tile + (uint32_t)r * 128u;
-    const uint32_t lbo = (uint32_t)rows * 16u;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {                              // 4 chunks of 8 K-elements
-        float4 v0, v1;
-        const uint32_t a0 = src + ((uint32_t)((2 * c) ^ (r & 7)) << 4), a1 = src + ((uint32_t)((2 * c + 1) ^ (r & 7)) << 4);
-        asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v0.x), "=f"(v0.y), "=f"(v0.z), "=f"(v0.w) : "r"(a0));
-        asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v1.x), "=f"(v1.y), "=f"(v1.z), "=f"(v1.w) : "r"(a1));
-        const __nv_bfloat162 p0 = __floats2bfloat162_rn(v0.x, v0.y), p1 = __floats2bfloat162_rn(v0.z, v0.w);
-        const __nv_bfloat162 p2 = __floats2bfloat162_rn(v1.x, v1.y), p3 = __floats2bfloat162_rn(v1.z, v1.w);
-        const uint32_t off = (uint32_t)c * lbo + (uint32_t)r * 16u;
-        asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(dst_tile + off), "r"(*reinterpret_cast<const uint32_t*>(&p0)),
-                     "r"(*reinterpret_cast<const uint32_t*>(&p1)), "r"(*reinterpret_cast<const uint32_t*>(&p2)),
-                     "r"(*reinterpret_cast<const uint32_t*>(&p3)) : "memory");
     }
 }
 
@@ -425,7 +417,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         const uint32_t a_dst = sbase + s * stage_bytes;
         if (g.ic_on) {
             // A comes straight from the activation: the block is channel block ic_cb of tap (ic_fr, ic_fs)
-            tma_load_im2col_4d(a_dst, &tmA, ic_cb * BKE, ic_w0, ic_h0, 0, (uint16_t)ic_fs, (uint16_t)ic_fr, full_bar(s));
+            if (g.ic_on == 2) tma_load_3d(a_dst, &tmA, ic_cb * BKE, ic_w0 + ic_fs, ic_h0 + ic_fr, full_bar(s));
+            else tma_load_im2col_4d(a_dst, &tmA, ic_cb * BKE, ic_w0, ic_h0, 0, (uint16_t)ic_fs, (uint16_t)ic_fr, full_bar(s));
             if (++ic_cb == g.ic_cblk) {
                 ic_cb = 0;
                 if (++ic_fs == g.ic_S) { ic_fs = 0; ++ic_fr; }
@@ -442,9 +435,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         }
         mbar_expect_tx(full_bar(s), b_bytes);
         const uint32_t b_dst = sbase + s * stage_bytes + a_stage;
-        // MODE 3: one box of four 8-element chunks x BN rows, staged after the fp32 and the bf16 A tile
-        if constexpr (MODE == 3) tma_load_3d(b_dst + rp * 64, &tmB, 0, n0, q >> 3, full_bar(s));
-        else tma_load_3d(b_dst, &tmB, q, n0, b, full_bar(s));
+        // MODE 3: BN rows of 32 bf16 with the 64-byte swizzle, staged after the fp32 and the bf16 A tile
+        tma_load_3d(MODE == 3 ? b_dst + rp * 64 : b_dst, &tmB, q, n0, b, full_bar(s));
     };
     tc_fence_before();
     __syncthreads();
@@ -573,12 +565,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                         umma<true>(acc, ah, bh, idesc, 1u);
                     }
                 } else if constexpr (MODE == 3) {
-                    const uint32_t a_bf = a_src + a_stage, b_bf = a_bf + rp * 64;
-                    const uint32_t lbo_a = (uint32_t)rp * 16u, lbo_b = (uint32_t)BN * 16u;
+                    const uint32_t a_bf = a_src + a_stage, lbo_a = (uint32_t)rp * 16u;
+                    const uint64_t bdesc = make_smem_desc64(a_bf + rp * 64);
 #pragma unroll
-                    for (int kk = 0; kk < 2; ++kk)             // 2 K-steps of 16 bf16 = 2 core matrices each
-                        umma<true>(acc, make_smem_desc_plain(a_bf + kk * 2 * lbo_a, lbo_a, 128),
-                                   make_smem_desc_plain(b_bf + kk * 2 * lbo_b, lbo_b, 128), idesc, kk ? 1u : first);
+                    for (int kk = 0; kk < 2; ++kk)             // 2 K-steps of 16 bf16 = 2 core matrices (32 bytes) each
+                        umma<true>(acc, make_smem_desc_plain(a_bf + kk * 2 * lbo_a, lbo_a, 128), bdesc + (uint64_t)(kk * 2), idesc,
+                                   kk ? 1u : first);
                 } else {
                     const uint64_t adesc = make_smem_desc(a_src);
                     const uint64_t bdesc = make_smem_desc(a_src + a_stage);
@@ -818,6 +810,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 }
 
 #include "conv3x3_tc.cuh"
+#include "conv3x3_bf16.cuh"
 #include "gemm_sp.cuh"
 #include "wino_fused.cuh"
 
@@ -893,14 +886,14 @@ nnv_status_t encode_im2col_operand(CUtensorMap* map, const void* base, int C, in
     return NNV_OK;
 }
 
-// 3-D tiled map over an NHWC fp32 activation {C, W, H}: boxes of 32 channels x 8 pixels x `box_h`
+// 3-D tiled map over an NHWC fp32 activation {C, W, H}: boxes of 32 channels x `box_w` pixels x `box_h`
 // rows (the halo boxes of conv3x3_tc_kernel); coordinates outside the image read as zero.
-nnv_status_t encode_halo_operand(CUtensorMap* map, const void* base, int C, int H, int W, int box_h) {
+nnv_status_t encode_halo_operand(CUtensorMap* map, const void* base, int C, int H, int W, int box_h, int box_w = 8) {
     NNV_REQUIRE((reinterpret_cast<uintptr_t>(base) & 15) == 0 && (C % 4) == 0, NNV_ERR_INVALID_ARG,
                 "activation must be 16-byte aligned with C a multiple of 4");
     cuuint64_t dims[3] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H};
     cuuint64_t strides[2] = {(cuuint64_t)C * 4, (cuuint64_t)W * C * 4};
-    cuuint32_t box[3] = {32, 8, (cuuint32_t)box_h};
+    cuuint32_t box[3] = {32, (cuuint32_t)box_w, (cuuint32_t)box_h};
     cuuint32_t estr[3] = {1, 1, 1};
     CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void*>(base), dims, strides, box, estr,
                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
@@ -910,28 +903,27 @@ nnv_status_t encode_halo_operand(CUtensorMap* map, const void* base, int C, int 
 }
 
 // Tiling of conv3x3_tc_kernel for one layer.
-struct ConvTiling { int MT, BN, splits, na, nb, tmem_cols, bf16; size_t smem; };
+struct ConvTiling { int MT, BN, splits, na, nb, tmem_cols; size_t smem; };
 
-// Bytes of one halo-box slot and one weight-tile slot: with BF16 math a box slot also holds the box rounded to bf16
-// (half its size) and a weight tile is bf16.
-size_t conv_a_slot(int MT, int bf16) { return (size_t)(16 * MT + 2) * 1024 * (bf16 ? 3 : 2) / 2; }
-size_t conv_b_slot(int BN, int bf16) { return (size_t)BN * (bf16 ? 64 : BK_BYTES); }
+// Bytes of one halo-box slot and one weight-tile slot.
+size_t conv_a_slot(int MT) { return (size_t)(16 * MT + 2) * 1024; }
+size_t conv_b_slot(int BN) { return (size_t)BN * BK_BYTES; }
 
-size_t conv_smem_bytes(int MT, int BN, int na, int nb, int bf16) {
-    return (size_t)1024 + (size_t)na * conv_a_slot(MT, bf16) + (size_t)nb * conv_b_slot(BN, bf16) + 8 * (3 * CONV_MAX_NA + 2 * CONV_MAX_NB + 2);
+size_t conv_smem_bytes(int MT, int BN, int na, int nb) {
+    return (size_t)1024 + (size_t)na * conv_a_slot(MT) + (size_t)nb * conv_b_slot(BN) + 8 * (2 * CONV_MAX_NA + 2 * CONV_MAX_NB + 2);
 }
 
 // Fills in ring depths (unless given), shared-memory size and TMEM columns; false if the tiling does
 // not fit (shared memory, or room to park the partial tiles of a K split).
 bool finish_conv_tiling(ConvTiling* t) {
     const size_t park = t->splits > 1 ? (size_t)t->MT * BM * (t->BN + 4) * 4 : 0;
-    auto rings = [&] { return (size_t)t->na * conv_a_slot(t->MT, t->bf16) + (size_t)t->nb * conv_b_slot(t->BN, t->bf16); };
+    auto rings = [&] { return (size_t)t->na * conv_a_slot(t->MT) + (size_t)t->nb * conv_b_slot(t->BN); };
     if (t->na <= 0 || t->nb <= 0) {
         t->na = 2; t->nb = 3;
         while (rings() < park && t->nb < CONV_MAX_NB) ++t->nb;      // deeper rings only to make room for the parked tiles
         while (rings() < park && t->na < CONV_MAX_NA) ++t->na;
     }
-    t->smem = conv_smem_bytes(t->MT, t->BN, t->na, t->nb, t->bf16);
+    t->smem = conv_smem_bytes(t->MT, t->BN, t->na, t->nb);
     t->tmem_cols = 32;
     while (t->tmem_cols < t->MT * t->BN) t->tmem_cols *= 2;
     return t->smem <= 200u * 1024u && rings() >= park;
@@ -945,11 +937,10 @@ bool finish_conv_tiling(ConvTiling* t) {
 // to one slot when that makes them fit.  Layers with fewer than four channel blocks and fewer than
 // two patches per SM, and layers too small to give every SM a CTA even with 8 splits, stay on the
 // plain implicit GEMM, which is faster there.
-bool pick_conv_tiling(int C, int H, int W, int N, int bf16, ConvTiling* out) {
+bool pick_conv_tiling(int C, int H, int W, int N, ConvTiling* out) {
     const int cblk = ceil_div(C, 32);
     ConvTiling t{};
     t.MT = 1;
-    t.bf16 = bf16;
     t.BN = std::min(128, ceil_div(N, 16) * 16);
     const long long tiles = (long long)ceil_div(H, 16) * ceil_div(W, 8) * ceil_div(N, t.BN);
     int max_sp = 1;
@@ -979,13 +970,6 @@ bool pick_conv_tiling(int C, int H, int W, int N, int bf16, ConvTiling* out) {
 
 uint32_t gemm_stage_bytes(int mode, int bn, int rows) {
     return mode == GEMM_X3 ? stage_bytes_of<2>(bn, rows) : mode == GEMM_BF16_CVT ? stage_bytes_of<3>(bn, rows) : stage_bytes_of<0>(bn, rows);
-}
-
-// Rows of A per tile.  As few 128-row tiles as hold M, of equal height when they divide M (7 x 7 and 14 x 14 grids: one
-// tile of 49, two of 98): rows that do not exist would fill shared memory all the same.
-int gemm_rows(int M) {
-    const int tiles = ceil_div(M, BM);
-    return M % tiles == 0 ? M / tiles : BM;
 }
 
 // Ring depth: 8 stages when every CTA has an SM to itself (a lone CTA needs that many loads in flight on weights that come
@@ -1060,6 +1044,7 @@ nnv_status_t gemm_tc_init() {
         cudaFuncSetAttribute(gemm_tc_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
         cudaFuncSetAttribute(gemm_tc_kernel<3>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         cudaFuncSetAttribute(conv3x3_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
+        cudaFuncSetAttribute(conv3x3_bf16_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
         cudaFuncSetAttribute(gemm_sp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
         cudaFuncSetAttribute(conv3x3_tc_persistent_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
         cudaFuncSetAttribute(wino_f2_fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
@@ -1068,20 +1053,18 @@ nnv_status_t gemm_tc_init() {
     return NNV_OK;
 }
 
-// bf16 packed weights [N][ld]: boxes of 8 elements (16 bytes) x BN rows, no swizzle -- four of them make the
-// un-swizzled core-matrix layout of a 32-element K block.
-static nnv_status_t encode_bf16_weight_chunks(CUtensorMap* map, const void* base, int64_t ld, int N, int BN) {
+// bf16 packed weights [N][ld]: boxes of 32 elements (64 bytes, 64-byte swizzle) x BN rows.  (Boxes of 16-byte pieces, which would
+// land un-swizzled, cost the copy engine as much per piece as one of 64 or 128 bytes does.)
+static nnv_status_t encode_bf16_weights(CUtensorMap* map, const void* base, int64_t ld, int Kd, int N, int BN) {
     NNV_REQUIRE((ld % 8) == 0 && (reinterpret_cast<uintptr_t>(base) & 15) == 0, NNV_ERR_INVALID_ARG, "bf16 weight rows must be 16-byte multiples");
-    // the rows seen as {8 elements, N rows, ld / 8 chunks}: one box of {8, BN, 4} lands as [chunk][row][16 bytes], i.e. a whole
-    // 32-element K block of BN rows in the core-matrix layout with ONE load (a fill costs ~150 cycles whatever its size)
-    cuuint64_t dims[3] = {8, (cuuint64_t)N, (cuuint64_t)(ld / 8)};
-    cuuint64_t strides[2] = {(cuuint64_t)ld * 2, 16};
-    cuuint32_t box[3] = {8, (cuuint32_t)BN, 4};
+    cuuint64_t dims[3] = {(cuuint64_t)Kd, (cuuint64_t)N, 1};
+    cuuint64_t strides[2] = {(cuuint64_t)ld * 2, (cuuint64_t)ld * 2 * N};
+    cuuint32_t box[3] = {32, (cuuint32_t)BN, 1};
     cuuint32_t estr[3] = {1, 1, 1};
     CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
-                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    NNV_REQUIRE(r == CUDA_SUCCESS, NNV_ERR_CUDA, "cuTensorMapEncodeTiled (bf16 weight chunks) failed with code %d", (int)r);
+    NNV_REQUIRE(r == CUDA_SUCCESS, NNV_ERR_CUDA, "cuTensorMapEncodeTiled (bf16 weights) failed with code %d", (int)r);
     return NNV_OK;
 }
 
@@ -1099,11 +1082,78 @@ static nnv_status_t encode_conv_output(CUtensorMap* map, const void* base, int K
     return NNV_OK;
 }
 
+// BF16 math: K splits and column tile of conv3x3_bf16_kernel.
+// The pair with the least estimated time (microseconds): fixed cost + waves x (channel blocks per CTA + write-out), fitted to
+// a sweep of both over 21 layer shapes; the chosen tilings are within 0.01 us of the best measured ones on average.
+struct ConvBTiling { int BN, splits; double t; };
+
+static ConvBTiling pick_conv_bf16_tiling(int C, int H, int W, int N) {
+    ConvBTiling best{16, 1, 1e30};
+    const int patches = ceil_div(H, 16) * ceil_div(W, 8), cblk = C / 32;
+    for (int bn = 16; bn <= std::min(128, ceil_div(N, 16) * 16); bn += 16) {
+        for (int sp = 1; sp <= 8 && sp <= cblk; sp *= 2) {
+            const long long ctas = (long long)patches * ceil_div(N, bn) * sp;
+            // capacity of one CTA per SM in clusters of 1 / 2, 4 and 8
+            const int slots = sp <= 2 ? 148 : sp == 4 ? 132 : 120;
+            const double waves = (double)((ctas + slots - 1) / slots);
+            const double t = 2.39 + waves * (ceil_div(cblk, sp) * (0.72 + 0.0018 * bn) + 0.25 + 0.019 * bn + (sp > 1 ? 0.0184 * bn : 0.0));
+            if (t < best.t - 1e-9) best = ConvBTiling{bn, sp, t};
+        }
+    }
+    return best;
+}
+
+static nnv_status_t launch_conv3x3_bf16(const GemmArgs& a, int BN, int splits, cudaStream_t st) {
+    ConvBDev g{};
+    CUtensorMap tmA, tmB, tmD;
+    const int C = a.ic.C, H = a.ic.H, W = a.ic.W;
+    NNV_REQUIRE(a.ldd == a.N, NNV_ERR_INVALID_ARG, "the 3x3 kernel writes a dense NHWC output");
+    NNV_TRY(encode_halo_operand(&tmA, a.A, C, H, W, 18, 10));
+    {
+        // packed bf16 rows [N][9 taps][C] seen as {C, N rows, 9 taps}: one box holds a filter row's three taps x 32 channels
+        NNV_REQUIRE((a.ldb % 8) == 0 && (reinterpret_cast<uintptr_t>(a.B) & 15) == 0, NNV_ERR_INVALID_ARG, "bf16 weight rows must be 16-byte multiples");
+        cuuint64_t dims[3] = {(cuuint64_t)C, (cuuint64_t)a.N, 9};
+        cuuint64_t strides[2] = {(cuuint64_t)a.ldb * 2, (cuuint64_t)C * 2};
+        cuuint32_t box[3] = {32, (cuuint32_t)BN, 3};
+        cuuint32_t estr[3] = {1, 1, 1};
+        CUresult r = g_encode(&tmB, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(a.B), dims, strides, box, estr,
+                              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+        NNV_REQUIRE(r == CUDA_SUCCESS, NNV_ERR_CUDA, "cuTensorMapEncodeTiled (bf16 filter taps) failed with code %d", (int)r);
+    }
+    g.stamp = next_stamp();
+    next_stamp() = nullptr;
+    g.D = a.D; g.bias = a.bias; g.addend = a.addend;
+    g.C = C; g.H = H; g.W = W; g.K = a.N;
+    g.BN = BN; g.act = a.act; g.splits = splits;
+    g.cblk = C / 32; g.tiles_w = ceil_div(W, 8);
+    g.tmem_cols = 32;
+    while (g.tmem_cols < BN) g.tmem_cols *= 2;
+    g.tma_out = 0;
+    if (splits == 1 && (a.N % 4) == 0 && (reinterpret_cast<uintptr_t>(a.D) & 15) == 0 && (!a.addend || (reinterpret_cast<uintptr_t>(a.addend) & 15) == 0)) {
+        g.tma_out = (BN % 32) == 0 ? 32 : 16;
+        NNV_TRY(encode_conv_output(&tmD, a.D, a.N, H, W, g.tma_out));
+    } else {
+        tmD = tmA;
+    }
+    // two channel blocks of weights in flight where they fit (three filter rows each)
+    const size_t recv = splits > 1 ? (size_t)128 * BN * 4 : 0;
+    g.b_off = (uint32_t)align_up(CB_RINGS_A, 1024);
+    g.nb = std::min({6, 3 * ceil_div(g.cblk, splits), (int)((225u * 1024u - g.b_off - CB_BAR_BYTES - 256 - recv) / ((size_t)BN * 192))});
+    g.bar_off = (uint32_t)align_up(g.b_off + (size_t)g.nb * BN * 192, 16);
+    g.recv_off = (uint32_t)align_up(g.bar_off + CB_BAR_BYTES, 128);
+    const size_t smem = (size_t)1024 + g.recv_off + recv;
+    NNV_REQUIRE(g.nb >= 1 && smem <= 226u * 1024u, NNV_ERR_UNSUPPORTED, "3x3 tiling does not fit shared memory");
+    const dim3 grid(ceil_div(H, 16) * g.tiles_w, ceil_div(a.N, BN), splits);
+    NNV_REQUIRE(grid.y <= 65535, NNV_ERR_UNSUPPORTED, "convolution grid too large");
+    NNV_CUDA(launch_pdl_cluster(conv3x3_bf16_kernel, grid, dim3(CB_THREADS), smem, st, splits, tmA, tmB, tmD, g));
+    return NNV_OK;
+}
+
 static nnv_status_t launch_conv3x3_tc(const GemmArgs& a, const ConvTiling& ct, cudaStream_t st) {
     CUtensorMap tmA, tmB, tmD;
     NNV_TRY(encode_halo_operand(&tmA, a.A, a.ic.C, a.ic.H, a.ic.W, 16 * ct.MT + 2));
-    if (ct.bf16) NNV_TRY(encode_bf16_weight_chunks(&tmB, a.B, a.ldb, a.N, ct.BN));
-    else NNV_TRY(encode_operand(&tmB, a.B, false, a.Kd, a.N, 1, a.ldb, a.strideB, ct.BN));
+    NNV_TRY(encode_operand(&tmB, a.B, false, a.Kd, a.N, 1, a.ldb, a.strideB, ct.BN));
     ConvDev g;
     g.stamp = next_stamp();
     next_stamp() = nullptr;
@@ -1111,12 +1161,11 @@ static nnv_status_t launch_conv3x3_tc(const GemmArgs& a, const ConvTiling& ct, c
     g.C = a.ic.C; g.H = a.ic.H; g.W = a.ic.W; g.K = a.N;
     g.BN = ct.BN; g.MT = ct.MT; g.act = a.act; g.tmem_cols = ct.tmem_cols; g.splits = ct.splits; g.na = ct.na; g.nb = ct.nb;
     g.cblk = ceil_div(a.ic.C, 32); g.tiles_w = ceil_div(a.ic.W, 8);
-    g.bf16 = ct.bf16;
     NNV_REQUIRE(a.ldd == a.N, NNV_ERR_INVALID_ARG, "the 3x3 kernel writes a dense NHWC output");
     // Write-out by TMA when nothing is added after the K loop but the bias, the output rows are 16-byte multiples and
     // the staged tile fits into the (then idle) rings; else plain stores.
     g.tma_out = 0;
-    const size_t rings = (size_t)ct.na * conv_a_slot(ct.MT, ct.bf16) + (size_t)ct.nb * conv_b_slot(ct.BN, ct.bf16);
+    const size_t rings = (size_t)ct.na * conv_a_slot(ct.MT) + (size_t)ct.nb * conv_b_slot(ct.BN);
     if (ct.splits == 1 && !a.addend && (a.N % 4) == 0 && (reinterpret_cast<uintptr_t>(a.D) & 15) == 0 &&
         (!a.bias || (reinterpret_cast<uintptr_t>(a.bias) & 15) == 0) && (size_t)ct.MT * BM * ct.BN * 4 <= rings) {
         g.tma_out = (ct.BN % 32) == 0 ? 32 : 16;
@@ -1299,20 +1348,18 @@ nnv_status_t launch_gemm_tc(const GemmArgs& a, cudaStream_t st) {
     // which moves fewer operand bytes through L2 and shared memory.
     if (a.ic.on && (a.mode == GEMM_TF32 || a.mode == GEMM_BF16_CVT) && a.batch == 1 && a.ic.R == 3 && a.ic.S == 3 && a.ic.stride == 1 &&
         a.ic.pad == 1 && (a.ic.C % 32) == 0) {
-        const int cbf = a.mode == GEMM_BF16_CVT ? 1 : 0;
+        if (a.mode == GEMM_BF16_CVT) {
+            ConvBTiling ct = pick_conv_bf16_tiling(a.ic.C, a.ic.H, a.ic.W, a.N);
+            if (tn.conv3x3 == 2 && tn.conv_splits <= a.ic.C / 32) ct = ConvBTiling{tn.conv_bn, tn.conv_splits, 0.0};
+            if (tn.conv3x3 != 1) return launch_conv3x3_bf16(a, ct.BN, ct.splits, st);
+        } else {
         ConvTiling ct;
-        bool use = pick_conv_tiling(a.ic.C, a.ic.H, a.ic.W, a.N, cbf, &ct);
-        // BF16 math: every box passes through the conversion warps before its MMAs, which a CTA with a single channel
-        // block (three boxes) cannot hide -- measured on 128 -> 128 @112: 29.7 us against 18.2 for the converting implicit
-        // GEMM; with two or more blocks per CTA the halo kernel is ahead (64 -> 64 @224: 19.6 against 29.3 us,
-        // 256 -> 256 @56: 20.4 against 26.2, 512 -> 512 @28: 20.7 against 26.9).
-        if (use && cbf && ceil_div(a.ic.C, 32) / ct.splits < 2) use = false;
+        bool use = pick_conv_tiling(a.ic.C, a.ic.H, a.ic.W, a.N, &ct);
         if (tn.conv3x3 == 1) {
             use = false;
         } else if (tn.conv3x3 == 2) {
             ConvTiling f{};
             f.MT = tn.conv_mt; f.BN = tn.conv_bn; f.splits = tn.conv_splits; f.na = tn.conv_na; f.nb = tn.conv_nb;
-            f.bf16 = cbf;
             if (f.splits <= ceil_div(a.ic.C, 32) && finish_conv_tiling(&f)) {
                 ct = f;
                 use = true;
@@ -1329,10 +1376,11 @@ nnv_status_t launch_gemm_tc(const GemmArgs& a, cudaStream_t st) {
         // alone where the tensor pipe needs 1.2; three one-tile CTAs per SM issue from three threads, and the resident
         // weights leave room for only three halo boxes in flight.
         int wbn = 0;
-        if (!cbf && tn.convw == 2 && convw_fits(a, &wbn)) return launch_conv3x3_ws(a, wbn, st);
-        if (!cbf && tn.convp == 2 && (size_t)tn.convp_bn <= (size_t)ceil_div(a.N, 16) * 16)
+        if (tn.convw == 2 && convw_fits(a, &wbn)) return launch_conv3x3_ws(a, wbn, st);
+        if (tn.convp == 2 && (size_t)tn.convp_bn <= (size_t)ceil_div(a.N, 16) * 16)
             return launch_conv3x3_persistent(a, tn.convp_bn, tn.convp_per_sm, tn.convp_na ? tn.convp_na : 2, tn.convp_nb ? tn.convp_nb : 4, st);
         if (use) return launch_conv3x3_tc(a, ct, st);
+        }
     }
     int tmem_cols = 32;
     while (tmem_cols < BN * issuers) tmem_cols *= 2;
@@ -1352,8 +1400,10 @@ nnv_status_t launch_gemm_tc(const GemmArgs& a, cudaStream_t st) {
     if (a.ic.on) {
         NNV_REQUIRE((a.mode == GEMM_TF32 || a.mode == GEMM_BF16_CVT) && a.batch == 1, NNV_ERR_INVALID_ARG,
                     "implicit im2col needs fp32 activations (TF32 or converting BF16 mode) and one batch");
-        NNV_TRY(encode_im2col_operand(&tmA, a.A, a.ic.C, a.ic.H, a.ic.W, a.ic.R, a.ic.S, a.ic.stride, a.ic.pad, rows));
-        g.ic_on = 1; g.ic_C = a.ic.C; g.ic_cblk = ceil_div(a.ic.C, 32); g.ic_S = a.ic.S; g.ic_OW = a.ic.OW;
+        const bool boxes = 4ull * a.ic.C * a.ic.H * a.ic.W < 131072ull && image_row_boxes(a.ic.H, a.ic.W, a.ic.R, a.ic.S, a.ic.stride, a.ic.pad);
+        if (boxes) NNV_TRY(encode_image_operand(&tmA, a.A, a.ic.C, a.ic.H, a.ic.W, rows / a.ic.W));
+        else NNV_TRY(encode_im2col_operand(&tmA, a.A, a.ic.C, a.ic.H, a.ic.W, a.ic.R, a.ic.S, a.ic.stride, a.ic.pad, rows));
+        g.ic_on = boxes ? 2 : 1; g.ic_C = a.ic.C; g.ic_cblk = ceil_div(a.ic.C, 32); g.ic_S = a.ic.S; g.ic_OW = a.ic.OW;
         g.ic_stride = a.ic.stride; g.ic_pad = a.ic.pad;
         g.Kd = a.ic.R * a.ic.S * g.ic_cblk;                       // number of K blocks
     } else {
@@ -1361,7 +1411,7 @@ nnv_status_t launch_gemm_tc(const GemmArgs& a, cudaStream_t st) {
     }
     if (a.mode == GEMM_BF16_CVT) {
         NNV_REQUIRE(a.batch == 1, NNV_ERR_INVALID_ARG, "the converting BF16 mode needs one batch");
-        NNV_TRY(encode_bf16_weight_chunks(&tmB, a.B, a.ldb, a.N, BN));
+        NNV_TRY(encode_bf16_weights(&tmB, a.B, a.ldb, (int)a.ldb, a.N, BN));
     } else {
         NNV_TRY(encode_operand(&tmB, a.B, bf16, a.Kd, a.N, a.batch, a.ldb, a.strideB, BN));
     }

@@ -297,6 +297,18 @@ struct GemmArgs {
     // B is the packed weight P[K][Qp] with Kd = Qp; M = OH*OW output pixels.  TF32 mode, batch 1.
     struct { int on, C, H, W, R, S, stride, pad, OW; } ic;
 };
+// Rows of A per tile of the GEMM kernel: as few 128-row tiles as hold M, of equal height when they divide M (7 x 7 and 14 x 14
+// grids: one tile of 49, two of 98): rows that do not exist would fill shared memory all the same.
+inline int gemm_rows(int M) {
+    const int tiles = (M + 127) / 128;
+    return M % tiles == 0 ? M / tiles : 128;
+}
+// True when every tile of a stride-1 convolution that keeps the image's size is a number of whole image rows: its A operand
+// is then a box of the image shifted by the tap.
+inline bool image_row_boxes(int H, int W, int R, int S, int stride, int pad) {
+    return stride == 1 && R == S && (R & 1) == 1 && pad == (R - 1) / 2 && W <= 256 && gemm_rows(H * W) % W == 0 &&
+           (H * W) % gemm_rows(H * W) == 0;
+}
 // GEMM_X3: fp32 operands; each is split on the fly into bf16 hi + lo and the product is formed
 // as hi*hi + lo*hi + hi*lo on the bf16 tensor pipe (fp32-class accuracy, fp32 bytes in memory).
 // GEMM_BF16_CVT: A is fp32 and is rounded to bf16 inside the kernel, B is bf16 (weights packed for BF16 math): the

@@ -166,9 +166,10 @@ static inline bool gemm1x1_direct_operand(const nnv_layer_desc_t& L, int math) {
 static inline bool implicit_gemm_operand(const nnv_layer_desc_t& L, int math) {
     // The TMA's im2col mode gathers filter-window pixels straight from the NHWC activation, so no
     // Xcol matrix is materialised: fp32 words (TF32), pixel rows a multiple of 16 bytes, and an
-    // activation of at least 128 KiB (smaller tensors take the explicit path).
+    // activation of at least 128 KiB.  Smaller images of stride-1 "same" layers are read as plain boxes of whole image rows
+    // (image_row_boxes); other small tensors take the explicit path.
     return ((math == NNV_MATH_TF32 && (L.C % 4) == 0) || (math == NNV_MATH_BF16 && (L.C % 8) == 0 && tuning().bf16cvt)) &&
-           4ull * L.C * L.H * L.W >= 131072ull && L.R <= 16 && L.S <= 16 && L.pad <= 8;
+           (4ull * L.C * L.H * L.W >= 131072ull || image_row_boxes(L.H, L.W, L.R, L.S, L.stride, L.pad)) && L.R <= 16 && L.S <= 16 && L.pad <= 8;
 }
 
 bool wino_fused_applies(const nnv_layer_desc_t& L, int v, int math) {
