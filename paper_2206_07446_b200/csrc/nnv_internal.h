@@ -248,7 +248,7 @@ struct XformDesc {
     int host_src;                    // src is pinned host memory read in place
 };
 constexpr int XF_BATCH_MAX = 56;
-struct XformBatch { unsigned long long* stamp; int n; int total_blocks; int host_src; XformDesc d[XF_BATCH_MAX]; };
+struct XformBatch { unsigned long long* stamp; int n; int total_blocks; int host_src; int follows; XformDesc d[XF_BATCH_MAX]; };
 nnv_status_t launch_transform_batch(XformDesc* descs, int n, cudaStream_t st);
 
 // Explicit im2col of an NHWC fp32 image: Xcol[P][Qp], q = (r*S+s)*C + c (fp32 or bf16).

@@ -44,71 +44,49 @@ template <> struct WinoG<6> {
     }
 };
 
-template <typename OutT, int NF> struct VecStore;
-template <> struct VecStore<float, 1> {
-    __device__ static void st(float* p, const float* v) { *p = v[0]; }
-};
-template <> struct VecStore<float, 2> {
-    __device__ static void st(float* p, const float* v) { *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]); }
-};
-template <> struct VecStore<float, 4> {
-    __device__ static void st(float* p, const float* v) {
-        *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
-    }
-};
-template <> struct VecStore<__nv_bfloat16, 2> {
-    __device__ static void st(__nv_bfloat16* p, const float* v) {
-        *reinterpret_cast<__nv_bfloat162*>(p) = __floats2bfloat162_rn(v[0], v[1]);
-    }
-};
-template <> struct VecStore<__nv_bfloat16, 4> {
-    __device__ static void st(__nv_bfloat16* p, const float* v) {
-        __nv_bfloat162 a = __floats2bfloat162_rn(v[0], v[1]);
-        __nv_bfloat162 b = __floats2bfloat162_rn(v[2], v[3]);
-        uint2 u;
-        u.x = *reinterpret_cast<uint32_t*>(&a);
-        u.y = *reinterpret_cast<uint32_t*>(&b);
-        *reinterpret_cast<uint2*>(p) = u;
-    }
-};
+// Four consecutive values of a plane: 16 bytes of fp32, 8 of bf16.
+__device__ __forceinline__ void store_plane4(float* p, const float* v) { *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]); }
+__device__ __forceinline__ void store_plane4(__nv_bfloat16* p, const float* v) {
+    __nv_bfloat162 a = __floats2bfloat162_rn(v[0], v[1]);
+    __nv_bfloat162 b = __floats2bfloat162_rn(v[2], v[3]);
+    uint2 u;
+    u.x = *reinterpret_cast<uint32_t*>(&a);
+    u.y = *reinterpret_cast<uint32_t*>(&b);
+    *reinterpret_cast<uint2*>(p) = u;
+}
 
-template <> struct VecStore<__nv_bfloat16, 8> {
-    __device__ static void st(__nv_bfloat16* p, const float* v) {
-        __nv_bfloat162 a = __floats2bfloat162_rn(v[0], v[1]), b = __floats2bfloat162_rn(v[2], v[3]);
-        __nv_bfloat162 c = __floats2bfloat162_rn(v[4], v[5]), d = __floats2bfloat162_rn(v[6], v[7]);
-        uint4 u;
-        u.x = *reinterpret_cast<uint32_t*>(&a);
-        u.y = *reinterpret_cast<uint32_t*>(&b);
-        u.z = *reinterpret_cast<uint32_t*>(&c);
-        u.w = *reinterpret_cast<uint32_t*>(&d);
-        *reinterpret_cast<uint4*>(p) = u;
-    }
-};
+// Shape of the filter transforms: threads of a block, filters (padded (k, c) pairs) of a thread, and the resident blocks
+// the registers are budgeted for.  The kernels stream (36 bytes of filter in, 4 alpha^2 out), so what counts is how many
+// warps an SM holds to keep loads and stores in flight.  The inner product is taken one column (nu) at a time, so that a
+// thread keeps its raw filters (9 words each) and three words of intermediate instead of 3 alpha: F(6,3) then runs in 64
+// registers, 32 warps an SM, where 84 held it to 16.  F(2,3) takes four filters a thread (16-byte fp32 stores; eight, for
+// 16-byte bf16 stores, need 128 registers: 512 -> 512 5.4 us against 4.0); the others two, which a pair of lanes turns
+// into 16-byte stores by exchanging halves: of every pair of planes the even lane stores one plane for both lanes'
+// filters and the odd lane the other (four filters a thread: 512 -> 512 F(6,3) 19.4 us against 14.5).
+// Whole models, cold L2, before / after with the staging below (us): ResNet-50-shaped F(6,3) 87 / 69, F(4,3) 101 / 52,
+// F(2,3) 81 / 42 (bf16 75 / 36); VGG-16-shaped F(4,3) 126 / 50.
+__host__ __device__ constexpr int ft_threads(int m) { return m == 2 ? 256 : 128; }
+__host__ __device__ constexpr int ft_per_thread(int m) { return m == 2 ? 4 : 2; }
+__host__ __device__ constexpr int ft_resident(int m) { return m == 2 ? 3 : 8; }
+__host__ __device__ constexpr int ft_filters(int m) { return ft_threads(m) * ft_per_thread(m); }
 
-constexpr int FT_THREADS = 256;
-constexpr int FT_FILTERS = 1024;                                // most filters (padded (k, c) pairs) a block takes
-// Filters of one block: every thread busy, at most FT_FILTERS (which the shared staging buffer holds).
-__host__ __device__ constexpr int ft_filters(int nf) { return FT_THREADS * nf > FT_FILTERS ? FT_FILTERS : FT_THREADS * nf; }
-// Filters per thread.  F(2x2,3x3): as many as make every store of a thread 16 bytes wide (4 fp32 or 8 bf16
-// values).  F(4x4,3x3) and F(6x6,3x3) keep 2 -- four filters' intermediates need 128 registers and halve the
-// resident warps (measured: 1024^2 filters 47 us against 41) -- and reach 16-byte stores by exchanging halves
-// between neighbouring lanes: of every pair of planes the even lane stores one plane for both lanes' filters
-// and the odd lane the other.
-template <int M_, typename OutT> struct FtNF { static constexpr int value = (M_ == 2) ? 4 : 2; };
-template <int M_> struct FtNF<M_, __nv_bfloat16> { static constexpr int value = (M_ == 2) ? 8 : 2; };
+// 16 bytes from global to shared memory without a register in between: a block's whole range is in flight at once,
+// whatever its register budget (staged through registers: 512 -> 512 F(2,3) 7.8 us against 5.4, repack 5.9 against 5.3).
+__device__ __forceinline__ void stage16(void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void stage_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// One thread transforms NF filters that are adjacent in the padded channel index, so that each of the alpha^2
-// output planes receives one NF-wide (16-byte) vector store per thread and a warp writes 32*NF consecutive
-// elements of the plane.  A block covers FT_FILTERS filters with FT_FILTERS / NF of its threads.  With C == Cp
-// the block's raw filters are one contiguous range, staged through shared memory with 128-bit loads by all
-// threads and read back with 128-bit loads (a thread's NF * 9 floats start on a 16-byte boundary; the eight
-// threads of a quarter warp then touch all 32 banks once).
-template <int M_, typename OutT, int NF>
+// One thread transforms NF filters that are adjacent in the padded channel index, so that a warp writes consecutive
+// elements of each of the alpha^2 output planes in 16-byte pieces.  With C == Cp
+// the block's raw filters are one contiguous range, staged through shared memory by all
+// threads and read back with 64- or 128-bit loads (a thread's NF * 9 floats start on such a boundary).
+template <int M_, typename OutT>
 __device__ __forceinline__ void filter_transform_block(const float* __restrict__ g, OutT* __restrict__ U, int K, int C,
                                                        int Cp, unsigned block, float* sg, bool late_wait) {
     constexpr int A = WinoG<M_>::A;
-    constexpr int FPB = ft_filters(NF);                          // filters of this block
-    constexpr int ACTIVE = FPB / NF;                              // threads that transform
+    constexpr int THREADS = ft_threads(M_), NF = ft_per_thread(M_);
+    constexpr int FPB = ft_filters(M_);                          // filters of this block
     const long long F = (long long)K * Cp;                      // padded filter count = plane size
     const long long f_block = (long long)block * FPB;
     const long long f0 = f_block + (long long)threadIdx.x * NF;
@@ -120,15 +98,16 @@ __device__ __forceinline__ void filter_transform_block(const float* __restrict__
         const float4* src = reinterpret_cast<const float4*>(g + base);
         float4* dst = reinterpret_cast<float4*>(sg);
         constexpr int NV = FPB * 9 / 4;
-        for (int i = threadIdx.x; i < NV; i += FT_THREADS) {
-            if (base + 4ll * i < total) dst[i] = __ldg(src + i);
-        }
+#pragma unroll
+        for (int i = threadIdx.x; i < NV; i += THREADS)
+            if (base + 4ll * i < total) stage16(dst + i, src + i);
+        stage_wait();
         __syncthreads();
     }
     // Weights read in place from host memory do not depend on the previous kernel of the stream: those loads were
     // issued above, before this wait (which then only orders the stores below).
     if (late_wait) pdl_wait();
-    if ((int)threadIdx.x >= ACTIVE || f0 >= F) return;
+    if (f0 >= F) return;
 
     float w[NF][9];
     bool pad[NF];
@@ -166,83 +145,82 @@ __device__ __forceinline__ void filter_transform_block(const float* __restrict__
         }
     }
 
-    // t[i][nu] = sum_j g[i][j] * G[nu][j]
-    float t[NF][3][A];
-#pragma unroll
-    for (int j = 0; j < NF; ++j)
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int nu = 0; nu < A; ++nu)
-                t[j][i][nu] = w[j][i * 3 + 0] * WinoG<M_>::g(nu, 0) + w[j][i * 3 + 1] * WinoG<M_>::g(nu, 1) +
-                              w[j][i * 3 + 2] * WinoG<M_>::g(nu, 2);
-
-    // U[xi][nu] = sum_i G[xi][i] * t[i][nu]; plane xi*A+nu, element f0..f0+NF-1
+    // U[xi][nu] = sum_i G[xi][i] * (sum_j g[i][j] * G[nu][j]); plane xi*A+nu, element f0..f0+NF-1
     OutT* out = U + f0;
-    auto plane_values = [&](int xi, int nu, float* v) {
+    auto column = [&](int nu, float (&t)[NF][3]) {
+#pragma unroll
+        for (int j = 0; j < NF; ++j)
+#pragma unroll
+            for (int i = 0; i < 3; ++i)
+                t[j][i] = w[j][i * 3 + 0] * WinoG<M_>::g(nu, 0) + w[j][i * 3 + 1] * WinoG<M_>::g(nu, 1) +
+                          w[j][i * 3 + 2] * WinoG<M_>::g(nu, 2);
+    };
+    auto plane_values = [&](int xi, const float (&t)[NF][3], float* v) {
 #pragma unroll
         for (int j = 0; j < NF; ++j) {
-            v[j] = WinoG<M_>::g(xi, 0) * t[j][0][nu] + WinoG<M_>::g(xi, 1) * t[j][1][nu] + WinoG<M_>::g(xi, 2) * t[j][2][nu];
+            v[j] = WinoG<M_>::g(xi, 0) * t[j][0] + WinoG<M_>::g(xi, 1) * t[j][1] + WinoG<M_>::g(xi, 2) * t[j][2];
             if (pad[j]) v[j] = 0.f;                              // padded channels hold +0, never -0
         }
     };
-    if constexpr (NF == 2 && sizeof(OutT) == 4) {
+    if constexpr (NF == 2) {
         // pairs of planes (A is even): lanes 2i and 2i+1 hold four adjacent filters between them (the plane size is a
         // multiple of 8, so both are live or neither); each sends the partner its two values of the plane the partner stores
         const unsigned live = __activemask();
         const bool odd = (threadIdx.x & 1) != 0;
+        OutT* lane_out = odd ? out + F - 2 : out;
 #pragma unroll
-        for (int xi = 0; xi < A; ++xi) {
+        for (int nu = 0; nu < A; nu += 2) {
+            float tp[NF][3], tq[NF][3];
+            column(nu, tp);
+            column(nu + 1, tq);
 #pragma unroll
-            for (int nu = 0; nu < A; nu += 2) {
+            for (int xi = 0; xi < A; ++xi) {
                 float vp[2], vq[2];
-                plane_values(xi, nu, vp);
-                plane_values(xi, nu + 1, vq);
+                plane_values(xi, tp, vp);
+                plane_values(xi, tq, vq);
                 const float s0 = __shfl_xor_sync(live, odd ? vp[0] : vq[0], 1);
                 const float s1 = __shfl_xor_sync(live, odd ? vp[1] : vq[1], 1);
                 float v4[4];
                 if (!odd) { v4[0] = vp[0]; v4[1] = vp[1]; v4[2] = s0; v4[3] = s1; }
                 else { v4[0] = s0; v4[1] = s1; v4[2] = vq[0]; v4[3] = vq[1]; }
-                OutT* dst = out + (long long)(xi * A + nu + (odd ? 1 : 0)) * F - (odd ? 2 : 0);
-                VecStore<OutT, 4>::st(dst, v4);
+                store_plane4(lane_out + (long long)(xi * A + nu) * F, v4);
             }
         }
     } else {
 #pragma unroll
-        for (int xi = 0; xi < A; ++xi) {
+        for (int nu = 0; nu < A; ++nu) {
+            float t[NF][3];
+            column(nu, t);
 #pragma unroll
-            for (int nu = 0; nu < A; ++nu) {
+            for (int xi = 0; xi < A; ++xi) {
                 float v[NF];
-                plane_values(xi, nu, v);
-                VecStore<OutT, NF>::st(out + (long long)(xi * A + nu) * F, v);
+                plane_values(xi, t, v);
+                store_plane4(out + (long long)(xi * A + nu) * F, v);
             }
         }
     }
 }
 
-constexpr int XF_SMEM_FLOATS = FT_FILTERS * 9;                   // 36 KB staging buffer shared by all transform kernels
-
-template <int M_, typename OutT, int NF>
-__global__ void __launch_bounds__(FT_THREADS)
+template <int M_, typename OutT>
+__global__ void __launch_bounds__(ft_threads(M_), ft_resident(M_))
 filter_transform_kernel(const float* __restrict__ g, OutT* __restrict__ U, int K, int C, int Cp, unsigned long long* stamp,
                         int host_src) {
     pdl_trigger();
     if (!host_src) pdl_wait();
     if (threadIdx.x == 0) stamp_start(stamp);
-    __shared__ __align__(16) float sg[XF_SMEM_FLOATS];
-    filter_transform_block<M_, OutT, NF>(g, U, K, C, Cp, blockIdx.x, sg, host_src != 0);
+    __shared__ __align__(16) float sg[ft_filters(M_) * 9];
+    filter_transform_block<M_, OutT>(g, U, K, C, Cp, blockIdx.x, sg, host_src != 0);
     __syncthreads();
     if (threadIdx.x == 0) stamp_end(stamp);
 }
 
 template <int M_, typename OutT>
 static nnv_status_t launch_ft(const float* g, void* U, int K, int C, int Cp, cudaStream_t st, bool host_src) {
-    constexpr int NF = FtNF<M_, OutT>::value;
     const long long F = (long long)K * Cp;
-    const unsigned grid = (unsigned)((F + ft_filters(NF) - 1) / ft_filters(NF));
+    const unsigned grid = (unsigned)((F + ft_filters(M_) - 1) / ft_filters(M_));
     unsigned long long* stamp = next_stamp();
     next_stamp() = nullptr;
-    NNV_LAUNCH((filter_transform_kernel<M_, OutT, NF>), grid, FT_THREADS, 0, st, g, reinterpret_cast<OutT*>(U), K, C, Cp, stamp,
+    NNV_LAUNCH((filter_transform_kernel<M_, OutT>), grid, ft_threads(M_), 0, st, g, reinterpret_cast<OutT*>(U), K, C, Cp, stamp,
                host_src ? 1 : 0);
     NNV_CUDA(cudaGetLastError());
     return NNV_OK;
@@ -275,7 +253,7 @@ template <> __device__ inline float cvt_out<float>(float v) { return round_tf32(
 template <> __device__ inline __nv_bfloat16 cvt_out<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
 
 constexpr int PACK_THREADS = 256;
-constexpr int PACK_SMEM_FLOATS = XF_SMEM_FLOATS;
+constexpr int PACK_SMEM_FLOATS = 9216;                           // 36 KB staging buffer: 1024 3x3 filters
 constexpr int PACK1X1_PER_BLOCK = PACK_THREADS * 16;            // elements of P one block of pack1x1 writes
 
 template <typename OutT> __device__ __forceinline__ void store4(OutT* p, float a, float b, float c, float d);
@@ -321,7 +299,8 @@ __device__ __forceinline__ void pack_fast_block(const float* __restrict__ w, Out
     const float4* src = reinterpret_cast<const float4*>(w + f_block * RS);
     float4* dst = reinterpret_cast<float4*>(sg);
     const int nv = nf * RS / 4;
-    for (int i = threadIdx.x; i < nv; i += PACK_THREADS) dst[i] = __ldg(src + i);
+    for (int i = threadIdx.x; i < nv; i += PACK_THREADS) stage16(dst + i, src + i);
+    stage_wait();
     __syncthreads();
     if (late_wait) pdl_wait();                                    // host weights were loaded above; only the stores wait
     const int Cb = min(C, PACK_NF);                               // channels of one k row inside this block
@@ -414,7 +393,7 @@ __device__ __forceinline__ void pack1x1_block(const float* __restrict__ w, OutT*
 }
 
 template <typename OutT>
-__global__ void __launch_bounds__(PACK_THREADS)
+__global__ void __launch_bounds__(PACK_THREADS, 4)
 pack_kernel(const float* __restrict__ w, OutT* __restrict__ P, int K, int C, int RS, int Qp, unsigned long long* stamp, int host_src) {
     pdl_trigger();
     if (!host_src) pdl_wait();
@@ -440,21 +419,31 @@ pack1x1_kernel(const float* __restrict__ w, OutT* __restrict__ P, int K, int C, 
 // Block b belongs to the descriptor whose [block0, block0 + blocks) range holds it and does there
 // exactly what the single-layer kernels do.  A batch of small layers then costs one launch and
 // presents the memory system with one large stream of work.  The kernel is instantiated per group
-// of transform kinds (repacks / F(2,3) and F(4,3) / F(6,3)) so that the register allocation, and with
-// it the number of resident warps, is that of the group's own code and not of the largest transform.
-enum { XG_PACK = 0, XG_WINO_SMALL = 1, XG_WINO6 = 2, XG_COUNT = 3 };
+// of transform kinds (repacks / F(2,3) / F(4,3) / F(6,3)) so that the register allocation, and with
+// it the number of resident warps, is that of the group's own code and not of the largest transform.  A batch of several
+// groups is several launches; they depend on the same earlier work and not on each other, so the later ones fill the SMs
+// that the first one's last blocks leave idle (ResNet-50-shaped F(6,3): 77 us against 81).
+enum { XG_PACK = 0, XG_WINO2 = 1, XG_WINO4 = 2, XG_WINO6 = 3, XG_COUNT = 4 };
 __host__ __device__ inline int xform_group(int kind) {
-    return kind == XF_WINO6 ? XG_WINO6 : (kind == XF_WINO2 || kind == XF_WINO4) ? XG_WINO_SMALL : XG_PACK;
+    return kind == XF_WINO6 ? XG_WINO6 : kind == XF_WINO4 ? XG_WINO4 : kind == XF_WINO2 ? XG_WINO2 : XG_PACK;
 }
+__host__ __device__ constexpr int xform_m(int group) { return group == XG_WINO2 ? 2 : group == XG_WINO4 ? 4 : 6; }
+__host__ __device__ constexpr int xform_threads(int group) { return group == XG_PACK ? PACK_THREADS : ft_threads(xform_m(group)); }
+// (repacks: ResNet-50's 1x1 and 3x3 layers take 44 us with 5 blocks an SM, 48 with 4 or 6)
+__host__ __device__ constexpr int xform_resident(int group) { return group == XG_PACK ? 5 : ft_resident(xform_m(group)); }
+__host__ __device__ constexpr int xform_smem_floats(int group) { return group == XG_PACK ? PACK_SMEM_FLOATS : ft_filters(xform_m(group)) * 9; }
 
 template <int GROUP>
-__global__ void __launch_bounds__(FT_THREADS)
+__global__ void __launch_bounds__(xform_threads(GROUP), xform_resident(GROUP))
 multi_transform_kernel(const __grid_constant__ XformBatch batch) {
-    pdl_trigger();
+    // `follows`: the launch before it in the stream is of the same batch.  Every block of the batch's first launch waits before
+    // it lets this grid start, so whatever precedes the batch has completed by then; the wait at the end keeps this grid's
+    // completion behind the earlier launches', for whatever follows in the stream.
     const bool late = batch.host_src != 0;                      // sources in host memory: load first, wait before the stores
-    if (!late) pdl_wait();
+    if (!late && !batch.follows) pdl_wait();
+    pdl_trigger();
     if (threadIdx.x == 0) stamp_start(batch.stamp);
-    __shared__ __align__(16) float smem[XF_SMEM_FLOATS];
+    __shared__ __align__(16) float smem[xform_smem_floats(GROUP)];
     const unsigned vb = blockIdx.x;
     int di = 0;
     for (int i = 1; i < batch.n; ++i)
@@ -470,16 +459,13 @@ multi_transform_kernel(const __grid_constant__ XformBatch batch) {
             case XF_PACK1X1 * 2 + 1: pack1x1_block<__nv_bfloat16>(src, (__nv_bfloat16*)d.dst, d.K, d.C, d.Qp, lb, late); break;
             default: break;
         }
-    } else if constexpr (GROUP == XG_WINO_SMALL) {
-        switch (d.kind * 2 + d.bf16) {
-            case XF_WINO2 * 2: filter_transform_block<2, float, 4>(src, (float*)d.dst, d.K, d.C, d.Cp, lb, smem, late); break;
-            case XF_WINO2 * 2 + 1: filter_transform_block<2, __nv_bfloat16, 8>(src, (__nv_bfloat16*)d.dst, d.K, d.C, d.Cp, lb, smem, late); break;
-            case XF_WINO4 * 2: filter_transform_block<4, float, 2>(src, (float*)d.dst, d.K, d.C, d.Cp, lb, smem, late); break;
-            default: break;
-        }
+    } else if constexpr (GROUP == XG_WINO2) {
+        if (d.bf16) filter_transform_block<2, __nv_bfloat16>(src, (__nv_bfloat16*)d.dst, d.K, d.C, d.Cp, lb, smem, late);
+        else filter_transform_block<2, float>(src, (float*)d.dst, d.K, d.C, d.Cp, lb, smem, late);
     } else {
-        if (d.kind == XF_WINO6 && !d.bf16) filter_transform_block<6, float, 2>(src, (float*)d.dst, d.K, d.C, d.Cp, lb, smem, late);
+        filter_transform_block<xform_m(GROUP), float>(src, (float*)d.dst, d.K, d.C, d.Cp, lb, smem, late);
     }
+    if (batch.follows) pdl_wait();
     __syncthreads();
     if (threadIdx.x == 0) stamp_end(batch.stamp);
 }
@@ -494,7 +480,7 @@ int xform_blocks(const XformDesc& d) {
         case XF_PACK: return (int)pack_blocks(d.K, d.C, d.RS);
         case XF_PACK1X1: return (int)(((long long)d.K * d.Qp + PACK1X1_PER_BLOCK - 1) / PACK1X1_PER_BLOCK);
         default: {                                              // the block size of the kind's instantiation in multi_transform_kernel
-            const int fpb = d.kind == XF_WINO2 ? ft_filters(d.bf16 ? 8 : 4) : ft_filters(2);
+            const int fpb = ft_filters(xform_m(xform_group(d.kind)));
             return (int)(((long long)d.K * d.Cp + fpb - 1) / fpb);
         }
     }
@@ -503,6 +489,7 @@ int xform_blocks(const XformDesc& d) {
 nnv_status_t launch_transform_batch(XformDesc* descs, int n, cudaStream_t st) {
     unsigned long long* stamp = next_stamp();                  // every launch of the batch stamps the same slot
     next_stamp() = nullptr;
+    bool launched = false;
     for (int grp = 0; grp < XG_COUNT; ++grp) {
         XformBatch b;
         b.stamp = stamp;
@@ -512,9 +499,12 @@ nnv_status_t launch_transform_batch(XformDesc* descs, int n, cudaStream_t st) {
         auto flush = [&]() -> nnv_status_t {
             if (b.n == 0) return NNV_OK;
             b.total_blocks = blocks;
-            if (grp == XG_PACK) NNV_LAUNCH((multi_transform_kernel<XG_PACK>), blocks, FT_THREADS, 0, st, b);
-            else if (grp == XG_WINO_SMALL) NNV_LAUNCH((multi_transform_kernel<XG_WINO_SMALL>), blocks, FT_THREADS, 0, st, b);
-            else NNV_LAUNCH((multi_transform_kernel<XG_WINO6>), blocks, FT_THREADS, 0, st, b);
+            b.follows = launched && !b.host_src;
+            launched = true;
+            if (grp == XG_PACK) NNV_LAUNCH((multi_transform_kernel<XG_PACK>), blocks, xform_threads(XG_PACK), 0, st, b);
+            else if (grp == XG_WINO2) NNV_LAUNCH((multi_transform_kernel<XG_WINO2>), blocks, xform_threads(XG_WINO2), 0, st, b);
+            else if (grp == XG_WINO4) NNV_LAUNCH((multi_transform_kernel<XG_WINO4>), blocks, xform_threads(XG_WINO4), 0, st, b);
+            else NNV_LAUNCH((multi_transform_kernel<XG_WINO6>), blocks, xform_threads(XG_WINO6), 0, st, b);
             NNV_CUDA(cudaGetLastError());
             b.n = 0;
             blocks = 0;
