@@ -82,9 +82,14 @@ nnv_status_t do_exec(const nnv_plan& p, int layer, int v, int math, const void* 
     // IM2COL and GEMM1X1: Y[P][K] = Xcol[P][Qp] * P[K][Qp]^T
     a.M = g.P; a.Kd = g.Qp; a.batch = 1;
     a.B = d_wt; a.ldb = g.Qp; a.strideB = (int64_t)L.K * g.Qp;
-    const bool direct_operand = (v == NNV_VAR_GEMM1X1) && need == 0 && L.stride == 1;
-    if ((direct_operand || need == 0) && bf16) a.mode = GEMM_BF16_CVT;   // fp32 activation rounded to bf16 inside the kernel
-    if (direct_operand) {
+    const bool gather = gather_operand(L, g, math);
+    const bool direct_operand = (v == NNV_VAR_GEMM1X1) && need == 0 && L.stride == 1 && !gather;
+    if (!gather && (direct_operand || need == 0) && bf16) a.mode = GEMM_BF16_CVT;   // fp32 activation rounded to bf16 inside the kernel
+    if (gather) {
+        a.A = x; a.lda = g.Qp;
+        a.ic.on = 1; a.ic.gather = 1; a.ic.C = L.C; a.ic.H = L.H; a.ic.W = L.W; a.ic.R = L.R; a.ic.S = L.S;
+        a.ic.stride = L.stride; a.ic.pad = L.pad; a.ic.OW = g.OW;
+    } else if (direct_operand) {
         a.A = x; a.lda = L.C; a.Kd = L.C;                      // rows of X are the GEMM's rows
     } else if (need == 0) {
         // implicit GEMM: the TMA gathers the filter-window pixels from the activation itself

@@ -13,12 +13,6 @@ __device__ __forceinline__ float apply_act(float v, int act) {
     return v;
 }
 
-// fp32 -> TF32 precision, round to nearest even (the tensor core would otherwise truncate).
-__device__ __forceinline__ float round_tf32(float v) {
-    uint32_t b = __float_as_uint(v);
-    b += 0xFFFu + ((b >> 13) & 1u);
-    return __uint_as_float(b & 0xFFFFE000u);
-}
 template <typename OutT> __device__ inline OutT to_out(float v);
 template <> __device__ inline float to_out<float>(float v) { return v; }
 template <> __device__ inline __nv_bfloat16 to_out<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }

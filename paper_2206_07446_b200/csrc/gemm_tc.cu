@@ -75,8 +75,10 @@ constexpr int BM = 128;                 // rows of A per tile = TMEM lanes
 constexpr int BK_BYTES = 128;           // bytes of K per stage row = one 128B swizzle atom
 constexpr int A_STAGE_BYTES = BM * BK_BYTES;
 constexpr int GEMM_THREADS = 192;
-// gemm_tc_kernel: a second MMA issuer and a second producer; splitting both operands (mode 2) takes four more warps
-constexpr int gemm_tc_threads(int mode) { return mode == 2 ? 384 : 256; }
+// gemm_tc_kernel: a second MMA issuer and a second producer; splitting both operands (mode 2) and gathering (modes 4 - 7) take
+// four more warps
+constexpr int gemm_tc_threads(int mode) { return mode == 2 || mode >= 4 ? 384 : 256; }
+constexpr int GATHER_WARPS = 8;
 constexpr int GEMM_BAR_BYTES = 8 * (3 * 8 + 4) + 512;         // barriers, TMEM address, bias of the tile's columns
 constexpr uint32_t WAIT_LIMIT = 1u << 20;
 
@@ -227,6 +229,20 @@ __device__ __forceinline__ bool elect_one() {
     return p != 0;
 }
 
+// Predicated loads (zero without the predicate) that the compiler cannot turn into branches: all of a thread's loads stay in
+// flight together.
+__device__ __forceinline__ float load_if(bool in, const void* p) {
+    float v;
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\t@p ld.global.nc.f32 %0, [%1];\n\t@!p mov.f32 %0, 0f00000000;\n\t}"
+                 : "=f"(v) : "l"(p), "r"((int)in));
+    return v;
+}
+__device__ __forceinline__ void load4_if(bool in, const void* p, float* v) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %5, 0;\n\t@p ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];\n\t"
+                 "@!p mov.f32 %0, 0f00000000;\n\t@!p mov.f32 %1, 0f00000000;\n\t@!p mov.f32 %2, 0f00000000;\n\t@!p mov.f32 %3, 0f00000000;\n\t}"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "l"(p), "r"((int)in));
+}
+
 struct GemmDev {
     unsigned long long* stamp;        // device-clock stamps of this launch, or null
     float* D;
@@ -243,6 +259,10 @@ struct GemmDev {
     // implicit im2col (A is the NHWC activation itself): 0 = off
     // (2: its tiles are whole image rows, fetched as plain boxes)
     int ic_on, ic_C, ic_cblk, ic_S, ic_OW, ic_stride, ic_pad;
+    // modes 4 - 7: the activation, its size and the window's length R * S * C; magic numbers that divide by C and S
+    const float* x;
+    int ic_H, ic_W, ic_Q;
+    uint32_t magic_c, magic_s;
 };
 
 __device__ __forceinline__ float act_fn(float v, int act) {
@@ -304,13 +324,18 @@ __device__ __forceinline__ void convert_chunk(const uint8_t* src_tile, uint8_t* 
 }
 
 // MODE 3: A is fp32 (the activation itself, direct or through the TMA's im2col mode) and is rounded to bf16 by the
-// epilogue warps on its way through shared memory; B is the bf16 packed weight, fetched straight into the
-// un-swizzled core-matrix layout by ONE TMA box per stage over the rows seen as {8 elements, N rows, chunks}.
+// epilogue warps on its way through shared memory; B is the bf16 packed weight, fetched with the 64-byte swizzle.
 // MODE 0: TF32 operands (fp32 words), 1: BF16 operands, 2: fp32 operands multiplied as
 // hi*hi + lo*hi + hi*lo of their bf16 splits (error-compensated, fp32-class accuracy).
+// MODE 4 - 7: A is gathered from the filter windows of the activation by eight warps, element by element (4: TF32, 5: BF16) or
+// four channels at a time (6, 7), and rounded to nearest even on the way; B as in mode 0 or 1.
+__host__ __device__ constexpr bool gather_mode(int mode) { return mode >= 4; }
+__host__ __device__ constexpr bool bf16_mode(int mode) { return mode == 1 || mode == 5 || mode == 7; }   // both operands staged as bf16
 template <int MODE> struct ModeTraits {
-    static constexpr int BKE = (MODE == 1) ? 64 : 32;          // K elements per stage
+    static constexpr int BKE = bf16_mode(MODE) ? 64 : 32;      // K elements per stage
 };
+// n / d for n * d < 2^32, with magic = ceil(2^32 / d)
+__device__ __forceinline__ int div_magic(int n, int d, uint32_t magic) { return d == 1 ? n : (int)__umulhi((uint32_t)n, magic); }
 
 // A stage holds the `rows` rows of A that are loaded (the MMA's other rows read whatever follows and are never written out)
 // and BN rows of B, 128 bytes each; the conversion modes add the bf16 tiles, `pad8(rows)` rows tall: A (hi, lo), B (hi, lo) in
@@ -326,7 +351,7 @@ __host__ __device__ constexpr uint32_t stage_bytes_of(int BN, int rows) {
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(gemm_tc_threads(MODE), MODE == 2 ? 2 : 3)
+__global__ void __launch_bounds__(gemm_tc_threads(MODE), MODE == 2 || gather_mode(MODE) ? 2 : 3)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmD, const __grid_constant__ CUtensorMap tmAdd, const GemmDev g) {
     extern __shared__ uint8_t smem_raw[];
@@ -379,7 +404,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmB)) : "memory");
         for (int s = 0; s < STAGES; ++s) {
-            mbar_init(full_bar(s), 2);
+            mbar_init(full_bar(s), gather_mode(MODE) ? GATHER_WARPS + 1 : 2);
             mbar_init(empty_bar(s), 1);
             mbar_init(conv_bar(s), MODE == 2 ? 8 : 4);
         }
@@ -438,6 +463,21 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         // MODE 3: BN rows of 32 bf16 with the 64-byte swizzle, staged after the fp32 and the bf16 A tile
         tma_load_3d(MODE == 3 ? b_dst + rp * 64 : b_dst, &tmB, q, n0, b, full_bar(s));
     };
+    // Gather modes: {byte offset of the first element, taps inside the image} of the window of each of the tile's output pixels;
+    // the taps as a bit for every filter row (0 - 15) and every filter column (16 - 30).  No bits: the pixel does not exist.
+    uint2* const windows = reinterpret_cast<uint2*>(smem_raw + (sbias - smem_u32(smem_raw)) + 512);
+    if constexpr (gather_mode(MODE)) {
+        if (threadIdx.x < BM) {
+            const int m = m0 + (int)threadIdx.x, oh = m / g.ic_OW;
+            const int ih = oh * g.ic_stride - g.ic_pad, iw = (m - oh * g.ic_OW) * g.ic_stride - g.ic_pad;
+            auto inside = [](int first, int size, int most) {  // bits i < most with 0 <= first + i < size
+                const int lo = min(max(-first, 0), most), hi = min(max(size - first, 0), most);
+                return hi > lo ? (1u << hi) - (1u << lo) : 0u;
+            };
+            const uint32_t taps = inside(ih, g.ic_H, 16) | inside(iw, g.ic_W, 15) << 16;
+            windows[threadIdx.x] = make_uint2((uint32_t)((ih * g.ic_W + iw) * g.ic_C) * 4u, (int)threadIdx.x < live ? taps : 0u);
+        }
+    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -490,12 +530,92 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         }
         return true;
     };
+    // Gather modes: A's tile of every K block, by eight warps.  A lane keeps its place in the row (and so its filter tap and channel)
+    // for the whole block and walks the rows: reads are contiguous along the window, the swizzled row is written in one piece.
+    // Issue slots bound it (per row a window, a test of the tap, an address, a load, the rounding, a store), and it replaces a pass
+    // that writes the R*S-fold matrix to memory and one that reads it back: 7x7 stem of a 224 x 224 image 10.5 -> 7.7 us (bf16
+    // 10.6 -> 7.1), its 3x3 one 6.0 -> 4.0, 3x3 stride-1 stem 12.1 -> 8.9; 37 -> 64 3x3 @56 10.9 -> 7.1 (bf16 8.2 -> 6.2).
+    auto gather_stages = [&](int gw) -> bool {
+        constexpr bool BF = bf16_mode(MODE);
+        constexpr int V = MODE >= 6 ? 4 : 1;                  // consecutive channels of one load
+        constexpr int E = V == 4 ? 4 : BF ? 2 : 1;            // elements of a row a lane writes
+        constexpr int LPR = BKE / E, RPS = 32 / LPR;          // lanes to a row, rows a warp writes at a time
+        constexpr int PITCH = GATHER_WARPS * RPS;             // rows all warps write at a time: a multiple of 8
+        constexpr int STEPS = BM / (2 * PITCH);               // half a tile's rows at a time: all loads of the half, then its stores
+        const int r0 = gw * RPS + lane / LPR, ql = (lane % LPR) * E;
+        const uint32_t byte = (uint32_t)(ql * (BF ? 2 : 4));  // of the row: its 16-byte word is swizzled by the row
+        const uint32_t dst0 = (uint32_t)r0 * 128u + (((byte >> 4) ^ (uint32_t)(r0 & 7)) << 4) + (byte & 15u);
+        const char* const x = reinterpret_cast<const char*>(g.x);
+        uint8_t* const sm0 = smem_raw + (sbase - smem_u32(smem_raw));
+        int s = 0;
+        uint32_t ph = 0;
+        for (int it = 0; it < nkb; ++it, s = (s + 1 == STAGES ? 0 : s + 1), ph ^= (s == 0 ? 1u : 0u)) {
+            uint32_t off[E / V], tap[E / V];
+#pragma unroll
+            for (int e = 0; e < E / V; ++e) {
+                const int q = (kb0 + it) * BKE + ql + e, t = div_magic(q, g.ic_C, g.magic_c), c = q - t * g.ic_C;
+                const int fr = div_magic(t, g.ic_S, g.magic_s), fs = t - fr * g.ic_S;
+                off[e] = (uint32_t)((fr * g.ic_W + fs) * g.ic_C + c) * 4u;
+                tap[e] = q < g.ic_Q ? (1u << fr | 0x10000u << fs) : 0x80000000u;   // (the row's padding reads as zero)
+            }
+            if (it >= STAGES && !mbar_wait(empty_bar(s), ph ^ 1u)) return false;
+            const uint2* win = windows + r0;
+            uint8_t* dst = sm0 + s * stage_bytes + dst0;
+#pragma unroll 1
+            for (int r = r0; r < g.rows; r += BM / 2, win += BM / 2, dst += BM / 2 * 128) {
+                float v[STEPS][E];
+#pragma unroll
+                for (int u = 0; u < STEPS; ++u) {
+                    const uint2 w = win[u * PITCH];
+#pragma unroll
+                    for (int e = 0; e < E / V; ++e) {
+                        const char* src = x + (w.x + off[e]);
+                        if constexpr (V == 4) load4_if((w.y & tap[e]) == tap[e], src, v[u]);
+                        else v[u][e] = load_if((w.y & tap[e]) == tap[e], src);
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < STEPS; ++u) {
+                    if (r + u * PITCH >= g.rows) continue;
+                    uint8_t* const d = dst + u * PITCH * 128;
+                    if constexpr (BF) {
+                        __nv_bfloat162 h[E / 2];
+#pragma unroll
+                        for (int e = 0; e < E / 2; ++e) h[e] = __floats2bfloat162_rn(v[u][2 * e], v[u][2 * e + 1]);
+                        if constexpr (E == 4) *reinterpret_cast<uint2*>(d) = make_uint2(*reinterpret_cast<uint32_t*>(&h[0]), *reinterpret_cast<uint32_t*>(&h[1]));
+                        else *reinterpret_cast<__nv_bfloat162*>(d) = h[0];
+                    } else if constexpr (E == 4) {
+                        *reinterpret_cast<float4*>(d) = make_float4(round_tf32(v[u][0]), round_tf32(v[u][1]), round_tf32(v[u][2]), round_tf32(v[u][3]));
+                    } else {
+                        *reinterpret_cast<float*>(d) = round_tf32(v[u][0]);
+                    }
+                }
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> visible to the MMA's reads
+            __syncwarp();
+            if (lane == 0) mbar_arrive(full_bar(s));
+        }
+        return true;
+    };
+    // One place that runs the gathering, for the epilogue's warps and the extra ones alike: a second copy of the code for the second
+    // group is fetched cold by every launch.  (The bias is fetched before it: 1x1 205 -> 96 @40 6.0 us against 6.7.)
+    bool gathered = true;
+    float early_bias = 0.f;
+    if constexpr (gather_mode(MODE)) {
+        if (warp >= 8 || (warp >= 2 && warp <= 5)) {
+            const int t = (int)threadIdx.x - 64;
+            if (g.bias && t < BN && n0 + t < g.N) early_bias = __ldg(g.bias + n0 + t);
+            gathered = gather_stages(warp >= 8 ? warp - 4 : warp - 2);
+            if (!gathered && lane == 0) atomicExch(&g_device_status, (int)NNV_ERR_TIMEOUT);
+            __syncwarp();
+        }
+    }
     bool cluster_arrived = false;                             // the epilogue warps arrive early, in their own code
     if (warp == 0 || warp == 7) {
         // Producers.  A load costs the thread that issues it ~157 cycles whatever its size, which for one thread issuing both
         // operands (314 cycles a K block) is more than the MMAs take: the activation's and the weights' loads come from a
         // warp each, the residual tile from the weights' one (it has fewer bytes to wait for).
-        if (elect_one()) {
+        if (!(gather_mode(MODE) && warp == 0) && elect_one()) {
             bool ok = true;
             int s = 0;
             uint32_t ph = 0;
@@ -537,7 +657,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         const int iss = warp == 1 ? 0 : warp - 5;
         if (iss < g.issuers && elect_one()) {
             // instruction descriptor: fp32 accumulate, A/B format, both K-major, N, M = 128
-            const uint32_t fmt = (MODE == 0) ? 2u : 1u;
+            const uint32_t fmt = (MODE == 0 || MODE == 4 || MODE == 6) ? 2u : 1u;
             const uint32_t idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
             const uint32_t acc = tmem_base + (uint32_t)(iss * BN);
             bool ok = true;
@@ -576,7 +696,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                     const uint64_t bdesc = make_smem_desc(a_src + a_stage);
 #pragma unroll
                     for (int kk = 0; kk < 4; ++kk)             // 4 MMAs of 32 bytes of K each
-                        umma<MODE == 1>(acc, adesc + (uint64_t)(kk * 2), bdesc + (uint64_t)(kk * 2), idesc, kk ? 1u : first);
+                        umma<bf16_mode(MODE)>(acc, adesc + (uint64_t)(kk * 2), bdesc + (uint64_t)(kk * 2), idesc, kk ? 1u : first);
                 }
                 umma_commit(empty_bar(s));
                 s += g.issuers;
@@ -593,7 +713,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         const int quarter = warp & 3;                         // the TMEM lanes this warp may read
         const int t = (int)threadIdx.x - 64;
         uint8_t* const sm = smem_raw + (sbase - smem_u32(smem_raw));
-        const float bias = (g.bias && t < BN && n0 + t < g.N) ? __ldg(g.bias + n0 + t) : 0.f;
+        float bias = early_bias;
+        if constexpr (!gather_mode(MODE)) bias = (g.bias && t < BN && n0 + t < g.N) ? __ldg(g.bias + n0 + t) : 0.f;
         const int naccs = min(g.issuers, nkb);
         const uint32_t tacc = tmem_base + ((uint32_t)(quarter * 32) << 16);
         const float hi = g.act == 2 ? 6.f : INFINITY;
@@ -619,8 +740,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
             }
         };
-        bool ok = true;
-        if constexpr (MODE >= 2) ok = convert_stages(warp - 2);
+        bool ok = gathered;
+        if constexpr (MODE == 2 || MODE == 3) ok = convert_stages(warp - 2);
         float* const s_bias = reinterpret_cast<float*>(sm + (sbias - sbase));
         if (t < BN) s_bias[t] = bias;
         asm volatile("barrier.sync 1, 128;" ::: "memory");
@@ -988,30 +1109,42 @@ int gemm_ring(int mode, int bn, int rows, long long ctas, int nkb) {
 // adds the pushes of the partial rows.  Constants (microseconds) fitted to a sweep of every BN and split over the 101 GEMM
 // layer shapes of the ResNet / MobileNetV2 / VGG configurations at several resolutions, chained launches: the chosen
 // tilings are 0.05 us a launch above the best measured ones on average.
-struct GemmTiling { int BN, splits; };
+// A gather mode's K block takes the eight warps time for every row, most of it in steps of half a tile; a second CTA on the SM adds
+// `share` of it.  Its tiles may be lower than 128 rows (any height that divides M), which spreads the rows over more SMs.  Fitted the
+// same way over 33 shapes: the chosen tilings are 3 % above the best measured ones on average.
+struct GemmTiling { int BN, splits, rows; };
 GemmTiling search_gemm_tiling(int mode, int M, int N, int batch, int nkb) {
-    const int m_tiles = ceil_div(M, BM), rows = gemm_rows(M);
-    GemmTiling best{16, 1};
+    constexpr struct { double row_us, share; } gather[4] = {{0.0064, 0.36}, {0.0054, 0.60}, {0.0025, 0.81}, {0.0042, 0.40}};   // modes 4 - 7
+    const double fixed = gather_mode(mode) ? 0.87 : 1.87, start = gather_mode(mode) ? 1.85 : 0.40;
+    const int least = ceil_div(M, BM);
+    const int most = gather_mode(mode) ? std::max(least, std::min(M / 16, 296)) : least;
+    GemmTiling best{16, 1, gemm_rows(M)};
     double best_t = 1e30;
-    for (int bn = 16; bn <= std::min(128, ceil_div(N, 16) * 16); bn += bn < 64 ? 16 : 32) {
-        const double kb_bytes = (double)(rows * BK_BYTES + bn * BK_BYTES);
-        for (int sp = 1; sp <= 16 && sp <= nkb; sp *= 2) {
-            const long long ctas = (long long)m_tiles * ceil_div(N, bn) * batch * sp;
-            const int nk = ceil_div(nkb, sp), ring = gemm_ring(mode, bn, rows, ctas, nk);
-            int tmem = 32;
-            while (tmem < 2 * bn) tmem *= 2;
-            const double smem = 2048.0 + (double)ring * gemm_stage_bytes(mode, bn, rows) + (sp > 1 ? 4.0 * rows * bn : 0.0);
-            const int occ = std::max(1, std::min({3, (int)(226.0 * 1024.0 / smem), 512 / tmem}));
-            // whole clusters must find free SMs inside one GPC: how many CTAs fit with one, two and three to an SM (as
-            // cudaOccupancyMaxActiveClusters reports)
-            static const int cap[5][3] = {{148, 296, 444}, {148, 296, 444}, {132, 284, 416}, {120, 264, 384}, {112, 224, 336}};
-            const long long slots = cap[sp == 16 ? 4 : sp == 8 ? 3 : sp == 4 ? 2 : sp - 1][occ - 1];
-            const double waves = (double)((ctas + slots - 1) / slots);
-            const double res = (double)std::min<long long>(occ, (ctas + 147) / 148);
-            const double kb = std::max({0.146 * res, kb_bytes * res / 108e3, kb_bytes * (double)std::min(ctas, slots) / 10.9e6});
-            const double split = sp > 1 ? 0.26 + 0.021 * std::log2((double)sp) + 1.22e-4 * bn * rows * res : 0.0;
-            const double t = 1.87 + waves * (nk * kb + 0.40 + 0.0093 * bn + split);
-            if (t < best_t - 1e-9) { best_t = t; best = GemmTiling{bn, sp}; }
+    for (int m_tiles = least; m_tiles <= most; ++m_tiles) {
+        if (m_tiles != least && M % m_tiles != 0) continue;
+        const int rows = M % m_tiles == 0 ? M / m_tiles : BM;
+        for (int bn = 16; bn <= std::min(128, ceil_div(N, 16) * 16); bn += bn < 64 ? 16 : 32) {
+            const double kb_bytes = (double)(rows * BK_BYTES + bn * BK_BYTES);
+            for (int sp = 1; sp <= 16 && sp <= nkb; sp *= 2) {
+                const long long ctas = (long long)m_tiles * ceil_div(N, bn) * batch * sp;
+                const int nk = ceil_div(nkb, sp), ring = gemm_ring(mode, bn, rows, ctas, nk);
+                int tmem = 32;
+                while (tmem < 2 * bn) tmem *= 2;
+                const double smem = 2048.0 + (double)ring * gemm_stage_bytes(mode, bn, rows) + (sp > 1 ? 4.0 * rows * bn : 0.0);
+                const int occ = std::max(1, std::min({gather_mode(mode) ? 2 : 3, (int)(226.0 * 1024.0 / smem), 512 / tmem}));
+                // whole clusters must find free SMs inside one GPC: how many CTAs fit with one, two and three to an SM (as
+                // cudaOccupancyMaxActiveClusters reports)
+                static const int cap[5][3] = {{148, 296, 444}, {148, 296, 444}, {132, 284, 416}, {120, 264, 384}, {112, 224, 336}};
+                const long long slots = cap[sp == 16 ? 4 : sp == 8 ? 3 : sp == 4 ? 2 : sp - 1][occ - 1];
+                const double waves = (double)((ctas + slots - 1) / slots);
+                const double res = (double)std::min<long long>(occ, (ctas + 147) / 148);
+                double kb = std::max({0.146 * res, kb_bytes * res / 108e3, kb_bytes * (double)std::min(ctas, slots) / 10.9e6});
+                if (gather_mode(mode))
+                    kb = std::max(kb, (0.2 + gather[mode & 3].row_us * (0.65 * 64 * ceil_div(rows, 64) + 0.35 * rows)) * (1 + gather[mode & 3].share * (res - 1)));
+                const double split = sp > 1 ? 0.26 + 0.021 * std::log2((double)sp) + 1.22e-4 * bn * rows * res : 0.0;
+                const double t = fixed + waves * (nk * kb + start + 0.0093 * bn + split);
+                if (t < best_t - 1e-9) { best_t = t; best = GemmTiling{bn, sp, rows}; }
+            }
         }
     }
     return best;
@@ -1035,14 +1168,11 @@ std::once_flag g_attr_once;
 nnv_status_t gemm_tc_init() {
     NNV_TRY(get_encoder());
     std::call_once(g_attr_once, [] {
-        cudaFuncSetAttribute(gemm_tc_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
-        cudaFuncSetAttribute(gemm_tc_kernel<0>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        cudaFuncSetAttribute(gemm_tc_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
-        cudaFuncSetAttribute(gemm_tc_kernel<1>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        cudaFuncSetAttribute(gemm_tc_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
-        cudaFuncSetAttribute(gemm_tc_kernel<2>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        cudaFuncSetAttribute(gemm_tc_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
-        cudaFuncSetAttribute(gemm_tc_kernel<3>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        for (auto* kernel : {gemm_tc_kernel<0>, gemm_tc_kernel<1>, gemm_tc_kernel<2>, gemm_tc_kernel<3>, gemm_tc_kernel<4>, gemm_tc_kernel<5>,
+                             gemm_tc_kernel<6>, gemm_tc_kernel<7>}) {
+            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
+            cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        }
         cudaFuncSetAttribute(conv3x3_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
         cudaFuncSetAttribute(conv3x3_bf16_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
         cudaFuncSetAttribute(gemm_sp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
@@ -1336,17 +1466,18 @@ nnv_status_t launch_gemm_tc(const GemmArgs& a, cudaStream_t st) {
     NNV_TRY(gemm_tc_init());
     // Tiling: column tile BN and K splits (a thread-block cluster of up to 8 CTAs) with the least estimated time.
     const int bke = (a.mode == GEMM_BF16) ? 64 : 32;
-    const int nkb_all = a.ic.on ? a.ic.R * a.ic.S * ceil_div(a.ic.C, 32) : ceil_div(a.Kd, bke);
-    const int m_tiles = ceil_div(a.M, BM);
+    const bool gather = a.ic.on && a.ic.gather;
+    const int mode = gather ? (a.mode == GEMM_BF16 ? 5 : 4) + ((a.ic.C % 4) == 0 ? 2 : 0) : a.mode;   // the kernel's
+    const int nkb_all = a.ic.on && !gather ? a.ic.R * a.ic.S * ceil_div(a.ic.C, 32) : ceil_div(a.Kd, bke);
     constexpr int issuers = 2;
-    const int rows = gemm_rows(a.M);
-    const GemmTiling tile = pick_gemm_tiling(a.mode, a.M, a.N, a.batch, nkb_all);
+    const GemmTiling tile = pick_gemm_tiling(mode, a.M, a.N, a.batch, nkb_all);
     int BN = tile.BN, splits = tile.splits;
+    const int rows = tile.rows, m_tiles = ceil_div(a.M, rows);
     const Tuning tn = tuning();
     if (tn.gemm_bn && tn.gemm_splits <= nkb_all) { BN = tn.gemm_bn; splits = tn.gemm_splits; }   // override (nnv_tuning_set)
     // A 3x3 / stride 1 / pad 1 layer large enough to fill the GPU runs on the halo-resident kernel,
     // which moves fewer operand bytes through L2 and shared memory.
-    if (a.ic.on && (a.mode == GEMM_TF32 || a.mode == GEMM_BF16_CVT) && a.batch == 1 && a.ic.R == 3 && a.ic.S == 3 && a.ic.stride == 1 &&
+    if (a.ic.on && !gather && (a.mode == GEMM_TF32 || a.mode == GEMM_BF16_CVT) && a.batch == 1 && a.ic.R == 3 && a.ic.S == 3 && a.ic.stride == 1 &&
         a.ic.pad == 1 && (a.ic.C % 32) == 0) {
         if (a.mode == GEMM_BF16_CVT) {
             ConvBTiling ct = pick_conv_bf16_tiling(a.ic.C, a.ic.H, a.ic.W, a.N);
@@ -1397,7 +1528,14 @@ nnv_status_t launch_gemm_tc(const GemmArgs& a, cudaStream_t st) {
     g.ldd = a.ldd; g.strideD = a.strideD;
     g.M = a.M; g.N = a.N; g.Kd = a.Kd; g.BN = BN; g.act = a.act; g.tmem_cols = tmem_cols; g.splits = splits; g.stages = ring; g.issuers = issuers;
     g.ic_on = 0; g.ic_C = g.ic_cblk = g.ic_S = g.ic_OW = g.ic_stride = g.ic_pad = 0;
-    if (a.ic.on) {
+    g.x = nullptr; g.ic_H = g.ic_W = g.ic_Q = 0; g.magic_c = g.magic_s = 0;
+    if (gather) {
+        g.x = static_cast<const float*>(a.A);
+        g.ic_C = a.ic.C; g.ic_S = a.ic.S; g.ic_OW = a.ic.OW; g.ic_stride = a.ic.stride; g.ic_pad = a.ic.pad;
+        g.ic_H = a.ic.H; g.ic_W = a.ic.W; g.ic_Q = a.ic.R * a.ic.S * a.ic.C;
+        g.magic_c = 0xFFFFFFFFu / (uint32_t)a.ic.C + 1u;
+        g.magic_s = 0xFFFFFFFFu / (uint32_t)a.ic.S + 1u;
+    } else if (a.ic.on) {
         NNV_REQUIRE((a.mode == GEMM_TF32 || a.mode == GEMM_BF16_CVT) && a.batch == 1, NNV_ERR_INVALID_ARG,
                     "implicit im2col needs fp32 activations (TF32 or converting BF16 mode) and one batch");
         const bool boxes = 4ull * a.ic.C * a.ic.H * a.ic.W < 131072ull && image_row_boxes(a.ic.H, a.ic.W, a.ic.R, a.ic.S, a.ic.stride, a.ic.pad);
@@ -1415,6 +1553,7 @@ nnv_status_t launch_gemm_tc(const GemmArgs& a, cudaStream_t st) {
     } else {
         NNV_TRY(encode_operand(&tmB, a.B, bf16, a.Kd, a.N, a.batch, a.ldb, a.strideB, BN));
     }
+    if (gather) tmA = tmB;                                       // unused by the kernel, but a kernel parameter must hold a valid object
 
     // Write-out by TMA through swizzled staging tiles when the output rows are 16-byte multiples (else plain stores), in
     // the ring once that is idle; with a residual addend, which is loaded while the ring works, in a place of their own.
@@ -1426,11 +1565,11 @@ nnv_status_t launch_gemm_tc(const GemmArgs& a, cudaStream_t st) {
     const size_t park = splits > 1 ? (size_t)rows * BN * 4 : (tma_out && !a.addend) ? staging : 0;
     const size_t behind = splits > 1 ? (size_t)splits * ceil_div(rows, splits) * BN * 4 : (tma_out && a.addend) ? staging + 1024 : 0;
     while (ring < 8 && (size_t)ring * sb < park) ++ring;
-    while (ring > 1 && (size_t)2048 + (size_t)ring * sb + GEMM_BAR_BYTES + behind > 226u * 1024u && (size_t)(ring - 1) * sb >= park) --ring;
+    while (ring > 1 && (size_t)2048 + (size_t)ring * sb + GEMM_BAR_BYTES + (gather ? BM * 8 : 0) + behind > 226u * 1024u && (size_t)(ring - 1) * sb >= park) --ring;
     g.stages = ring;
     g.rows = rows;
     g.bar_off = (uint32_t)ring * sb;
-    const size_t ring_and_bars = (size_t)ring * sb + GEMM_BAR_BYTES;
+    const size_t ring_and_bars = (size_t)ring * sb + GEMM_BAR_BYTES + (gather ? BM * 8 : 0);
     g.recv_off = (uint32_t)align_up(ring_and_bars, 128);
     g.tma_out = tma_out ? ((BN % 32) == 0 ? 32 : 16) : 0;
     g.stage_off = a.addend ? (uint32_t)align_up(ring_and_bars, 1024) : 0;
@@ -1453,16 +1592,10 @@ nnv_status_t launch_gemm_tc(const GemmArgs& a, cudaStream_t st) {
 
     dim3 grid(m_tiles, ceil_div(a.N, BN), a.batch * splits);
     NNV_REQUIRE(grid.y <= 65535 && grid.z <= 65535, NNV_ERR_UNSUPPORTED, "GEMM grid too large");
-    if (a.mode == GEMM_TF32)
-        (void)launch_pdl_cluster(gemm_tc_kernel<0>, grid, dim3(gemm_tc_threads(0)), smem_bytes, st, splits, tmA, tmB, tmD, tmAdd, g);
-    else if (a.mode == GEMM_BF16)
-        (void)launch_pdl_cluster(gemm_tc_kernel<1>, grid, dim3(gemm_tc_threads(1)), smem_bytes, st, splits, tmA, tmB, tmD, tmAdd, g);
-    else if (a.mode == GEMM_BF16_CVT)
-        (void)launch_pdl_cluster(gemm_tc_kernel<3>, grid, dim3(gemm_tc_threads(3)), smem_bytes, st, splits, tmA, tmB, tmD, tmAdd, g);
-    else if (a.mode == GEMM_X3)
-        (void)launch_pdl_cluster(gemm_tc_kernel<2>, grid, dim3(gemm_tc_threads(2)), smem_bytes, st, splits, tmA, tmB, tmD, tmAdd, g);
-    else
-        return fail(NNV_ERR_INVALID_ARG, "unknown GEMM mode %d", a.mode);
+    static constexpr decltype(&gemm_tc_kernel<0>) kernels[8] = {gemm_tc_kernel<GEMM_TF32>, gemm_tc_kernel<GEMM_BF16>, gemm_tc_kernel<GEMM_X3>,
+        gemm_tc_kernel<GEMM_BF16_CVT>, gemm_tc_kernel<4>, gemm_tc_kernel<5>, gemm_tc_kernel<6>, gemm_tc_kernel<7>};
+    NNV_REQUIRE(a.mode >= GEMM_TF32 && a.mode <= GEMM_BF16_CVT, NNV_ERR_INVALID_ARG, "unknown GEMM mode %d", a.mode);
+    (void)launch_pdl_cluster(kernels[mode], grid, dim3(gemm_tc_threads(mode)), smem_bytes, st, splits, tmA, tmB, tmD, tmAdd, g);
     NNV_CUDA(cudaGetLastError());
     return NNV_OK;
 }

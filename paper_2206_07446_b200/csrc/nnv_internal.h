@@ -89,6 +89,16 @@ inline cudaError_t launch_pdl_cluster(void (*kernel)(Params...), dim3 grid, dim3
     (void)::nnv::launch_pdl(kernel, dim3(grid), dim3(block), (size_t)(smem), st, __VA_ARGS__)
 #endif
 
+#ifdef __CUDACC__
+// fp32 -> TF32 precision (10 explicit mantissa bits), round to nearest even, by integer arithmetic; the result is an fp32
+// word whose low 13 mantissa bits are zero (the tensor core would otherwise truncate).
+__device__ __forceinline__ float round_tf32(float v) {
+    uint32_t b = __float_as_uint(v);
+    b += 0xFFFu + ((b >> 13) & 1u);
+    return __uint_as_float(b & 0xFFFFE000u);
+}
+#endif
+
 // ---- device-clock stamps of kernels ----------------------------------------------------------
 // A kernel given a non-null `stamp` pointer records the device-wide nanosecond clock when its first
 // block starts working (after the wait on the previous kernel) and when its last block has finished:
@@ -251,6 +261,7 @@ constexpr int XF_BATCH_MAX = 56;
 struct XformBatch { unsigned long long* stamp; int n; int total_blocks; int host_src; int follows; XformDesc d[XF_BATCH_MAX]; };
 nnv_status_t launch_transform_batch(XformDesc* descs, int n, cudaStream_t st);
 
+bool gather_operand(const nnv_layer_desc_t& L, const LayerGeom& g, int math);   // the GEMM gathers the filter windows itself
 // Explicit im2col of an NHWC fp32 image: Xcol[P][Qp], q = (r*S+s)*C + c (fp32 or bf16).
 nnv_status_t launch_im2col(bool bf16, const float* d_x, void* d_col, int C, int H, int W, int R, int S,
                            int stride, int pad, int OH, int OW, int Qp, cudaStream_t st);
@@ -295,7 +306,8 @@ struct GemmArgs {
     int mode;                         // GEMM_TF32, GEMM_BF16 or GEMM_X3
     // Implicit im2col: A is the NHWC fp32 activation (C % 4 == 0) read by the TMA in im2col mode;
     // B is the packed weight P[K][Qp] with Kd = Qp; M = OH*OW output pixels.  TF32 mode, batch 1.
-    struct { int on, C, H, W, R, S, stride, pad, OW; } ic;
+    // gather: windows the TMA cannot fetch (any C), gathered by the kernel's warps; TF32 or BF16 mode, Kd = Qp.
+    struct { int on, C, H, W, R, S, stride, pad, OW, gather; } ic;
 };
 // Rows of A per tile of the GEMM kernel: as few 128-row tiles as hold M, of equal height when they divide M (7 x 7 and 14 x 14
 // grids: one tile of 49, two of 98): rows that do not exist would fill shared memory all the same.

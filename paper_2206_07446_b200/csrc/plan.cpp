@@ -172,6 +172,19 @@ static inline bool implicit_gemm_operand(const nnv_layer_desc_t& L, int math) {
            (4ull * L.C * L.H * L.W >= 131072ull || image_row_boxes(L.H, L.W, L.R, L.S, L.stride, L.pad)) && L.R <= 16 && L.S <= 16 && L.pad <= 8;
 }
 
+// What neither of those reads in place -- channel counts that are no multiple of 16 bytes (network stems), small strided images --
+// is gathered by the GEMM's own warps.  The exception is fp32 words one by one for many output channels: every column tile
+// gathers the windows again, and the explicit matrix pays or is as good (303 -> 300 3x3 @7: 6.7 us against 7.2, 102 -> 400 @56 28.2
+// and 28.3, 1x1 333 -> 1024 @28 9.3 against 9.8; at 250 channels, 250 -> 250 @56, the gathering wins 37 to 58).
+bool gather_operand(const nnv_layer_desc_t& L, const LayerGeom& g, int math) {
+    if (L.R * L.S == 1 ? gemm1x1_direct_operand(L, math) || implicit_gemm_operand(L, math) : implicit_gemm_operand(L, math)) return false;
+    if (math == NNV_MATH_BF16 && !tuning().bf16cvt) return false;
+    if (math == NNV_MATH_TF32 && (L.C % 4) != 0 && L.K > 256) return false;
+    // 32-bit byte offsets, a bit for every filter row and column, exact division by magic numbers
+    return ((double)g.Qp + 64.0) * L.C < 4.0e9 && ((double)L.H + 2.0 * L.pad) * ((double)L.W + 2.0 * L.pad) * L.C < 5.0e8 &&
+           L.R <= 16 && L.S <= 15;
+}
+
 bool wino_fused_applies(const nnv_layer_desc_t& L, int v, int math) {
     return v == NNV_VAR_WINO_F2 && math == NNV_MATH_TF32 && L.groups == 1 && L.R == 3 && L.S == 3 && L.stride == 1 &&
            (L.C % 8) == 0 && (L.K % 8) == 0;
@@ -220,6 +233,7 @@ uint64_t exec_ws_bytes(const nnv_plan& p, int layer, int v, int math) {
         const uint64_t T = (uint64_t)ceil_div(g.OH, m) * ceil_div(g.OW, m);
         return align_up(a2 * T * g.Cp * es, 256) + align_up(a2 * T * L.K * 4, 256);
     }
+    if ((v == NNV_VAR_IM2COL || v == NNV_VAR_GEMM1X1) && gather_operand(L, g, math)) return 0;
     if (v == NNV_VAR_IM2COL) return implicit_gemm_operand(L, math) ? 0 : align_up((uint64_t)g.P * g.Qp * es, 256);
     if (v == NNV_VAR_GEMM1X1)
         return (gemm1x1_direct_operand(L, math) || implicit_gemm_operand(L, math)) ? 0

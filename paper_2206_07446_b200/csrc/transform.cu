@@ -241,13 +241,6 @@ nnv_status_t launch_filter_transform(int m, bool bf16, const float* g, void* U, 
 // ---- GEMM-ready repack ----------------------------------------------------------------------
 // Elements are rounded to the precision the tensor core will use: TF32 (stored as fp32 words) or
 // bf16, round to nearest even, so the hardware never truncates the weights.
-// fp32 -> TF32 precision (10 explicit mantissa bits), round to nearest even, by integer arithmetic;
-// the result is an fp32 word whose low 13 mantissa bits are zero.
-__device__ __forceinline__ float round_tf32(float v) {
-    uint32_t b = __float_as_uint(v);
-    b += 0xFFFu + ((b >> 13) & 1u);
-    return __uint_as_float(b & 0xFFFFE000u);
-}
 template <typename OutT> __device__ inline OutT cvt_out(float v);
 template <> __device__ inline float cvt_out<float>(float v) { return round_tf32(v); }
 template <> __device__ inline __nv_bfloat16 cvt_out<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
