@@ -229,20 +229,6 @@ __device__ __forceinline__ bool elect_one() {
     return p != 0;
 }
 
-// Predicated loads (zero without the predicate) that the compiler cannot turn into branches: all of a thread's loads stay in
-// flight together.
-__device__ __forceinline__ float load_if(bool in, const void* p) {
-    float v;
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\t@p ld.global.nc.f32 %0, [%1];\n\t@!p mov.f32 %0, 0f00000000;\n\t}"
-                 : "=f"(v) : "l"(p), "r"((int)in));
-    return v;
-}
-__device__ __forceinline__ void load4_if(bool in, const void* p, float* v) {
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %5, 0;\n\t@p ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];\n\t"
-                 "@!p mov.f32 %0, 0f00000000;\n\t@!p mov.f32 %1, 0f00000000;\n\t@!p mov.f32 %2, 0f00000000;\n\t@!p mov.f32 %3, 0f00000000;\n\t}"
-                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "l"(p), "r"((int)in));
-}
-
 struct GemmDev {
     unsigned long long* stamp;        // device-clock stamps of this launch, or null
     float* D;
@@ -533,8 +519,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     // Gather modes: A's tile of every K block, by eight warps.  A lane keeps its place in the row (and so its filter tap and channel)
     // for the whole block and walks the rows: reads are contiguous along the window, the swizzled row is written in one piece.
     // Issue slots bound it (per row a window, a test of the tap, an address, a load, the rounding, a store), and it replaces a pass
-    // that writes the R*S-fold matrix to memory and one that reads it back: 7x7 stem of a 224 x 224 image 10.5 -> 7.7 us (bf16
-    // 10.6 -> 7.1), its 3x3 one 6.0 -> 4.0, 3x3 stride-1 stem 12.1 -> 8.9; 37 -> 64 3x3 @56 10.9 -> 7.1 (bf16 8.2 -> 6.2).
+    // that writes the R*S-fold matrix to memory and one that reads it back: 7x7 stem of a 224 x 224 image 10.5 -> 7.6 us (bf16
+    // 10.6 -> 6.5), its 3x3 one 6.0 -> 4.0, 3x3 stride-1 stem 12.1 -> 8.9; 37 -> 64 3x3 @56 10.9 -> 7.0 (bf16 8.2 -> 5.7).
     auto gather_stages = [&](int gw) -> bool {
         constexpr bool BF = bf16_mode(MODE);
         constexpr int V = MODE >= 6 ? 4 : 1;                  // consecutive channels of one load
@@ -569,9 +555,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                     const uint2 w = win[u * PITCH];
 #pragma unroll
                     for (int e = 0; e < E / V; ++e) {
+                        const bool in = (w.y & tap[e]) == tap[e];
                         const char* src = x + (w.x + off[e]);
-                        if constexpr (V == 4) load4_if((w.y & tap[e]) == tap[e], src, v[u]);
-                        else v[u][e] = load_if((w.y & tap[e]) == tap[e], src);
+                        if constexpr (V == 4) {
+                            const float4 f = in ? __ldg(reinterpret_cast<const float4*>(src)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                            v[u][0] = f.x; v[u][1] = f.y; v[u][2] = f.z; v[u][3] = f.w;
+                        } else {
+                            v[u][e] = in ? __ldg(reinterpret_cast<const float*>(src)) : 0.f;
+                        }
                     }
                 }
 #pragma unroll
