@@ -1103,10 +1103,14 @@ int gemm_ring(int mode, int bn, int rows, long long ctas, int nkb) {
 // A gather mode's K block takes the eight warps time for every row, most of it in steps of half a tile; a second CTA on the SM adds
 // `share` of it.  Its tiles may be lower than 128 rows (any height that divides M), which spreads the rows over more SMs.  Fitted the
 // same way over 33 shapes: the chosen tilings are 3 % above the best measured ones on average.
+// X3's K block waits for the split of both operands (by pieces of 32 rows), most of which a second CTA on the SM overlaps: fitted over
+// 68 F(4,3) / F(6,3) layers, 1 % above the best measured tilings (the constants of the other modes: 2.5 %, and 20 % on 512 -> 512
+// F(4,3) @7, 22.9 us against 19.1).
 struct GemmTiling { int BN, splits, rows; };
 GemmTiling search_gemm_tiling(int mode, int M, int N, int batch, int nkb) {
     constexpr struct { double row_us, share; } gather[4] = {{0.0064, 0.36}, {0.0054, 0.60}, {0.0025, 0.81}, {0.0042, 0.40}};   // modes 4 - 7
-    const double fixed = gather_mode(mode) ? 0.87 : 1.87, start = gather_mode(mode) ? 1.85 : 0.40;
+    const bool x3 = mode == GEMM_X3;
+    const double fixed = gather_mode(mode) ? 0.87 : 1.87, start = gather_mode(mode) ? 1.85 : x3 ? 0.80 : 0.40, column = x3 ? 0.005 : 0.0093;
     const int least = ceil_div(M, BM);
     const int most = gather_mode(mode) ? std::max(least, std::min(M / 16, 296)) : least;
     GemmTiling best{16, 1, gemm_rows(M)};
@@ -1122,18 +1126,19 @@ GemmTiling search_gemm_tiling(int mode, int M, int N, int batch, int nkb) {
                 int tmem = 32;
                 while (tmem < 2 * bn) tmem *= 2;
                 const double smem = 2048.0 + (double)ring * gemm_stage_bytes(mode, bn, rows) + (sp > 1 ? 4.0 * rows * bn : 0.0);
-                const int occ = std::max(1, std::min({gather_mode(mode) ? 2 : 3, (int)(226.0 * 1024.0 / smem), 512 / tmem}));
+                const int occ = std::max(1, std::min({gather_mode(mode) || x3 ? 2 : 3, (int)(226.0 * 1024.0 / smem), 512 / tmem}));
                 // whole clusters must find free SMs inside one GPC: how many CTAs fit with one, two and three to an SM (as
                 // cudaOccupancyMaxActiveClusters reports)
                 static const int cap[5][3] = {{148, 296, 444}, {148, 296, 444}, {132, 284, 416}, {120, 264, 384}, {112, 224, 336}};
                 const long long slots = cap[sp == 16 ? 4 : sp == 8 ? 3 : sp == 4 ? 2 : sp - 1][occ - 1];
                 const double waves = (double)((ctas + slots - 1) / slots);
                 const double res = (double)std::min<long long>(occ, (ctas + 147) / 148);
-                double kb = std::max({0.146 * res, kb_bytes * res / 108e3, kb_bytes * (double)std::min(ctas, slots) / 10.9e6});
+                double kb = std::max({(x3 ? 0.37 : 0.146) * res, kb_bytes * res / 108e3, kb_bytes * (double)std::min(ctas, slots) / (x3 ? 4.6e6 : 10.9e6)});
+                if (x3) kb = std::max(kb, (0.40 + 0.07 * (ceil_div(rows, 32) + ceil_div(bn, 32))) * (1 + 0.15 * (res - 1)));
                 if (gather_mode(mode))
                     kb = std::max(kb, (0.2 + gather[mode & 3].row_us * (0.65 * 64 * ceil_div(rows, 64) + 0.35 * rows)) * (1 + gather[mode & 3].share * (res - 1)));
-                const double split = sp > 1 ? 0.26 + 0.021 * std::log2((double)sp) + 1.22e-4 * bn * rows * res : 0.0;
-                const double t = fixed + waves * (nk * kb + start + 0.0093 * bn + split);
+                const double split = sp > 1 ? (x3 ? 0.73 : 0.26 + 0.021 * std::log2((double)sp)) + 1.22e-4 * bn * rows * res : 0.0;
+                const double t = fixed + waves * (nk * kb + start + column * bn + split);
                 if (t < best_t - 1e-9) { best_t = t; best = GemmTiling{bn, sp, rows}; }
             }
         }
