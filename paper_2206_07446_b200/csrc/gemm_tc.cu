@@ -1041,30 +1041,23 @@ bool finish_conv_tiling(ConvTiling* t) {
     return t->smem <= 200u * 1024u && rings() >= park;
 }
 
-// Measured on B200 (sweeps over tilings, ring depths and K splits at the 3x3 shapes of the VGG / ResNet
-// configurations, L2 flushed before each launch): the kernel runs best with one MMA tile per CTA,
-// channel tiles of 128, shallow rings (two or three CTAs then share an SM, and one CTA's fill and
-// write-out overlap another's MMAs) and enough K splits for ~1.5 CTAs per SM; all CTAs should be
-// resident at once (a second, mostly empty wave costs as much as the first), so the box ring drops
-// to one slot when that makes them fit.  Layers with fewer than four channel blocks and fewer than
-// two patches per SM, and layers too small to give every SM a CTA even with 8 splits, stay on the
-// plain implicit GEMM, which is faster there.
-bool pick_conv_tiling(int C, int H, int W, int N, ConvTiling* out) {
+// The TF32 halo kernel's tiling, if it is to be used: one MMA tile per CTA, channel tiles of up to 128, shallow rings (two or three
+// CTAs then share an SM, and one CTA's fill and write-out overlap another's MMAs), all CTAs resident at once: the box ring drops to
+// one slot when that makes them fit.  Its K split is dear (7 us), so it splits only to fill the GPU.
+// It moves fewer operand bytes than the implicit GEMM but has one issuing thread where that has two.  Measured (us, halo kernel /
+// implicit GEMM): it wins where the implicit GEMM's tiles do not fit the GPU at once -- 64 -> 64 @224 12.7 / 17.1, 128 -> 256 @112
+// 18.4 / 24.8, 64 -> 128 @180 12.6 / 17.9, 64 -> 112 @160 11.8 / 23.3, 512 -> 512 @72 58 / 84 -- and on deep layers with some 50
+// patches, 512 -> 256 @56 22.7 / 25.4; it loses where they fit: 128 -> 128 @112 15.4 / 13.3, 64 -> 64 @180 11.8 / 10.0,
+// 256 -> 512 @56 26.1 / 22.0.
+bool pick_conv_tiling(int C, int H, int W, int N, bool gemm_fits, ConvTiling* out) {
     const int cblk = ceil_div(C, 32);
     ConvTiling t{};
     t.MT = 1;
     t.BN = std::min(128, ceil_div(N, 16) * 16);
     const long long tiles = (long long)ceil_div(H, 16) * ceil_div(W, 8) * ceil_div(N, t.BN);
-    int max_sp = 1;
-    while (max_sp * 2 <= std::min(8, cblk)) max_sp *= 2;
-    if (tiles * max_sp < 148 || (cblk < 4 && tiles < 296)) return false;
-    // Against the implicit GEMM with its refit tiling model (kernel stamps, L2 flushed; halo kernel / implicit GEMM, us):
-    // 64 -> 64 @224 13.4 / 18.0 and 256 -> 256 @56 18.8 / 24.0, but 128 -> 128 @112 17.7 / 14.9, 128 -> 256 @56 14.7 / 12.8,
-    // 256 -> 512 @28 14.7 / 12.9, 512 -> 512 @28 19.0 / 18.6: the halo kernel keeps the layers with two or more patches per SM
-    // and the deep ones (eight or more channel blocks) that still have ~50 tiles.
-    if (tiles < 296 && !(cblk >= 8 && tiles >= 48)) return false;
+    if (gemm_fits && !(cblk >= 12 && tiles >= 48)) return false;
     t.splits = 1;
-    while (t.splits < max_sp && tiles * t.splits < 224) t.splits *= 2;
+    while (t.splits * 2 <= std::min(8, cblk) && tiles * t.splits < 148) t.splits *= 2;
     const long long ctas = tiles * t.splits;
     bool found = false;
     const int rings[2][2] = {{2, 3}, {1, 3}};
@@ -1106,14 +1099,14 @@ int gemm_ring(int mode, int bn, int rows, long long ctas, int nkb) {
 // X3's K block waits for the split of both operands (by pieces of 32 rows), most of which a second CTA on the SM overlaps: fitted over
 // 68 F(4,3) / F(6,3) layers, 1 % above the best measured tilings (the constants of the other modes: 2.5 %, and 20 % on 512 -> 512
 // F(4,3) @7, 22.9 us against 19.1).
-struct GemmTiling { int BN, splits, rows; };
+struct GemmTiling { int BN, splits, rows, waves; };
 GemmTiling search_gemm_tiling(int mode, int M, int N, int batch, int nkb) {
     constexpr struct { double row_us, share; } gather[4] = {{0.0064, 0.36}, {0.0054, 0.60}, {0.0025, 0.81}, {0.0042, 0.40}};   // modes 4 - 7
     const bool x3 = mode == GEMM_X3;
     const double fixed = gather_mode(mode) ? 0.87 : 1.87, start = gather_mode(mode) ? 1.85 : x3 ? 0.80 : 0.40, column = x3 ? 0.005 : 0.0093;
     const int least = ceil_div(M, BM);
     const int most = gather_mode(mode) ? std::max(least, std::min(M / 16, 296)) : least;
-    GemmTiling best{16, 1, gemm_rows(M)};
+    GemmTiling best{16, 1, gemm_rows(M), 1};
     double best_t = 1e30;
     for (int m_tiles = least; m_tiles <= most; ++m_tiles) {
         if (m_tiles != least && M % m_tiles != 0) continue;
@@ -1139,7 +1132,7 @@ GemmTiling search_gemm_tiling(int mode, int M, int N, int batch, int nkb) {
                     kb = std::max(kb, (0.2 + gather[mode & 3].row_us * (0.65 * 64 * ceil_div(rows, 64) + 0.35 * rows)) * (1 + gather[mode & 3].share * (res - 1)));
                 const double split = sp > 1 ? (x3 ? 0.73 : 0.26 + 0.021 * std::log2((double)sp)) + 1.22e-4 * bn * rows * res : 0.0;
                 const double t = fixed + waves * (nk * kb + start + column * bn + split);
-                if (t < best_t - 1e-9) { best_t = t; best = GemmTiling{bn, sp, rows}; }
+                if (t < best_t - 1e-9) { best_t = t; best = GemmTiling{bn, sp, rows, (int)waves}; }
             }
         }
     }
@@ -1483,7 +1476,7 @@ nnv_status_t launch_gemm_tc(const GemmArgs& a, cudaStream_t st) {
             if (tn.conv3x3 != 1) return launch_conv3x3_bf16(a, ct.BN, ct.splits, st);
         } else {
         ConvTiling ct;
-        bool use = pick_conv_tiling(a.ic.C, a.ic.H, a.ic.W, a.N, &ct);
+        bool use = pick_conv_tiling(a.ic.C, a.ic.H, a.ic.W, a.N, tile.waves == 1, &ct);
         if (tn.conv3x3 == 1) {
             use = false;
         } else if (tn.conv3x3 == 2) {
