@@ -1464,7 +1464,7 @@ nnv_status_t launch_gemm_tc(const GemmArgs& a, cudaStream_t st) {
     const GemmTiling tile = pick_gemm_tiling(mode, a.M, a.N, a.batch, nkb_all);
     int BN = tile.BN, splits = tile.splits;
     const int rows = tile.rows, m_tiles = ceil_div(a.M, rows);
-    const Tuning tn = tuning();
+    const Tuning& tn = tuning();
     if (tn.gemm_bn && tn.gemm_splits <= nkb_all) { BN = tn.gemm_bn; splits = tn.gemm_splits; }   // override (nnv_tuning_set)
     // A 3x3 / stride 1 / pad 1 layer large enough to fill the GPU runs on the halo-resident kernel,
     // which moves fewer operand bytes through L2 and shared memory.

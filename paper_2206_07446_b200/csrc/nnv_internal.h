@@ -169,7 +169,7 @@ struct Tuning {
     int smallp_splits = 0;                    // 0 = the cost model decides
     uint64_t generation = 0;
 };
-Tuning tuning();                              // a copy of the current overrides (thread safe)
+const Tuning& tuning();                       // the calling thread's copy of the current overrides, valid until its next call
 
 struct GraphKey {
     uint64_t tuning_gen = 0;
@@ -254,11 +254,10 @@ enum { XF_PACK = 0, XF_PACK1X1 = 1, XF_WINO2 = 2, XF_WINO4 = 3, XF_WINO6 = 4 };
 struct XformDesc {
     const void* src; void* dst;
     int K, C, Cp, RS, Qp;
-    int kind, bf16, block0;
+    int kind, bf16;
     int host_src;                    // src is pinned host memory read in place
 };
-constexpr int XF_BATCH_MAX = 56;
-struct XformBatch { unsigned long long* stamp; int n; int total_blocks; int host_src; int follows; XformDesc d[XF_BATCH_MAX]; };
+constexpr int XF_CHUNK_MAX = 56;        // layers of one copy chunk, transformed by one batch
 nnv_status_t launch_transform_batch(XformDesc* descs, int n, cudaStream_t st);
 
 bool gather_operand(const nnv_layer_desc_t& L, const LayerGeom& g, int math);   // the GEMM gathers the filter windows itself

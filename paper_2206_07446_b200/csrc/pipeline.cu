@@ -190,7 +190,7 @@ static nnv_status_t run_model(nnv_plan* p, const nnv_choice_t* choices, const vo
                                                                           // transform and execution then follows the last byte
                 CopyChunk& c = chunks.back();
                 if (src >= c.src + c.bytes && (uint64_t)(src - (c.src + c.bytes)) <= kMaxGap && src - c.src == dst - c.dst &&
-                    c.bytes < target && i - c.first < XF_BATCH_MAX) {
+                    c.bytes < target && i - c.first < XF_CHUNK_MAX) {
                     c.bytes = (uint64_t)(src - c.src) + len;
                     c.last = i;
                     joined = true;
@@ -456,8 +456,9 @@ static nnv_status_t run_model(nnv_plan* p, const nnv_choice_t* choices, const vo
         }
 
         // execute
-        // (one wait serves all layers of a chunk on a stream: the event is the chunk's)
-        if (ready && ready != waited[on_side[i]]) {
+        // (one wait serves all layers of a chunk on a stream: the event is the chunk's, and its transforms' event implies its copy's)
+        const bool covered = merge && chunk_of[i] >= 0 && waited[on_side[i]] == EV(chunks[chunk_of[i]].first, 1);
+        if (ready && ready != waited[on_side[i]] && !covered) {
             NNV_CUDA(cudaStreamWaitEvent(se, ready, 0));
             waited[on_side[i]] = ready;
         }

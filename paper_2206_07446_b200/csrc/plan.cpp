@@ -1,6 +1,7 @@
 // Host-side plan logic: validation, eligibility, size queries, arena layout and the
 // integer cold-cost selection.  No device work happens in this file.
 #include <algorithm>
+#include <atomic>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
@@ -23,10 +24,16 @@ nnv_status_t fail(nnv_status_t code, const char* fmt, ...) {
 
 static std::mutex g_tuning_mu;
 static Tuning g_tuning;
+static std::atomic<uint64_t> g_tuning_generation{0};
 
-Tuning tuning() {
-    std::lock_guard<std::mutex> lk(g_tuning_mu);
-    return g_tuning;
+// (asked several times a launch: a thread takes the lock and the copy only when something has been set since)
+const Tuning& tuning() {
+    static thread_local Tuning seen;
+    if (seen.generation != g_tuning_generation.load(std::memory_order_acquire)) {
+        std::lock_guard<std::mutex> lk(g_tuning_mu);
+        seen = g_tuning;
+    }
+    return seen;
 }
 
 // "key=value;key=value" -> *t.  Returns the offending item on a parse / range error, else nullptr.
@@ -192,7 +199,7 @@ bool wino_fused_applies(const nnv_layer_desc_t& L, int v, int math) {
 
 SmallPPlan small_p_plan(const nnv_layer_desc_t& L, const LayerGeom& g, int v, int math) {
     SmallPPlan sp{};
-    const Tuning tn = tuning();
+    const Tuning& tn = tuning();
     if (!tn.smallp || (v != NNV_VAR_IM2COL && v != NNV_VAR_GEMM1X1) || math != NNV_MATH_TF32 || L.groups != 1 || L.stride != 1 ||
         L.R != L.S || (L.R & 1) == 0 || L.pad != (L.R - 1) / 2 || L.H * L.W > 256 || (L.C % 32) != 0 || (L.K % 4) != 0)
         return sp;
@@ -390,6 +397,7 @@ nnv_status_t nnv_tuning_set(const char* spec) {
     std::lock_guard<std::mutex> lk(g_tuning_mu);
     t.generation = g_tuning.generation + 1;
     g_tuning = t;
+    g_tuning_generation.store((uint64_t)t.generation, std::memory_order_release);
     return NNV_OK;
 }
 

@@ -3,6 +3,9 @@
 // transformation" stage (its Section 2 and Figure 3), run on the device.
 #include <cuda_bf16.h>
 
+#include <algorithm>
+#include <type_traits>
+
 #include "nnv_internal.h"
 
 namespace nnv {
@@ -426,9 +429,15 @@ __host__ __device__ constexpr int xform_threads(int group) { return group == XG_
 __host__ __device__ constexpr int xform_resident(int group) { return group == XG_PACK ? 5 : ft_resident(xform_m(group)); }
 __host__ __device__ constexpr int xform_smem_floats(int group) { return group == XG_PACK ? PACK_SMEM_FLOATS : ft_filters(xform_m(group)) * 9; }
 
-template <int GROUP>
+// The descriptors travel as kernel parameters, which cost the host ~0.7 us a kilobyte to launch with: 36 bytes each, in one of two sizes
+// (a chunk of a cold run rarely holds more than 16 layers; its launch takes the host 3 us instead of 5.4).
+struct XformItem { const void* src; void* dst; int K, C, pitch, block0; uint16_t RS; uint8_t kind, bf16; };   // pitch: Cp, or Qp of a repack
+constexpr int XF_BATCH_SMALL = 16, XF_BATCH_MAX = 56;
+template <int N> struct XformBatch { unsigned long long* stamp; int n, host_src, follows; XformItem d[N]; };
+
+template <int GROUP, int N>
 __global__ void __launch_bounds__(xform_threads(GROUP), xform_resident(GROUP))
-multi_transform_kernel(const __grid_constant__ XformBatch batch) {
+multi_transform_kernel(const __grid_constant__ XformBatch<N> batch) {
     // `follows`: the launch before it in the stream is of the same batch.  Every block of the batch's first launch waits before
     // it lets this grid start, so whatever precedes the batch has completed by then; the wait at the end keeps this grid's
     // completion behind the earlier launches', for whatever follows in the stream.
@@ -441,22 +450,22 @@ multi_transform_kernel(const __grid_constant__ XformBatch batch) {
     int di = 0;
     for (int i = 1; i < batch.n; ++i)
         if (vb >= (unsigned)batch.d[i].block0) di = i;
-    const XformDesc& d = batch.d[di];
+    const XformItem& d = batch.d[di];
     const unsigned lb = vb - (unsigned)d.block0;
     const float* src = static_cast<const float*>(d.src);
     if constexpr (GROUP == XG_PACK) {
         switch (d.kind * 2 + d.bf16) {
-            case XF_PACK * 2: pack_block<float>(src, (float*)d.dst, d.K, d.C, d.RS, d.Qp, lb, smem, late); break;
-            case XF_PACK * 2 + 1: pack_block<__nv_bfloat16>(src, (__nv_bfloat16*)d.dst, d.K, d.C, d.RS, d.Qp, lb, smem, late); break;
-            case XF_PACK1X1 * 2: pack1x1_block<float>(src, (float*)d.dst, d.K, d.C, d.Qp, lb, late); break;
-            case XF_PACK1X1 * 2 + 1: pack1x1_block<__nv_bfloat16>(src, (__nv_bfloat16*)d.dst, d.K, d.C, d.Qp, lb, late); break;
+            case XF_PACK * 2: pack_block<float>(src, (float*)d.dst, d.K, d.C, d.RS, d.pitch, lb, smem, late); break;
+            case XF_PACK * 2 + 1: pack_block<__nv_bfloat16>(src, (__nv_bfloat16*)d.dst, d.K, d.C, d.RS, d.pitch, lb, smem, late); break;
+            case XF_PACK1X1 * 2: pack1x1_block<float>(src, (float*)d.dst, d.K, d.C, d.pitch, lb, late); break;
+            case XF_PACK1X1 * 2 + 1: pack1x1_block<__nv_bfloat16>(src, (__nv_bfloat16*)d.dst, d.K, d.C, d.pitch, lb, late); break;
             default: break;
         }
     } else if constexpr (GROUP == XG_WINO2) {
-        if (d.bf16) filter_transform_block<2, __nv_bfloat16>(src, (__nv_bfloat16*)d.dst, d.K, d.C, d.Cp, lb, smem, late);
-        else filter_transform_block<2, float>(src, (float*)d.dst, d.K, d.C, d.Cp, lb, smem, late);
+        if (d.bf16) filter_transform_block<2, __nv_bfloat16>(src, (__nv_bfloat16*)d.dst, d.K, d.C, d.pitch, lb, smem, late);
+        else filter_transform_block<2, float>(src, (float*)d.dst, d.K, d.C, d.pitch, lb, smem, late);
     } else {
-        filter_transform_block<xform_m(GROUP), float>(src, (float*)d.dst, d.K, d.C, d.Cp, lb, smem, late);
+        filter_transform_block<xform_m(GROUP), float>(src, (float*)d.dst, d.K, d.C, d.pitch, lb, smem, late);
     }
     if (batch.follows) pdl_wait();
     __syncthreads();
@@ -483,21 +492,31 @@ nnv_status_t launch_transform_batch(XformDesc* descs, int n, cudaStream_t st) {
     unsigned long long* stamp = next_stamp();                  // every launch of the batch stamps the same slot
     next_stamp() = nullptr;
     bool launched = false;
+    XformBatch<XF_BATCH_MAX> b;
+    b.stamp = stamp;
+    b.host_src = (n > 0 && descs[0].host_src) ? 1 : 0;          // a batch is all device or all host sources
     for (int grp = 0; grp < XG_COUNT; ++grp) {
-        XformBatch b;
-        b.stamp = stamp;
-        b.host_src = (n > 0 && descs[0].host_src) ? 1 : 0;      // a batch is all device or all host sources
         b.n = 0;
         int blocks = 0;
         auto flush = [&]() -> nnv_status_t {
             if (b.n == 0) return NNV_OK;
-            b.total_blocks = blocks;
             b.follows = launched && !b.host_src;
             launched = true;
-            if (grp == XG_PACK) NNV_LAUNCH((multi_transform_kernel<XG_PACK>), blocks, xform_threads(XG_PACK), 0, st, b);
-            else if (grp == XG_WINO2) NNV_LAUNCH((multi_transform_kernel<XG_WINO2>), blocks, xform_threads(XG_WINO2), 0, st, b);
-            else if (grp == XG_WINO4) NNV_LAUNCH((multi_transform_kernel<XG_WINO4>), blocks, xform_threads(XG_WINO4), 0, st, b);
-            else NNV_LAUNCH((multi_transform_kernel<XG_WINO6>), blocks, xform_threads(XG_WINO6), 0, st, b);
+            auto launch = [&](auto group) {
+                constexpr int G = decltype(group)::value;
+                if (b.n > XF_BATCH_SMALL) {
+                    NNV_LAUNCH((multi_transform_kernel<G, XF_BATCH_MAX>), blocks, xform_threads(G), 0, st, b);
+                } else {
+                    XformBatch<XF_BATCH_SMALL> small;
+                    small.stamp = b.stamp; small.n = b.n; small.host_src = b.host_src; small.follows = b.follows;
+                    std::copy(b.d, b.d + b.n, small.d);
+                    NNV_LAUNCH((multi_transform_kernel<G, XF_BATCH_SMALL>), blocks, xform_threads(G), 0, st, small);
+                }
+            };
+            if (grp == XG_PACK) launch(std::integral_constant<int, XG_PACK>{});
+            else if (grp == XG_WINO2) launch(std::integral_constant<int, XG_WINO2>{});
+            else if (grp == XG_WINO4) launch(std::integral_constant<int, XG_WINO4>{});
+            else launch(std::integral_constant<int, XG_WINO6>{});
             NNV_CUDA(cudaGetLastError());
             b.n = 0;
             blocks = 0;
@@ -505,12 +524,11 @@ nnv_status_t launch_transform_batch(XformDesc* descs, int n, cudaStream_t st) {
         };
         for (int i = 0; i < n; ++i) {
             if (xform_group(descs[i].kind) != grp) continue;
-            XformDesc d = descs[i];
+            const XformDesc& d = descs[i];
             NNV_REQUIRE(d.kind != XF_PACK || 8 * d.RS <= PACK_SLICE, NNV_ERR_UNSUPPORTED,
                         "filter window of %d taps is too large to repack", d.RS);
-            d.block0 = blocks;
+            b.d[b.n++] = XformItem{d.src, d.dst, d.K, d.C, grp == XG_PACK ? d.Qp : d.Cp, blocks, (uint16_t)d.RS, (uint8_t)d.kind, (uint8_t)d.bf16};
             blocks += xform_blocks(d);
-            b.d[b.n++] = d;
             if (b.n == XF_BATCH_MAX) NNV_TRY(flush());
         }
         NNV_TRY(flush());
