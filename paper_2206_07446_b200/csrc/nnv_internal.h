@@ -162,7 +162,7 @@ struct Tuning {
     int convw = 0;                            // weights-stationary 3x3 kernel: 0 the library decides, 1 off, 2 wherever it fits
     int side = 1, merge = 1, group = 1;       // pipeline features: side stream, merged reads, grouped transforms
     int copies_first = 1;                     // merged reads all enqueued before the first kernel
-    int chunk_first_kb = 256, chunk_max_kb = 16384;   // merged reads: size target of the first chunk, doubling up to the maximum
+    int chunk_first_kb = 1024, chunk_max_kb = 32768;   // merged reads: size target of the first chunk, doubling up to the maximum
     int winofused = -1;                       // the one-kernel F(2x2,3x3) path: -1 the library decides, 0 off, 1 on where it applies
     int bf16cvt = 1;                          // BF16 math straight from the fp32 activation (rounded inside the GEMM); 0: explicit bf16 im2col
     int smallp = 1;                           // the weights-on-rows kernel for layers with few pixels
