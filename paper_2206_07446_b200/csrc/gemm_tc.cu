@@ -1150,6 +1150,60 @@ GemmTiling pick_gemm_tiling(int mode, int M, int N, int batch, int nkb) {
     return e.t;
 }
 
+// Ring, issuers and shared-memory layout of one launch of gemm_tc_kernel (host arithmetic only; `mode` is the kernel's).
+struct GemmShape {
+    int BN, splits, rows, m_tiles, issuers, ring, tmem_cols;
+    uint32_t bar_off, recv_off, stage_off;
+    size_t smem_bytes;
+};
+
+nnv_status_t gemm_shape(int mode, const GemmTiling& tile, int M, int N, int batch, int nkb, bool tma_out, bool addend, GemmShape* out) {
+    GemmShape g{};
+    const Tuning& tn = tuning();
+    g.BN = tile.BN; g.splits = tile.splits; g.rows = tile.rows;
+    g.m_tiles = ceil_div(M, g.rows);
+    if (tn.gemm_bn && tn.gemm_splits <= nkb) { g.BN = tn.gemm_bn; g.splits = tn.gemm_splits; }   // override (nnv_tuning_set)
+    // (BF16 on fp32 activations: two MMAs a K block wait for the conversion, not for their issuer; one accumulator then adds the
+    // blocks in order, and 3x3/2 256 -> 512 @28 takes 8.4 us against 8.5, 5x5 64 -> 64 @56 8.8 against 8.9)
+    g.issuers = mode == GEMM_BF16_CVT ? 1 : 2;
+    g.tmem_cols = 32;
+    while (g.tmem_cols < g.BN * g.issuers) g.tmem_cols *= 2;
+    const bool split = g.splits > 1;
+    const size_t sb = gemm_stage_bytes(mode, g.BN, g.rows), bars = GEMM_BAR_BYTES + (gather_mode(mode) ? BM * 8 : 0);
+    const int nkb_cta = ceil_div(nkb, g.splits);
+    g.ring = gemm_ring(mode, g.BN, g.rows, (long long)g.m_tiles * ceil_div(N, g.BN) * batch * g.splits, nkb_cta);
+    if (tn.gemm_ring && (size_t)tn.gemm_ring * sb <= 210u * 1024u) g.ring = tn.gemm_ring;
+    // Write-out by TMA through swizzled staging tiles when the output rows are 16-byte multiples (else plain stores), in
+    // the ring once that is idle; with a residual addend, which is loaded while the ring works, in a place of their own.
+    const size_t staging = (size_t)ceil_div(g.rows, 32) * 32 * g.BN * 4;
+    // Split K: room to park the partial tile in the ring, and for the rows this CTA receives (its share from every CTA).
+    const size_t park = split ? (size_t)g.rows * g.BN * 4 : (tma_out && !addend) ? staging : 0;
+    const size_t behind = split ? (size_t)g.splits * ceil_div(g.rows, g.splits) * g.BN * 4 : (tma_out && addend) ? staging + 1024 : 0;
+    while (g.ring < 8 && g.ring * sb < park) ++g.ring;
+    while (g.ring > 1 && 2048 + g.ring * sb + bars + behind > 226u * 1024u && (g.ring - 1) * sb >= park) --g.ring;
+    // Two issuers take alternate K blocks, so in a ring of odd depth the blocks of one slot go to one and the other in turn.  A wait
+    // by parity only tells neighbouring phases apart: an issuer that is through with block i - 2 takes the slot of block i for full
+    // while the load of its former block, i - depth, is still on its way (loads may land in any order).  It would multiply what
+    // is there and release the slot; the producers then arrive at a barrier whose phase already has all its arrivals, and loads
+    // land in a CTA that has gone.  So a ring that is refilled has an even depth: an issuer then has its slots for itself.
+    // (X3's issuers wait for eight warps that convert the blocks in order: block i - 2 converted means block i - depth is, from
+    // two slots on.)
+    if (g.issuers == 2 && nkb_cta > g.ring && (mode == GEMM_X3 ? g.ring == 1 : (g.ring & 1) == 1)) {
+        if (g.ring > 1 && (g.ring - 1) * sb >= park) --g.ring;
+        else g.issuers = 1;
+    }
+    g.bar_off = (uint32_t)(g.ring * sb);
+    const size_t ring_and_bars = g.ring * sb + bars;
+    g.recv_off = (uint32_t)align_up(ring_and_bars, 128);
+    g.stage_off = addend ? (uint32_t)align_up(ring_and_bars, 1024) : 0;
+    g.smem_bytes = (size_t)1024 + (split ? g.recv_off + behind : (tma_out && addend) ? g.stage_off + staging : ring_and_bars);
+    // the MMAs read 128 rows of A from every stage, the last one included
+    g.smem_bytes = std::max(g.smem_bytes, (size_t)1024 + (g.ring - 1) * sb + A_STAGE_BYTES);
+    NNV_REQUIRE(g.smem_bytes <= 226u * 1024u, NNV_ERR_UNSUPPORTED, "GEMM tiling does not fit shared memory");
+    *out = g;
+    return NNV_OK;
+}
+
 std::once_flag g_attr_once;
 
 }  // namespace
@@ -1453,19 +1507,13 @@ static nnv_status_t launch_conv3x3_persistent(const GemmArgs& a, int BN, int per
 nnv_status_t launch_gemm_tc(const GemmArgs& a, cudaStream_t st) {
     NNV_REQUIRE(a.M > 0 && a.N > 0 && a.Kd > 0 && a.batch > 0, NNV_ERR_INVALID_ARG, "empty GEMM");
     NNV_TRY(gemm_tc_init());
-    // Tiling: column tile BN and K splits (a thread-block cluster of up to 8 CTAs) with the least estimated time.
+    // Tiling: column tile BN and K splits (a thread-block cluster of up to 16 CTAs) with the least estimated time.
     const int bke = (a.mode == GEMM_BF16) ? 64 : 32;
     const bool gather = a.ic.on && a.ic.gather;
     const int mode = gather ? (a.mode == GEMM_BF16 ? 5 : 4) + ((a.ic.C % 4) == 0 ? 2 : 0) : a.mode;   // the kernel's
     const int nkb_all = a.ic.on && !gather ? a.ic.R * a.ic.S * ceil_div(a.ic.C, 32) : ceil_div(a.Kd, bke);
-    // (BF16 on fp32 activations: two MMAs a K block wait for the conversion, not for their issuer; one accumulator then adds the
-    // blocks in order, and 3x3/2 256 -> 512 @28 takes 8.4 us against 8.5, 5x5 64 -> 64 @56 8.8 against 8.9)
-    const int issuers = a.mode == GEMM_BF16_CVT ? 1 : 2;
     const GemmTiling tile = pick_gemm_tiling(mode, a.M, a.N, a.batch, nkb_all);
-    int BN = tile.BN, splits = tile.splits;
-    const int rows = tile.rows, m_tiles = ceil_div(a.M, rows);
     const Tuning& tn = tuning();
-    if (tn.gemm_bn && tn.gemm_splits <= nkb_all) { BN = tn.gemm_bn; splits = tn.gemm_splits; }   // override (nnv_tuning_set)
     // A 3x3 / stride 1 / pad 1 layer large enough to fill the GPU runs on the halo-resident kernel,
     // which moves fewer operand bytes through L2 and shared memory.
     if (a.ic.on && !gather && (a.mode == GEMM_TF32 || a.mode == GEMM_BF16_CVT) && a.batch == 1 && a.ic.R == 3 && a.ic.S == 3 && a.ic.stride == 1 &&
@@ -1504,11 +1552,12 @@ nnv_status_t launch_gemm_tc(const GemmArgs& a, cudaStream_t st) {
         if (use) return launch_conv3x3_tc(a, ct, st);
         }
     }
-    int tmem_cols = 32;
-    while (tmem_cols < BN * issuers) tmem_cols *= 2;
-    const uint32_t sb = gemm_stage_bytes(a.mode, BN, rows);
-    int ring = gemm_ring(a.mode, BN, rows, (long long)m_tiles * ceil_div(a.N, BN) * a.batch * splits, ceil_div(nkb_all, splits));
-    if (tn.gemm_ring && (size_t)tn.gemm_ring * sb <= 210u * 1024u) ring = tn.gemm_ring;
+    const bool tma_ok = (a.N % 4) == 0 && (a.ldd % 4) == 0 && (a.strideD % 4) == 0 && (reinterpret_cast<uintptr_t>(a.D) & 15) == 0 &&
+                        (!a.addend || ((reinterpret_cast<uintptr_t>(a.addend) & 15) == 0 && a.batch == 1));
+    GemmShape sh;
+    NNV_TRY(gemm_shape(mode, tile, a.M, a.N, a.batch, nkb_all, tma_ok, a.addend != nullptr, &sh));
+    const int BN = sh.BN, splits = sh.splits, rows = sh.rows, m_tiles = sh.m_tiles;
+    const bool tma_out = tma_ok && splits == 1;
 
     const bool bf16 = a.mode == GEMM_BF16;
     CUtensorMap tmA, tmB, tmD, tmAdd;
@@ -1517,7 +1566,9 @@ nnv_status_t launch_gemm_tc(const GemmArgs& a, cudaStream_t st) {
     next_stamp() = nullptr;
     g.D = a.D; g.bias = a.bias; g.addend = a.addend;
     g.ldd = a.ldd; g.strideD = a.strideD;
-    g.M = a.M; g.N = a.N; g.Kd = a.Kd; g.BN = BN; g.act = a.act; g.tmem_cols = tmem_cols; g.splits = splits; g.stages = ring; g.issuers = issuers;
+    g.M = a.M; g.N = a.N; g.Kd = a.Kd; g.BN = BN; g.act = a.act; g.tmem_cols = sh.tmem_cols; g.splits = splits; g.stages = sh.ring; g.issuers = sh.issuers;
+    g.rows = rows; g.bar_off = sh.bar_off; g.recv_off = sh.recv_off; g.stage_off = sh.stage_off;
+    g.tma_out = tma_out ? ((BN % 32) == 0 ? 32 : 16) : 0;
     g.ic_on = 0; g.ic_C = g.ic_cblk = g.ic_S = g.ic_OW = g.ic_stride = g.ic_pad = 0;
     g.x = nullptr; g.ic_H = g.ic_W = g.ic_Q = 0; g.magic_c = g.magic_s = 0;
     if (gather) {
@@ -1546,32 +1597,10 @@ nnv_status_t launch_gemm_tc(const GemmArgs& a, cudaStream_t st) {
     }
     if (gather) tmA = tmB;                                       // unused by the kernel, but a kernel parameter must hold a valid object
 
-    // Write-out by TMA through swizzled staging tiles when the output rows are 16-byte multiples (else plain stores), in
-    // the ring once that is idle; with a residual addend, which is loaded while the ring works, in a place of their own.
-    const size_t staging = (size_t)ceil_div(rows, 32) * 32 * BN * 4;
-    const bool tma_out = splits == 1 && (a.N % 4) == 0 && (a.ldd % 4) == 0 && (a.strideD % 4) == 0 &&
-                         (reinterpret_cast<uintptr_t>(a.D) & 15) == 0 && (!a.addend || (reinterpret_cast<uintptr_t>(a.addend) & 15) == 0) &&
-                         (!a.addend || a.batch == 1);
-    // Split K: room to park the partial tile in the ring, and for the rows this CTA receives (its share from every CTA).
-    const size_t park = splits > 1 ? (size_t)rows * BN * 4 : (tma_out && !a.addend) ? staging : 0;
-    const size_t behind = splits > 1 ? (size_t)splits * ceil_div(rows, splits) * BN * 4 : (tma_out && a.addend) ? staging + 1024 : 0;
-    while (ring < 8 && (size_t)ring * sb < park) ++ring;
-    while (ring > 1 && (size_t)2048 + (size_t)ring * sb + GEMM_BAR_BYTES + (gather ? BM * 8 : 0) + behind > 226u * 1024u && (size_t)(ring - 1) * sb >= park) --ring;
-    g.stages = ring;
-    g.rows = rows;
-    g.bar_off = (uint32_t)ring * sb;
-    const size_t ring_and_bars = (size_t)ring * sb + GEMM_BAR_BYTES + (gather ? BM * 8 : 0);
-    g.recv_off = (uint32_t)align_up(ring_and_bars, 128);
-    g.tma_out = tma_out ? ((BN % 32) == 0 ? 32 : 16) : 0;
-    g.stage_off = a.addend ? (uint32_t)align_up(ring_and_bars, 1024) : 0;
     // equal tiles: the output is addressed as {N, rows, tiles}, so that the hardware clips a tile's last 32-row box
     const bool equal = a.M == m_tiles * rows && (a.batch == 1 || a.strideD == (int64_t)a.M * a.ldd);
     NNV_REQUIRE(equal || rows == BM, NNV_ERR_INVALID_ARG, "batched GEMM outputs must be dense");
     g.z_tiles = equal ? m_tiles : 0;
-    size_t smem_bytes = (size_t)1024 + (splits > 1 ? g.recv_off + behind : (tma_out && a.addend) ? g.stage_off + staging : ring_and_bars);
-    // the MMAs read 128 rows of A from every stage, the last one included
-    smem_bytes = std::max(smem_bytes, (size_t)1024 + (size_t)(ring - 1) * sb + A_STAGE_BYTES);
-    NNV_REQUIRE(smem_bytes <= 226u * 1024u, NNV_ERR_UNSUPPORTED, "GEMM tiling does not fit shared memory");
     auto encode_out = [&](CUtensorMap* map, const void* base) {
         if (equal) return encode_output(map, base, a.N, rows, m_tiles * a.batch, a.ldd, (int64_t)rows * a.ldd, g.tma_out);
         return encode_output(map, base, a.N, a.M, a.batch, a.ldd, a.batch > 1 ? a.strideD : (int64_t)a.M * a.ldd, g.tma_out);
@@ -1586,9 +1615,21 @@ nnv_status_t launch_gemm_tc(const GemmArgs& a, cudaStream_t st) {
     static constexpr decltype(&gemm_tc_kernel<0>) kernels[8] = {gemm_tc_kernel<GEMM_TF32>, gemm_tc_kernel<GEMM_BF16>, gemm_tc_kernel<GEMM_X3>,
         gemm_tc_kernel<GEMM_BF16_CVT>, gemm_tc_kernel<4>, gemm_tc_kernel<5>, gemm_tc_kernel<6>, gemm_tc_kernel<7>};
     NNV_REQUIRE(a.mode >= GEMM_TF32 && a.mode <= GEMM_BF16_CVT, NNV_ERR_INVALID_ARG, "unknown GEMM mode %d", a.mode);
-    (void)launch_pdl_cluster(kernels[mode], grid, dim3(gemm_tc_threads(mode)), smem_bytes, st, splits, tmA, tmB, tmD, tmAdd, g);
+    (void)launch_pdl_cluster(kernels[mode], grid, dim3(gemm_tc_threads(mode)), sh.smem_bytes, st, splits, tmA, tmB, tmD, tmAdd, g);
     NNV_CUDA(cudaGetLastError());
     return NNV_OK;
 }
 
 }  // namespace nnv
+
+// Host-side launch shape of gemm_tc_kernel for the tests (kernel mode, K blocks of 128 bytes).
+extern "C" int nnv_internal_gemm_shape(int mode, int M, int N, int batch, int nkb, int tma_out, int addend, int32_t* out) {
+    using namespace nnv;
+    GemmShape s;
+    const nnv_status_t st = gemm_shape(mode, pick_gemm_tiling(mode, M, N, batch, nkb), M, N, batch, nkb, tma_out != 0, addend != 0, &s);
+    if (st != NNV_OK) return st;
+    const int32_t v[] = {s.BN, s.splits, s.rows, s.m_tiles, s.issuers, s.ring, s.tmem_cols, (int32_t)s.bar_off, (int32_t)s.recv_off,
+                         (int32_t)s.stage_off, (int32_t)s.smem_bytes, (int32_t)gemm_stage_bytes(mode, s.BN, s.rows), gemm_tc_threads(mode)};
+    std::copy(std::begin(v), std::end(v), out);
+    return NNV_OK;
+}
