@@ -169,10 +169,10 @@ conv3x3_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                             umma<true>(tmem_base, make_smem_desc_plain(a + (uint32_t)(r * 10 + s) * 16u + kk * 2u * lbo_a, lbo_a, 160),
                                        make_smem_desc64(b + (uint32_t)s * BN * 64u) + (uint64_t)(kk * 2), idesc,
                                        (it | r | s | kk) ? 1u : 0u);
-                    umma_commit(b_empty(sb));
+                    if (3 * it + r + NB < 3 * ncb) umma_commit(b_empty(sb));           // the slot is refilled: somebody waits
                     if (++sb == NB) { sb = 0; pb ^= 1u; }
                 }
-                if (ok) umma_commit(a_empty(sa));
+                if (ok && it + 2 < ncb) umma_commit(a_empty(sa));
             }
             if (ok) umma_commit(tmem_full_bar);
             else atomicExch(&g_device_status, (int)NNV_ERR_TIMEOUT);

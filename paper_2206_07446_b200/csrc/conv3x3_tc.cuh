@@ -116,6 +116,7 @@ conv3x3_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
             const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
             bool ok = true;
             int sa = 0, sb = 0;
+            int refill_a = 3 * ncb - NA, refill_b = 9 * ncb - NB;    // releases that a producer waits for
             uint32_t pa = 0, pb = 0;
             for (int cbi = 0; cbi < ncb && ok; ++cbi) {
                 for (int s = 0; s < 3 && ok; ++s) {
@@ -134,10 +135,10 @@ conv3x3_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                                 umma<false>(tmem_base + (uint32_t)(mt * BN), adesc + (uint64_t)(kk * 2), bdesc + (uint64_t)(kk * 2),
                                             idesc, (cbi | s | r | kk) ? 1u : 0u);
                         }
-                        umma_commit(b_empty(sb));
+                        if (refill_b-- > 0) umma_commit(b_empty(sb));
                         if (++sb == NB) { sb = 0; pb ^= 1u; }
                     }
-                    if (ok) umma_commit(a_empty(sa));
+                    if (ok && refill_a-- > 0) umma_commit(a_empty(sa));
                     if (++sa == NA) { sa = 0; pa ^= 1u; }
                 }
             }
@@ -453,6 +454,8 @@ conv3x3_tc_persistent_kernel(const __grid_constant__ CUtensorMap tmA, const __gr
             int sa = 0, sb = 0;
             uint32_t pa = 0, pb = 0;
             int lt = 0;                                           // this CTA's tile count so far
+            const int boxes = 3 * g.cblk * ((g.tiles_total - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x);
+            int refill_a = boxes - NA, refill_b = 3 * boxes - NB;     // releases that the producer waits for
             for (int t = blockIdx.x; t < g.tiles_total && ok; t += gridDim.x, ++lt) {
                 const int acc = lt & 1;
                 ok = mbar_wait(t_empty(acc), (((uint32_t)lt >> 1) & 1u) ^ 1u);   // the epilogue has drained this accumulator
@@ -473,10 +476,10 @@ conv3x3_tc_persistent_kernel(const __grid_constant__ CUtensorMap tmA, const __gr
 #pragma unroll
                             for (int kk = 0; kk < 4; ++kk)
                                 umma<false>(tmem_d, adesc + (uint64_t)(kk * 2), bdesc + (uint64_t)(kk * 2), idesc, (cbi | s | r | kk) ? 1u : 0u);
-                            umma_commit(b_empty(sb));
+                            if (refill_b-- > 0) umma_commit(b_empty(sb));
                             if (++sb == NB) { sb = 0; pb ^= 1u; }
                         }
-                        if (ok) umma_commit(a_empty(sa));
+                        if (ok && refill_a-- > 0) umma_commit(a_empty(sa));
                         if (++sa == NA) { sa = 0; pa ^= 1u; }
                     }
                 }
@@ -668,6 +671,7 @@ conv3x3_tc_ws_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
             int sa = 0;
             uint32_t pa = 0;
             int lt = 0;                                           // this CTA's patch count so far
+            int refill_a = 3 * g.cblk * ((g.patches - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x) - CONVW_NA;   // releases that the producer waits for
             for (int t = blockIdx.x; t < g.patches && ok; t += gridDim.x, ++lt) {
                 const int acc = lt & 1;
                 ok = mbar_wait(t_empty(acc), (((uint32_t)lt >> 1) & 1u) ^ 1u);   // the epilogue has drained this accumulator
@@ -692,7 +696,7 @@ conv3x3_tc_ws_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                             for (int kk = 0; kk < 4; ++kk)
                                 umma<false>(tmem_d, adesc + (uint64_t)(kk * 2), bdesc + (uint64_t)(kk * 2), idesc, (cbi | s | r | kk) ? 1u : 0u);
                         }
-                        if (ok) umma_commit(a_empty(sa));
+                        if (ok && refill_a-- > 0) umma_commit(a_empty(sa));
                         if (++sa == CONVW_NA) { sa = 0; pa ^= 1u; }
                     }
                 }

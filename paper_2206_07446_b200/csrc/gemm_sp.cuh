@@ -117,7 +117,7 @@ gemm_sp_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk)                 // 4 MMAs of 32 bytes of K each
                     umma<false>(tmem_base, adesc + (uint64_t)(kk * 2), bdesc + (uint64_t)(kk * 2), idesc, (it | kk) ? 1u : 0u);
-                umma_commit(empty_bar(s));
+                if (it + STAGES < nkb) umma_commit(empty_bar(s));   // the slot is refilled: the producer waits
                 if (++s == STAGES) { s = 0; ph ^= 1u; }
             }
             if (ok) umma_commit(tmem_full_bar);

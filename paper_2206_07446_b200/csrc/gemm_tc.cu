@@ -9,7 +9,8 @@
 //   warps 0, 7  TMA producers of A and B: cp.async.bulk.tensor loads of 128-byte-wide K slices into a ring of
 //            shared-memory stages (128B swizzle), completion on "full" mbarriers
 //   warps 1, 6  issue tcgen05.mma (one lane each) from shared-memory descriptors for alternate K blocks, each into its own
-//            fp32 accumulator in TMEM, and release stages with tcgen05.commit on "empty" mbarriers; warp 1 allocates TMEM
+//            fp32 accumulator in TMEM, and release the stages that are refilled with tcgen05.commit on "empty" mbarriers (an
+//            arrival that nobody waits for could meet a CTA that has left); warp 1 allocates TMEM
 //   warps 2-5  epilogue: tcgen05.ld the accumulators (each warp its own 32 TMEM lanes), apply
 //            bias / residual / activation, store fp32 rows
 // These layers are latency-bound (5 - 10 dependent phases of ~0.1 - 0.5 us each); what bounds each phase was read from
@@ -689,7 +690,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                     for (int kk = 0; kk < 4; ++kk)             // 4 MMAs of 32 bytes of K each
                         umma<bf16_mode(MODE)>(acc, adesc + (uint64_t)(kk * 2), bdesc + (uint64_t)(kk * 2), idesc, kk ? 1u : first);
                 }
-                umma_commit(empty_bar(s));
+                if (it + STAGES < nkb) umma_commit(empty_bar(s));
                 s += g.issuers;
                 while (s >= STAGES) { s -= STAGES; ph ^= 1u; }
             }

@@ -113,7 +113,7 @@ wino_f2_fused_kernel(const __grid_constant__ CUtensorMap tmU, const WfDev g) {
                     const uint64_t bdesc = make_smem_desc_plain(b_s + (uint32_t)p * (uint32_t)BN * 16u, b_chunk, 128u);
                     umma<false>(tmem_base + (uint32_t)(p * BN), adesc, bdesc, idesc, it ? 1u : 0u);
                 }
-                umma_commit(empty_bar(s));
+                if (it + STAGES < g.nsteps) umma_commit(empty_bar(s));   // the slot is refilled: its writers wait
                 if (++s == STAGES) { s = 0; ph ^= 1u; }
             }
             if (ok) umma_commit(tmem_full_bar);

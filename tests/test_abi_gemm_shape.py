@@ -2,12 +2,15 @@
 them, held against a model of the kernel's barrier protocol."""
 import ctypes
 import functools
+import os
 import random
+import re
 
 import pytest
 
 from paper_2206_07446_b200 import binding as nb
 
+CSRC = os.path.join(os.path.dirname(nb.LIB_PATH), "csrc")
 FIELDS = ("BN", "splits", "rows", "m_tiles", "issuers", "ring", "tmem_cols", "bar_off", "recv_off", "stage_off", "smem",
           "stage_bytes", "threads")
 X3, BF16_CVT = 2, 3
@@ -90,3 +93,16 @@ def test_no_issuer_runs_ahead_of_a_load(tuning):
         assert seen > 3000
     finally:
         nb.nnv_tuning_set("")
+
+
+def test_no_arrival_without_a_waiter():
+    """A tcgen05.commit arrives on its own time: on a slot's "empty" barrier only where the slot is refilled, that is, where a
+    producer waits for it before the CTA can leave."""
+    found = 0
+    for f in sorted(os.listdir(CSRC)):
+        if f.endswith((".cu", ".cuh")):
+            for line in open(os.path.join(CSRC, f)):
+                if re.search(r"umma_commit\(\w*empty", line):
+                    found += 1
+                    assert re.search(r"if \(.*(\+ .* < |refill_[ab]-- > 0).*\) umma_commit", line), (f, line)
+    assert found >= 9
