@@ -1015,6 +1015,13 @@ nnv_status_t encode_halo_operand(CUtensorMap* map, const void* base, int C, int 
     return NNV_OK;
 }
 
+// Shared memory of a cluster's CTA is at least the share of the SM's 228 KB (1 KB of it the system's) that its TMEM columns are of
+// 512, so that CTAs that fit an SM find their columns free, whichever launches they come from.  tcgen05.alloc waits without a limit:
+// where more CTAs fit than have columns, each of three clusters may hold columns on some SMs and wait for them on another.
+// (A CTA without a cluster waits for nobody else once it has its columns and needs no such rule.)
+constexpr size_t tmem_share_bytes(int cols) { return (size_t)228 * 1024 * cols / 512 - 1024; }
+static_assert(CB_RINGS_A >= tmem_share_bytes(128), "the BF16 3x3 kernel's rings alone are the share of its columns");
+
 // Tiling of conv3x3_tc_kernel for one layer.
 struct ConvTiling { int MT, BN, splits, na, nb, tmem_cols; size_t smem; };
 
@@ -1036,9 +1043,10 @@ bool finish_conv_tiling(ConvTiling* t) {
         while (rings() < park && t->nb < CONV_MAX_NB) ++t->nb;      // deeper rings only to make room for the parked tiles
         while (rings() < park && t->na < CONV_MAX_NA) ++t->na;
     }
-    t->smem = conv_smem_bytes(t->MT, t->BN, t->na, t->nb);
     t->tmem_cols = 32;
     while (t->tmem_cols < t->MT * t->BN) t->tmem_cols *= 2;
+    t->smem = conv_smem_bytes(t->MT, t->BN, t->na, t->nb);
+    if (t->splits > 1) t->smem = std::max(t->smem, tmem_share_bytes(t->tmem_cols));
     return t->smem <= 200u * 1024u && rings() >= park;
 }
 
@@ -1200,6 +1208,7 @@ nnv_status_t gemm_shape(int mode, const GemmTiling& tile, int M, int N, int batc
     g.smem_bytes = (size_t)1024 + (split ? g.recv_off + behind : (tma_out && addend) ? g.stage_off + staging : ring_and_bars);
     // the MMAs read 128 rows of A from every stage, the last one included
     g.smem_bytes = std::max(g.smem_bytes, (size_t)1024 + (g.ring - 1) * sb + A_STAGE_BYTES);
+    if (split) g.smem_bytes = std::max(g.smem_bytes, tmem_share_bytes(g.tmem_cols));
     NNV_REQUIRE(g.smem_bytes <= 226u * 1024u, NNV_ERR_UNSUPPORTED, "GEMM tiling does not fit shared memory");
     *out = g;
     return NNV_OK;

@@ -95,6 +95,24 @@ def test_no_issuer_runs_ahead_of_a_load(tuning):
         nb.nnv_tuning_set("")
 
 
+@pytest.mark.parametrize("tuning", ["", "gemm_tile=128,8", "gemm_tile=96,2;gemm_ring=2"])
+def test_clusters_that_fit_an_sm_find_their_tmem_columns(tuning):
+    """A cluster's CTA takes at least the share of an SM's 228 KB of shared memory (1 KB of it the system's) that its TMEM
+    columns are of 512: tcgen05.alloc then never waits for a CTA that waits for a member of its own cluster."""
+    nb.nnv_tuning_set(tuning)
+    try:
+        split = 0
+        for c in cases(4000, 11):
+            s = shape(*c)
+            if s is None or s["splits"] == 1:
+                continue
+            split += 1
+            assert (s["smem"] + 1024) * 512 >= 228 * 1024 * s["tmem_cols"], (c, s)
+        assert split > 500
+    finally:
+        nb.nnv_tuning_set("")
+
+
 def test_no_arrival_without_a_waiter():
     """A tcgen05.commit arrives on its own time: on a slot's "empty" barrier only where the slot is refilled, that is, where a
     producer waits for it before the CTA can leave."""
