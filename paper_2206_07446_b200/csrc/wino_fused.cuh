@@ -43,7 +43,6 @@ __device__ __forceinline__ float wf_round_tf32(float v) {
 __global__ void __launch_bounds__(GEMM_THREADS)
 wino_f2_fused_kernel(const __grid_constant__ CUtensorMap tmU, const WfDev g) {
     extern __shared__ uint8_t smem_raw[];
-    pdl_trigger();
     const int STAGES = g.stages, BN = g.BN;
     const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t b_chunk = 16u * (uint32_t)BN * 16u;             // one k-chunk of U: 16 planes x BN rows x 16 bytes
@@ -75,6 +74,7 @@ wino_f2_fused_kernel(const __grid_constant__ CUtensorMap tmU, const WfDev g) {
     tc_fence_after();
     const uint32_t tmem_base = *holder_ptr;
     pdl_wait();
+    pdl_trigger();                                            // not before the TMEM is ours: the next kernel's CTAs would keep theirs while they wait for this one
     if (threadIdx.x == 32) stamp_start(g.stamp);
 
     if (warp == 0) {

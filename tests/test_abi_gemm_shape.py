@@ -124,3 +124,15 @@ def test_no_arrival_without_a_waiter():
                     found += 1
                     assert re.search(r"if \(.*(\+ .* < |refill_[ab]-- > 0).*\) umma_commit", line), (f, line)
     assert found >= 9
+
+
+def test_the_next_kernel_is_let_in_after_the_tmem_allocation():
+    """CTAs let in earlier could take columns that this grid's still need, and keep them until this grid is done."""
+    kernels = 0
+    for f in sorted(os.listdir(CSRC)):
+        if f.endswith((".cu", ".cuh")):
+            for body in open(os.path.join(CSRC, f)).read().split("__global__")[1:]:
+                if "tcgen05.alloc" in body:
+                    kernels += 1
+                    assert body.index("tcgen05.alloc") < body.rindex("pdl_wait();", 0, body.index("pdl_trigger();")), (f, body[:200])
+    assert kernels == 7
