@@ -348,6 +348,7 @@ conv3x3_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                 }
             }
         }
+        __syncwarp();
         cluster_sync_all();                                   // nobody leaves while its tiles may still be read
     }
     tc_fence_before();

@@ -191,6 +191,7 @@ direct_conv_kernel(const DirectDev g) {
             const int row = idx / (T / 4), c4 = (idx % (T / 4)) * 4;
             *reinterpret_cast<float4*>(red + row * RP + c4) = group_sum(row, c4);
         }
+        __syncwarp();                                          // the cluster barrier is one instruction of the whole warp
         asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
         asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     }
@@ -232,6 +233,7 @@ direct_conv_kernel(const DirectDev g) {
         if (vec) *reinterpret_cast<float4*>(g.y + o) = make_float4(v[0], v[1], v[2], v[3]);
     }
     if (g.splits > 1) {                                        // nobody leaves while its partial tile may still be read
+        __syncwarp();
         asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
         asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     }

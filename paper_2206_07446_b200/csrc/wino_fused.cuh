@@ -28,6 +28,7 @@ constexpr int WF_MAX_STAGES = 3;
 constexpr uint32_t WF_A_STAGE = 16u * 2u * 2048u;               // 16 planes x 2 k-chunks x (128 rows x 16 bytes)
 
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
+    __syncwarp();
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
                  : "r"(taddr)

@@ -136,3 +136,20 @@ def test_the_next_kernel_is_let_in_after_the_tmem_allocation():
                     kernels += 1
                     assert body.index("tcgen05.alloc") < body.rindex("pdl_wait();", 0, body.index("pdl_trigger();")), (f, body[:200])
     assert kernels == 7
+
+
+def test_warp_wide_instructions_follow_a_reconvergence():
+    """tcgen05.ld and the cluster barriers are .aligned: one instruction of a whole warp, whose lanes may just have left a loop or
+    a branch on their own."""
+    for f in sorted(os.listdir(CSRC)):
+        if f.endswith((".cu", ".cuh")):
+            src = open(os.path.join(CSRC, f)).read()
+            for m in re.finditer(r"void (tmem_ld\w+)\(uint32_t", src):
+                assert src[m.end():].split("{", 1)[1].lstrip().startswith("__syncwarp();"), (f, m.group(1))
+            lines = [ln.split("//")[0].strip() for ln in src.split("\n")]
+            code = [ln for ln in lines if ln]
+            for i, ln in enumerate(code):
+                own = re.match(r"(asm volatile\(.barrier\.cluster\.arrive|cluster_arrive\w*\(\);|cluster_sync_all\(\);)", ln)
+                if own and "cluster_arrive();" not in ln:
+                    back = code[max(0, i - 3):i]
+                    assert any("__syncwarp();" in b or "__syncthreads();" in b for b in back) or "cluster_arrived" in code[i + 1], (f, ln, back)
