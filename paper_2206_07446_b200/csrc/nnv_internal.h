@@ -91,11 +91,12 @@ inline cudaError_t launch_pdl_cluster(void (*kernel)(Params...), dim3 grid, dim3
 
 #ifdef __CUDACC__
 // fp32 -> TF32 precision (10 explicit mantissa bits), round to nearest even, by integer arithmetic; the result is an fp32
-// word whose low 13 mantissa bits are zero (the tensor core would otherwise truncate).
+// word whose low 13 mantissa bits are zero (the tensor core would otherwise truncate).  NaNs stay as they are: the sum would carry
+// those with all mantissa bits set, which the GPU's own arithmetic gives, out of the exponent and into a zero.
 __device__ __forceinline__ float round_tf32(float v) {
     uint32_t b = __float_as_uint(v);
     b += 0xFFFu + ((b >> 13) & 1u);
-    return __uint_as_float(b & 0xFFFFE000u);
+    return v == v ? __uint_as_float(b & 0xFFFFE000u) : v;
 }
 #endif
 

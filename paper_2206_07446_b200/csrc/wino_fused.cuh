@@ -35,12 +35,6 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
                  : "memory");
 }
 
-__device__ __forceinline__ float wf_round_tf32(float v) {
-    uint32_t b = __float_as_uint(v);
-    b += 0xFFFu + ((b >> 13) & 1u);
-    return __uint_as_float(b & 0xFFFFE000u);
-}
-
 __global__ void __launch_bounds__(GEMM_THREADS)
 wino_f2_fused_kernel(const __grid_constant__ CUtensorMap tmU, const WfDev g) {
     extern __shared__ uint8_t smem_raw[];
@@ -168,8 +162,8 @@ wino_f2_fused_kernel(const __grid_constant__ CUtensorMap tmU, const WfDev g) {
 #pragma unroll
                     for (int b = 0; b < 4; ++b) {
                         const uint32_t addr = a_s + (uint32_t)((a * 4 + b) * 2 + j) * 2048u;
-                        asm volatile("st.shared.v4.f32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "f"(wf_round_tf32(v[b].x)), "f"(wf_round_tf32(v[b].y)),
-                                     "f"(wf_round_tf32(v[b].z)), "f"(wf_round_tf32(v[b].w)) : "memory");
+                        asm volatile("st.shared.v4.f32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "f"(round_tf32(v[b].x)), "f"(round_tf32(v[b].y)),
+                                     "f"(round_tf32(v[b].z)), "f"(round_tf32(v[b].w)) : "memory");
                     }
                 }
             }

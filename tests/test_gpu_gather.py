@@ -35,3 +35,26 @@ def test_gathered_windows(C, K, R, stride, pad, H, W, resid, math):
     assert nb.nnv_exec_workspace_bytes(plan, 0, v, math) == 0      # no matrix of the windows in memory
     y = run_conv(plan, 0, L, v, math, x, w, b, add)
     assert_conv_close(y, omodel.run_layer(L, x, w, b, add), TOL[math])
+
+
+@pytest.mark.parametrize("math", [nb.MATH_TF32, nb.MATH_BF16])
+@pytest.mark.parametrize("C,K,R,stride,pad,H,W", [
+    (3, 16, 3, 2, 1, 19, 23),           # gathered word by word
+    (64, 48, 3, 2, 1, 8, 8),            # gathered four channels at a time
+    (64, 40, 3, 1, 1, 7, 7),            # boxes of a small image
+    (64, 64, 3, 1, 1, 40, 40),          # read in place by the TMA
+    (333, 300, 1, 1, 0, 7, 7),          # explicit im2col (TF32)
+])
+def test_nan_pixels_stay_nan(C, K, R, stride, pad, H, W, math):
+    """A NaN input -- with the bits the GPU's own arithmetic gives it, which integer rounding carries out of the exponent -- reaches
+    exactly the outputs whose window holds it."""
+    L = dict(op=nb.OP_CONV, C=C, K=K, R=R, S=R, stride=stride, pad=pad, groups=1, H=H, W=W, in0=-1, in1=-1, act=0, has_bias=0)
+    rng = np.random.default_rng([C, K, 5])
+    x = rng.uniform(-1, 1, (C, H, W)).astype(np.float32)
+    h, w0, c = H // 2, W // 2, C - 1
+    x.view(np.uint32)[c, h, w0] = 0x7FFFFFFF
+    w = (rng.standard_normal((K, C, R, R)) * np.sqrt(2.0 / (C * R * R))).astype(np.float32)
+    y = run_conv(nb.Plan([L]), 0, L, nb.VAR_GEMM1X1 if R == 1 else nb.VAR_IM2COL, math, x, w)
+    p, q = np.arange(y.shape[1]) * stride - pad, np.arange(y.shape[2]) * stride - pad
+    hit = ((p <= h) & (h < p + R))[:, None] & ((q <= w0) & (w0 < q + R))[None, :]
+    assert hit.any() and np.array_equal(np.isnan(y), np.broadcast_to(hit, y.shape))
