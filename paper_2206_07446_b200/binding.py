@@ -233,6 +233,8 @@ def nnv_exec_workspace_bytes(plan, layer, variant, math):
 
 def _choices_array(plan, choices):
     if isinstance(choices, ctypes.Array):                 # already marshalled (choices_array): latency-critical callers
+        if choices._type_ is not Choice or len(choices) < plan.n:
+            raise ValueError("an array of one Choice per layer expected")
         return choices
     arr = (Choice * plan.n)()
     for i, c in enumerate(choices):
@@ -641,7 +643,7 @@ try:
     from . import _nnvcall
 except ImportError as e:
     raise ImportError("_nnvcall.so is not built (%s). Run `python -m paper_2206_07446_b200.build`." % e)
-_nnvcall.set_fallbacks(nnv_conv_exec, nnv_transform_weights, nnv_transform_all, _check)
+_nnvcall.set_fallbacks(nnv_conv_exec, nnv_transform_weights, nnv_transform_all, _check, ctypes.Array, Choice)
 nnv_conv_exec = _nnvcall.nnv_conv_exec
 nnv_transform_weights = _nnvcall.nnv_transform_weights
 nnv_transform_all = _nnvcall.nnv_transform_all

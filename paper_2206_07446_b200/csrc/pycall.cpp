@@ -17,6 +17,10 @@ namespace {
 PyObject* s_data_ptr;
 PyObject* s_cuda_stream;
 PyObject* s_address;
+PyObject* s_n;
+PyObject* s_type;
+PyObject* g_array;                                            // ctypes.Array and the binding's Choice
+PyObject* g_choice;
 
 // One converted argument; ok = false: not a kind that is handled here.
 struct Arg {
@@ -54,14 +58,20 @@ Arg stream(PyObject* o) {
 }
 Arg plan(PyObject* o) { return from_call(PyObject_GetAttr(o, s_address)); }
 
-// Buffer address of a ctypes array (choices already laid out by choices_array), as long as the plan's layers need.
-Arg choices(PyObject* o, Py_ssize_t want) {
+// Address of the choices already laid out by choices_array: a ctypes array of Choice with one entry for each of the plan's layers.
+// Nothing else that exports a buffer will do: a numpy array's rows are another layout, for the Python function to convert.
+Arg choices(PyObject* o, PyObject* plan) {
+    const Arg no{0, false};
+    const int is_array = PyObject_IsInstance(o, g_array);
+    PyObject* type = is_array == 1 ? PyObject_GetAttr(o, s_type) : nullptr;
+    const Arg n = type == g_choice ? from_call(PyObject_GetAttr(plan, s_n)) : no;
+    Py_XDECREF(type);
     Py_buffer b;
-    if (!PyObject_CheckBuffer(o) || PyObject_GetBuffer(o, &b, PyBUF_SIMPLE) != 0) {
+    if (!n.ok || PyObject_GetBuffer(o, &b, PyBUF_SIMPLE) != 0) {
         PyErr_Clear();
-        return {0, false};
+        return no;
     }
-    const Arg a{(uint64_t)(uintptr_t)b.buf, b.len >= want};
+    const Arg a{(uint64_t)(uintptr_t)b.buf, (uint64_t)b.len / sizeof(nnv_choice_t) >= n.v};
     PyBuffer_Release(&b);
     return a;
 }
@@ -123,7 +133,7 @@ PyObject* transform_weights(PyObject*, PyObject* const* args, Py_ssize_t n, PyOb
 PyObject* transform_all(PyObject*, PyObject* const* args, Py_ssize_t n, PyObject* kw) {
     uint64_t v[6];
     if (n < 6 || n > 7 || (kw && PyTuple_GET_SIZE(kw) != 0)) return PyObject_Vectorcall(g_fallback[2], args, n, kw);
-    const Arg c = choices(args[1], 0);
+    const Arg c = choices(args[1], args[0]);
     PyObject* rest[6] = {args[0], args[2], args[3], args[4], args[5], n == 7 ? args[6] : Py_None};
     if (!c.ok || !convert("paiais", rest, 6, nullptr, v)) return PyObject_Vectorcall(g_fallback[2], args, n, kw);
     nnv_status_t st;
@@ -134,12 +144,14 @@ PyObject* transform_all(PyObject*, PyObject* const* args, Py_ssize_t n, PyObject
 }
 
 PyObject* set_fallbacks(PyObject*, PyObject* const* args, Py_ssize_t n) {
-    if (n != 4) {
-        PyErr_SetString(PyExc_TypeError, "four functions expected");
+    if (n != 6) {
+        PyErr_SetString(PyExc_TypeError, "four functions and two classes expected");
         return nullptr;
     }
     for (int i = 0; i < 3; ++i) Py_XSETREF(g_fallback[i], Py_NewRef(args[i]));
     Py_XSETREF(g_check, Py_NewRef(args[3]));
+    Py_XSETREF(g_array, Py_NewRef(args[4]));
+    Py_XSETREF(g_choice, Py_NewRef(args[5]));
     Py_RETURN_NONE;
 }
 
@@ -158,5 +170,7 @@ PyMODINIT_FUNC PyInit__nnvcall(void) {
     s_data_ptr = PyUnicode_InternFromString("data_ptr");
     s_cuda_stream = PyUnicode_InternFromString("cuda_stream");
     s_address = PyUnicode_InternFromString("address");
+    s_n = PyUnicode_InternFromString("n");
+    s_type = PyUnicode_InternFromString("_type_");
     return PyModule_Create(&g_module);
 }

@@ -221,3 +221,34 @@ def test_tuning_overrides_parse_and_reject():
             assert e.value.status == 1, bad
     finally:
         nb.nnv_tuning_set(None)
+
+
+def test_choices_reach_the_library_as_what_they_are():
+    """Every form of per-layer choices -- tuples, a Choice array, numpy rows of any integer type -- means the same, and one that is too
+    short is refused before the library reads it.  (An output of no bytes: the message names the size the choices ask for.)"""
+    layers = wl.tiny_net()
+    plan = _plan(layers)
+    rows = []
+    for i, L in enumerate(layers):
+        v = max(nb.nnv_eligible(plan, i)) if L["op"] == wl.OP_CONV else 0
+        rows.append((v, nb.MATH_FP32 if v in (nb.VAR_DIRECT, nb.VAR_DEPTHWISE) else nb.MATH_TF32, 0))
+    need = nb.nnv_transformed_layout(plan, rows)[1]
+    marshalled = nb.choices_array(plan, rows)
+    longer = (nb.Choice * (plan.n + 3))(*marshalled)
+
+    def error(choices, **kw):
+        with pytest.raises(nb.NnvError) as e:
+            nb.nnv_transform_all(plan, choices, 256, 0, 256, 0, **kw)
+        return str(e.value)
+
+    want = error(rows)
+    assert "needs %d bytes" % need in want
+    for form in (marshalled, longer, np.array(rows, np.int32), np.array(rows, np.int64), np.array(rows, np.uint8)):
+        assert error(form) == want and error(form, stream=None) == want
+    short = (nb.Choice * (plan.n - 1))(*marshalled[:plan.n - 1])
+    words = (ctypes.c_int32 * (3 * plan.n))()
+    for bad in (short, words):
+        for call in (lambda: nb.nnv_transform_all(plan, bad, 256, 0, 256, 0), lambda: nb.nnv_arena_bytes(plan, bad, 0),
+                     lambda: nb.nnv_transformed_layout(plan, bad)):
+            with pytest.raises(ValueError):
+                call()
