@@ -15,7 +15,8 @@ switched OFF, and every call is enqueued eagerly (no recorded graph: a cold infe
   roofline*  kernel durations come from the per-layer events of the TIMED headline steps
 
 `python bench.py` (1 GPU) or under torch.distributed.run with --gpus N (independent replicas; the path
-does not shard).  `--impl reference` times the CPU oracle instead.  `--kernel ...` times one kernel
+does not shard).  One JSON line on standard output; the whole report goes to --report FILE or standard error.
+`--impl reference` times the CPU oracle instead.  `--kernel ...` times one kernel
 (or a sweep of shapes) through the C ABI instead of a whole step.
 """
 import argparse
@@ -64,6 +65,7 @@ def parse():
     ap.add_argument("--file-reps", type=int, default=5, help="cold runs fed from a model file on local storage (0 = skip)")
     ap.add_argument("--also", default="cfg2_resnet18,cfg5_vgg16", help="other workloads measured beside --config (headline, e2e and rooflines only)")
     ap.add_argument("--minimal", action="store_true", help="headline + e2e + rooflines only (no side arms or sections)")
+    ap.add_argument("--report", default=None, help="write the whole report (per layer, arms, sections; JSON) to this file instead of standard error")
     ap.add_argument("--save-costs", default=None, help="write the profiled cost table (JSON) to this file")
     ap.add_argument("--load-costs", default=None, help="use a cost table saved earlier instead of profiling (e.g. under a profiler)")
     # single-kernel timing through the C ABI
@@ -357,8 +359,37 @@ def run_ours(args):
         others[name]["e2e"] = {k: o["e2e"][k] for k in ("value", "h2d_bytes_per_step", "host_link")}
     line["other_workloads"] = others
     if rank == 0:
-        print(json.dumps(line))
+        report = json.dumps(line)
+        if args.report:
+            with open(args.report, "w") as f:
+                f.write(report + "\n")
+        else:
+            print(report, file=sys.stderr)
+        print(json.dumps(finite(headline(line)), allow_nan=False))
     ranks.close()
+
+
+def finite(v):
+    """v with every number that strict JSON has no text for replaced by null."""
+    if isinstance(v, dict):
+        return {k: finite(x) for k, x in v.items()}
+    if isinstance(v, (list, tuple)):
+        return [finite(x) for x in v]
+    return None if isinstance(v, float) and not np.isfinite(v) else v
+
+
+def headline(line):
+    """The one line of standard output: the result, without what explains it.  The whole report is over 20 KB, more than a reader
+    of the output's end keeps."""
+    out = {k: v for k, v in line.items() if k in (
+        "metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "ms_per_step_median", "higher_is_better", "scaling",
+        "vs_baseline", "dtype", "data", "config", "gpu_launches", "clocks", "cpu_baseline", "parity_rel_l2_end_to_end")}
+    out["e2e"] = {k: v for k, v in line["e2e"].items() if k != "what"}
+    for k in ("roofline", "roofline_transform", "transform_all"):
+        if line.get(k):
+            out[k] = {f: line[k].get(f) for f in ("bound", "achieved", "peak", "unit", "frac", "traffic") if f in line[k]}
+    out["other_workloads"] = {n: {"value": o["value"], "e2e": o["e2e"]["value"]} for n, o in line.get("other_workloads", {}).items()}
+    return out
 
 
 def measure(args, config, steps, warmup, minimal, rank, world, local, ranks):

@@ -1,0 +1,31 @@
+"""The line that bench.py prints, cut from a whole report: small, strict JSON, with everything a reader of the result needs."""
+import json
+
+import bench
+
+
+def _report():
+    roof = {"kernel": "k" * 100, "bound": "hbm", "achieved": 1.0, "peak": 2.0, "unit": "GB/s", "frac": 0.5, "traffic": None, "durations": "d" * 90}
+    e2e = {"value": 1.8, "unit": "ms", "h2d_bytes_per_step": 94000000, "d2h_bytes_per_step": 4000, "host_wall_ms": 1.9, "host_enqueue_ms": 0.3,
+           "what": "w" * 80, "host_link": {"bound": "pcie", "bulk_copy_gbs": 55.2, "floor_ms": 1.7, "frac_of_floor": float("inf")}}
+    other = {"value": 0.9, "unit": "ms", "steps": 20, "e2e": dict(e2e), "roofline": dict(roof), "per_layer": [{"layer": i, "shape": "s" * 40} for i in range(20)]}
+    return {"metric": bench.METRIC, "value": 1.8, "unit": "ms", "n_gpus": 1, "steps": 20, "warmup": 5, "ms_per_step": 1.8,
+            "ms_per_step_median": float("nan"), "higher_is_better": False, "scaling": "weak", "vs_baseline": None, "dtype": "tf32",
+            "data": "synthetic", "config": {"workload": "cfg4_resnet50", "batch": 1, "math": "tf32", "weights": "w" * 90, "l2": "l" * 60},
+            "run": {"what": "r" * 120}, "e2e": e2e, "gpu_launches": 4000, "clocks": {"sm_mhz": 1965.0, "sm_max_mhz": 1965.0, "reasons": [], "samples": 9},
+            "roofline": roof, "roofline_transform": dict(roof), "transform_all": dict(roof), "kernel_rooflines": [dict(roof)] * 8,
+            "per_layer": [{"layer": i, "shape": "s" * 40} for i in range(60)], "arms": {"a": "x" * 4000}, "algorithm1": None, "breakdown": {"choices": [["im2col", "tf32", 0]] * 60},
+            "cpu_baseline": {"value": 1588.0, "unit": "ms", "cores": 16, "kind": "oracle", "sample": "s" * 120}, "other_workloads": {"cfg2_resnet18": other, "cfg5_vgg16": other}}
+
+
+def test_the_printed_line_is_small_strict_and_complete():
+    line = _report()
+    text = json.dumps(bench.finite(bench.headline(line)), allow_nan=False)
+    assert len(text) < 3000 < len(json.dumps(line)) and "\n" not in text
+    got = json.loads(text)
+    for k in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling", "vs_baseline", "dtype", "data",
+              "config", "gpu_launches", "cpu_baseline"):
+        assert got[k] == line[k], k
+    assert {"value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step"} <= set(got["e2e"]) and {"sm_mhz", "sm_max_mhz", "reasons"} <= set(got["clocks"])
+    assert got["ms_per_step_median"] is None and got["e2e"]["host_link"]["frac_of_floor"] is None       # not NaN, not Infinity
+    assert got["other_workloads"]["cfg5_vgg16"] == {"value": 0.9, "e2e": 1.8} and got["roofline"]["frac"] == 0.5
