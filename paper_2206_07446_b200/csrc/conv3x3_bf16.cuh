@@ -150,7 +150,7 @@ conv3x3_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | (8u << 24);
             constexpr uint32_t lbo_a = CB_PIX * 16u;
             bool ok = true;
-            int sb = 0;
+            int sb = 0, refill_b = 3 * ncb - NB;              // releases that the producer waits for
             uint32_t pb = 0;
             for (int it = 0; it < ncb && ok; ++it) {
                 const int sa = it & 1;
@@ -169,7 +169,7 @@ conv3x3_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                             umma<true>(tmem_base, make_smem_desc_plain(a + (uint32_t)(r * 10 + s) * 16u + kk * 2u * lbo_a, lbo_a, 160),
                                        make_smem_desc64(b + (uint32_t)s * BN * 64u) + (uint64_t)(kk * 2), idesc,
                                        (it | r | s | kk) ? 1u : 0u);
-                    if (3 * it + r + NB < 3 * ncb) umma_commit(b_empty(sb));           // the slot is refilled: somebody waits
+                    if (refill_b-- > 0) umma_commit(b_empty(sb));
                     if (++sb == NB) { sb = 0; pb ^= 1u; }
                 }
                 if (ok && it + 2 < ncb) umma_commit(a_empty(sa));
