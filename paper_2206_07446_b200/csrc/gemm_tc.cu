@@ -1052,36 +1052,11 @@ bool finish_conv_tiling(ConvTiling* t) {
     return t->smem <= 200u * 1024u && rings() >= park;
 }
 
-// The TF32 halo kernel's tiling, if it is to be used: one MMA tile per CTA, channel tiles of up to 128, shallow rings (two or three
-// CTAs then share an SM, and one CTA's fill and write-out overlap another's MMAs), all CTAs resident at once: the box ring drops to
-// one slot when that makes them fit.  Its K split is dear (7 us), so it splits only to fill the GPU.
-// It moves fewer operand bytes than the implicit GEMM but has one issuing thread where that has two.  Measured (us, halo kernel /
-// implicit GEMM): it wins where the implicit GEMM's tiles do not fit the GPU at once -- 64 -> 64 @224 12.7 / 17.1, 128 -> 256 @112
-// 18.4 / 24.8, 64 -> 128 @180 12.6 / 17.9, 64 -> 112 @160 11.8 / 23.3, 512 -> 512 @72 58 / 84 -- and on deep layers with some 50
-// patches, 512 -> 256 @56 22.7 / 25.4; it loses where they fit: 128 -> 128 @112 15.4 / 13.3, 64 -> 64 @180 11.8 / 10.0,
-// 256 -> 512 @56 26.1 / 22.0.
-bool pick_conv_tiling(int C, int H, int W, int N, bool gemm_fits, ConvTiling* out) {
-    const int cblk = ceil_div(C, 32);
-    ConvTiling t{};
-    t.MT = 1;
-    t.BN = std::min(128, ceil_div(N, 16) * 16);
-    const long long tiles = (long long)ceil_div(H, 16) * ceil_div(W, 8) * ceil_div(N, t.BN);
-    if (gemm_fits && !(cblk >= 12 && tiles >= 48)) return false;
-    t.splits = 1;
-    while (t.splits * 2 <= std::min(8, cblk) && tiles * t.splits < 148) t.splits *= 2;
-    const long long ctas = tiles * t.splits;
-    bool found = false;
-    const int rings[2][2] = {{2, 3}, {1, 3}};
-    for (int i = 0; i < 2 && !found; ++i) {
-        ConvTiling c = t;
-        c.na = rings[i][0]; c.nb = rings[i][1];
-        if (!finish_conv_tiling(&c)) continue;
-        const int occ = std::max(1, std::min((int)(227u * 1024u / (c.smem + 1024)), 512 / c.tmem_cols));
-        if (ctas <= 148ll * occ) { t = c; found = true; }
-    }
-    if (!found) { t.na = 0; t.nb = 0; found = finish_conv_tiling(&t); }
-    if (found) *out = t;
-    return found;
+// CTAs that run at once in clusters of `splits`, `occ` to an SM: whole clusters must find room inside one GPC (as
+// cudaOccupancyMaxActiveClusters reports).
+int cluster_slots(int splits, int occ) {
+    static constexpr int slots[5][3] = {{148, 296, 444}, {148, 296, 444}, {132, 284, 416}, {120, 264, 384}, {112, 224, 336}};
+    return slots[splits == 16 ? 4 : splits == 8 ? 3 : splits == 4 ? 2 : splits - 1][std::min(occ, 3) - 1];
 }
 
 uint32_t gemm_stage_bytes(int mode, int bn, int rows) {
@@ -1131,10 +1106,7 @@ GemmTiling search_gemm_tiling(int mode, int M, int N, int batch, int nkb) {
                 while (tmem < 2 * bn) tmem *= 2;
                 const double smem = 2048.0 + (double)ring * gemm_stage_bytes(mode, bn, rows) + (sp > 1 ? 4.0 * rows * bn : 0.0);
                 const int occ = std::max(1, std::min({gather_mode(mode) || x3 ? 2 : 3, (int)(226.0 * 1024.0 / smem), 512 / tmem}));
-                // whole clusters must find free SMs inside one GPC: how many CTAs fit with one, two and three to an SM (as
-                // cudaOccupancyMaxActiveClusters reports)
-                static const int cap[5][3] = {{148, 296, 444}, {148, 296, 444}, {132, 284, 416}, {120, 264, 384}, {112, 224, 336}};
-                const long long slots = cap[sp == 16 ? 4 : sp == 8 ? 3 : sp == 4 ? 2 : sp - 1][occ - 1];
+                const long long slots = cluster_slots(sp, occ);
                 const double waves = (double)((ctas + slots - 1) / slots);
                 const double res = (double)std::min<long long>(occ, (ctas + 147) / 148);
                 double kb = std::max({(x3 ? 0.37 : 0.146) * res, kb_bytes * res / 108e3, kb_bytes * (double)std::min(ctas, slots) / (x3 ? 4.6e6 : 10.9e6)});
@@ -1159,6 +1131,51 @@ GemmTiling pick_gemm_tiling(int mode, int M, int N, int batch, int nkb) {
     if (e.mode != mode || e.M != M || e.N != N || e.batch != batch || e.nkb != nkb)
         e = Entry{mode, M, N, batch, nkb, search_gemm_tiling(mode, M, N, batch, nkb)};
     return e.t;
+}
+
+// The TF32 halo kernel's tiling, if it is to be used: one MMA tile per CTA, channel tiles of up to 128, two or one box slots and three
+// weight tiles (two or three CTAs then share an SM, and one CTA's fill and write-out overlap another's MMAs).  It moves fewer operand
+// bytes than the implicit GEMM but has one issuing thread where that has two, and its K split is dear.  Of the tilings the one with
+// the least estimated time (us), if that is below the GEMM's: waves x (channel blocks per CTA x time per block + start and write-out).
+// A block's time depends on the CTAs that share the SM and on the box slots, 2.4 with an SM to itself, 3.1 for two (2.7 at 64 columns),
+// 5.2 for three on one slot; an even spread is not to be had with room for three CTAs to an SM or in clusters of eight.  A K block of
+// the GEMM is 0.25, 0.31 with two CTAs to an SM.  Where the GEMM's tiles need a second wave the halo kernel is always ahead.  A K
+// split runs in one wave of whole clusters or not at all: a second one costs as much as the first (72 clusters of four on 71 places:
+// 384 -> 512 @48 34.7 us, with one box slot and three CTAs to an SM 27.4).
+// Fitted to 240 layers (64 - 768 channels, 28 - 224 pixels a side), the chosen kernel and tiling 0.4 % above the best measured on
+// average.  Measured, halo kernel / implicit GEMM: 64 -> 64 @224 12.3 / 16.8, 128 -> 256 @112 18.2 / 25.2, 512 -> 512 @72 54 / 80, 384 -> 256
+// @80 27.5 / 32.2, 512 -> 256 @56 23.2 / 26.5, 768 -> 64 @112 30.5 / 56; the GEMM's: 128 -> 128 @112 15.4 / 13.3, 64 -> 64 @180 11.2 / 10.0,
+// 384 -> 512 @48 27.4 / 21.8, 512 -> 512 @28 16.6 / 15.8.
+double halo_us(const ConvTiling& t, long long tiles, int cblk) {
+    const int occ = std::max(1, std::min({(int)(227u * 1024u / (t.smem + 1024)), 512 / t.tmem_cols, 3}));
+    const long long ctas = tiles * t.splits, slots = cluster_slots(t.splits, occ);
+    if (t.splits > 1 && ctas > slots) return 1e30;
+    const int r = t.splits == 8 ? occ : (int)std::min<double>(occ, std::ceil((double)ctas / cluster_slots(t.splits, 1) + (occ == 3 ? 0.3 : 0.0)));
+    const double bn = t.BN;
+    const double block = t.na >= 2 ? (r == 1 ? 2.44 : r == 2 ? std::max(2.44, 2.25 + 0.00625 * bn) : std::max(2.6, 2.6 + 0.0164 * bn))
+                                   : (r == 1 ? 2.6 + 0.0057 * bn : r == 2 ? 2.5 + 0.0125 * bn : 5.2);
+    const double rest = t.splits == 1 ? 3.5 + 0.0155 * bn : t.splits == 2 ? 5.4 + 0.06 * bn : t.splits == 4 ? 5.0 + 0.045 * bn : 5.8 + 0.045 * bn;
+    return (double)((ctas + slots - 1) / slots) * (ceil_div(cblk, t.splits) * block + rest);
+}
+bool pick_conv_tiling(int C, int H, int W, int N, const GemmTiling& gemm, ConvTiling* out) {
+    const int cblk = ceil_div(C, 32), BN = std::min(128, ceil_div(N, 16) * 16);
+    const long long tiles = (long long)ceil_div(H, 16) * ceil_div(W, 8) * ceil_div(N, BN);
+    double best = 1e30;
+    if (gemm.waves == 1) {
+        const long long ctas = (long long)ceil_div(H * W, gemm.rows) * ceil_div(N, gemm.BN) * gemm.splits;
+        best = ceil_div(9 * cblk, gemm.splits) * (ctas <= 148 ? 0.247 : 0.31) + 1.4 + 0.033 * gemm.BN +
+               (gemm.splits == 1 ? 0.0 : gemm.splits == 2 ? 0.9 + 0.0172 * gemm.BN : 0.7 + 0.0093 * gemm.BN);
+    }
+    bool found = false;
+    for (int splits = 1; splits <= 8 && splits <= cblk; splits *= 2)
+        for (int na = 2; na >= 1; --na) {
+            ConvTiling c{};
+            c.MT = 1; c.BN = BN; c.splits = splits; c.na = na; c.nb = 3;
+            if (!finish_conv_tiling(&c)) continue;
+            const double t = halo_us(c, tiles, cblk);
+            if (t < best - 1e-9) { best = t; *out = c; found = true; }
+        }
+    return found;
 }
 
 // Ring, issuers and shared-memory layout of one launch of gemm_tc_kernel (host arithmetic only; `mode` is the kernel's).
@@ -1536,7 +1553,7 @@ nnv_status_t launch_gemm_tc(const GemmArgs& a, cudaStream_t st) {
             if (tn.conv3x3 != 1) return launch_conv3x3_bf16(a, ct.BN, ct.splits, st);
         } else {
         ConvTiling ct;
-        bool use = pick_conv_tiling(a.ic.C, a.ic.H, a.ic.W, a.N, tile.waves == 1, &ct);
+        bool use = pick_conv_tiling(a.ic.C, a.ic.H, a.ic.W, a.N, tile, &ct);
         if (tn.conv3x3 == 1) {
             use = false;
         } else if (tn.conv3x3 == 2) {
@@ -1642,6 +1659,17 @@ extern "C" int nnv_internal_gemm_shape(int mode, int M, int N, int batch, int nk
     if (st != NNV_OK) return st;
     const int32_t v[] = {s.BN, s.splits, s.rows, s.m_tiles, s.issuers, s.ring, s.tmem_cols, (int32_t)s.bar_off, (int32_t)s.recv_off,
                          (int32_t)s.stage_off, (int32_t)s.smem_bytes, (int32_t)gemm_stage_bytes(mode, s.BN, s.rows), gemm_tc_threads(mode)};
+    std::copy(std::begin(v), std::end(v), out);
+    return NNV_OK;
+}
+
+// The 3x3 halo kernel's tiling for a TF32 layer, for the tests; out[0] = 0: the implicit GEMM takes the layer.
+extern "C" int nnv_internal_conv3x3_shape(int C, int H, int W, int N, int32_t* out) {
+    using namespace nnv;
+    ConvTiling t{};
+    const GemmTiling gemm = pick_gemm_tiling(GEMM_TF32, H * W, N, 1, 9 * ceil_div(C, 32));
+    const bool use = pick_conv_tiling(C, H, W, N, gemm, &t);
+    const int32_t v[] = {use, t.MT, t.BN, t.splits, t.na, t.nb, t.tmem_cols, (int32_t)t.smem, gemm.waves};
     std::copy(std::begin(v), std::end(v), out);
     return NNV_OK;
 }

@@ -153,3 +153,39 @@ def test_warp_wide_instructions_follow_a_reconvergence():
                 if own and "cluster_arrive();" not in ln:
                     back = code[max(0, i - 3):i]
                     assert any("__syncwarp();" in b or "__syncthreads();" in b for b in back) or "cluster_arrived" in code[i + 1], (f, ln, back)
+
+
+def halo_shape(C, H, W, N):
+    out = (ctypes.c_int32 * 9)()
+    assert ctypes.CDLL(nb.LIB_PATH).nnv_internal_conv3x3_shape(C, H, W, N, out) == 0
+    return dict(zip(("use", "MT", "BN", "splits", "na", "nb", "tmem_cols", "smem", "gemm_waves"), out))
+
+
+def test_split_halo_layers_run_in_one_wave_of_whole_clusters():
+    """A second wave costs the split 3x3 kernel as much as the first.  Clusters of 2 / 4 / 8 CTAs that run at once with one, two and
+    three CTAs to an SM, as the occupancy API reports them on this GPU (132 ... 416 for four: GPCs hold no whole number of them)."""
+    slots = {1: (148, 296, 444), 2: (148, 296, 444), 4: (132, 284, 416), 8: (120, 264, 384)}
+    rng, used, split = random.Random(3), 0, 0
+    layers = [(32 * rng.randrange(1, 25), rng.randrange(7, 240), rng.randrange(7, 240), rng.randrange(1, 520)) for _ in range(4000)]
+    layers += [(384, 48, 48, 512), (512, 40, 56, 512), (384, 80, 80, 256), (512, 160, 160, 64)]
+    for C, H, W, N in layers:
+        t = halo_shape(C, H, W, N)
+        if not t["use"]:
+            assert t["gemm_waves"] == 1
+            continue
+        used += 1
+        tiles = -(-H // 16) * -(-W // 8) * -(-N // t["BN"])
+        occ = min(3, 227 * 1024 // (t["smem"] + 1024), 512 // t["tmem_cols"])
+        assert t["splits"] <= -(-C // 32) and t["smem"] <= 200 * 1024
+        if t["splits"] > 1:
+            split += 1
+            assert tiles * t["splits"] <= slots[t["splits"]][occ - 1], (C, H, W, N, t)
+    assert used > 1000 and split > 100
+
+
+@pytest.mark.parametrize("C,N,H,W,splits", [
+    (64, 64, 224, 224, 1), (128, 256, 112, 112, 1), (512, 512, 72, 72, 1), (512, 256, 56, 56, 4), (384, 256, 80, 80, 4),   # the halo kernel's
+    (128, 128, 112, 112, 0), (64, 64, 180, 180, 0), (384, 512, 48, 48, 0), (512, 512, 40, 56, 0), (256, 512, 56, 56, 0)])  # the GEMM's
+def test_halo_kernel_takes_the_layers_it_was_measured_to_win(C, N, H, W, splits):
+    t = halo_shape(C, H, W, N)
+    assert (t["splits"] if t["use"] else 0) == splits
