@@ -62,8 +62,8 @@ Arg plan(PyObject* o) { return from_call(PyObject_GetAttr(o, s_address)); }
 // Nothing else that exports a buffer will do: a numpy array's rows are another layout, for the Python function to convert.
 Arg choices(PyObject* o, PyObject* plan) {
     const Arg no{0, false};
-    const int is_array = PyObject_IsInstance(o, g_array);
-    PyObject* type = is_array == 1 ? PyObject_GetAttr(o, s_type) : nullptr;
+    if (!PyType_IsSubtype(Py_TYPE(o), (PyTypeObject*)g_array)) return no;
+    PyObject* type = PyObject_GetAttr((PyObject*)Py_TYPE(o), s_type);
     const Arg n = type == g_choice ? from_call(PyObject_GetAttr(plan, s_n)) : no;
     Py_XDECREF(type);
     Py_buffer b;
