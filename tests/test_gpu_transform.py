@@ -144,3 +144,24 @@ def test_random_filter_banks(K, C):
             nb.nnv_transform_weights(planr, 0, variant, math, dev(wr), d_out, torch.cuda.current_stream())
             torch.cuda.synchronize()
             assert np.array_equal(d_out[:nbytes].cpu().numpy(), ref.view(np.uint8).reshape(-1)), (R, bf16)
+
+
+def test_tf32_rounding_of_every_kind_of_word():
+    """Words of every exponent, subnormals, ties, the largest finite numbers (which round to infinity) and infinities: bit for bit the
+    oracle's rounding; NaNs stay NaN."""
+    rng = np.random.default_rng(17)
+    bits = rng.integers(0, 1 << 32, 256 * 256, dtype=np.uint64).astype(np.uint32)
+    bits[:8192] = (bits[:8192] & np.uint32(0xFFFFE000)) | rng.choice(np.array([0xFFF, 0x1000, 0x1001], np.uint32), 8192)   # around a tie
+    bits[8192:8200] = [0x7F7FFFFF, 0xFF7FFFFF, 0x7F800000, 0xFF800000, 0x00000001, 0x80000000, 0x00000FFF, 0x7F7FEFFF]
+    bits[8200:8204] = [0x7FFFFFFF, 0xFFFFFFFF, 0x7F800001, 0x7FC00000]
+    w = bits.view(np.float32).reshape(256, 256, 1, 1)
+    L = _layer(256, 256, 1)
+    L["pad"] = 0
+    plan = nb.Plan([L], [0], [0])
+    d_out = poisoned(w.nbytes)
+    nb.nnv_transform_weights(plan, 0, nb.VAR_GEMM1X1, nb.MATH_TF32, dev(w), d_out, torch.cuda.current_stream())
+    got = d_out[:w.nbytes].cpu().numpy().view(np.float32).reshape(-1)
+    nan = np.isnan(w).reshape(-1)
+    assert np.array_equal(np.isnan(got), nan) and nan.sum() > 100
+    ref = opack.tf32_round_rne(w).reshape(-1)
+    assert np.array_equal(got.view(np.uint32)[~nan], ref.view(np.uint32)[~nan])
