@@ -208,10 +208,12 @@ SmallPPlan small_p_plan(const nnv_layer_desc_t& L, const LayerGeom& g, int v, in
     if (!tn.smallp || (v != NNV_VAR_IM2COL && v != NNV_VAR_GEMM1X1) || math != NNV_MATH_TF32 || L.groups != 1 || L.stride != 1 ||
         L.R != L.S || (L.R & 1) == 0 || L.pad != (L.R - 1) / 2 || L.H * L.W > 256 || (L.C % 32) != 0 || (L.K % 4) != 0)
         return sp;
-    // Unless forced, only for deep 3x3 (and larger) filters on up to 64 pixels, where every K block of the pixel-on-rows GEMM
-    // spends its MMAs on 128 rows of which half do not exist: 512 -> 512 3x3 @7 takes 7.0 us against 7.4, @5 6.0 against
-    // 6.9.  Every 1x1 layer is faster there (2048 -> 512 @7: 4.3 us against 6.2; 960 -> 160 @7: 3.3 against 5.3).
-    if (!tn.smallp_splits && (L.H * L.W > 64 || L.R == 1 || L.R * L.S * (L.C / 32) < 128)) return sp;
+    // Unless forced, only for deep 3x3 (and larger) filters on up to 64 pixels of an activation below 128 KiB, which the pixel-on-rows
+    // GEMM would gather: 512 -> 512 3x3 @7 takes 7.6 us against 8.7, 512 -> 256 6.8 against 8.4, 512 -> 512 @5 6.5 against 8.4, 256 -> 256
+    // 5x5 @5 6.6 against 10.1.  Larger activations the TMA brings, and that is faster (768 -> 512 @7: 6.9 us against 8.0, 512 -> 512 @8:
+    // 7.1 against 7.7), and so is every 1x1 layer (2048 -> 512 @7: 4.6 us against 6.2; 960 -> 160 @7: 3.5 against 5.7).  (From ~100 K
+    // blocks on it would be ahead of the gathering, 384 -> 384 @7 6.7 against 7.6, but the gathering rounds the activation.)
+    if (!tn.smallp_splits && (L.H * L.W > 64 || L.R == 1 || L.R * L.S * (L.C / 32) < 128 || 4ull * L.C * L.H * L.W >= 131072ull)) return sp;
     sp.Npad = ceil_div(g.P, 16) * 16;
     sp.b_slot_bytes = (uint32_t)align_up((uint64_t)sp.Npad * 128, 1024);
     const double stage = 16384.0 + sp.b_slot_bytes;

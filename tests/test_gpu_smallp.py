@@ -63,3 +63,18 @@ def test_every_split_matches_the_oracle(shape):
     assert ran >= min(2, nkb)
     auto, _ = _run(L, x, w, b, add, None, variant)              # whatever the library picks by itself
     assert_conv_close(auto, ref, TOL[nb.MATH_TF32], "library's choice")
+
+
+@pytest.mark.parametrize("C,K,H,taken", [(512, 64, 7, True), (640, 64, 7, True), (672, 36, 7, False), (512, 40, 8, False)])
+def test_both_sides_of_the_size_rule(C, K, H, taken):
+    """Deep filters on few pixels: the weights-on-rows kernel (its partial tiles are scratch) below 128 KiB of activation, the implicit
+    GEMM from there on."""
+    L = dict(op=nb.OP_CONV, C=C, K=K, R=3, S=3, stride=1, pad=1, groups=1, H=H, W=H, in0=-1, in1=-1, act=1, has_bias=1)
+    plan = nb.Plan([L], [0], [0])
+    assert (nb.nnv_exec_workspace_bytes(plan, 0, nb.VAR_IM2COL, nb.MATH_TF32) > 0) == taken
+    rng = np.random.default_rng([C, K, H])
+    x = rng.uniform(-1, 1, (C, H, H)).astype(np.float32)
+    w = (rng.standard_normal((K, C, 3, 3)) * np.sqrt(2.0 / (C * 9))).astype(np.float32)
+    b = rng.uniform(-0.1, 0.1, K).astype(np.float32)
+    y = run_conv(plan, 0, L, nb.VAR_IM2COL, nb.MATH_TF32, x, w, b)
+    assert_conv_close(y, omodel.run_layer(L, x, w, b), TOL[nb.MATH_TF32])
