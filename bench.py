@@ -38,7 +38,7 @@ import workloads as wl  # noqa: E402
 # DRAM bytes per tensor-core GEMM launch (dram__bytes_read.sum + dram__bytes_write.sum, averaged over the
 # launches of one step) from an ncu capture of this command; the file under profiles/ gives the command.
 # An entry is dropped (traffic = null) whenever the kernel changes after the capture.
-NCU_GEMM_TRAFFIC_BYTES = {("cfg4_resnet50", "tf32"): 3380086}   # profiles/gemm_cfg4_dram_traffic.md
+NCU_GEMM_TRAFFIC_BYTES = {("cfg4_resnet50", "tf32"): 2357933}   # profiles/gemm_cfg4_dram_traffic.md
 
 METRIC = "cold_inference_ms_batch1"
 UNIT = "ms"
@@ -256,19 +256,18 @@ class ClockSampler:
         return out
 
 
-def count_launches(layers, choices, plan, nb):
-    """Kernels of this library launched by one pass (layout conversion in, per-layer kernels, out)."""
-    n = 2
+def count_launches(layers, choices, plan, nb, transforms):
+    """Kernels of this library launched by one pass: layout conversion in and out, `transforms` weight transforms (layers of one
+    copy share a launch), and the layers' own kernels."""
+    n = 2 + transforms
     for i, L in enumerate(layers):
         if L["op"] != wl.OP_CONV:
             n += 1
             continue
-        v, m, cached = choices[i]
+        v, m, _ = choices[i]
         if v in (nb.VAR_DIRECT, nb.VAR_DEPTHWISE):
             n += 1
             continue
-        if not cached:
-            n += 1                                           # transform
         if v in (nb.VAR_WINO_F2, nb.VAR_WINO_F4, nb.VAR_WINO_F6):
             n += 3
         else:
@@ -803,8 +802,8 @@ def measure(args, config, steps, warmup, minimal, rank, world, local, ranks):
     flops = sum(layer_flops(i) for i in ex)
     exec_ns = sum(avg(v) for v in ex.values())
     xform_ns = sum(avg(v) for v in xf.values())
-    n_xf = sum(1 for c in choices_raw if c is not None and c[0] not in (nb.VAR_DIRECT, nb.VAR_DEPTHWISE))
-    per_step_launches = count_launches(layers, choices_raw, model.plan, nb)
+    n_xf = len(xf)                                               # a grouped launch stamps its first layer
+    per_step_launches = count_launches(layers, choices_raw, model.plan, nb, n_xf)
 
     h2d_value = h2d_bytes(layers, choices_raw, model.plan, nb, 0)
     h2d_e2e = h2d_bytes(layers, choices_raw, model.plan, nb, x.nbytes)
