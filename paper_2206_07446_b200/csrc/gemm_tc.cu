@@ -76,8 +76,8 @@ constexpr int BM = 128;                 // rows of A per tile = TMEM lanes
 constexpr int BK_BYTES = 128;           // bytes of K per stage row = one 128B swizzle atom
 constexpr int A_STAGE_BYTES = BM * BK_BYTES;
 constexpr int GEMM_THREADS = 192;
-// gemm_tc_kernel: a second MMA issuer and a second producer; splitting both operands (mode 2) and gathering (modes 4 - 7) take
-// four more warps
+// gemm_tc_kernel: a second MMA issuer and a second producer; splitting both operands (mode 2), gathering (modes 4 - 7) and rounding
+// (mode 8) take four more warps
 constexpr int gemm_tc_threads(int mode) { return mode == 2 || mode >= 4 ? 384 : 256; }
 constexpr int GATHER_WARPS = 8;
 constexpr int GEMM_BAR_BYTES = 8 * (3 * 8 + 4) + 512;         // barriers, TMEM address, bias of the tile's columns
@@ -319,7 +319,14 @@ __device__ __forceinline__ void convert_chunk(const uint8_t* src_tile, uint8_t* 
 // hi*hi + lo*hi + hi*lo of their bf16 splits (error-compensated, fp32-class accuracy).
 // MODE 4 - 7: A is gathered from the filter windows of the activation by eight warps, element by element (4: TF32, 5: BF16) or
 // four channels at a time (6, 7), and rounded to nearest even on the way; B as in mode 0 or 1.
-__host__ __device__ constexpr bool gather_mode(int mode) { return mode >= 4; }
+// MODE 8: TF32 on the boxes of a small image (below 128 KiB), whose tiles warps 2-5 and 8-11 round to nearest even where they lie;
+// the tensor core would truncate them, an error of 4.3e-4 a layer against 2.9e-4.  The two groups of warps take the K blocks in
+// turn, as the issuers do: all eight on every block take 5 % longer, four 20 %.  Bound: the pass through shared memory (25 KB a
+// block of 98 rows) behind each load.  us, gathered / this / truncated: 64 -> 64 3x3 @14 4.2 / 3.9 / 3.6, 160 -> 160 @14 6.6 / 5.4 / 4.3,
+// 256 -> 256 @7 6.0 / 4.8 / 4.2, 320 -> 320 @10 8.4 / 6.4 / 5.1.
+constexpr int ROUNDED = 8;
+__host__ __device__ constexpr bool gather_mode(int mode) { return mode >= 4 && mode <= 7; }
+__host__ __device__ constexpr bool converting_mode(int mode) { return mode == 2 || mode == 3 || mode == ROUNDED; }
 __host__ __device__ constexpr bool bf16_mode(int mode) { return mode == 1 || mode == 5 || mode == 7; }   // both operands staged as bf16
 template <int MODE> struct ModeTraits {
     static constexpr int BKE = bf16_mode(MODE) ? 64 : 32;      // K elements per stage
@@ -341,7 +348,7 @@ __host__ __device__ constexpr uint32_t stage_bytes_of(int BN, int rows) {
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(gemm_tc_threads(MODE), MODE == 2 || gather_mode(MODE) ? 2 : 3)
+__global__ void __launch_bounds__(gemm_tc_threads(MODE), MODE == 2 || MODE >= 4 ? 2 : 3)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmD, const __grid_constant__ CUtensorMap tmAdd, const GemmDev g) {
     extern __shared__ uint8_t smem_raw[];
@@ -481,8 +488,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     pdl_trigger();
     if (threadIdx.x == 32) stamp_start(g.stamp);
 
-    // Operand conversion (modes 2 and 3), by warps 2-5 (and 8-11 in mode 2) together: MODE 3 rounds A to bf16 (the weights arrive as
-    // bf16), MODE 2 splits both operands into bf16 hi / lo tiles.  The work of a stage is dealt to the warps in pieces of
+    // Operand conversion (modes 2, 3 and 8), by warps 2-5 (and 8-11 in modes 2 and 8): MODE 3 rounds A to bf16 (the weights arrive as
+    // bf16), MODE 8 to TF32 in place, MODE 2 splits both operands into bf16 hi / lo tiles.  The work of a stage is dealt to the warps in pieces of
     // 32 rows x 8 elements: a thread that converted whole rows of A and B alone paid ~3400 cycles a K block in dependent
     // instructions, most of the kernel's time (512 -> 512 F(4,3) @7, whole layer: 38.7 -> 23.5 us).
     auto convert_stages = [&](int cw) -> bool {
@@ -491,6 +498,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         int s = 0;
         uint32_t ph = 0;
         for (int it = 0; it < nkb; ++it, s = (s + 1 == STAGES ? 0 : s + 1), ph ^= (s == 0 ? 1u : 0u)) {
+            if (MODE == ROUNDED && (g.issuers == 2 ? it & 1 : 0) != cw >> 2) continue;
             if (!mbar_wait(full_bar(s), ph)) return false;
             uint8_t* const st = sm0 + s * stage_bytes;
             uint8_t* const cv = st + a_stage + (MODE == 2 ? b_stage_bytes : 0u);      // converted tiles: A hi, A lo, B hi, B lo
@@ -499,6 +507,17 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 if (r < g.rows) {
 #pragma unroll
                     for (int c = 0; c < 4; ++c) convert_chunk<false>(st, cv, cv, r, c, rp);
+                }
+            } else if constexpr (MODE == ROUNDED) {
+                const int r = (cw & 3) * 32 + lane;           // a row of A per thread, its words in another order for each of eight lanes
+                if (r < g.rows) {
+                    float4 v[8];                              // all loads first: the compiler keeps them behind earlier stores
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) v[c] = *reinterpret_cast<const float4*>(st + r * 128 + ((c ^ (r & 7)) << 4));
+#pragma unroll
+                    for (int c = 0; c < 8; ++c)
+                        *reinterpret_cast<float4*>(st + r * 128 + ((c ^ (r & 7)) << 4)) =
+                            make_float4(round_tf32(v[c].x), round_tf32(v[c].y), round_tf32(v[c].z), round_tf32(v[c].w));
                 }
             } else {
 #pragma unroll 2
@@ -640,7 +659,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         __syncwarp();
         if (splits > 1) cluster_wait();
     } else if (warp >= 8) {
-        if constexpr (MODE == 2) {
+        if constexpr (MODE == 2 || MODE == ROUNDED) {
             if (!convert_stages(warp - 4) && lane == 0) atomicExch(&g_device_status, (int)NNV_ERR_TIMEOUT);
         }
         __syncwarp();
@@ -652,14 +671,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         const int iss = warp == 1 ? 0 : warp - 5;
         if (iss < g.issuers && elect_one()) {
             // instruction descriptor: fp32 accumulate, A/B format, both K-major, N, M = 128
-            const uint32_t fmt = (MODE == 0 || MODE == 4 || MODE == 6) ? 2u : 1u;
+            const uint32_t fmt = (MODE == 0 || MODE == 4 || MODE == 6 || MODE == ROUNDED) ? 2u : 1u;
             const uint32_t idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
             const uint32_t acc = tmem_base + (uint32_t)(iss * BN);
             bool ok = true;
             int s = iss % STAGES;
             uint32_t ph = (uint32_t)(iss / STAGES) & 1u;
             for (int it = iss; it < nkb; it += g.issuers) {
-                ok = mbar_wait((MODE == 2 || MODE == 3) ? conv_bar(s) : full_bar(s), ph);
+                ok = mbar_wait(converting_mode(MODE) ? conv_bar(s) : full_bar(s), ph);
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t first = it != iss ? 1u : 0u;     // 0: the accumulator's first MMA overwrites it
@@ -736,7 +755,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             }
         };
         bool ok = gathered;
-        if constexpr (MODE == 2 || MODE == 3) ok = convert_stages(warp - 2);
+        if constexpr (converting_mode(MODE)) ok = convert_stages(warp - 2);
         float* const s_bias = reinterpret_cast<float*>(sm + (sbias - sbase));
         if (t < BN) s_bias[t] = bias;
         asm volatile("barrier.sync 1, 128;" ::: "memory");
@@ -1085,11 +1104,14 @@ int gemm_ring(int mode, int bn, int rows, long long ctas, int nkb) {
 // X3's K block waits for the split of both operands (by pieces of 32 rows), most of which a second CTA on the SM overlaps: fitted over
 // 68 F(4,3) / F(6,3) layers, 1 % above the best measured tilings (the constants of the other modes: 2.5 %, and 20 % on 512 -> 512
 // F(4,3) @7, 22.9 us against 19.1).
+// Mode 8's K block waits for the rounding; CTAs that share an SM count by the clusters that fit (clusters of 16 put 128 CTAs on 112
+// places): fitted to 34 layers, 0.6 % above the best measured tilings (the TF32 constants: 5.6 %).
 struct GemmTiling { int BN, splits, rows, waves; };
 GemmTiling search_gemm_tiling(int mode, int M, int N, int batch, int nkb) {
     constexpr struct { double row_us, share; } gather[4] = {{0.0064, 0.36}, {0.0054, 0.60}, {0.0025, 0.81}, {0.0042, 0.40}};   // modes 4 - 7
     const bool x3 = mode == GEMM_X3;
-    const double fixed = gather_mode(mode) ? 0.87 : 1.87, start = gather_mode(mode) ? 1.85 : x3 ? 0.80 : 0.40, column = x3 ? 0.005 : 0.0093;
+    const bool rounded = mode == ROUNDED;
+    const double fixed = gather_mode(mode) ? 0.87 : 1.87, start = gather_mode(mode) ? 1.85 : x3 || rounded ? 0.80 : 0.40, column = x3 ? 0.005 : 0.0093;
     const int least = ceil_div(M, BM);
     const int most = gather_mode(mode) ? std::max(least, std::min(M / 16, 296)) : least;
     GemmTiling best{16, 1, gemm_rows(M), 1};
@@ -1105,15 +1127,17 @@ GemmTiling search_gemm_tiling(int mode, int M, int N, int batch, int nkb) {
                 int tmem = 32;
                 while (tmem < 2 * bn) tmem *= 2;
                 const double smem = 2048.0 + (double)ring * gemm_stage_bytes(mode, bn, rows) + (sp > 1 ? 4.0 * rows * bn : 0.0);
-                const int occ = std::max(1, std::min({gather_mode(mode) || x3 ? 2 : 3, (int)(226.0 * 1024.0 / smem), 512 / tmem}));
+                const int occ = std::max(1, std::min({mode == 2 || mode >= 4 ? 2 : 3, (int)(226.0 * 1024.0 / smem), 512 / tmem}));
                 const long long slots = cluster_slots(sp, occ);
                 const double waves = (double)((ctas + slots - 1) / slots);
-                const double res = (double)std::min<long long>(occ, (ctas + 147) / 148);
+                const int lone = rounded ? cluster_slots(sp, 1) : 148;
+                const double res = (double)std::min<long long>(occ, (ctas + lone - 1) / lone);
                 double kb = std::max({(x3 ? 0.37 : 0.146) * res, kb_bytes * res / 108e3, kb_bytes * (double)std::min(ctas, slots) / (x3 ? 4.6e6 : 10.9e6)});
                 if (x3) kb = std::max(kb, (0.40 + 0.07 * (ceil_div(rows, 32) + ceil_div(bn, 32))) * (1 + 0.15 * (res - 1)));
                 if (gather_mode(mode))
                     kb = std::max(kb, (0.2 + gather[mode & 3].row_us * (0.65 * 64 * ceil_div(rows, 64) + 0.35 * rows)) * (1 + gather[mode & 3].share * (res - 1)));
-                const double split = sp > 1 ? (x3 ? 0.73 : 0.26 + 0.021 * std::log2((double)sp)) + 1.22e-4 * bn * rows * res : 0.0;
+                if (rounded) kb = std::max(kb, (0.25 + 0.0005 * rows) * (1 + 0.8 * (res - 1)));
+                const double split = sp > 1 ? (x3 ? 0.73 : 0.26 + (rounded ? 0.0 : 0.021) * std::log2((double)sp)) + 1.22e-4 * bn * rows * res : 0.0;
                 const double t = fixed + waves * (nk * kb + start + column * bn + split);
                 if (t < best_t - 1e-9) { best_t = t; best = GemmTiling{bn, sp, rows, (int)waves}; }
             }
@@ -1215,7 +1239,7 @@ nnv_status_t gemm_shape(int mode, const GemmTiling& tile, int M, int N, int batc
     // is there and release the slot; the producers then arrive at a barrier whose phase already has all its arrivals, and loads
     // land in a CTA that has gone.  So a ring that is refilled has an even depth: an issuer then has its slots for itself.
     // (X3's issuers wait for eight warps that convert the blocks in order: block i - 2 converted means block i - depth is, from
-    // two slots on.)
+    // two slots on.  Mode 8's two groups of warps take the blocks in turn like the issuers; with one issuer one group takes all.)
     if (g.issuers == 2 && nkb_cta > g.ring && (mode == GEMM_X3 ? g.ring == 1 : (g.ring & 1) == 1)) {
         if (g.ring > 1 && (g.ring - 1) * sb >= park) --g.ring;
         else g.issuers = 1;
@@ -1241,7 +1265,7 @@ nnv_status_t gemm_tc_init() {
     NNV_TRY(get_encoder());
     std::call_once(g_attr_once, [] {
         for (auto* kernel : {gemm_tc_kernel<0>, gemm_tc_kernel<1>, gemm_tc_kernel<2>, gemm_tc_kernel<3>, gemm_tc_kernel<4>, gemm_tc_kernel<5>,
-                             gemm_tc_kernel<6>, gemm_tc_kernel<7>}) {
+                             gemm_tc_kernel<6>, gemm_tc_kernel<7>, gemm_tc_kernel<ROUNDED>}) {
             cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
             cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         }
@@ -1539,7 +1563,11 @@ nnv_status_t launch_gemm_tc(const GemmArgs& a, cudaStream_t st) {
     // Tiling: column tile BN and K splits (a thread-block cluster of up to 16 CTAs) with the least estimated time.
     const int bke = (a.mode == GEMM_BF16) ? 64 : 32;
     const bool gather = a.ic.on && a.ic.gather;
-    const int mode = gather ? (a.mode == GEMM_BF16 ? 5 : 4) + ((a.ic.C % 4) == 0 ? 2 : 0) : a.mode;   // the kernel's
+    // an activation below 128 KiB comes as boxes of whole image rows
+    const bool boxes = a.ic.on && !gather && 4ull * a.ic.C * a.ic.H * a.ic.W < 131072ull &&
+                       image_row_boxes(a.ic.H, a.ic.W, a.ic.R, a.ic.S, a.ic.stride, a.ic.pad);
+    const int mode = gather ? (a.mode == GEMM_BF16 ? 5 : 4) + ((a.ic.C % 4) == 0 ? 2 : 0)
+                            : boxes && a.mode == GEMM_TF32 ? ROUNDED : a.mode;   // the kernel's
     const int nkb_all = a.ic.on && !gather ? a.ic.R * a.ic.S * ceil_div(a.ic.C, 32) : ceil_div(a.Kd, bke);
     const GemmTiling tile = pick_gemm_tiling(mode, a.M, a.N, a.batch, nkb_all);
     const Tuning& tn = tuning();
@@ -1609,7 +1637,6 @@ nnv_status_t launch_gemm_tc(const GemmArgs& a, cudaStream_t st) {
     } else if (a.ic.on) {
         NNV_REQUIRE((a.mode == GEMM_TF32 || a.mode == GEMM_BF16_CVT) && a.batch == 1, NNV_ERR_INVALID_ARG,
                     "implicit im2col needs fp32 activations (TF32 or converting BF16 mode) and one batch");
-        const bool boxes = 4ull * a.ic.C * a.ic.H * a.ic.W < 131072ull && image_row_boxes(a.ic.H, a.ic.W, a.ic.R, a.ic.S, a.ic.stride, a.ic.pad);
         if (boxes) NNV_TRY(encode_image_operand(&tmA, a.A, a.ic.C, a.ic.H, a.ic.W, rows / a.ic.W));
         else NNV_TRY(encode_im2col_operand(&tmA, a.A, a.ic.C, a.ic.H, a.ic.W, a.ic.R, a.ic.S, a.ic.stride, a.ic.pad, rows));
         g.ic_on = boxes ? 2 : 1; g.ic_C = a.ic.C; g.ic_cblk = ceil_div(a.ic.C, 32); g.ic_S = a.ic.S; g.ic_OW = a.ic.OW;
@@ -1641,8 +1668,9 @@ nnv_status_t launch_gemm_tc(const GemmArgs& a, cudaStream_t st) {
 
     dim3 grid(m_tiles, ceil_div(a.N, BN), a.batch * splits);
     NNV_REQUIRE(grid.y <= 65535 && grid.z <= 65535, NNV_ERR_UNSUPPORTED, "GEMM grid too large");
-    static constexpr decltype(&gemm_tc_kernel<0>) kernels[8] = {gemm_tc_kernel<GEMM_TF32>, gemm_tc_kernel<GEMM_BF16>, gemm_tc_kernel<GEMM_X3>,
-        gemm_tc_kernel<GEMM_BF16_CVT>, gemm_tc_kernel<4>, gemm_tc_kernel<5>, gemm_tc_kernel<6>, gemm_tc_kernel<7>};
+    static constexpr decltype(&gemm_tc_kernel<0>) kernels[9] = {gemm_tc_kernel<GEMM_TF32>, gemm_tc_kernel<GEMM_BF16>, gemm_tc_kernel<GEMM_X3>,
+        gemm_tc_kernel<GEMM_BF16_CVT>, gemm_tc_kernel<4>, gemm_tc_kernel<5>, gemm_tc_kernel<6>, gemm_tc_kernel<7>,
+        gemm_tc_kernel<ROUNDED>};
     NNV_REQUIRE(a.mode >= GEMM_TF32 && a.mode <= GEMM_BF16_CVT, NNV_ERR_INVALID_ARG, "unknown GEMM mode %d", a.mode);
     (void)launch_pdl_cluster(kernels[mode], grid, dim3(gemm_tc_threads(mode)), sh.smem_bytes, st, splits, tmA, tmB, tmD, tmAdd, g);
     NNV_CUDA(cudaGetLastError());

@@ -173,18 +173,13 @@ static inline bool gemm1x1_direct_operand(const nnv_layer_desc_t& L, int math) {
 static inline bool implicit_gemm_operand(const nnv_layer_desc_t& L, int math) {
     // The TMA's im2col mode gathers filter-window pixels straight from the NHWC activation, so no
     // Xcol matrix is materialised: fp32 words (TF32), pixel rows a multiple of 16 bytes, and an
-    // activation of at least 128 KiB.  With BF16 math, whose kernel rounds the activation itself, smaller images of stride-1
-    // "same" layers are read as plain boxes of whole image rows (image_row_boxes).  All other small tensors are gathered (below),
-    // which rounds them to nearest even; the tensor core would truncate fp32 words that the TMA brings (relative error of a layer
-    // 4.3e-4 against 2.9e-4).  The rounding costs 0.5 - 3.5 us a layer (64 -> 64 3x3 @14 4.3 us against 3.6, 160 -> 160 @14 6.7
-    // against 4.3, 320 -> 320 @10 8.6 against 5.1); boxes whose tiles four warps round in shared memory are no faster (4.3, 6.1, 7.0,
-    // but 128 -> 128 @14 6.3 against 5.4, 256 -> 256 @7 6.4 against 6.0).
+    // activation of at least 128 KiB.  Smaller images of stride-1 "same" layers are read as plain boxes of whole image rows
+    // (image_row_boxes), which the kernel rounds; all other small tensors are gathered (below).
     return ((math == NNV_MATH_TF32 && (L.C % 4) == 0) || (math == NNV_MATH_BF16 && (L.C % 8) == 0 && tuning().bf16cvt)) &&
-           (4ull * L.C * L.H * L.W >= 131072ull ||
-            (math == NNV_MATH_BF16 && image_row_boxes(L.H, L.W, L.R, L.S, L.stride, L.pad))) && L.R <= 16 && L.S <= 16 && L.pad <= 8;
+           (4ull * L.C * L.H * L.W >= 131072ull || image_row_boxes(L.H, L.W, L.R, L.S, L.stride, L.pad)) && L.R <= 16 && L.S <= 16 && L.pad <= 8;
 }
 
-// What neither of those reads in place -- channel counts that are no multiple of 16 bytes (network stems), small images --
+// What neither of those reads in place -- channel counts that are no multiple of 16 bytes (network stems), other small images --
 // is gathered by the GEMM's own warps.  The exception is fp32 words one by one for many output channels: every column tile
 // gathers the windows again, and the explicit matrix pays or is as good (303 -> 300 3x3 @7: 6.7 us against 7.2, 102 -> 400 @56 28.2
 // and 28.3, 1x1 333 -> 1024 @28 9.3 against 9.8; at 250 channels, 250 -> 250 @56, the gathering wins 37 to 58).

@@ -1,5 +1,5 @@
-"""GPU parity of im2col GEMMs whose activation is small: gathered and rounded (TF32), fetched as boxes of whole image rows or gathered
-(BF16, also through the 3x3 halo kernel)."""
+"""GPU parity of im2col GEMMs whose activation is small: tiles of whole image rows fetched as boxes and rounded by the kernel, and the
+shapes next to them, which are gathered; BF16 math also through the 3x3 halo kernel."""
 import numpy as np
 import pytest
 
@@ -44,3 +44,21 @@ def test_small_tf32_activations_are_rounded(C, K, R, H, W):
         w = (rng.standard_normal((K, C, R, R)) * np.sqrt(2.0 / (C * R * R))).astype(np.float32)
         y = run_conv(nb.Plan([L]), 0, L, nb.VAR_IM2COL, nb.MATH_TF32, x, w)
         assert_conv_close(y, omodel.run_layer(L, x, w, None, None), 3.4e-4, seed)
+
+
+@pytest.mark.parametrize("tuning", ["gemm_tile=16,1;gemm_ring=2", "gemm_tile=48,1;gemm_ring=3", "gemm_tile=32,1", "gemm_tile=32,2;gemm_ring=5",
+                                    "gemm_tile=48,16", "gemm_tile=16,8;gemm_ring=2"])
+def test_rounded_boxes_in_rings_that_wrap(tuning):
+    """75 K blocks in rings of every kind, by one CTA or a cluster: two groups of warps round them in turn."""
+    C, K, R, H, W = 96, 48, 5, 14, 14
+    L = dict(op=nb.OP_CONV, C=C, K=K, R=R, S=R, stride=1, pad=2, groups=1, H=H, W=W, in0=-1, in1=-1, act=2, has_bias=1)
+    rng = np.random.default_rng(3)
+    x = rng.uniform(-1, 1, (C, H, W)).astype(np.float32)
+    w = (rng.standard_normal((K, C, R, R)) * np.sqrt(2.0 / (C * R * R))).astype(np.float32)
+    b, add = rng.uniform(-0.1, 0.1, K).astype(np.float32), rng.uniform(-1, 1, (K, H, W)).astype(np.float32)
+    nb.nnv_tuning_set(tuning)
+    try:
+        y = run_conv(nb.Plan([L]), 0, L, nb.VAR_IM2COL, nb.MATH_TF32, x, w, b, add)
+    finally:
+        nb.nnv_tuning_set(None)
+    assert_conv_close(y, omodel.run_layer(L, x, w, b, add), 3.4e-4, tuning)
