@@ -1,7 +1,9 @@
 // 3x3 / stride 1 / pad 1 convolution with BF16 math straight from the fp32 activation.  Included by gemm_tc.cu (inside namespace
 // nnv, after the PTX helpers).
 //
-// Bound: the tensor pipe (18 MMAs of ~82 cycles per patch and 32 input channels; M = 128, N <= 128, K = 16).  A CTA owns an
+// Bound: the issue of 18 MMAs (M = 128, N <= 128, K = 16), ~82 cycles each, per patch and 32 input channels by one thread; the chain
+// of box load, rounding and MMAs comes right behind (256 -> 256 @56: without the rounding after two boxes, or without the weights'
+// loads after the first ring, the same time within 1 %; with half the MMAs 9.3 us instead of 11.0).  A CTA owns an
 // output patch of 16 rows x 8 columns and BN output channels.  Per block of 32 input channels it fetches ONE fp32 halo box of
 // 18 x 10 pixels, eight warps round it to bf16 into the un-swizzled core-matrix layout [8-channel chunk][pixel][16 bytes],
 // and all nine taps read that one copy: a tap (r, s) is a shift of the descriptor's start address by 10 r + s pixels, and the

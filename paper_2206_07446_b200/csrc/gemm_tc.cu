@@ -684,7 +684,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 const uint32_t first = it != iss ? 1u : 0u;     // 0: the accumulator's first MMA overwrites it
                 const uint32_t a_src = sbase + s * stage_bytes;
                 if constexpr (MODE == 2) {
-                    // converted tiles follow the staged ones: A_hi, A_lo (8 KB each), B_hi, B_lo
+                    // converted tiles follow the staged ones: A_hi, A_lo (64 bytes a row), B_hi, B_lo
                     const uint32_t a_hi = a_src + a_stage + b_stage_bytes, a_lo = a_hi + rp * 64;
                     const uint32_t b_hi = a_lo + rp * 64, b_lo = b_hi + b_stage_bytes / 2;
                     const uint32_t lbo_a = (uint32_t)rp * 16u, lbo_b = (uint32_t)BN * 16u;

@@ -158,9 +158,9 @@ static nnv_status_t run_model(nnv_plan* p, const nnv_choice_t* choices, const vo
     // its stream (measured: 96 MB as 1 MB copies moves at 45 GB/s, as 4 MB copies at 51, as 16 MB copies at 53, as one copy at
     // 55), so at depth 0 (where the arena mirrors the host blobs' layouts) consecutive layers whose source
     // and destination ranges line up are read by ONE copy.  The chunks start at 1 MB, so that execution
-    // begins early, and double up to 32 MB (256 KB ... 16 MB / 1 ... 32 MB / 2 ... 32 MB, us: ResNet-50-shaped @224 1809 / 1796 /
-    // 1791, ResNet-18-shaped 903 / 894 / 890, MobileNetV2-shaped @224, whose 8.8 MB run as fast as the host enqueues them, 264 / 264 /
-    // 276, @120 254 / 239 / 250; 1710 us for one bulk copy of the ResNet-50-shaped model's bytes); all layers of a chunk become ready
+    // begins early, and double up to 32 MB (256 KB ... 16 MB / 1 ... 32 MB / 2 ... 32 MB, us: ResNet-50-shaped @224 1813 / 1800 /
+    // 1794, ResNet-18-shaped 907 / 897 / 896, MobileNetV2-shaped @224, whose 8.8 MB run as fast as the host enqueues them, 290 / 281 /
+    // 291, @120 269 / 256 / 259; 1710 us for one bulk copy of the ResNet-50-shaped model's bytes); all layers of a chunk become ready
     // when it lands, and their weight transforms are one grouped launch.
     struct CopyChunk { const uint8_t* src; uint8_t* dst; uint64_t bytes; int first, last; bool zero_copy; };
     std::vector<CopyChunk> chunks;

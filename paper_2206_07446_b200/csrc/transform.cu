@@ -429,7 +429,7 @@ __host__ __device__ constexpr int xform_threads(int group) { return group == XG_
 __host__ __device__ constexpr int xform_resident(int group) { return group == XG_PACK ? 5 : ft_resident(xform_m(group)); }
 __host__ __device__ constexpr int xform_smem_floats(int group) { return group == XG_PACK ? PACK_SMEM_FLOATS : ft_filters(xform_m(group)) * 9; }
 
-// The descriptors travel as kernel parameters, which cost the host ~0.7 us a kilobyte to launch with: 36 bytes each, in one of two sizes
+// The descriptors travel as kernel parameters, which cost the host ~0.7 us a kilobyte to launch with: 40 bytes each, in one of two sizes
 // (a chunk of a cold run rarely holds more than 16 layers; its launch takes the host 3 us instead of 5.4).
 struct XformItem { const void* src; void* dst; int K, C, pitch, block0; uint16_t RS; uint8_t kind, bf16; };   // pitch: Cp, or Qp of a repack
 constexpr int XF_BATCH_SMALL = 16, XF_BATCH_MAX = 56;

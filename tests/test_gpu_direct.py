@@ -14,7 +14,7 @@ pytestmark = pytest.mark.gpu
     (12, 33, 3, 3, 1, 1, 7, 5),          # half a chunk of channels, ragged tiles, K not a multiple of 4
     (64, 128, 3, 3, 2, 1, 57, 55),       # 32 x 32 tiles
     (512, 36, 3, 3, 1, 1, 7, 7),         # 64 chunks over a cluster of eight
-    (64, 64, 3, 3, 1, 1, 151, 149),      # 64 x 64 tiles
+    (64, 64, 3, 3, 1, 1, 151, 149),      # 703 x 2 tiles, the last ones ragged
     (4, 5, 1, 1, 1, 0, 1, 1),            # a single output pixel
     (68, 40, 1, 1, 2, 0, 15, 13),        # 1x1, one channel word beyond a chunk
     (256, 512, 1, 1, 1, 0, 14, 14),
