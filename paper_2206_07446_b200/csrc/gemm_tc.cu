@@ -11,8 +11,8 @@
 //   warps 1, 6  issue tcgen05.mma (one lane each) from shared-memory descriptors for alternate K blocks, each into its own
 //            fp32 accumulator in TMEM, and release the stages that are refilled with tcgen05.commit on "empty" mbarriers (an
 //            arrival that nobody waits for could meet a CTA that has left); warp 1 allocates TMEM
-//   warps 2-5  epilogue: tcgen05.ld the accumulators (each warp its own 32 TMEM lanes), apply
-//            bias / residual / activation, store fp32 rows
+//   warps 4, 5  every other load of deep K loops; warps 2-5  the bias, and the conversion of operands
+//   all eight  write out: tcgen05.ld the accumulators (each warp 32 TMEM lanes), apply bias / residual / activation, store fp32 rows
 // These layers are latency-bound (5 - 10 dependent phases of ~0.1 - 0.5 us each); what bounds each phase was read from
 // device-clock probes.  Two producers and two issuers: one thread pays 157 cycles per load and ~560 per K block of waiting,
 // issuing four MMAs and committing, more than the fill (~320 cycles of 24 KB) or the tensor pipe need.  Their loops run under
@@ -80,7 +80,7 @@ constexpr int GEMM_THREADS = 192;
 // (mode 8) take four more warps
 constexpr int gemm_tc_threads(int mode) { return mode == 2 || mode >= 4 ? 384 : 256; }
 constexpr int GATHER_WARPS = 8;
-constexpr int GEMM_BAR_BYTES = 8 * (3 * 8 + 4) + 512;         // barriers, TMEM address, bias of the tile's columns
+constexpr int GEMM_BAR_BYTES = 8 * (3 * 8 + 6) + 512;         // barriers, TMEM address, bias of the tile's columns
 constexpr uint32_t WAIT_LIMIT = 1u << 20;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -233,6 +233,15 @@ __device__ __forceinline__ bool elect_one() {
     return p != 0;
 }
 
+__device__ __forceinline__ float4 lds128(uint32_t addr) {
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ void sts128(uint32_t addr, const float4& v) {
+    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+}
+
 struct GemmDev {
     unsigned long long* stamp;        // device-clock stamps of this launch, or null
     float* D;
@@ -243,7 +252,7 @@ struct GemmDev {
     int rows;                         // rows of A per tile, at most 128
     int z_tiles;                      // output map: 0 = {N, M, batch}; else {N, rows, tiles} with this many tiles per batch entry
     uint32_t bar_off;                 // byte offset (from the aligned base) of the barriers
-    int tma_out;                      // 0: plain stores; else the column width (16 or 32) of the staged tiles stored by TMA
+    int chunk;                        // unsplit: columns of a staging sub-tile (16); 0: plain stores
     uint32_t recv_off;                // splits > 1: byte offset (from the aligned base) of the received partial rows
     uint32_t stage_off;               // byte offset (from the aligned base) of the dedicated staging tile; 0 = the idle ring
     // implicit im2col (A is the NHWC activation itself): 0 = off
@@ -347,10 +356,10 @@ __host__ __device__ constexpr uint32_t stage_bytes_of(int BN, int rows) {
     return a + b;
 }
 
-template <int MODE>
+template <int MODE, bool SPLIT>
 __global__ void __launch_bounds__(gemm_tc_threads(MODE), MODE == 2 || MODE >= 4 ? 2 : 3)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-               const __grid_constant__ CUtensorMap tmD, const __grid_constant__ CUtensorMap tmAdd, const GemmDev g) {
+               const __grid_constant__ CUtensorMap tmAdd, const GemmDev g) {
     extern __shared__ uint8_t smem_raw[];
     const int STAGES = g.stages;                              // depth of the shared-memory ring (2..8)
     constexpr int MAXS = 8;
@@ -370,12 +379,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const uint32_t holder = bars + 8u * (3 * MAXS + 1);
     const uint32_t addend_bar = bars + 8u * (3 * MAXS + 2);
     const uint32_t recv_bar = bars + 8u * (3 * MAXS + 3);
-    const uint32_t sbias = bars + 8u * (3 * MAXS + 4);        // the tile's BN bias values (zeros without a bias)
-    // Write-out through shared memory (g.tma_out): the tile is staged as [column chunk][warp quarter] sub-tiles of
-    // 32 rows x CW columns in the swizzled layout of the output tensor map and stored by TMA.  With a residual
-    // addend the sub-tiles live in their own region and the addend is loaded INTO them while the K loop runs, so
-    // the epilogue adds in place; without one they reuse the ring, which is idle by then.
-    const int CW = g.tma_out;
+    const uint32_t bias_bar = bars + 8u * (3 * MAXS + 4);
+    const uint32_t sbias = bars + 8u * (3 * MAXS + 6);        // the tile's BN bias values (zeros without a bias)
+    // Write-out through shared memory (g.chunk): the tile is staged as [16-column chunk][warp quarter] sub-tiles of 32 rows, their
+    // 16-byte words in the 64-byte swizzle.  With a residual addend the sub-tiles live in their own region and the addend is loaded
+    // INTO them while the K loop runs, so the write-out adds in place; without one they reuse the ring, which is idle by then.
+    // (The width is a launch parameter although it is always 16: as a constant it let the compiler rearrange the loop, 256 -> 1024 1x1
+    // @14 3.14 us against 3.05, 24 -> 144 @40 2.38 against 2.32.)
+    const int CW = g.chunk;
     const uint32_t chunk_bytes = 32u * (uint32_t)CW * 4u;
     const uint32_t stg0 = sbase + g.stage_off;
     const int quarters = (g.rows + 31) >> 5;                  // 32-row sub-tiles of the tile
@@ -385,7 +396,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     // blockIdx.z = batch * splits + split; the `splits` CTAs of one output tile form a thread-block
     // cluster, each reducing its own contiguous range of K blocks.
-    const int splits = g.splits;
+    const int splits = SPLIT ? g.splits : 1;
     const int sp = (int)blockIdx.z % splits, b = (int)blockIdx.z / splits;
     const int zd = g.z_tiles ? b * g.z_tiles + (int)blockIdx.x : b;
     const int m0 = blockIdx.x * g.rows, n0 = blockIdx.y * BN;
@@ -408,10 +419,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         mbar_init(tmem_full_bar, (uint32_t)g.issuers);
         mbar_init(addend_bar, 1);
         mbar_init(recv_bar, 1);
-        if (CW) {
-            asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmD)) : "memory");
-            if (g.addend) asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmAdd)) : "memory");
-        }
+        mbar_init(bias_bar, 4);
+        if (CW && g.addend) asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmAdd)) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
@@ -475,10 +484,54 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             windows[threadIdx.x] = make_uint2((uint32_t)((ih * g.ic_W + iw) * g.ic_C) * 4u, (int)threadIdx.x < live ? taps : 0u);
         }
     }
+    // What the write-out needs besides the accumulator is worked out here, where it costs nothing: a warp that has its scheduler to
+    // itself pays 5 - 30 cycles for every dependent instruction.  (The pins keep the compiler from moving it behind the waits.)
+    auto pin = [](auto& v) {
+        if constexpr (sizeof(v) == 8) asm volatile("" : "+l"(v));
+        else asm volatile("" : "+r"(v));
+    };
+    int quarter = warp & 3, grp = warp >= 2 && warp <= 5 ? 0 : 1, t = grp * 128 + quarter * 32 + lane;
+    uint32_t tacc_off = (uint32_t)(quarter * 32) << 16;
+    pin(t); pin(tacc_off);
+    int rows_live = live - quarter * 32;                      // unsplit: rows of this warp's quarter, its first sub-tile, its lane's first word in memory
+    uint32_t out_sub = 0;
+    float* out_dst = nullptr;
+    // split: see below
+    int nch = 0, rot0 = 0, qstep = 0, rstep = 0, rot_step = 0, rr = 0, cc = 0, rot = 0, vec = 0;
+    uint32_t prow = 0, push_dst = 0, push_bar = 0, push_src = 0, push_bytes = 0;
+    float* dbase = nullptr;
+    const float* abase = nullptr;
+    if constexpr (!SPLIT) {
+        out_sub = stg0 + (uint32_t)(grp * quarters + quarter) * chunk_bytes;
+        out_dst = g.D + (long long)b * g.strideD + (long long)(m0 + quarter * 32 + (lane >> 2)) * g.ldd + n0 + grp * 16 + (lane & 3) * 4;
+        pin(rows_live); pin(out_sub); pin(out_dst);
+    } else {
+        const int r0 = sp * rows_per, q0 = quarter * 32;
+        nch = BN / 4;
+        rot0 = (q0 + lane) % nch;
+        prow = sbase + (uint32_t)(q0 + lane) * (uint32_t)BN * 4u;
+        const int a0 = max(q0, lane * rows_per), a1 = min(min(q0 + 32, live), (lane + 1) * rows_per);
+        if (grp == 0 && lane < splits && a1 > a0) {
+            push_dst = cluster_addr(sbase + g.recv_off + (uint32_t)((r0 + a0 - lane * rows_per) * BN) * 4u, lane);
+            push_bar = cluster_addr(recv_bar, lane);
+            push_src = sbase + (uint32_t)(a0 * BN) * 4u;
+            push_bytes = (uint32_t)((a1 - a0) * BN) * 4u;
+        }
+        vec = ((g.ldd & 3) == 0) && ((g.N & 3) == 0) && ((reinterpret_cast<uintptr_t>(g.D) & 15) == 0) &&
+              (!g.addend || (reinterpret_cast<uintptr_t>(g.addend) & 15) == 0);
+        // thread t walks the (row, 4-column group) grid of its CTA's rows in steps of 256
+        qstep = 256 / nch; rstep = 256 - qstep * nch;
+        rr = t / nch; cc = t - rr * nch; rot = (r0 + rr) % nch;
+        rot_step = qstep % nch;
+        dbase = g.D + (long long)b * g.strideD + (long long)(m0 + r0) * g.ldd + n0;
+        abase = g.addend ? g.addend + (long long)(m0 + r0) * g.ldd + n0 : nullptr;
+        pin(nch); pin(rot0); pin(prow); pin(push_dst); pin(push_bar); pin(push_src); pin(push_bytes); pin(vec);
+        pin(qstep); pin(rstep); pin(rr); pin(cc); pin(rot); pin(rot_step); pin(dbase); pin(abase);
+    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (splits > 1) {
+    if constexpr (SPLIT) {
         if (threadIdx.x == 64 && my_rows) mbar_expect_tx(recv_bar, (uint32_t)(splits * my_rows * BN) * 4u);
         __syncwarp();
         cluster_arrive_relaxed();                             // this CTA's (fenced) barriers may be signalled from here on
@@ -624,46 +677,55 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             __syncwarp();
         }
     }
-    bool cluster_arrived = false;                             // the epilogue warps arrive early, in their own code
-    if (warp == 0 || warp == 7) {
-        // Producers.  A load costs the thread that issues it ~157 cycles whatever its size, which for one thread issuing both
-        // operands (314 cycles a K block) is more than the MMAs take: the activation's and the weights' loads come from a
-        // warp each, the residual tile from the weights' one (it has fewer bytes to wait for).
-        if (!(gather_mode(MODE) && warp == 0) && elect_one()) {
-            bool ok = true;
-            int s = 0;
-            uint32_t ph = 0;
-            const int first = min(nkb, STAGES);
-            for (int it = 0; it < nkb; ++it) {
-                if (it >= STAGES) ok = mbar_wait(empty_bar(s), ph ^ 1u);
-                if (!ok) break;
-                if (warp == 0) {
-                    issue_a(it, s);
-                } else {
-                    issue_b(it, s);
-                    if (it == first - 1 && CW && g.addend) {  // straight into the staging sub-tiles
-                        const int nch = BN / CW;
-                        mbar_expect_tx(addend_bar, (uint32_t)(nch * quarters) * chunk_bytes);
-                        for (int j = 0; j < nch; ++j)
-                            for (int q = 0; q < quarters; ++q)
-                                tma_load_3d(stg0 + (uint32_t)(j * quarters + q) * chunk_bytes, &tmAdd, n0 + j * CW, y0 + q * 32, zd, addend_bar);
-                    }
+    // Producers.  A load costs the thread that issues it ~165 cycles whatever its size, more than the copy engine needs for it (1.1
+    // cycles a row of 128 bytes) or the MMAs of its K block: the activation's and the weights' loads come from a warp each, and where
+    // warps 4 and 5 have nothing to convert they take every other block (64 -> 64 3x3 @56, nine blocks a CTA,
+    // 4.81 -> 4.55 us, 256 -> 512 3x3 @28 10.1 -> 9.8; five blocks and fewer are slower that way).
+    constexpr bool FOUR = MODE == 0 || MODE == 1;
+    const int step = FOUR && nkb >= 6 && STAGES >= 2 ? 2 : 1;
+    auto produce = [&](bool is_a, int first_it) {
+        bool ok = true;
+        int s = first_it;                                     // (a ring that two producers share has two slots or more)
+        uint32_t ph = 0;
+        const int first = min(nkb, STAGES);
+        auto skip = [&]() {                                   // the other warp's block
+            if (!g.ic_on || ++ic_cb != g.ic_cblk) return;
+            ic_cb = 0;
+            ++ic_tap;
+            if (++ic_fs == g.ic_S) { ic_fs = 0; ++ic_fr; }
+        };
+        if (first_it) skip();
+        for (int it = first_it; it < nkb; it += step) {
+            if (it >= STAGES) ok = mbar_wait(empty_bar(s), ph ^ 1u);
+            if (!ok) break;
+            if (is_a) {
+                issue_a(it, s);
+            } else {
+                issue_b(it, s);
+                if (first_it == 0 && it < first && it + step >= first && CW && g.addend) {   // straight into the staging sub-tiles
+                    const int nch = BN / CW;
+                    mbar_expect_tx(addend_bar, (uint32_t)(nch * quarters) * chunk_bytes);
+                    for (int j = 0; j < nch; ++j)             // (a box is as high as the tile's sub-tiles together)
+                        tma_load_3d(stg0 + (uint32_t)(j * quarters) * chunk_bytes, &tmAdd, n0 + j * CW, y0, zd, addend_bar);
                 }
-                if (++s == STAGES) { s = 0; ph ^= 1u; }
             }
-            if (!ok) {
-                atomicExch(&g_device_status, (int)NNV_ERR_TIMEOUT);
-                for (int i = 0; i < 1000; ++i) __nanosleep(1000);   // let loads already in flight land
-            }
+            if (FOUR && step == 2) skip();
+            s += step;
+            if (s >= STAGES) { s -= STAGES; ph ^= 1u; }
         }
-        __syncwarp();
-        if (splits > 1) cluster_wait();
+        if (!ok) {
+            atomicExch(&g_device_status, (int)NNV_ERR_TIMEOUT);
+            for (int i = 0; i < 1000; ++i) __nanosleep(1000);       // let loads already in flight land
+        }
+    };
+    if (warp == 0 || warp == 7) {
+        if (!(gather_mode(MODE) && warp == 0) && elect_one()) produce(warp == 0, 0);
     } else if (warp >= 8) {
         if constexpr (MODE == 2 || MODE == ROUNDED) {
             if (!convert_stages(warp - 4) && lane == 0) atomicExch(&g_device_status, (int)NNV_ERR_TIMEOUT);
         }
         __syncwarp();
-        if (splits > 1) cluster_wait();
+        if constexpr (SPLIT) cluster_wait();
     } else if (warp == 1 || warp == 6) {
         // MMA issuers.  One thread that waits for a stage, issues its four MMAs into one accumulator and commits takes
         // ~560 cycles a K block (device-clock probes), several times what the tensor pipe needs at these tile widths, so
@@ -719,113 +781,115 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             if (ok) umma_commit(tmem_full_bar);
             else atomicExch(&g_device_status, (int)NNV_ERR_TIMEOUT);
         }
-        __syncwarp();
-        if (splits > 1) cluster_wait();
     } else {
-        // Epilogue warps.  A warp that has its scheduler to itself pays 5 - 30 cycles for every dependent instruction, so
-        // whatever does not need the accumulator -- indices, addresses, the bias -- is worked out before the wait for it.
-        const int quarter = warp & 3;                         // the TMEM lanes this warp may read
-        const int t = (int)threadIdx.x - 64;
-        uint8_t* const sm = smem_raw + (sbase - smem_u32(smem_raw));
+        const int c = (int)threadIdx.x - 64;
         float bias = early_bias;
-        if constexpr (!gather_mode(MODE)) bias = (g.bias && t < BN && n0 + t < g.N) ? __ldg(g.bias + n0 + t) : 0.f;
-        const int naccs = min(g.issuers, nkb);
-        const uint32_t tacc = tmem_base + ((uint32_t)(quarter * 32) << 16);
-        const float hi = g.act == 2 ? 6.f : INFINITY;
+        if constexpr (!gather_mode(MODE)) bias = (g.bias && c < BN && n0 + c < g.N) ? __ldg(g.bias + n0 + c) : 0.f;
+        if constexpr (FOUR)
+            if (step == 2 && warp >= 4 && elect_one()) produce(warp == 4, 1);
+        __syncwarp();
+        if constexpr (converting_mode(MODE)) gathered = convert_stages(warp - 2);
+        if (c < BN) *reinterpret_cast<float*>(smem_raw + (sbias - smem_u32(smem_raw)) + 4 * c) = bias;
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bias_bar);
+    }
+    __syncwarp();
+    if (warp < 8) {
+        // Write-out, by the eight warps that led here: the TMEM lanes a warp may read are those of its number modulo four, so each
+        // quarter of the tile's rows has two (one of warps 2-5, one of the producers and issuers, whose work is done by then),
+        // which take the column chunks in turn.
+        bool ok = gathered;
         auto act4 = [&](float4& v) {
             if (g.act) {
+                const float hi = g.act == 2 ? 6.f : INFINITY;
                 v.x = fminf(fmaxf(v.x, 0.f), hi); v.y = fminf(fmaxf(v.y, 0.f), hi);
                 v.z = fminf(fmaxf(v.z, 0.f), hi); v.w = fminf(fmaxf(v.w, 0.f), hi);
             }
         };
-        // 16 accumulator columns of this lane's row, the issuers' accumulators added in order
-        auto acc16 = [&](int c0, float (&v)[16]) {
-            uint32_t r[16];
-            tmem_ld16_nowait(tacc + (uint32_t)c0, r);
-            if (naccs > 1) {
-                uint32_t q[16];
-                tmem_ld16_nowait(tacc + (uint32_t)(BN + c0), q);
-                tmem_wait_ld();
-#pragma unroll
-                for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]) + __uint_as_float(q[i]);
-            } else {
-                tmem_wait_ld();
-#pragma unroll
-                for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-            }
-        };
-        bool ok = gathered;
-        if constexpr (converting_mode(MODE)) ok = convert_stages(warp - 2);
-        float* const s_bias = reinterpret_cast<float*>(sm + (sbias - sbase));
-        if (t < BN) s_bias[t] = bias;
-        asm volatile("barrier.sync 1, 128;" ::: "memory");
         auto wait_acc = [&]() {
-            ok = ok && mbar_wait(tmem_full_bar, 0);
+            ok = ok && mbar_wait(bias_bar, 0) && mbar_wait(tmem_full_bar, 0);
+            if constexpr (!SPLIT)
+                if (g.addend && CW) ok = ok && mbar_wait(addend_bar, 0);
             tc_fence_after();
             if (!ok && lane == 0) atomicExch(&g_device_status, (int)NNV_ERR_TIMEOUT);
             ok = __all_sync(0xffffffffu, ok);
         };
-        if (splits == 1 && CW) {
-            // lane = one accumulator row; per 16 columns: TMEM -> registers -> (+ bias, + addend from the staging sub-tile,
-            // activation) -> staging sub-tile, and per sub-tile one TMA store per warp
-            const uint32_t swz = CW == 32 ? (uint32_t)(lane & 7) : (uint32_t)((lane >> 1) & 3);
-            const bool row_live = quarter * 32 < live;
-            uint8_t* row0 = sm + g.stage_off + (uint32_t)quarter * chunk_bytes + (uint32_t)lane * (uint32_t)CW * 4u;
-            wait_acc();
-            if (ok && g.addend) ok = mbar_wait(addend_bar, 0);
-            ok = __all_sync(0xffffffffu, ok);
-            if (ok && row_live) {
-#pragma unroll 1
-                for (int c0 = 0; c0 < BN; c0 += 16) {
-                    float v[16];
-                    acc16(c0, v);
-                    const uint32_t half = CW == 32 ? (uint32_t)(c0 >> 2) & 4u : 0u;      // 16-byte word of the sub-tile's row
-                    float4 o[4];
+        const uint32_t tacc = tmem_base + tacc_off;
+        const bool two = min(g.issuers, nkb) > 1;
+        // 16 accumulator columns of this lane's row, the issuers' accumulators added in order
+        auto acc16 = [&](int c0, float (&v)[16]) {
+            uint32_t r[16], q[16];
+            tmem_ld16_nowait(tacc + (uint32_t)c0, r);
+            tmem_ld16_nowait(tacc + (uint32_t)(two ? BN + c0 : c0), q);
+            tmem_wait_ld();
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        const float4 bb = *reinterpret_cast<const float4*>(s_bias + c0 + c * 4);
-                        o[c] = make_float4(v[c * 4] + bb.x, v[c * 4 + 1] + bb.y, v[c * 4 + 2] + bb.z, v[c * 4 + 3] + bb.w);
-                    }
-                    if (g.addend) {
+            for (int i = 0; i < 16; ++i) v[i] = two ? __uint_as_float(r[i]) + __uint_as_float(q[i]) : __uint_as_float(r[i]);
+        };
+        if constexpr (!SPLIT) {
+            // Per 16 columns: lane = one accumulator row, TMEM -> registers -> (+ bias, + addend from the staging sub-tile, activation) ->
+            // staging sub-tile; then its rows from there to memory, 64 bytes each.  (One compact loop: code that a launch runs once
+            // costs more to fetch than to execute.)
+            if (CW && grp * 16 < BN) {
+                wait_acc();
+                if (ok && rows_live > 0) {
+                    const uint32_t sub_step = 2u * (uint32_t)quarters * chunk_bytes;
+#pragma unroll 1
+                    for (int c0 = grp * 16; c0 < BN; c0 += 32, out_sub += sub_step, out_dst += 32) {
+                        float v[16];
+                        acc16(c0, v);
+                        const uint32_t row0 = out_sub + (uint32_t)lane * 64u, swz = (uint32_t)((lane >> 1) & 3) << 4;
 #pragma unroll
                         for (int c = 0; c < 4; ++c) {
-                            const float4 aa = *reinterpret_cast<const float4*>(row0 + (((half + (uint32_t)c) ^ swz) << 4));
-                            o[c].x += aa.x; o[c].y += aa.y; o[c].z += aa.z; o[c].w += aa.w;
+                            const float4 bb = lds128(sbias + (uint32_t)(c0 + 4 * c) * 4u);
+                            v[c * 4] += bb.x; v[c * 4 + 1] += bb.y; v[c * 4 + 2] += bb.z; v[c * 4 + 3] += bb.w;
                         }
-                    }
+                        if (g.addend) {
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        act4(o[c]);
-                        *reinterpret_cast<float4*>(row0 + (((half + (uint32_t)c) ^ swz) << 4)) = o[c];
-                    }
-                    if (CW == 16 || half) {                   // the sub-tile is complete
-                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> visible to the TMA's reads
-                        __syncwarp();
-                        if (lane == 0 && row_live && n0 + c0 + 16 - CW < g.N) {
-                            tma_store_3d(&tmD, smem_u32(row0), n0 + c0 + 16 - CW, y0 + quarter * 32, zd);
-                            tma_store_commit();
+                            for (int c = 0; c < 4; ++c) {
+                                const float4 aa = lds128(row0 + (((uint32_t)c << 4) ^ swz));
+                                v[c * 4] += aa.x; v[c * 4 + 1] += aa.y; v[c * 4 + 2] += aa.z; v[c * 4 + 3] += aa.w;
+                            }
                         }
-                        row0 += (uint32_t)quarters * chunk_bytes;
+                        if (g.act) {
+                            const float hi = g.act == 2 ? 6.f : INFINITY;
+#pragma unroll
+                            for (int c = 0; c < 16; ++c) v[c] = fminf(fmaxf(v[c], 0.f), hi);
+                        }
+#pragma unroll
+                        for (int c = 0; c < 4; ++c)
+                            sts128(row0 + (((uint32_t)c << 4) ^ swz), make_float4(v[c * 4], v[c * 4 + 1], v[c * 4 + 2], v[c * 4 + 3]));
+                        __syncwarp();
+                        const int r1 = lane >> 2, w1 = lane & 3;
+                        const uint32_t src = out_sub + (uint32_t)r1 * 64u + (uint32_t)((w1 ^ ((r1 >> 1) & 3)) << 4);
+                        if (n0 + c0 + 4 * w1 < g.N) {
+                            float4 q[4];
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) q[i] = lds128(src + (uint32_t)i * 512u);
+#pragma unroll
+                            for (int i = 0; i < 4; ++i)
+                                if (r1 + i * 8 < rows_live) *reinterpret_cast<float4*>(out_dst + (long long)(i * 8) * g.ldd) = q[i];
+                        }
                     }
                 }
-                if (lane == 0) tma_store_wait_read();
-            }
-        } else if (splits == 1) {
-            wait_acc();
-            if (ok) {
-                const int m = m0 + quarter * 32 + lane;
-                float* drow = g.D + (long long)b * g.strideD + (long long)m * g.ldd;
-                const float* arow = g.addend ? g.addend + (long long)m * g.ldd : nullptr;
-                for (int c0 = 0; c0 < BN; c0 += 16) {
-                    float v[16];
-                    acc16(c0, v);
+            } else if (!CW) {
+                wait_acc();
+                if (ok) {
+                    const int m = m0 + quarter * 32 + lane;
+                    float* drow = g.D + (long long)b * g.strideD + (long long)m * g.ldd;
+                    const float* arow = g.addend ? g.addend + (long long)m * g.ldd : nullptr;
+                    for (int c0 = grp * 16; c0 < BN; c0 += 32) {
+                        float v[16];
+                        acc16(c0, v);
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const int n = n0 + c0 + j;
-                        if (quarter * 32 + lane < live && n < g.N) {
-                            float o = v[j] + s_bias[c0 + j];
-                            if (arow) o += __ldg(arow + n);
-                            drow[n] = act_fn(o, g.act);
+                        for (int j = 0; j < 16; ++j) {
+                            const int n = n0 + c0 + j;
+                            if (quarter * 32 + lane < live && n < g.N) {
+                                float bb;
+                                asm volatile("ld.shared.f32 %0, [%1];" : "=f"(bb) : "r"(sbias + (uint32_t)(c0 + j) * 4u) : "memory");
+                                float o = v[j] + bb;
+                                if (arow) o += __ldg(arow + n);
+                                drow[n] = act_fn(o, g.act);
+                            }
                         }
                     }
                 }
@@ -833,83 +897,75 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         } else {
             // Split K, sender: park the partial tile in the stage ring (idle by then) as rows of BN words, the 16-byte words
             // of a row rotated by its index so that the lanes' stores meet different banks, and let the copy engine push
-            // every owner its rows of this warp's 32.  Owner: the rows arrive from every CTA of the cluster (its own
+            // every owner its rows of this quarter's 32.  Owner: the rows arrive from every CTA of the cluster (its own
             // included); they are added in rank order (a fixed order: the result does not depend on timing), bias /
             // residual / activation are applied and row-contiguous 128-bit words are stored.
-            const int nch = BN / 4, r0 = sp * rows_per, q0 = quarter * 32;
-            uint8_t* const prow = sm + (uint32_t)(q0 + lane) * (uint32_t)BN * 4u;
-            int pos = (q0 + lane) % nch;
-            const int a0 = max(q0, lane * rows_per), a1 = min(min(q0 + 32, live), (lane + 1) * rows_per);
-            const bool sends = lane < splits && a1 > a0;
-            uint32_t push_dst = 0, push_bar = 0;
-            if (sends) {
-                push_dst = cluster_addr(sbase + g.recv_off + (uint32_t)((r0 + a0 - lane * rows_per) * BN) * 4u, lane);
-                push_bar = cluster_addr(recv_bar, lane);
-            }
-            const bool vec = ((g.ldd & 3) == 0) && ((g.N & 3) == 0) && ((reinterpret_cast<uintptr_t>(g.D) & 15) == 0) &&
-                             (!g.addend || (reinterpret_cast<uintptr_t>(g.addend) & 15) == 0);
-            // thread t walks the (row, 4-column group) grid of its CTA's rows in steps of 128
-            const int qstep = 128 / nch, rstep = 128 - qstep * nch;
-            int rr = t / nch, cc = t - rr * nch, rot = (r0 + rr) % nch;
-            const int rot_step = qstep % nch;
-            const uint8_t* const recv = sm + g.recv_off;
-            const uint32_t part_stride = (uint32_t)(rows_per * BN) * 4u;
-            float* const dbase = g.D + (long long)b * g.strideD + (long long)(m0 + r0) * g.ldd + n0;
-            const float* const abase = g.addend ? g.addend + (long long)(m0 + r0) * g.ldd + n0 : nullptr;
+            const int q0 = quarter * 32;
             cluster_wait();                                   // every CTA's barriers are initialised
             wait_acc();
             if (ok && q0 < live) {
 #pragma unroll 1
-                for (int c0 = 0; c0 < BN; c0 += 16) {
+                for (int c0 = grp * 16; c0 < BN; c0 += 32) {
                     float v[16];
                     acc16(c0, v);
+                    int pos = rot0 + (c0 >> 2);
+                    if (pos >= nch) pos -= nch;
 #pragma unroll
                     for (int j = 0; j < 16; j += 4) {
-                        if (q0 + lane < live) *reinterpret_cast<float4*>(prow + pos * 16) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+                        if (q0 + lane < live) sts128(prow + (uint32_t)pos * 16u, make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]));
                         pos = pos + 1 == nch ? 0 : pos + 1;
                     }
                 }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> visible to the bulk copies
-                __syncwarp();
-                if (sends) bulk_push(push_dst, sbase + (uint32_t)(a0 * BN) * 4u, (uint32_t)((a1 - a0) * BN) * 4u, push_bar);
             }
+            __syncwarp();
+            asm volatile("barrier.sync %0, 64;" ::"r"(2 + quarter) : "memory");    // both warps' columns of these rows are parked
+            if (ok && push_bytes) bulk_push(push_dst, push_src, push_bytes, push_bar);
             int total = my_rows * nch;
+            // (the residual's words are fetched one step ahead, the first ones while the rows are on their way)
+            auto fetch_addend = [&](int idx) {
+                return vec && abase && idx < total && n0 + cc * 4 < g.N ? __ldg(reinterpret_cast<const float4*>(abase + (long long)rr * g.ldd + cc * 4))
+                                                                        : make_float4(0.f, 0.f, 0.f, 0.f);
+            };
+            float4 ahead = fetch_addend(t);
             if (my_rows && !mbar_wait(recv_bar, 0)) {
                 if (lane == 0) atomicExch(&g_device_status, (int)NNV_ERR_TIMEOUT);
                 total = 0;
             }
             __syncwarp();
             cluster_arrive_relaxed();                         // this CTA's rows have arrived: their senders may leave
-            cluster_arrived = true;
+            const uint32_t recv = sbase + g.recv_off, part_stride = (uint32_t)(rows_per * BN) * 4u;
             auto reduce = [&](auto nsplits) {
                 constexpr int NS = decltype(nsplits)::value;
-#pragma unroll 2
-                for (int idx = t; idx < total; idx += 128) {
+#pragma unroll 1
+                for (int idx = t; idx < total; idx += 256) {
                     const int p = cc + rot >= nch ? cc + rot - nch : cc + rot;
-                    const uint8_t* src = recv + (uint32_t)(rr * BN) * 4u + (uint32_t)p * 16u;
+                    const uint32_t src = recv + (uint32_t)(rr * BN) * 4u + (uint32_t)p * 16u;
                     constexpr int NB = NS < 8 ? NS : 8;       // loads in flight
                     float4 v[NB];
 #pragma unroll
-                    for (int rk = 0; rk < NB; ++rk) v[rk] = *reinterpret_cast<const float4*>(src + rk * part_stride);
-                    float4 o = *reinterpret_cast<const float4*>(s_bias + cc * 4);
+                    for (int rk = 0; rk < NB; ++rk) v[rk] = lds128(src + (uint32_t)rk * part_stride);
+                    float4 o = lds128(sbias + (uint32_t)cc * 16u);
                     const int n = cc * 4;
                     const long long off = (long long)rr * g.ldd + n;
+                    const float4 aa = ahead;
+                    rr += qstep; cc += rstep; rot += rot_step;
+                    if (cc >= nch) { cc -= nch; ++rr; ++rot; }
+                    if (rot >= nch) rot -= nch;
+                    ahead = fetch_addend(idx + 256);
                     float4 a = v[0];
 #pragma unroll
                     for (int rk = 1; rk < NB; ++rk) { a.x += v[rk].x; a.y += v[rk].y; a.z += v[rk].z; a.w += v[rk].w; }
                     if constexpr (NS > 8) {
 #pragma unroll
-                        for (int rk = 0; rk < 8; ++rk) v[rk] = *reinterpret_cast<const float4*>(src + (rk + 8) * part_stride);
+                        for (int rk = 0; rk < 8; ++rk) v[rk] = lds128(src + (uint32_t)(rk + 8) * part_stride);
 #pragma unroll
                         for (int rk = 0; rk < 8; ++rk) { a.x += v[rk].x; a.y += v[rk].y; a.z += v[rk].z; a.w += v[rk].w; }
                     }
                     o.x += a.x; o.y += a.y; o.z += a.z; o.w += a.w;
                     if (n0 + n < g.N) {
                         if (vec) {
-                            if (abase) {
-                                const float4 aa = __ldg(reinterpret_cast<const float4*>(abase + off));
-                                o.x += aa.x; o.y += aa.y; o.z += aa.z; o.w += aa.w;
-                            }
+                            if (abase) { o.x += aa.x; o.y += aa.y; o.z += aa.z; o.w += aa.w; }
                             act4(o);
                             *reinterpret_cast<float4*>(dbase + off) = o;
                         } else {
@@ -918,9 +974,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                                 dbase[off + j] = act_fn(abase ? vv[j] + __ldg(abase + off + j) : vv[j], g.act);
                         }
                     }
-                    rr += qstep; cc += rstep; rot += rot_step;
-                    if (cc >= nch) { cc -= nch; ++rr; ++rot; }
-                    if (rot >= nch) rot -= nch;
                 }
             };
             if (splits == 16) reduce(std::integral_constant<int, 16>());
@@ -930,8 +983,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         }
     }
     __syncwarp();
-    if (splits > 1) {
-        if (!cluster_arrived) cluster_arrive_relaxed();
+    if constexpr (SPLIT) {
+        if (warp >= 8) cluster_arrive_relaxed();
         cluster_wait();                                       // nobody leaves while its rows may still be on their way
     }
     tc_fence_before();
@@ -988,17 +1041,17 @@ nnv_status_t encode_operand(CUtensorMap* map, const void* base, bool bf16, int K
     return NNV_OK;
 }
 
-// 3-D map over the fp32 output (or the residual addend, same geometry): dims {N, M, batch}, boxes of
-// `cw` columns (32 with the 128-byte swizzle, 16 with the 64-byte one) x 32 rows.
-nnv_status_t encode_output(CUtensorMap* map, const void* base, int N, int M, int batch, int64_t ld, int64_t batch_stride, int cw) {
+// 3-D map over the residual addend (the output's geometry): dims {N, M, batch}, boxes of 16 columns, 64-byte swizzle, x `box_rows`
+// rows: what a column chunk's staging sub-tiles hold together.
+nnv_status_t encode_addend_tiles(CUtensorMap* map, const void* base, int N, int M, int batch, int64_t ld, int64_t batch_stride, int box_rows) {
     cuuint64_t dims[3] = {(cuuint64_t)N, (cuuint64_t)M, (cuuint64_t)batch};    // or {N, rows of a tile, tiles}
     cuuint64_t strides[2] = {(cuuint64_t)(ld * 4), (cuuint64_t)(batch_stride * 4)};
-    cuuint32_t box[3] = {(cuuint32_t)cw, 32, 1};
+    cuuint32_t box[3] = {16, (cuuint32_t)box_rows, 1};
     cuuint32_t estr[3] = {1, 1, 1};
     CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void*>(base), dims, strides, box, estr,
-                          CU_TENSOR_MAP_INTERLEAVE_NONE, cw == 32 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
                           CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    NNV_REQUIRE(r == CUDA_SUCCESS, NNV_ERR_CUDA, "cuTensorMapEncodeTiled (output tiles) failed with code %d", (int)r);
+    NNV_REQUIRE(r == CUDA_SUCCESS, NNV_ERR_CUDA, "cuTensorMapEncodeTiled (residual tiles) failed with code %d", (int)r);
     return NNV_OK;
 }
 
@@ -1209,7 +1262,7 @@ struct GemmShape {
     size_t smem_bytes;
 };
 
-nnv_status_t gemm_shape(int mode, const GemmTiling& tile, int M, int N, int batch, int nkb, bool tma_out, bool addend, GemmShape* out) {
+nnv_status_t gemm_shape(int mode, const GemmTiling& tile, int M, int N, int batch, int nkb, bool staged, bool addend, GemmShape* out) {
     GemmShape g{};
     const Tuning& tn = tuning();
     g.BN = tile.BN; g.splits = tile.splits; g.rows = tile.rows;
@@ -1225,12 +1278,12 @@ nnv_status_t gemm_shape(int mode, const GemmTiling& tile, int M, int N, int batc
     const int nkb_cta = ceil_div(nkb, g.splits);
     g.ring = gemm_ring(mode, g.BN, g.rows, (long long)g.m_tiles * ceil_div(N, g.BN) * batch * g.splits, nkb_cta);
     if (tn.gemm_ring && (size_t)tn.gemm_ring * sb <= 210u * 1024u) g.ring = tn.gemm_ring;
-    // Write-out by TMA through swizzled staging tiles when the output rows are 16-byte multiples (else plain stores), in
+    // Write-out through swizzled staging tiles when the output rows are 16-byte multiples (else plain stores), in
     // the ring once that is idle; with a residual addend, which is loaded while the ring works, in a place of their own.
     const size_t staging = (size_t)ceil_div(g.rows, 32) * 32 * g.BN * 4;
     // Split K: room to park the partial tile in the ring, and for the rows this CTA receives (its share from every CTA).
-    const size_t park = split ? (size_t)g.rows * g.BN * 4 : (tma_out && !addend) ? staging : 0;
-    const size_t behind = split ? (size_t)g.splits * ceil_div(g.rows, g.splits) * g.BN * 4 : (tma_out && addend) ? staging + 1024 : 0;
+    const size_t park = split ? (size_t)g.rows * g.BN * 4 : (staged && !addend) ? staging : 0;
+    const size_t behind = split ? (size_t)g.splits * ceil_div(g.rows, g.splits) * g.BN * 4 : (staged && addend) ? staging + 1024 : 0;
     while (g.ring < 8 && g.ring * sb < park) ++g.ring;
     while (g.ring > 1 && 2048 + g.ring * sb + bars + behind > 226u * 1024u && (g.ring - 1) * sb >= park) --g.ring;
     // Two issuers take alternate K blocks, so in a ring of odd depth the blocks of one slot go to one and the other in turn.  A wait
@@ -1248,7 +1301,7 @@ nnv_status_t gemm_shape(int mode, const GemmTiling& tile, int M, int N, int batc
     const size_t ring_and_bars = g.ring * sb + bars;
     g.recv_off = (uint32_t)align_up(ring_and_bars, 128);
     g.stage_off = addend ? (uint32_t)align_up(ring_and_bars, 1024) : 0;
-    g.smem_bytes = (size_t)1024 + (split ? g.recv_off + behind : (tma_out && addend) ? g.stage_off + staging : ring_and_bars);
+    g.smem_bytes = (size_t)1024 + (split ? g.recv_off + behind : (staged && addend) ? g.stage_off + staging : ring_and_bars);
     // the MMAs read 128 rows of A from every stage, the last one included
     g.smem_bytes = std::max(g.smem_bytes, (size_t)1024 + (g.ring - 1) * sb + A_STAGE_BYTES);
     if (split) g.smem_bytes = std::max(g.smem_bytes, tmem_share_bytes(g.tmem_cols));
@@ -1259,16 +1312,25 @@ nnv_status_t gemm_shape(int mode, const GemmTiling& tile, int M, int N, int batc
 
 std::once_flag g_attr_once;
 
+// [kernel mode][K split over a cluster]
+constexpr decltype(&gemm_tc_kernel<0, false>) gemm_kernels[9][2] = {
+    {gemm_tc_kernel<0, false>, gemm_tc_kernel<0, true>}, {gemm_tc_kernel<1, false>, gemm_tc_kernel<1, true>},
+    {gemm_tc_kernel<2, false>, gemm_tc_kernel<2, true>}, {gemm_tc_kernel<3, false>, gemm_tc_kernel<3, true>},
+    {gemm_tc_kernel<4, false>, gemm_tc_kernel<4, true>}, {gemm_tc_kernel<5, false>, gemm_tc_kernel<5, true>},
+    {gemm_tc_kernel<6, false>, gemm_tc_kernel<6, true>}, {gemm_tc_kernel<7, false>, gemm_tc_kernel<7, true>},
+    {gemm_tc_kernel<ROUNDED, false>, gemm_tc_kernel<ROUNDED, true>}};
+static_assert(GEMM_TF32 == 0 && GEMM_BF16 == 1 && GEMM_X3 == 2 && GEMM_BF16_CVT == 3, "the table's order");
+
 }  // namespace
 
 nnv_status_t gemm_tc_init() {
     NNV_TRY(get_encoder());
     std::call_once(g_attr_once, [] {
-        for (auto* kernel : {gemm_tc_kernel<0>, gemm_tc_kernel<1>, gemm_tc_kernel<2>, gemm_tc_kernel<3>, gemm_tc_kernel<4>, gemm_tc_kernel<5>,
-                             gemm_tc_kernel<6>, gemm_tc_kernel<7>, gemm_tc_kernel<ROUNDED>}) {
-            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
-            cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        }
+        for (auto& forms : gemm_kernels)
+            for (auto* kernel : forms) {
+                cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
+                cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+            }
         cudaFuncSetAttribute(conv3x3_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
         cudaFuncSetAttribute(conv3x3_bf16_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
         cudaFuncSetAttribute(gemm_sp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
@@ -1609,15 +1671,15 @@ nnv_status_t launch_gemm_tc(const GemmArgs& a, cudaStream_t st) {
         if (use) return launch_conv3x3_tc(a, ct, st);
         }
     }
-    const bool tma_ok = (a.N % 4) == 0 && (a.ldd % 4) == 0 && (a.strideD % 4) == 0 && (reinterpret_cast<uintptr_t>(a.D) & 15) == 0 &&
+    const bool vec_ok = (a.N % 4) == 0 && (a.ldd % 4) == 0 && (a.strideD % 4) == 0 && (reinterpret_cast<uintptr_t>(a.D) & 15) == 0 &&
                         (!a.addend || ((reinterpret_cast<uintptr_t>(a.addend) & 15) == 0 && a.batch == 1));
     GemmShape sh;
-    NNV_TRY(gemm_shape(mode, tile, a.M, a.N, a.batch, nkb_all, tma_ok, a.addend != nullptr, &sh));
+    NNV_TRY(gemm_shape(mode, tile, a.M, a.N, a.batch, nkb_all, vec_ok, a.addend != nullptr, &sh));
     const int BN = sh.BN, splits = sh.splits, rows = sh.rows, m_tiles = sh.m_tiles;
-    const bool tma_out = tma_ok && splits == 1;
+    const bool staged = vec_ok && splits == 1;
 
     const bool bf16 = a.mode == GEMM_BF16;
-    CUtensorMap tmA, tmB, tmD, tmAdd;
+    CUtensorMap tmA, tmB, tmAdd;
     GemmDev g;
     g.stamp = next_stamp();
     next_stamp() = nullptr;
@@ -1625,7 +1687,7 @@ nnv_status_t launch_gemm_tc(const GemmArgs& a, cudaStream_t st) {
     g.ldd = a.ldd; g.strideD = a.strideD;
     g.M = a.M; g.N = a.N; g.Kd = a.Kd; g.BN = BN; g.act = a.act; g.tmem_cols = sh.tmem_cols; g.splits = splits; g.stages = sh.ring; g.issuers = sh.issuers;
     g.rows = rows; g.bar_off = sh.bar_off; g.recv_off = sh.recv_off; g.stage_off = sh.stage_off;
-    g.tma_out = tma_out ? ((BN % 32) == 0 ? 32 : 16) : 0;
+    g.chunk = staged ? 16 : 0;
     g.ic_on = 0; g.ic_C = g.ic_cblk = g.ic_S = g.ic_OW = g.ic_stride = g.ic_pad = 0;
     g.x = nullptr; g.ic_H = g.ic_W = g.ic_Q = 0; g.magic_c = g.magic_s = 0;
     if (gather) {
@@ -1657,22 +1719,18 @@ nnv_status_t launch_gemm_tc(const GemmArgs& a, cudaStream_t st) {
     const bool equal = a.M == m_tiles * rows && (a.batch == 1 || a.strideD == (int64_t)a.M * a.ldd);
     NNV_REQUIRE(equal || rows == BM, NNV_ERR_INVALID_ARG, "batched GEMM outputs must be dense");
     g.z_tiles = equal ? m_tiles : 0;
-    auto encode_out = [&](CUtensorMap* map, const void* base) {
-        if (equal) return encode_output(map, base, a.N, rows, m_tiles * a.batch, a.ldd, (int64_t)rows * a.ldd, g.tma_out);
-        return encode_output(map, base, a.N, a.M, a.batch, a.ldd, a.batch > 1 ? a.strideD : (int64_t)a.M * a.ldd, g.tma_out);
+    auto encode_addend = [&](CUtensorMap* map, const void* base) {
+        const int box_rows = ceil_div(rows, 32) * 32;
+        if (equal) return encode_addend_tiles(map, base, a.N, rows, m_tiles * a.batch, a.ldd, (int64_t)rows * a.ldd, box_rows);
+        return encode_addend_tiles(map, base, a.N, a.M, a.batch, a.ldd, a.batch > 1 ? a.strideD : (int64_t)a.M * a.ldd, box_rows);
     };
-    if (tma_out) NNV_TRY(encode_out(&tmD, a.D));
-    else tmD = tmA;                                              // unused by the kernel, but a kernel parameter must hold a valid object
-    if (tma_out && a.addend) NNV_TRY(encode_out(&tmAdd, a.addend));
+    if (staged && a.addend) NNV_TRY(encode_addend(&tmAdd, a.addend));
     else tmAdd = tmA;
 
     dim3 grid(m_tiles, ceil_div(a.N, BN), a.batch * splits);
     NNV_REQUIRE(grid.y <= 65535 && grid.z <= 65535, NNV_ERR_UNSUPPORTED, "GEMM grid too large");
-    static constexpr decltype(&gemm_tc_kernel<0>) kernels[9] = {gemm_tc_kernel<GEMM_TF32>, gemm_tc_kernel<GEMM_BF16>, gemm_tc_kernel<GEMM_X3>,
-        gemm_tc_kernel<GEMM_BF16_CVT>, gemm_tc_kernel<4>, gemm_tc_kernel<5>, gemm_tc_kernel<6>, gemm_tc_kernel<7>,
-        gemm_tc_kernel<ROUNDED>};
     NNV_REQUIRE(a.mode >= GEMM_TF32 && a.mode <= GEMM_BF16_CVT, NNV_ERR_INVALID_ARG, "unknown GEMM mode %d", a.mode);
-    (void)launch_pdl_cluster(kernels[mode], grid, dim3(gemm_tc_threads(mode)), sh.smem_bytes, st, splits, tmA, tmB, tmD, tmAdd, g);
+    (void)launch_pdl_cluster(gemm_kernels[mode][splits > 1], grid, dim3(gemm_tc_threads(mode)), sh.smem_bytes, st, splits, tmA, tmB, tmAdd, g);
     NNV_CUDA(cudaGetLastError());
     return NNV_OK;
 }
@@ -1680,10 +1738,10 @@ nnv_status_t launch_gemm_tc(const GemmArgs& a, cudaStream_t st) {
 }  // namespace nnv
 
 // Host-side launch shape of gemm_tc_kernel for the tests (kernel mode, K blocks of 128 bytes).
-extern "C" int nnv_internal_gemm_shape(int mode, int M, int N, int batch, int nkb, int tma_out, int addend, int32_t* out) {
+extern "C" int nnv_internal_gemm_shape(int mode, int M, int N, int batch, int nkb, int staged, int addend, int32_t* out) {
     using namespace nnv;
     GemmShape s;
-    const nnv_status_t st = gemm_shape(mode, pick_gemm_tiling(mode, M, N, batch, nkb), M, N, batch, nkb, tma_out != 0, addend != 0, &s);
+    const nnv_status_t st = gemm_shape(mode, pick_gemm_tiling(mode, M, N, batch, nkb), M, N, batch, nkb, staged != 0, addend != 0, &s);
     if (st != NNV_OK) return st;
     const int32_t v[] = {s.BN, s.splits, s.rows, s.m_tiles, s.issuers, s.ring, s.tmem_cols, (int32_t)s.bar_off, (int32_t)s.recv_off,
                          (int32_t)s.stage_off, (int32_t)s.smem_bytes, (int32_t)gemm_stage_bytes(mode, s.BN, s.rows), gemm_tc_threads(mode)};
