@@ -1146,11 +1146,11 @@ int gemm_ring(int mode, int bn, int rows, long long ctas, int nkb) {
     return std::max(2, std::min(most, nkb));
 }
 
-// Tiling of gemm_tc_kernel: fixed cost + waves x (K blocks per CTA x time per block + write-out).  A K block costs a CTA four
-// MMAs of ~82 cycles whatever BN <= 128 is, or the fill of its shared memory (per SM, and from L2 over all SMs); a split
-// adds the pushes of the partial rows.  Constants (microseconds) fitted to a sweep of every BN and split over the 101 GEMM
-// layer shapes of the ResNet / MobileNetV2 / VGG configurations at several resolutions, chained launches: the chosen
-// tilings are 0.05 us a launch above the best measured ones on average.
+// Tiling of gemm_tc_kernel: waves x (K blocks per CTA x time per block + start and write-out).  A K block costs a CTA the issue of
+// its MMAs (or the wait for its conversion) whatever BN <= 128 is, or the fill of its shared memory (per SM, and from L2 over all
+// SMs); a split adds the pushes of the partial rows.  Constants (microseconds) fitted to sweeps of every BN and split, chained
+// launches, by the excess of the chosen tilings over the best measured ones: TF32 1.3 % over 213 layers (the former constants 2.1 %),
+// BF16 operands 0.4 % over 28 (1.8 %), BF16 math on fp32 activations 1.3 % over 79 (3.7 %).
 // A gather mode's K block takes the eight warps time for every row, most of it in steps of half a tile; a second CTA on the SM adds
 // `share` of it.  Its tiles may be lower than 128 rows (any height that divides M), which spreads the rows over more SMs.  Fitted the
 // same way over 33 shapes: the chosen tilings are 3 % above the best measured ones on average.
@@ -1159,12 +1159,21 @@ int gemm_ring(int mode, int bn, int rows, long long ctas, int nkb) {
 // F(4,3) @7, 22.9 us against 19.1).
 // Mode 8's K block waits for the rounding; CTAs that share an SM count by the clusters that fit (clusters of 16 put 128 CTAs on 112
 // places): fitted to 34 layers, 0.6 % above the best measured tilings (the TF32 constants: 5.6 %).
+struct TilingCost { double fixed, block, sm_rate, l2_rate, start, column, shared_column, split, split_word; };
+constexpr TilingCost tiling_cost(int mode) {
+    return gather_mode(mode) ? TilingCost{0.87, 0.146, 108e3, 10.9e6, 1.85, 0.0093, 0.0, 0.28, 1.22e-4}
+           : mode == 2       ? TilingCost{1.87, 0.37, 108e3, 4.6e6, 0.80, 0.005, 0.0, 0.73, 1.22e-4}
+           : mode == ROUNDED ? TilingCost{1.87, 0.146, 108e3, 10.9e6, 0.80, 0.0093, 0.0, 0.26, 1.22e-4}
+           : mode == 1       ? TilingCost{1.87, 0.366, 26.8e3, 2.9e6, 0.0, 0.0022, 0.0, 0.0, 2.32e-3}
+           : mode == 3       ? TilingCost{1.87, 0.372, 48.9e3, 5.02e6, 0.0, 0.0065, 0.0, 0.67, 1.53e-4}
+                             : TilingCost{1.87, 0.10, 114e3, 11.8e6, 2.97, 0.010, 0.0247, 0.546, 1.69e-4};
+}
 struct GemmTiling { int BN, splits, rows, waves; };
 GemmTiling search_gemm_tiling(int mode, int M, int N, int batch, int nkb) {
     constexpr struct { double row_us, share; } gather[4] = {{0.0064, 0.36}, {0.0054, 0.60}, {0.0025, 0.81}, {0.0042, 0.40}};   // modes 4 - 7
     const bool x3 = mode == GEMM_X3;
     const bool rounded = mode == ROUNDED;
-    const double fixed = gather_mode(mode) ? 0.87 : 1.87, start = gather_mode(mode) ? 1.85 : x3 || rounded ? 0.80 : 0.40, column = x3 ? 0.005 : 0.0093;
+    const TilingCost c = tiling_cost(mode);
     const int least = ceil_div(M, BM);
     const int most = gather_mode(mode) ? std::max(least, std::min(M / 16, 296)) : least;
     GemmTiling best{16, 1, gemm_rows(M), 1};
@@ -1185,13 +1194,13 @@ GemmTiling search_gemm_tiling(int mode, int M, int N, int batch, int nkb) {
                 const double waves = (double)((ctas + slots - 1) / slots);
                 const int lone = rounded ? cluster_slots(sp, 1) : 148;
                 const double res = (double)std::min<long long>(occ, (ctas + lone - 1) / lone);
-                double kb = std::max({(x3 ? 0.37 : 0.146) * res, kb_bytes * res / 108e3, kb_bytes * (double)std::min(ctas, slots) / (x3 ? 4.6e6 : 10.9e6)});
+                double kb = std::max({c.block * res, kb_bytes * res / c.sm_rate, kb_bytes * (double)std::min(ctas, slots) / c.l2_rate});
                 if (x3) kb = std::max(kb, (0.40 + 0.07 * (ceil_div(rows, 32) + ceil_div(bn, 32))) * (1 + 0.15 * (res - 1)));
                 if (gather_mode(mode))
                     kb = std::max(kb, (0.2 + gather[mode & 3].row_us * (0.65 * 64 * ceil_div(rows, 64) + 0.35 * rows)) * (1 + gather[mode & 3].share * (res - 1)));
                 if (rounded) kb = std::max(kb, (0.25 + 0.0005 * rows) * (1 + 0.8 * (res - 1)));
-                const double split = sp > 1 ? (x3 ? 0.73 : 0.26 + (rounded ? 0.0 : 0.021) * std::log2((double)sp)) + 1.22e-4 * bn * rows * res : 0.0;
-                const double t = fixed + waves * (nk * kb + start + column * bn + split);
+                const double split = sp > 1 ? c.split + c.split_word * bn * rows * res : 0.0;
+                const double t = c.fixed + waves * (nk * kb + c.start + (c.column + c.shared_column * (res - 1)) * bn + split);
                 if (t < best_t - 1e-9) { best_t = t; best = GemmTiling{bn, sp, rows, (int)waves}; }
             }
         }
@@ -1216,13 +1225,13 @@ GemmTiling pick_gemm_tiling(int mode, int M, int N, int batch, int nkb) {
 // the least estimated time (us), if that is below the GEMM's: waves x (channel blocks per CTA x time per block + start and write-out).
 // A block's time depends on the CTAs that share the SM and on the box slots, 2.4 with an SM to itself, 3.1 for two (2.7 at 64 columns),
 // 5.2 for three on one slot; an even spread is not to be had with room for three CTAs to an SM or in clusters of eight.  A K block of
-// the GEMM is 0.25, 0.31 with two CTAs to an SM.  Where the GEMM's tiles need a second wave the halo kernel is always ahead.  A K
-// split runs in one wave of whole clusters or not at all: a second one costs as much as the first (72 clusters of four on 71 places:
-// 384 -> 512 @48 34.7 us, with one box slot and three CTAs to an SM 27.4).
-// Fitted to 240 layers (64 - 768 channels, 28 - 224 pixels a side), the chosen kernel and tiling 0.4 % above the best measured on
-// average.  Measured, halo kernel / implicit GEMM: 64 -> 64 @224 12.3 / 16.8, 128 -> 256 @112 18.2 / 25.2, 512 -> 512 @72 54 / 80, 384 -> 256
-// @80 27.5 / 32.2, 512 -> 256 @56 23.2 / 26.5, 768 -> 64 @112 30.5 / 56; the GEMM's: 128 -> 128 @112 15.4 / 13.3, 64 -> 64 @180 11.2 / 10.0,
-// 384 -> 512 @48 27.4 / 21.8, 512 -> 512 @28 16.6 / 15.8.
+// the GEMM is 0.155 at 64 columns, 0.235 at 128, 0.32 with two CTAs to an SM.  Where the GEMM's tiles need a second wave the halo kernel
+// is always ahead.  A K split runs in one wave of whole clusters or not at all: a second one costs as much as the first (72 clusters of
+// four on 71 places: 384 -> 512 @48 34.7 us, with one box slot and three CTAs to an SM 27.4).
+// The halo kernel's figures are fitted to 240 layers (64 - 768 channels, 28 - 224 pixels a side), the GEMM's to 20.  Measured, halo kernel
+// / implicit GEMM: 64 -> 64 @224 12.1 / 16.3, 128 -> 256 @112 18.1 / 20.4, 512 -> 512 @72 54 / 74, 768 -> 64 @112 29.8 / 34.6, 512 -> 256
+// @56 23.0 / 22.7; the GEMM's: 128 -> 128 @112 13.6 / 11.6, 256 -> 256 @56 16.9 / 14.7, 384 -> 512 @48 21.6 / 18.9, 192 -> 192 @96 17.1 / 13.9,
+// 512 -> 512 @28 15.7 / 14.0.
 double halo_us(const ConvTiling& t, long long tiles, int cblk) {
     const int occ = std::max(1, std::min({(int)(227u * 1024u / (t.smem + 1024)), 512 / t.tmem_cols, 3}));
     const long long ctas = tiles * t.splits, slots = cluster_slots(t.splits, occ);
@@ -1240,8 +1249,8 @@ bool pick_conv_tiling(int C, int H, int W, int N, const GemmTiling& gemm, ConvTi
     double best = 1e30;
     if (gemm.waves == 1) {
         const long long ctas = (long long)ceil_div(H * W, gemm.rows) * ceil_div(N, gemm.BN) * gemm.splits;
-        best = ceil_div(9 * cblk, gemm.splits) * (ctas <= 148 ? 0.247 : 0.31) + 1.4 + 0.033 * gemm.BN +
-               (gemm.splits == 1 ? 0.0 : gemm.splits == 2 ? 0.9 + 0.0172 * gemm.BN : 0.7 + 0.0093 * gemm.BN);
+        best = ceil_div(9 * cblk, gemm.splits) * (ctas <= 148 ? 0.075 + 0.00125 * gemm.BN : 0.324) + 1.98 + 0.023 * gemm.BN +
+               (gemm.splits == 1 ? 0.0 : gemm.splits == 2 ? 0.64 + 0.0137 * gemm.BN : 1.02 + 0.0021 * gemm.BN);
     }
     bool found = false;
     for (int splits = 1; splits <= 8 && splits <= cblk; splits *= 2)
