@@ -1,19 +1,22 @@
 // 3x3 / stride 1 / pad 1 convolution with BF16 math straight from the fp32 activation.  Included by gemm_tc.cu (inside namespace
 // nnv, after the PTX helpers).
 //
-// Bound: the issue of 18 MMAs (M = 128, N <= 128, K = 16), ~82 cycles each, per patch and 32 input channels by one thread; the chain
-// of box load, rounding and MMAs comes right behind (256 -> 256 @56: without the rounding after two boxes, or without the weights'
-// loads after the first ring, the same time within 1 %; with half the MMAs 9.3 us instead of 11.0).  A CTA owns an
+// Bound: shared memory.  Per patch and block of 32 input channels the copies write 60 KB (64 output channels), the rounding reads 23 and
+// writes 12, and 18 MMAs (M = 128, N = 64, K = 16) read 6 KB each: 200 KB, 1590 cycles at 128 bytes a cycle, where a block takes 1500
+// (device-clock probes, 256 -> 256 @56).  One thread issues an MMA per 82 cycles; two, with an accumulator each and the filter rows in
+// turn, reach that bound, and four boxes in flight keep it fed.  (A copy of the box for each filter column, so that the rows of the A
+// operand start on 128 bytes, costs more traffic than it saves: 11.5 us against 10.8.)  A CTA owns an
 // output patch of 16 rows x 8 columns and BN output channels.  Per block of 32 input channels it fetches ONE fp32 halo box of
 // 18 x 10 pixels, eight warps round it to bf16 into the un-swizzled core-matrix layout [8-channel chunk][pixel][16 bytes],
 // and all nine taps read that one copy: a tap (r, s) is a shift of the descriptor's start address by 10 r + s pixels, and the
 // eight-row groups of the A operand (the image rows of the patch) lie 160 bytes apart.  The implicit GEMM converts and fetches
-// every tap's tile by itself (9 x 16 KB against 23 KB), the earlier form of this kernel three boxes.
+// every tap's tile by itself (9 x 16 KB against 23 KB).
 // The weights of a filter row's three taps arrive as bf16, 64-byte swizzled, through one three-dimensional box.  K splits over
 // the channel blocks use a cluster whose CTAs push their partial rows to the rows' owners, as in gemm_tc_kernel.
-// Measured (chained launches, with bias, us; the better of the converting implicit GEMM and the earlier form -> this one):
-// 256 -> 256 @56 21.0 -> 11.0, 64 -> 64 @224 20.3 -> 17.5, 128 -> 128 @112 20.5 -> 9.1, 512 -> 512 @28 19.7 -> 11.9, 64 -> 64 @56
-// 6.9 -> 4.7, 128 -> 128 @28 6.7 -> 4.7, 256 -> 256 @14 7.4 -> 5.2.
+// The write-out is that of gemm_tc_kernel: eight warps, rows from shared memory as coalesced stores.  It took 1.7 us of the 10.8.
+// Measured (chained launches, with bias, us; one issuer, two boxes, TMA stores by four warps -> this one): 256 -> 256 @56 10.9 -> 9.9,
+// 64 -> 64 @224 16.8 -> 15.0, 128 -> 128 @112 9.1 -> 8.2, 64 -> 64 @56 4.55 -> 4.16, 320 -> 640 @24 9.7 -> 8.7, 128 -> 128 @28 4.53 -> 4.37,
+// 512 -> 512 @14 7.3 -> 7.0.
 #pragma once
 
 struct ConvBDev {
@@ -21,8 +24,7 @@ struct ConvBDev {
     float* D;
     const float* bias;
     const float* addend;
-    int C, H, W, K, BN, act, tmem_cols, splits, nb, cblk, tiles_w;
-    int tma_out;                      // 0: plain stores; else the column width of the sub-tiles stored by TMA
+    int C, H, W, K, BN, act, tmem_cols, splits, na, nb, cblk, tiles_w, issuers;
     uint32_t b_off, bar_off, recv_off;
 };
 
@@ -30,26 +32,29 @@ constexpr int CB_THREADS = 384;
 constexpr int CB_PIX = 180;                                   // pixels of a halo box: 18 rows x 10
 constexpr uint32_t CB_A32 = 23 * 1024;                        // fp32 box slot (180 x 128 bytes, padded)
 constexpr uint32_t CB_ABF = 92 * 128;                         // bf16 box slot (4 x 180 x 16 bytes, padded)
-constexpr uint32_t CB_RINGS_A = 2 * (CB_A32 + CB_ABF);
+constexpr int CB_MAX_NA = 4;
 constexpr int CB_MAX_NB = 8;
-constexpr int CB_BAR_BYTES = 8 * (6 + 2 * CB_MAX_NB + 4) + 512;
+constexpr int CB_BAR_BYTES = 8 * (2 * CB_MAX_NA + 4 + 2 * CB_MAX_NB + 4) + 512;
 
+template <bool SPLIT>
 __global__ void __launch_bounds__(CB_THREADS, 1)
 conv3x3_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                    const __grid_constant__ CUtensorMap tmD, const ConvBDev g) {
+                    const ConvBDev g) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* const sm = smem_raw + (sbase - smem_u32(smem_raw));
-    const int BN = g.BN, NB = g.nb, splits = g.splits;
+    const int BN = g.BN, NA = g.na, NB = g.nb, splits = SPLIT ? g.splits : 1;
+    const uint32_t abf0 = (uint32_t)NA * CB_A32;              // the bf16 boxes lie behind the fp32 ones
     const uint32_t b_slot = (uint32_t)BN * 192u;              // three taps x BN rows x 64 bytes
     const uint32_t bars = sbase + g.bar_off;
-    auto a_full = [&](int s) { return bars + 8u * s; };
-    auto a_conv = [&](int s) { return bars + 8u * (2 + s); };
-    auto a_empty = [&](int s) { return bars + 8u * (4 + s); };
-    auto b_full = [&](int s) { return bars + 8u * (6 + s); };
-    auto b_empty = [&](int s) { return bars + 8u * (6 + CB_MAX_NB + s); };
-    const uint32_t tmem_full_bar = bars + 8u * (6 + 2 * CB_MAX_NB), recv_bar = tmem_full_bar + 8u, holder = recv_bar + 8u;
-    float* const s_bias = reinterpret_cast<float*>(sm + g.bar_off + 8 * (6 + 2 * CB_MAX_NB + 4));
+    auto a_full = [&](int s) { return bars + 8u * s; };                        // an fp32 box has landed
+    auto a_free = [&](int s) { return bars + 8u * (CB_MAX_NA + s); };          // it has been rounded
+    auto a_conv = [&](int s) { return bars + 8u * (2 * CB_MAX_NA + s); };      // a bf16 box is complete
+    auto a_empty = [&](int s) { return bars + 8u * (2 * CB_MAX_NA + 2 + s); }; // it has been multiplied
+    auto b_full = [&](int s) { return bars + 8u * (2 * CB_MAX_NA + 4 + s); };
+    auto b_empty = [&](int s) { return bars + 8u * (2 * CB_MAX_NA + 4 + CB_MAX_NB + s); };
+    const uint32_t tmem_full_bar = bars + 8u * (2 * CB_MAX_NA + 4 + 2 * CB_MAX_NB), recv_bar = tmem_full_bar + 8u, holder = recv_bar + 8u;
+    const uint32_t sbias = bars + (uint32_t)CB_BAR_BYTES - 512u;
     const volatile uint32_t* holder_ptr = reinterpret_cast<const volatile uint32_t*>(sm + (holder - sbase));
 
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
@@ -61,10 +66,10 @@ conv3x3_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     if (warp == 0 && lane == 0) {
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmB)) : "memory");
-        if (g.tma_out) asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmD)) : "memory");
-        for (int s = 0; s < 2; ++s) { mbar_init(a_full(s), 1); mbar_init(a_conv(s), 8); mbar_init(a_empty(s), 1); }
+        for (int s = 0; s < NA; ++s) { mbar_init(a_full(s), 1); mbar_init(a_free(s), 8); }
+        for (int s = 0; s < 2; ++s) { mbar_init(a_conv(s), 8); mbar_init(a_empty(s), (uint32_t)g.issuers); }
         for (int s = 0; s < NB; ++s) { mbar_init(b_full(s), 1); mbar_init(b_empty(s), 1); }
-        mbar_init(tmem_full_bar, 1);
+        mbar_init(tmem_full_bar, (uint32_t)g.issuers);
         mbar_init(recv_bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -72,11 +77,38 @@ conv3x3_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(holder), "r"((uint32_t)g.tmem_cols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    // What the write-out needs besides the accumulator is worked out here, under the previous kernel's tail.
+    const int cw = warp >= 8 ? warp - 4 : warp - 2;           // of the eight converting warps
+    const int quarter = warp & 3, q0 = quarter * 32, half = warp >> 3, t = half * 128 + (cw & 3) * 32 + lane;
+    const bool vec = (g.K & 3) == 0 && (reinterpret_cast<uintptr_t>(g.D) & 15) == 0 && (!g.addend || (reinterpret_cast<uintptr_t>(g.addend) & 15) == 0);
+    uint32_t sub = sbase + (uint32_t)(cw & 7) * 2048u;        // a warp's sub-tile: 32 pixels x 16 columns
+    long long row_pitch = (long long)g.W * g.K;
+    int rows_live = ow0 + (lane >> 2) < g.W ? g.H - oh0 - quarter * 4 : 0;        // image rows of the quarter that exist where this lane stores
+    float* out = g.D + ((long long)(oh0 + quarter * 4) * g.W + ow0 + (lane >> 2)) * g.K + n0 + half * 16 + (lane & 3) * 4;
+    const int rows_per = 128 / splits, r0 = sp * rows_per;
+    int nch = BN / 4, rot0 = 0, qstep = 0, rstep = 0, rot_step = 0, rr = 0, cc = 0, rot = 0;
+    uint32_t push_dst = 0, push_bar = 0, push_src = 0, push_bytes = 0;
+    if constexpr (!SPLIT) {
+        asm volatile("" : "+r"(sub), "+l"(row_pitch), "+r"(rows_live), "+l"(out));
+    } else {
+        rot0 = (q0 + lane) % nch;
+        const int a0 = max(q0, lane * rows_per), a1 = min(q0 + 32, (lane + 1) * rows_per);
+        if (half == 0 && lane < splits && a1 > a0) {
+            push_dst = cluster_addr(sbase + g.recv_off + (uint32_t)((r0 + a0 - lane * rows_per) * BN) * 4u, lane);
+            push_bar = cluster_addr(recv_bar, lane);
+            push_src = sbase + (uint32_t)(a0 * BN) * 4u;
+            push_bytes = (uint32_t)((a1 - a0) * BN) * 4u;
+        }
+        qstep = 256 / nch; rstep = 256 - qstep * nch;
+        rr = t / nch; cc = t - rr * nch; rot = (r0 + rr) % nch;
+        rot_step = qstep % nch;
+        asm volatile("" : "+r"(nch), "+r"(rot0), "+r"(push_dst), "+r"(push_bar), "+r"(push_src), "+r"(push_bytes));
+        asm volatile("" : "+r"(qstep), "+r"(rstep), "+r"(rr), "+r"(cc), "+r"(rot), "+r"(rot_step));
+    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const int rows_per = 128 / splits, r0 = sp * rows_per, nch = BN / 4;
-    if (splits > 1) {
+    if constexpr (SPLIT) {
         if (threadIdx.x == 64) mbar_expect_tx(recv_bar, (uint32_t)(splits * rows_per * BN) * 4u);
         __syncwarp();
         cluster_arrive_relaxed();
@@ -88,13 +120,14 @@ conv3x3_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
 
     // Warps 2-5 and 8-11: round box after box, 32 pixels x 8 channels at a time.
     auto convert_boxes = [&](int cw) -> bool {
+        int sa = 0;
+        uint32_t pa = 0;
         for (int it = 0; it < ncb; ++it) {
             const int s = it & 1;
-            const uint32_t ph = (uint32_t)(it >> 1) & 1u;
-            if (!mbar_wait(a_full(s), ph)) return false;
-            if (it >= 2 && !mbar_wait(a_empty(s), ph ^ 1u)) return false;      // the slot's former bf16 box has been multiplied
-            const uint8_t* const src = sm + (uint32_t)s * CB_A32;
-            uint8_t* const dst = sm + 2 * CB_A32 + (uint32_t)s * CB_ABF;
+            if (!mbar_wait(a_full(sa), pa)) return false;
+            if (it >= 2 && !mbar_wait(a_empty(s), ((uint32_t)(it >> 1) & 1u) ^ 1u)) return false;      // the slot's former bf16 box has been multiplied
+            const uint8_t* const src = sm + (uint32_t)sa * CB_A32;
+            uint8_t* const dst = sm + abf0 + (uint32_t)s * CB_ABF;
 #pragma unroll
             for (int i = 0; i < 3; ++i) {
                 const int item = cw + 8 * i;                                   // 6 groups of 32 pixels x 4 chunks
@@ -103,7 +136,11 @@ conv3x3_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");       // generic writes -> visible to the MMA's reads
             __syncwarp();
-            if (lane == 0) mbar_arrive(a_conv(s));
+            if (lane == 0) {
+                mbar_arrive(a_conv(s));
+                if (it + NA < ncb) mbar_arrive(a_free(sa));                    // only where the producer waits for it
+            }
+            if (++sa == NA) { sa = 0; pa ^= 1u; }
         }
         return true;
     };
@@ -112,12 +149,14 @@ conv3x3_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     if (warp == 0) {
         if (elect_one()) {
             bool ok = true;
+            int s = 0;
+            uint32_t ph = 0;
             for (int it = 0; it < ncb; ++it) {
-                const int s = it & 1;
-                if (it >= 2) ok = mbar_wait(a_conv(s), ((uint32_t)(it >> 1) & 1u) ^ 1u);   // the slot's former fp32 box has been rounded
+                if (it >= NA) ok = mbar_wait(a_free(s), ph ^ 1u);
                 if (!ok) break;
                 mbar_expect_tx(a_full(s), CB_PIX * 128u);
                 tma_load_3d(sbase + (uint32_t)s * CB_A32, &tmA, (cb0 + it) * 32, ow0 - 1, oh0 - 1, a_full(s));
+                if (++s == NA) { s = 0; ph ^= 1u; }
             }
             if (!ok) {
                 atomicExch(&g_device_status, (int)NNV_ERR_TIMEOUT);
@@ -125,7 +164,7 @@ conv3x3_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             }
         }
         __syncwarp();
-        if (splits > 1) cluster_wait();
+        if constexpr (SPLIT) cluster_wait();
     } else if (warp == 7) {
         if (elect_one()) {
             bool ok = true;
@@ -145,21 +184,24 @@ conv3x3_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             }
         }
         __syncwarp();
-        if (splits > 1) cluster_wait();
-    } else if (warp == 1) {
-        if (elect_one()) {
+        if constexpr (SPLIT) cluster_wait();
+    } else if (warp == 1 || warp == 6) {
+        const int iss = warp == 1 ? 0 : 1;
+        if (iss < g.issuers && elect_one()) {
             // instruction descriptor: fp32 accumulate, bf16 operands, both K-major, N = BN, M = 128
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | (8u << 24);
             constexpr uint32_t lbo_a = CB_PIX * 16u;
             bool ok = true;
-            int sb = 0, refill_b = 3 * ncb - NB;              // releases that the producer waits for
-            uint32_t pb = 0;
+            const uint32_t acc = tmem_base + (uint32_t)(iss * BN);
+            int sb = 0, stage = 0;                            // filter rows are stages; with two issuers, this one's are the even or the odd ones
+            uint32_t pb = 0, more = 0;                        // 0: the accumulator's first MMA overwrites it
             for (int it = 0; it < ncb && ok; ++it) {
                 const int sa = it & 1;
                 ok = mbar_wait(a_conv(sa), (uint32_t)(it >> 1) & 1u);
                 if (!ok) break;
-                const uint32_t a = sbase + 2 * CB_A32 + (uint32_t)sa * CB_ABF;
-                for (int r = 0; r < 3; ++r) {
+                const uint32_t a = sbase + abf0 + (uint32_t)sa * CB_ABF;
+                for (int r = 0; r < 3; ++r, ++stage, sb = sb + 1 == NB ? 0 : sb + 1, pb ^= sb == 0 ? 1u : 0u) {
+                    if (g.issuers == 2 && (stage & 1) != iss) continue;
                     ok = mbar_wait(b_full(sb), pb);
                     if (!ok) break;
                     tc_fence_after();
@@ -168,11 +210,11 @@ conv3x3_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                     for (int s = 0; s < 3; ++s)
 #pragma unroll
                         for (int kk = 0; kk < 2; ++kk)
-                            umma<true>(tmem_base, make_smem_desc_plain(a + (uint32_t)(r * 10 + s) * 16u + kk * 2u * lbo_a, lbo_a, 160),
+                            umma<true>(acc, make_smem_desc_plain(a + (uint32_t)(r * 10 + s) * 16u + kk * 2u * lbo_a, lbo_a, 160),
                                        make_smem_desc64(b + (uint32_t)s * BN * 64u) + (uint64_t)(kk * 2), idesc,
-                                       (it | r | s | kk) ? 1u : 0u);
-                    if (refill_b-- > 0) umma_commit(b_empty(sb));
-                    if (++sb == NB) { sb = 0; pb ^= 1u; }
+                                       (s | kk) ? 1u : more);
+                    more = 1u;
+                    if (stage + NB < 3 * ncb) umma_commit(b_empty(sb));   // only where the producer waits for it
                 }
                 if (ok && it + 2 < ncb) umma_commit(a_empty(sa));
             }
@@ -180,123 +222,124 @@ conv3x3_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             else atomicExch(&g_device_status, (int)NNV_ERR_TIMEOUT);
         }
         __syncwarp();
-        if (splits > 1) cluster_wait();
-    } else if (warp == 6) {
-        if (splits > 1) cluster_wait();
-    } else if (warp >= 8) {
-        if (!convert_boxes(warp - 4) && lane == 0) atomicExch(&g_device_status, (int)NNV_ERR_TIMEOUT);
-        __syncwarp();
-        if (splits > 1) cluster_wait();
+        if constexpr (SPLIT) cluster_wait();
     } else {
-        // Warps 2-5: conversion, then the write-out (the indices and the bias before the wait for the accumulator).
-        const int quarter = warp & 3, q0 = quarter * 32, t = (int)threadIdx.x - 64;
+        // Warps 2-5 and 8-11: conversion, then the write-out.  The TMEM lanes a warp may read are those of its number modulo four, so
+        // each quarter of the tile's rows (4 image rows x 8 pixels) has two warps, which take the 16-column chunks in turn.
         const float bias = (g.bias && t < BN && n0 + t < g.K) ? __ldg(g.bias + n0 + t) : 0.f;
-        const float hi = g.act == 2 ? 6.f : INFINITY;
         auto act4 = [&](float4& v) {
             if (g.act) {
+                const float hi = g.act == 2 ? 6.f : INFINITY;
                 v.x = fminf(fmaxf(v.x, 0.f), hi); v.y = fminf(fmaxf(v.y, 0.f), hi);
                 v.z = fminf(fmaxf(v.z, 0.f), hi); v.w = fminf(fmaxf(v.w, 0.f), hi);
             }
         };
+        const uint32_t tacc = tmem_base + ((uint32_t)q0 << 16);
+        const bool two = g.issuers == 2;
+        // 16 columns of this lane's row, the issuers' accumulators added in order
         auto acc16 = [&](int c0, float (&v)[16]) {
-            uint32_t r[16];
-            tmem_ld16_nowait(tmem_base + ((uint32_t)q0 << 16) + (uint32_t)c0, r);
+            uint32_t r[16], q[16];
+            tmem_ld16_nowait(tacc + (uint32_t)c0, r);
+            tmem_ld16_nowait(tacc + (uint32_t)(two ? BN + c0 : c0), q);
             tmem_wait_ld();
 #pragma unroll
-            for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+            for (int i = 0; i < 16; ++i) v[i] = two ? __uint_as_float(r[i]) + __uint_as_float(q[i]) : __uint_as_float(r[i]);
         };
-        bool ok = convert_boxes(warp - 2);
-        if (t < BN) s_bias[t] = bias;
-        asm volatile("barrier.sync 1, 128;" ::: "memory");
-        const bool vec = (g.K & 3) == 0 && (reinterpret_cast<uintptr_t>(g.D) & 15) == 0 && (!g.addend || (reinterpret_cast<uintptr_t>(g.addend) & 15) == 0);
+        bool ok = convert_boxes(cw);
+        if (t < BN) asm volatile("st.shared.f32 [%0], %1;" ::"r"(sbias + 4u * (uint32_t)t), "f"(bias) : "memory");
+        asm volatile("barrier.sync 1, 256;" ::: "memory");
         auto wait_acc = [&]() {
             ok = ok && mbar_wait(tmem_full_bar, 0);
             tc_fence_after();
             if (!ok && lane == 0) atomicExch(&g_device_status, (int)NNV_ERR_TIMEOUT);
             ok = __all_sync(0xffffffffu, ok);
         };
-        if (splits == 1) {
-            // MMA row = 8 * (patch row) + (patch column): a warp holds 4 image rows x 8 pixels
+        if (!SPLIT && vec) {
+            // Per 16 columns: TMEM -> registers (lane = one pixel), + bias -> a sub-tile in shared memory (both A rings are idle by then)
+            // -> (+ residual, activation) -> memory, an image row of 8 pixels x 64 bytes at a time.
+            auto fetch_addend = [&](int c0, float4 (&a)[4]) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    a[i] = g.addend && c0 < BN && i < rows_live && n0 + c0 + 4 * (lane & 3) < g.K
+                               ? __ldg(reinterpret_cast<const float4*>(g.addend + (out - g.D) + (c0 - half * 16) + (long long)i * row_pitch))
+                               : make_float4(0.f, 0.f, 0.f, 0.f);
+            };
+            float4 aa[4];
+            fetch_addend(half * 16, aa);
+            wait_acc();
+            if (ok && half * 16 < BN) {
+#pragma unroll 1
+                for (int c0 = half * 16; c0 < BN; c0 += 32) {
+                    float v[16];
+                    acc16(c0, v);
+                    const uint32_t swz = (uint32_t)((lane >> 1) & 3) << 4;
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        const float4 bb = lds128(sbias + (uint32_t)(c0 + 4 * c) * 4u);
+                        sts128(sub + (uint32_t)lane * 64u + (((uint32_t)c << 4) ^ swz),
+                               make_float4(v[c * 4] + bb.x, v[c * 4 + 1] + bb.y, v[c * 4 + 2] + bb.z, v[c * 4 + 3] + bb.w));
+                    }
+                    __syncwarp();
+                    const int r1 = lane >> 2;
+                    const uint32_t src = sub + (uint32_t)r1 * 64u + (uint32_t)(((lane & 3) ^ ((r1 >> 1) & 3)) << 4);
+                    float4 q[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        q[i] = lds128(src + (uint32_t)i * 512u);
+                        if (g.addend) { q[i].x += aa[i].x; q[i].y += aa[i].y; q[i].z += aa[i].z; q[i].w += aa[i].w; }
+                        act4(q[i]);
+                    }
+                    float* const at = out + (c0 - half * 16);
+                    if (n0 + c0 + 4 * (lane & 3) < g.K) {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            if (i < rows_live) *reinterpret_cast<float4*>(at + (long long)i * row_pitch) = q[i];
+                    }
+                    if (g.addend) fetch_addend(c0 + 32, aa);
+                    __syncwarp();                             // the sub-tile is free again
+                }
+            }
+        } else if (!SPLIT) {
             const int oh = oh0 + quarter * 4 + (lane >> 3), ow = ow0 + (lane & 7);
-            const bool inside = oh < g.H && ow < g.W;
             const long long off = ((long long)oh * g.W + ow) * g.K + n0;
-            const int CW = g.tma_out ? g.tma_out : 16;
-            const uint32_t swz = CW == 32 ? (uint32_t)(lane & 7) : (uint32_t)((lane >> 1) & 3);
-            const uint32_t sub = 32u * (uint32_t)CW * 4u;
-            uint8_t* row0 = sm + (uint32_t)quarter * sub + (uint32_t)lane * (uint32_t)CW * 4u;    // both A rings are idle by then
             wait_acc();
             if (ok) {
 #pragma unroll 1
-                for (int c0 = 0; c0 < BN; c0 += 16) {
+                for (int c0 = half * 16; c0 < BN; c0 += 32) {
                     float v[16];
-                    float4 aa[4];
-                    if (g.addend && vec) {
-#pragma unroll
-                        for (int c = 0; c < 4; ++c)
-                            aa[c] = inside && n0 + c0 + 4 * c < g.K ? __ldg(reinterpret_cast<const float4*>(g.addend + off + c0 + 4 * c)) : make_float4(0.f, 0.f, 0.f, 0.f);
-                    }
                     acc16(c0, v);
-                    const uint32_t h = CW == 32 ? (uint32_t)(c0 >> 2) & 4u : 0u;
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        const float4 bb = *reinterpret_cast<const float4*>(s_bias + c0 + c * 4);
-                        float4 o = make_float4(v[c * 4] + bb.x, v[c * 4 + 1] + bb.y, v[c * 4 + 2] + bb.z, v[c * 4 + 3] + bb.w);
-                        if (g.addend && vec) { o.x += aa[c].x; o.y += aa[c].y; o.z += aa[c].z; o.w += aa[c].w; }
-                        if (vec) act4(o);
-                        if (g.tma_out) {
-                            *reinterpret_cast<float4*>(row0 + (((h + (uint32_t)c) ^ swz) << 4)) = o;
-                        } else if (inside) {
-                            const float vv[4] = {o.x, o.y, o.z, o.w};
-                            for (int j = 0; j < 4 && n0 + c0 + 4 * c + j < g.K; ++j) {
-                                const long long at = off + c0 + 4 * c + j;
-                                g.D[at] = vec ? vv[j] : act_fn(g.addend ? vv[j] + __ldg(g.addend + at) : vv[j], g.act);
-                            }
+                    for (int j = 0; j < 16; ++j)
+                        if (oh < g.H && ow < g.W && n0 + c0 + j < g.K) {
+                            float bb;
+                            asm volatile("ld.shared.f32 %0, [%1];" : "=f"(bb) : "r"(sbias + (uint32_t)(c0 + j) * 4u) : "memory");
+                            const float o = v[j] + bb;
+                            g.D[off + c0 + j] = act_fn(g.addend ? o + __ldg(g.addend + off + c0 + j) : o, g.act);
                         }
-                    }
-                    if (g.tma_out && (CW == 16 || h)) {       // the sub-tile is complete
-                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                        __syncwarp();
-                        if (lane == 0 && oh0 + quarter * 4 < g.H && n0 + c0 + 16 - CW < g.K) {
-                            tma_store_3d(&tmD, smem_u32(row0), n0 + c0 + 16 - CW, ow0, oh0 + quarter * 4);
-                            tma_store_commit();
-                        }
-                        row0 += 4u * sub;
-                    }
                 }
-                if (g.tma_out && lane == 0) tma_store_wait_read();
             }
         } else {
-            uint8_t* const prow = sm + (uint32_t)(q0 + lane) * (uint32_t)BN * 4u;
-            int pos = (q0 + lane) % nch;
-            const int a0 = max(q0, lane * rows_per), a1 = min(q0 + 32, (lane + 1) * rows_per);
-            const bool sends = lane < splits && a1 > a0;
-            uint32_t push_dst = 0, push_bar = 0;
-            if (sends) {
-                push_dst = cluster_addr(sbase + g.recv_off + (uint32_t)((r0 + a0 - lane * rows_per) * BN) * 4u, lane);
-                push_bar = cluster_addr(recv_bar, lane);
-            }
-            const int qstep = 128 / nch, rstep = 128 - qstep * nch;
-            int rr = t / nch, cc = t - rr * nch, rot = (r0 + rr) % nch;
-            const int rot_step = qstep % nch;
-            const uint8_t* const recv = sm + g.recv_off;
-            const uint32_t part_stride = (uint32_t)(rows_per * BN) * 4u;
+            const uint32_t prow = sbase + (uint32_t)(q0 + lane) * (uint32_t)BN * 4u, recv = sbase + g.recv_off, part_stride = (uint32_t)(rows_per * BN) * 4u;
             cluster_wait();                                   // every CTA's barriers are initialised
             wait_acc();
             if (ok) {
 #pragma unroll 1
-                for (int c0 = 0; c0 < BN; c0 += 16) {
+                for (int c0 = half * 16; c0 < BN; c0 += 32) {
                     float v[16];
                     acc16(c0, v);
+                    int pos = rot0 + c0 / 4;
+                    if (pos >= nch) pos -= nch;
 #pragma unroll
                     for (int j = 0; j < 16; j += 4) {
-                        *reinterpret_cast<float4*>(prow + pos * 16) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+                        sts128(prow + (uint32_t)pos * 16u, make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]));
                         pos = pos + 1 == nch ? 0 : pos + 1;
                     }
                 }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> visible to the bulk copies
-                __syncwarp();
-                if (sends) bulk_push(push_dst, sbase + (uint32_t)(a0 * BN) * 4u, (uint32_t)((a1 - a0) * BN) * 4u, push_bar);
             }
+            __syncwarp();
+            asm volatile("barrier.sync %0, 64;" ::"r"(2 + quarter) : "memory");   // both warps' columns of these rows are parked
+            if (ok && push_bytes) bulk_push(push_dst, push_src, push_bytes, push_bar);
             int total = rows_per * nch;
             if (!mbar_wait(recv_bar, 0)) {
                 if (lane == 0) atomicExch(&g_device_status, (int)NNV_ERR_TIMEOUT);
@@ -308,13 +351,13 @@ conv3x3_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             auto reduce = [&](auto nsplits) {
                 constexpr int NS = decltype(nsplits)::value;
 #pragma unroll 1
-                for (int idx = t; idx < total; idx += 128) {
+                for (int idx = t; idx < total; idx += 256) {
                     const int p = cc + rot >= nch ? cc + rot - nch : cc + rot;
-                    const uint8_t* src = recv + (uint32_t)(rr * BN) * 4u + (uint32_t)p * 16u;
+                    const uint32_t src = recv + (uint32_t)(rr * BN) * 4u + (uint32_t)p * 16u;
                     float4 v[NS];
 #pragma unroll
-                    for (int rk = 0; rk < NS; ++rk) v[rk] = *reinterpret_cast<const float4*>(src + rk * part_stride);
-                    float4 o = *reinterpret_cast<const float4*>(s_bias + cc * 4);
+                    for (int rk = 0; rk < NS; ++rk) v[rk] = lds128(src + (uint32_t)rk * part_stride);
+                    float4 o = lds128(sbias + (uint32_t)cc * 16u);
                     float4 a = v[0];
 #pragma unroll
                     for (int rk = 1; rk < NS; ++rk) { a.x += v[rk].x; a.y += v[rk].y; a.z += v[rk].z; a.w += v[rk].w; }
@@ -346,7 +389,7 @@ conv3x3_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         }
     }
     __syncwarp();
-    if (splits > 1) {
+    if constexpr (SPLIT) {
         if (!cluster_arrived) cluster_arrive_relaxed();
         cluster_wait();                                       // nobody leaves while its rows may still be on their way
     }

@@ -1094,7 +1094,6 @@ nnv_status_t encode_halo_operand(CUtensorMap* map, const void* base, int C, int 
 // where more CTAs fit than have columns, each of three clusters may hold columns on some SMs and wait for them on another.
 // (A CTA without a cluster waits for nobody else once it has its columns and needs no such rule.)
 constexpr size_t tmem_share_bytes(int cols) { return (size_t)228 * 1024 * cols / 512 - 1024; }
-static_assert(CB_RINGS_A >= tmem_share_bytes(128), "the BF16 3x3 kernel's rings alone are the share of its columns");
 
 // Tiling of conv3x3_tc_kernel for one layer.
 struct ConvTiling { int MT, BN, splits, na, nb, tmem_cols; size_t smem; };
@@ -1341,7 +1340,8 @@ nnv_status_t gemm_tc_init() {
                 cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
             }
         cudaFuncSetAttribute(conv3x3_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
-        cudaFuncSetAttribute(conv3x3_bf16_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
+        cudaFuncSetAttribute(conv3x3_bf16_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
+        cudaFuncSetAttribute(conv3x3_bf16_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
         cudaFuncSetAttribute(gemm_sp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
         cudaFuncSetAttribute(conv3x3_tc_persistent_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
         cudaFuncSetAttribute(wino_f2_fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
@@ -1402,7 +1402,7 @@ static ConvBTiling pick_conv_bf16_tiling(int C, int H, int W, int N) {
 
 static nnv_status_t launch_conv3x3_bf16(const GemmArgs& a, int BN, int splits, cudaStream_t st) {
     ConvBDev g{};
-    CUtensorMap tmA, tmB, tmD;
+    CUtensorMap tmA, tmB;
     const int C = a.ic.C, H = a.ic.H, W = a.ic.W;
     NNV_REQUIRE(a.ldd == a.N, NNV_ERR_INVALID_ARG, "the 3x3 kernel writes a dense NHWC output");
     NNV_TRY(encode_halo_operand(&tmA, a.A, C, H, W, 18, 10));
@@ -1425,25 +1425,30 @@ static nnv_status_t launch_conv3x3_bf16(const GemmArgs& a, int BN, int splits, c
     g.BN = BN; g.act = a.act; g.splits = splits;
     g.cblk = C / 32; g.tiles_w = ceil_div(W, 8);
     g.tmem_cols = 32;
-    while (g.tmem_cols < BN) g.tmem_cols *= 2;
-    g.tma_out = 0;
-    if (splits == 1 && (a.N % 4) == 0 && (reinterpret_cast<uintptr_t>(a.D) & 15) == 0 && (!a.addend || (reinterpret_cast<uintptr_t>(a.addend) & 15) == 0)) {
-        g.tma_out = (BN % 32) == 0 ? 32 : 16;
-        NNV_TRY(encode_conv_output(&tmD, a.D, a.N, H, W, g.tma_out));
-    } else {
-        tmD = tmA;
-    }
+    while (g.tmem_cols < 2 * BN) g.tmem_cols *= 2;
     // two channel blocks of weights in flight where they fit (three filter rows each)
     const size_t recv = splits > 1 ? (size_t)128 * BN * 4 : 0;
-    g.b_off = (uint32_t)align_up(CB_RINGS_A, 1024);
-    g.nb = std::min({6, 3 * ceil_div(g.cblk, splits), (int)((225u * 1024u - g.b_off - CB_BAR_BYTES - 256 - recv) / ((size_t)BN * 192))});
+    // boxes in flight: as many as the channel blocks, where six weight boxes still fit (and at least two, whose room the write-out uses)
+    const int ncb = ceil_div(g.cblk, splits);
+    g.na = std::max(2, std::min(CB_MAX_NA, ncb));
+    auto b_off = [&](int na) { return (uint32_t)align_up((size_t)na * CB_A32 + 2 * CB_ABF, 1024); };
+    while (g.na > 2 && b_off(g.na) + CB_BAR_BYTES + 256 + recv + (size_t)6 * BN * 192 > 225u * 1024u) --g.na;
+    g.b_off = b_off(g.na);
+    const int stages = 3 * ncb;
+    g.nb = std::min({6, stages, (int)((225u * 1024u - g.b_off - CB_BAR_BYTES - 256 - recv) / ((size_t)BN * 192))});
+    // (two issuers take alternate filter rows: a ring that is refilled has an even depth, as in gemm_tc_kernel)
+    g.issuers = 2;
+    if (stages > g.nb && (g.nb & 1)) {
+        if (g.nb > 1) --g.nb;
+        else g.issuers = 1;
+    }
     g.bar_off = (uint32_t)align_up(g.b_off + (size_t)g.nb * BN * 192, 16);
     g.recv_off = (uint32_t)align_up(g.bar_off + CB_BAR_BYTES, 128);
-    const size_t smem = (size_t)1024 + g.recv_off + recv;
+    const size_t smem = std::max((size_t)1024 + g.recv_off + recv, splits > 1 ? tmem_share_bytes(g.tmem_cols) : 0);
     NNV_REQUIRE(g.nb >= 1 && smem <= 226u * 1024u, NNV_ERR_UNSUPPORTED, "3x3 tiling does not fit shared memory");
     const dim3 grid(ceil_div(H, 16) * g.tiles_w, ceil_div(a.N, BN), splits);
     NNV_REQUIRE(grid.y <= 65535, NNV_ERR_UNSUPPORTED, "convolution grid too large");
-    NNV_CUDA(launch_pdl_cluster(conv3x3_bf16_kernel, grid, dim3(CB_THREADS), smem, st, splits, tmA, tmB, tmD, g));
+    NNV_CUDA(launch_pdl_cluster(splits > 1 ? conv3x3_bf16_kernel<true> : conv3x3_bf16_kernel<false>, grid, dim3(CB_THREADS), smem, st, splits, tmA, tmB, g));
     return NNV_OK;
 }
 
