@@ -69,7 +69,8 @@ nnv_status_t do_exec(const nnv_plan& p, int layer, int v, int math, const void* 
         // F(2,3) runs as one TF32 / BF16 pass; F(4,3) and F(6,3) amplify operand rounding too much for
         // that, so their tile GEMM multiplies fp32 operands with the compensated bf16 scheme.
         if (m != 2) a.mode = GEMM_X3;
-        NNV_TRY(launch_wino_input(m, bf16, x, V, L.C, g.Cp, L.H, L.W, L.pad, TH, TW, st));
+        a.split_a = m != 2 && (g.Cp % 32) == 0;
+        NNV_TRY(launch_wino_input(m, bf16, a.split_a, x, V, L.C, g.Cp, L.H, L.W, L.pad, TH, TW, st));
         a.A = V; a.B = d_wt; a.D = Mt;
         a.M = T; a.Kd = g.Cp; a.batch = a2;
         a.lda = g.Cp; a.ldb = g.Cp; a.ldd = L.K;
@@ -203,7 +204,7 @@ nnv_status_t nnv_wino_input_transform(const nnv_plan_t* p, int32_t layer, int32_
     NNV_REQUIRE(aligned256(d_in) && aligned256(d_V), NNV_ERR_INVALID_ARG, "device pointers must be 256-byte aligned");
     const nnv_layer_desc_t& L = p->layers[layer];
     const LayerGeom& g = p->geom[layer];
-    return launch_wino_input(m, math == NNV_MATH_BF16, (const float*)d_in, d_V, L.C, g.Cp, L.H, L.W, L.pad, ceil_div(g.OH, m),
+    return launch_wino_input(m, math == NNV_MATH_BF16, false, (const float*)d_in, d_V, L.C, g.Cp, L.H, L.W, L.pad, ceil_div(g.OH, m),
                              ceil_div(g.OW, m), (cudaStream_t)stream);
 }
 

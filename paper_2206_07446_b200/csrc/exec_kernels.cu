@@ -181,7 +181,9 @@ template <> struct WinoBA<6> {
 
 // One thread per (tile, padded channel); channel is the fastest index so that every load and
 // store of a warp covers 32 consecutive channels.  V[(xi*A+nu)][t][cp].
-template <int M_, typename OutT>
+// SPLIT (Cp % 32 == 0): a block of 32 words holds its 32 elements as bf16 hi = rn(v), then lo = rn(v - hi), the operand of the
+// compensated GEMM; neighbouring lanes swap halves, so that each stores one word.
+template <int M_, typename OutT, bool SPLIT>
 __global__ void __launch_bounds__(128)
 wino_input_kernel(const float* __restrict__ x, OutT* __restrict__ V, int C, int Cp, int H, int W, int pad, int TH,
                   int TW) {
@@ -214,7 +216,8 @@ wino_input_kernel(const float* __restrict__ x, OutT* __restrict__ V, int C, int 
                 if (WinoBA<M_>::bt(i, l) != 0.f) s += WinoBA<M_>::bt(i, l) * d[l][j];
             tmp[i][j] = s;
         }
-    OutT* out = V + (long long)t * Cp + c;
+    const int word = SPLIT ? (c & ~31) + ((c & 1) << 4) + ((c & 31) >> 1) : c;
+    OutT* out = V + (long long)t * Cp + word;
 #pragma unroll
     for (int i = 0; i < A; ++i)
 #pragma unroll
@@ -223,18 +226,27 @@ wino_input_kernel(const float* __restrict__ x, OutT* __restrict__ V, int C, int 
 #pragma unroll
             for (int l = 0; l < A; ++l)
                 if (WinoBA<M_>::bt(j, l) != 0.f) s += tmp[i][l] * WinoBA<M_>::bt(j, l);
-            out[(long long)(i * A + j) * T * Cp] = to_out<OutT>((sizeof(OutT) == 4 && M_ == 2) ? round_tf32(s) : s);
+            if constexpr (SPLIT) {
+                const __nv_bfloat16 hi = __float2bfloat16_rn(s), lo = __float2bfloat16_rn(s - __bfloat162float(hi));
+                const uint32_t own = (uint32_t)__bfloat16_as_ushort(hi) | (uint32_t)__bfloat16_as_ushort(lo) << 16;
+                const uint32_t other = __shfl_xor_sync(0xffffffffu, own, 1);
+                out[(long long)(i * A + j) * T * Cp] = __uint_as_float((c & 1) ? __byte_perm(other, own, 0x7632) : __byte_perm(own, other, 0x5410));
+            } else {
+                out[(long long)(i * A + j) * T * Cp] = to_out<OutT>((sizeof(OutT) == 4 && M_ == 2) ? round_tf32(s) : s);
+            }
         }
 }
 
-nnv_status_t launch_wino_input(int m, bool bf16, const float* x, void* V, int C, int Cp, int H, int W, int pad,
+nnv_status_t launch_wino_input(int m, bool bf16, bool split, const float* x, void* V, int C, int Cp, int H, int W, int pad,
                                int TH, int TW, cudaStream_t st) {
     const long long n = (long long)TH * TW * Cp;
     const unsigned grid = (unsigned)((n + 127) / 128);
 #define NNV_WI(MM)                                                                                              \
-    if (bf16) NNV_LAUNCH((wino_input_kernel<MM, __nv_bfloat16>), grid, 128, 0, st, x, (__nv_bfloat16*)V, C, Cp, H, W, pad, TH, TW); \
-    else NNV_LAUNCH((wino_input_kernel<MM, float>), grid, 128, 0, st, x, (float*)V, C, Cp, H, W, pad, TH, TW);
-    if (m == 2) { NNV_WI(2) } else if (m == 4) { NNV_WI(4) } else if (m == 6) { NNV_WI(6) }
+    if (bf16) NNV_LAUNCH((wino_input_kernel<MM, __nv_bfloat16, false>), grid, 128, 0, st, x, (__nv_bfloat16*)V, C, Cp, H, W, pad, TH, TW); \
+    else NNV_LAUNCH((wino_input_kernel<MM, float, false>), grid, 128, 0, st, x, (float*)V, C, Cp, H, W, pad, TH, TW);
+    if (split && m == 4) NNV_LAUNCH((wino_input_kernel<4, float, true>), grid, 128, 0, st, x, (float*)V, C, Cp, H, W, pad, TH, TW);
+    else if (split && m == 6) NNV_LAUNCH((wino_input_kernel<6, float, true>), grid, 128, 0, st, x, (float*)V, C, Cp, H, W, pad, TH, TW);
+    else if (m == 2) { NNV_WI(2) } else if (m == 4) { NNV_WI(4) } else if (m == 6) { NNV_WI(6) }
     else return fail(NNV_ERR_INVALID_ARG, "no Winograd tile size %d", m);
 #undef NNV_WI
     NNV_CUDA(cudaGetLastError());

@@ -78,7 +78,7 @@ constexpr int A_STAGE_BYTES = BM * BK_BYTES;
 constexpr int GEMM_THREADS = 192;
 // gemm_tc_kernel: a second MMA issuer and a second producer; splitting both operands (mode 2), gathering (modes 4 - 7) and rounding
 // (mode 8) take four more warps
-constexpr int gemm_tc_threads(int mode) { return mode == 2 || mode >= 4 ? 384 : 256; }
+constexpr int gemm_tc_threads(int mode) { return mode == 2 || mode >= 4 ? 384 : 256; }   // (3: the write-out's warps convert)
 constexpr int GATHER_WARPS = 8;
 constexpr int GEMM_BAR_BYTES = 8 * (3 * 8 + 6) + 512;         // barriers, TMEM address, bias of the tile's columns
 constexpr uint32_t WAIT_LIMIT = 1u << 20;
@@ -334,8 +334,13 @@ __device__ __forceinline__ void convert_chunk(const uint8_t* src_tile, uint8_t* 
 // block of 98 rows) behind each load.  us, gathered / this / truncated: 64 -> 64 3x3 @14 4.2 / 3.9 / 3.6, 160 -> 160 @14 6.6 / 5.4 / 4.3,
 // 256 -> 256 @7 6.0 / 4.8 / 4.2, 320 -> 320 @10 8.4 / 6.4 / 5.1.
 constexpr int ROUNDED = 8;
+// MODE 9: mode 2 on an A that is split already: a row's block of 32 words holds its elements' bf16 hi parts, then their lo parts (the
+// Winograd input transform writes it so where the channels come in whole blocks), and only B's rows are split here, a third of the work
+// or less.  The same products in the same order as mode 2.
+constexpr int SPLIT_A = 9;
+__host__ __device__ constexpr bool x3_mode(int mode) { return mode == 2 || mode == SPLIT_A; }
 __host__ __device__ constexpr bool gather_mode(int mode) { return mode >= 4 && mode <= 7; }
-__host__ __device__ constexpr bool converting_mode(int mode) { return mode == 2 || mode == 3 || mode == ROUNDED; }
+__host__ __device__ constexpr bool converting_mode(int mode) { return x3_mode(mode) || mode == 3 || mode == ROUNDED; }
 __host__ __device__ constexpr bool bf16_mode(int mode) { return mode == 1 || mode == 5 || mode == 7; }   // both operands staged as bf16
 template <int MODE> struct ModeTraits {
     static constexpr int BKE = bf16_mode(MODE) ? 64 : 32;      // K elements per stage
@@ -353,11 +358,14 @@ __host__ __device__ constexpr uint32_t stage_bytes_of(int BN, int rows) {
     const uint32_t a = a_stage_of(rows), b = (uint32_t)(BN * BK_BYTES);
     if (MODE == 3) return (a + (uint32_t)(pad8(rows) * 64) + b / 2 + 1023u) & ~1023u;
     if (MODE == 2) return (a + b + (uint32_t)(pad8(rows) * 128) + b + 1023u) & ~1023u;
+    if (MODE == SPLIT_A) return (a + 2 * b + 1023u) & ~1023u;
     return a + b;
 }
 
+// (Four CTAs to an SM, 64 registers a thread, for unsplit launches without conversion, whose grids may be many waves of short K loops:
+// 17 -> 24 F(2,3) @180 BF16 20.3 us with three, 18.5 with four.)
 template <int MODE, bool SPLIT>
-__global__ void __launch_bounds__(gemm_tc_threads(MODE), MODE == 2 || MODE >= 4 ? 2 : 3)
+__global__ void __launch_bounds__(gemm_tc_threads(MODE), MODE == 2 || MODE >= 4 ? 2 : MODE == 3 || SPLIT ? 3 : 4)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmAdd, const GemmDev g) {
     extern __shared__ uint8_t smem_raw[];
@@ -414,7 +422,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(full_bar(s), gather_mode(MODE) ? GATHER_WARPS + 1 : 2);
             mbar_init(empty_bar(s), 1);
-            mbar_init(conv_bar(s), MODE == 2 ? 8 : 4);
+            mbar_init(conv_bar(s), x3_mode(MODE) ? 8 : 4);
         }
         mbar_init(tmem_full_bar, (uint32_t)g.issuers);
         mbar_init(addend_bar, 1);
@@ -554,7 +562,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             if (MODE == ROUNDED && (g.issuers == 2 ? it & 1 : 0) != cw >> 2) continue;
             if (!mbar_wait(full_bar(s), ph)) return false;
             uint8_t* const st = sm0 + s * stage_bytes;
-            uint8_t* const cv = st + a_stage + (MODE == 2 ? b_stage_bytes : 0u);      // converted tiles: A hi, A lo, B hi, B lo
+            uint8_t* const cv = st + a_stage + (x3_mode(MODE) ? b_stage_bytes : 0u);      // converted tiles: A hi, A lo, B hi, B lo
             if constexpr (MODE == 3) {
                 const int r = cw * 32 + lane;                 // a row of A per thread
                 if (r < g.rows) {
@@ -571,6 +579,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                     for (int c = 0; c < 8; ++c)
                         *reinterpret_cast<float4*>(st + r * 128 + ((c ^ (r & 7)) << 4)) =
                             make_float4(round_tf32(v[c].x), round_tf32(v[c].y), round_tf32(v[c].z), round_tf32(v[c].w));
+                }
+            } else if constexpr (MODE == SPLIT_A) {
+                for (int i = cw; i < 4 * gb; i += 8) {
+                    const int r = (i >> 2) * 32 + lane;
+                    if (r < BN) convert_chunk<true>(st + a_stage, cv, cv + b_stage_bytes / 2, r, i & 3, BN);
                 }
             } else {
 #pragma unroll 2
@@ -685,7 +698,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const int step = FOUR && nkb >= 6 && STAGES >= 2 ? 2 : 1;
     auto produce = [&](bool is_a, int first_it) {
         bool ok = true;
-        int s = first_it;                                     // (a ring that two producers share has two slots or more)
+        int s = first_it;                                     // (a ring that two loaders share has two slots or more; a slot's next block is one phase on, whosever it is)
         uint32_t ph = 0;
         const int first = min(nkb, STAGES);
         auto skip = [&]() {                                   // the other warp's block
@@ -721,7 +734,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     if (warp == 0 || warp == 7) {
         if (!(gather_mode(MODE) && warp == 0) && elect_one()) produce(warp == 0, 0);
     } else if (warp >= 8) {
-        if constexpr (MODE == 2 || MODE == ROUNDED) {
+        if constexpr (x3_mode(MODE) || MODE == ROUNDED) {
             if (!convert_stages(warp - 4) && lane == 0) atomicExch(&g_device_status, (int)NNV_ERR_TIMEOUT);
         }
         __syncwarp();
@@ -754,6 +767,18 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                     for (int kk = 0; kk < 2; ++kk) {            // 2 K-steps of 16 bf16 = 2 core matrices each
                         const uint64_t ah = make_smem_desc_plain(a_hi + kk * 2 * lbo_a, lbo_a, 128);
                         const uint64_t al = make_smem_desc_plain(a_lo + kk * 2 * lbo_a, lbo_a, 128);
+                        const uint64_t bh = make_smem_desc_plain(b_hi + kk * 2 * lbo_b, lbo_b, 128);
+                        const uint64_t bl = make_smem_desc_plain(b_lo + kk * 2 * lbo_b, lbo_b, 128);
+                        umma<true>(acc, al, bh, idesc, kk ? 1u : first);   // small terms first
+                        umma<true>(acc, ah, bl, idesc, 1u);
+                        umma<true>(acc, ah, bh, idesc, 1u);
+                    }
+                } else if constexpr (MODE == SPLIT_A) {
+                    const uint32_t b_hi = a_src + a_stage + b_stage_bytes, b_lo = b_hi + b_stage_bytes / 2, lbo_b = (uint32_t)BN * 16u;
+                    const uint64_t adesc = make_smem_desc(a_src);      // a row: 64 bytes of hi, 64 of lo
+#pragma unroll
+                    for (int kk = 0; kk < 2; ++kk) {
+                        const uint64_t ah = adesc + (uint64_t)(kk * 2), al = adesc + (uint64_t)(4 + kk * 2);
                         const uint64_t bh = make_smem_desc_plain(b_hi + kk * 2 * lbo_b, lbo_b, 128);
                         const uint64_t bl = make_smem_desc_plain(b_lo + kk * 2 * lbo_b, lbo_b, 128);
                         umma<true>(acc, al, bh, idesc, kk ? 1u : first);   // small terms first
@@ -1131,7 +1156,7 @@ int cluster_slots(int splits, int occ) {
 }
 
 uint32_t gemm_stage_bytes(int mode, int bn, int rows) {
-    return mode == GEMM_X3 ? stage_bytes_of<2>(bn, rows) : mode == GEMM_BF16_CVT ? stage_bytes_of<3>(bn, rows) : stage_bytes_of<0>(bn, rows);
+    return mode == GEMM_X3 ? stage_bytes_of<2>(bn, rows) : mode == SPLIT_A ? stage_bytes_of<SPLIT_A>(bn, rows) : mode == GEMM_BF16_CVT ? stage_bytes_of<3>(bn, rows) : stage_bytes_of<0>(bn, rows);
 }
 
 // Ring depth: 8 stages when every CTA has an SM to itself (a lone CTA needs that many loads in flight on weights that come
@@ -1140,7 +1165,7 @@ uint32_t gemm_stage_bytes(int mode, int bn, int rows) {
 int gemm_ring(int mode, int bn, int rows, long long ctas, int nkb) {
     const int sb = (int)gemm_stage_bytes(mode, bn, rows);
     // (X3 stages are twice as large: as many as fit one CTA, or two CTAs on an SM)
-    if (mode == GEMM_X3) return std::max(2, std::min({4, (ctas <= 148 ? 200 : 104) * 1024 / sb, nkb}));
+    if (x3_mode(mode)) return std::max(2, std::min({4, (ctas <= 148 ? 200 : 104) * 1024 / sb, nkb}));
     const int most = (ctas <= 148 && 8 * sb <= 200 * 1024) ? 8 : 4;
     return std::max(2, std::min(most, nkb));
 }
@@ -1153,15 +1178,15 @@ int gemm_ring(int mode, int bn, int rows, long long ctas, int nkb) {
 // A gather mode's K block takes the eight warps time for every row, most of it in steps of half a tile; a second CTA on the SM adds
 // `share` of it.  Its tiles may be lower than 128 rows (any height that divides M), which spreads the rows over more SMs.  Fitted the
 // same way over 33 shapes: the chosen tilings are 3 % above the best measured ones on average.
-// X3's K block waits for the split of both operands (by pieces of 32 rows), most of which a second CTA on the SM overlaps: fitted over
-// 68 F(4,3) / F(6,3) layers, 1 % above the best measured tilings (the constants of the other modes: 2.5 %, and 20 % on 512 -> 512
-// F(4,3) @7, 22.9 us against 19.1).
+// X3's K block waits for the split of its operands (by pieces of 32 rows), most of which a second CTA on the SM overlaps: fitted over
+// 106 F(4,3) / F(6,3) layers with A split already, 0.2 % above the best measured tilings on average, and 23 without, 1.3 %.
 // Mode 8's K block waits for the rounding; CTAs that share an SM count by the clusters that fit (clusters of 16 put 128 CTAs on 112
 // places): fitted to 34 layers, 0.6 % above the best measured tilings (the TF32 constants: 5.6 %).
 struct TilingCost { double fixed, block, sm_rate, l2_rate, start, column, shared_column, split, split_word; };
 constexpr TilingCost tiling_cost(int mode) {
     return gather_mode(mode) ? TilingCost{0.87, 0.146, 108e3, 10.9e6, 1.85, 0.0093, 0.0, 0.28, 1.22e-4}
-           : mode == 2       ? TilingCost{1.87, 0.37, 108e3, 4.6e6, 0.80, 0.005, 0.0, 0.73, 1.22e-4}
+           : mode == SPLIT_A ? TilingCost{1.87, 0.434, 28.2e3, 7.4e6, 0.0, 0.0098, 0.0, 1.46, 2.4e-5}
+           : mode == 2       ? TilingCost{1.87, 0.91, 27.2e3, 6.9e6, 0.0, 0.0188, 0.0, 1.47, 0.9e-5}
            : mode == ROUNDED ? TilingCost{1.87, 0.146, 108e3, 10.9e6, 0.80, 0.0093, 0.0, 0.26, 1.22e-4}
            : mode == 1       ? TilingCost{1.87, 0.366, 26.8e3, 2.9e6, 0.0, 0.0022, 0.0, 0.0, 2.32e-3}
            : mode == 3       ? TilingCost{1.87, 0.372, 48.9e3, 5.02e6, 0.0, 0.0065, 0.0, 0.67, 1.53e-4}
@@ -1170,7 +1195,7 @@ constexpr TilingCost tiling_cost(int mode) {
 struct GemmTiling { int BN, splits, rows, waves; };
 GemmTiling search_gemm_tiling(int mode, int M, int N, int batch, int nkb) {
     constexpr struct { double row_us, share; } gather[4] = {{0.0064, 0.36}, {0.0054, 0.60}, {0.0025, 0.81}, {0.0042, 0.40}};   // modes 4 - 7
-    const bool x3 = mode == GEMM_X3;
+    const bool x3 = x3_mode(mode);
     const bool rounded = mode == ROUNDED;
     const TilingCost c = tiling_cost(mode);
     const int least = ceil_div(M, BM);
@@ -1194,7 +1219,7 @@ GemmTiling search_gemm_tiling(int mode, int M, int N, int batch, int nkb) {
                 const int lone = rounded ? cluster_slots(sp, 1) : 148;
                 const double res = (double)std::min<long long>(occ, (ctas + lone - 1) / lone);
                 double kb = std::max({c.block * res, kb_bytes * res / c.sm_rate, kb_bytes * (double)std::min(ctas, slots) / c.l2_rate});
-                if (x3) kb = std::max(kb, (0.40 + 0.07 * (ceil_div(rows, 32) + ceil_div(bn, 32))) * (1 + 0.15 * (res - 1)));
+                if (x3) kb = std::max(kb, (0.40 + 0.07 * ((mode == 2 ? ceil_div(rows, 32) : 0) + ceil_div(bn, 32))) * (1 + 0.15 * (res - 1)));
                 if (gather_mode(mode))
                     kb = std::max(kb, (0.2 + gather[mode & 3].row_us * (0.65 * 64 * ceil_div(rows, 64) + 0.35 * rows)) * (1 + gather[mode & 3].share * (res - 1)));
                 if (rounded) kb = std::max(kb, (0.25 + 0.0005 * rows) * (1 + 0.8 * (res - 1)));
@@ -1301,7 +1326,7 @@ nnv_status_t gemm_shape(int mode, const GemmTiling& tile, int M, int N, int batc
     // land in a CTA that has gone.  So a ring that is refilled has an even depth: an issuer then has its slots for itself.
     // (X3's issuers wait for eight warps that convert the blocks in order: block i - 2 converted means block i - depth is, from
     // two slots on.  Mode 8's two groups of warps take the blocks in turn like the issuers; with one issuer one group takes all.)
-    if (g.issuers == 2 && nkb_cta > g.ring && (mode == GEMM_X3 ? g.ring == 1 : (g.ring & 1) == 1)) {
+    if (g.issuers == 2 && nkb_cta > g.ring && (x3_mode(mode) ? g.ring == 1 : (g.ring & 1) == 1)) {
         if (g.ring > 1 && (g.ring - 1) * sb >= park) --g.ring;
         else g.issuers = 1;
     }
@@ -1321,12 +1346,12 @@ nnv_status_t gemm_shape(int mode, const GemmTiling& tile, int M, int N, int batc
 std::once_flag g_attr_once;
 
 // [kernel mode][K split over a cluster]
-constexpr decltype(&gemm_tc_kernel<0, false>) gemm_kernels[9][2] = {
+constexpr decltype(&gemm_tc_kernel<0, false>) gemm_kernels[10][2] = {
     {gemm_tc_kernel<0, false>, gemm_tc_kernel<0, true>}, {gemm_tc_kernel<1, false>, gemm_tc_kernel<1, true>},
     {gemm_tc_kernel<2, false>, gemm_tc_kernel<2, true>}, {gemm_tc_kernel<3, false>, gemm_tc_kernel<3, true>},
     {gemm_tc_kernel<4, false>, gemm_tc_kernel<4, true>}, {gemm_tc_kernel<5, false>, gemm_tc_kernel<5, true>},
     {gemm_tc_kernel<6, false>, gemm_tc_kernel<6, true>}, {gemm_tc_kernel<7, false>, gemm_tc_kernel<7, true>},
-    {gemm_tc_kernel<ROUNDED, false>, gemm_tc_kernel<ROUNDED, true>}};
+    {gemm_tc_kernel<ROUNDED, false>, gemm_tc_kernel<ROUNDED, true>}, {gemm_tc_kernel<SPLIT_A, false>, gemm_tc_kernel<SPLIT_A, true>}};
 static_assert(GEMM_TF32 == 0 && GEMM_BF16 == 1 && GEMM_X3 == 2 && GEMM_BF16_CVT == 3, "the table's order");
 
 }  // namespace
@@ -1643,7 +1668,7 @@ nnv_status_t launch_gemm_tc(const GemmArgs& a, cudaStream_t st) {
     const bool boxes = a.ic.on && !gather && 4ull * a.ic.C * a.ic.H * a.ic.W < 131072ull &&
                        image_row_boxes(a.ic.H, a.ic.W, a.ic.R, a.ic.S, a.ic.stride, a.ic.pad);
     const int mode = gather ? (a.mode == GEMM_BF16 ? 5 : 4) + ((a.ic.C % 4) == 0 ? 2 : 0)
-                            : boxes && a.mode == GEMM_TF32 ? ROUNDED : a.mode;   // the kernel's
+                            : boxes && a.mode == GEMM_TF32 ? ROUNDED : a.mode == GEMM_X3 && a.split_a ? SPLIT_A : a.mode;   // the kernel's
     const int nkb_all = a.ic.on && !gather ? a.ic.R * a.ic.S * ceil_div(a.ic.C, 32) : ceil_div(a.Kd, bke);
     const GemmTiling tile = pick_gemm_tiling(mode, a.M, a.N, a.batch, nkb_all);
     const Tuning& tn = tuning();

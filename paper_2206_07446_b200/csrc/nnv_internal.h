@@ -275,7 +275,7 @@ bool gather_operand(const nnv_layer_desc_t& L, const LayerGeom& g, int math);   
 nnv_status_t launch_im2col(bool bf16, const float* d_x, void* d_col, int C, int H, int W, int R, int S,
                            int stride, int pad, int OH, int OW, int Qp, cudaStream_t st);
 // Winograd input transform V[alpha^2][T][Cp] = B^T d B per tile and channel.
-nnv_status_t launch_wino_input(int m, bool bf16, const float* d_x, void* d_V, int C, int Cp, int H, int W,
+nnv_status_t launch_wino_input(int m, bool bf16, bool split, const float* d_x, void* d_V, int C, int Cp, int H, int W,
                                int pad, int TH, int TW, cudaStream_t st);
 // Winograd output transform Y = A^T M A with the layer epilogue.
 nnv_status_t launch_wino_output(int m, const float* d_M, float* d_y, const float* d_bias, const float* d_add,
@@ -313,6 +313,7 @@ struct GemmArgs {
     int64_t strideA, strideB, strideD;  // batch strides (elements)
     const float* bias; const float* addend; int act;
     int mode;                         // GEMM_TF32, GEMM_BF16 or GEMM_X3
+    bool split_a;                     // GEMM_X3: A's blocks of 32 words hold 32 bf16 hi parts, then 32 lo parts (Kd % 32 == 0)
     // Implicit im2col: A is the NHWC fp32 activation (C % 4 == 0) read by the TMA in im2col mode;
     // B is the packed weight P[K][Qp] with Kd = Qp; M = OH*OW output pixels.  TF32 mode, batch 1.
     // gather: windows the TMA cannot fetch (any C), gathered by the kernel's warps; TF32 or BF16 mode, Kd = Qp.
