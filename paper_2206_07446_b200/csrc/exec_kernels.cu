@@ -3,6 +3,8 @@
 // Activations are NHWC fp32 (batch 1).
 #include <cuda_bf16.h>
 
+#include <type_traits>
+
 #include "nnv_internal.h"
 
 namespace nnv {
@@ -179,10 +181,34 @@ template <> struct WinoBA<6> {
     }
 };
 
+// Two forms of each data transform.  A thread per (tile, channel) loads A*A values, works through ~2 A*A*A multiply-adds and stores as
+// many: on a layer of a few thousand of them (512 -> 512 @7, F(4,3): 16 blocks) a handful of warps do everything one after the other.
+// So up to WT_BLOCKS blocks the work of a tile is dealt to A warps: a warp for every column of the tile and then, through shared memory,
+// for every row of its transform, a lane a channel.  More blocks than that cost more than they spread.
+// us a layer (three kernels, chained), a thread per tile and channel / a block per tile and 32 channels: F(4,3) 64 -> 64 @56 10.4 / 7.3,
+// 128 -> 128 @28 9.9 / 7.6, 512 -> 512 @7 16.5 / 15.6, F(6,3) 128 -> 128 @28 15.0 / 8.0, 64 -> 128 @112 22.4 / 15.9; F(2,3) 64 -> 64 @200 38 / 59,
+// F(4,3) 64 -> 64 @224 37.7 / 40.2.
+template <int M_> struct WinoTileLimit { static constexpr long long BLOCKS = M_ == 4 ? 3000 : 2000; };
+template <int M_> static bool wino_tile_blocks(int TH, int TW, int channels) {
+    return (long long)TH * TW * ceil_div(channels, 32) <= WinoTileLimit<M_>::BLOCKS;
+}
+
+// What the transform writes.  V[(xi*A+nu)][t][cp]; SPLIT (Cp % 32 == 0): a block of 32 words holds its 32 elements as bf16 hi = rn(v), then
+// lo = rn(v - hi), the operand of the compensated GEMM; neighbouring lanes swap halves, so that each stores one word.
+template <bool SPLIT> __device__ __forceinline__ int wino_word(int c) { return SPLIT ? (c & ~31) + ((c & 1) << 4) + ((c & 31) >> 1) : c; }
+template <int M_, typename OutT, bool SPLIT> __device__ __forceinline__ OutT wino_operand(float s, int c) {
+    if constexpr (SPLIT) {
+        const __nv_bfloat16 hi = __float2bfloat16_rn(s), lo = __float2bfloat16_rn(s - __bfloat162float(hi));
+        const uint32_t own = (uint32_t)__bfloat16_as_ushort(hi) | (uint32_t)__bfloat16_as_ushort(lo) << 16;
+        const uint32_t other = __shfl_xor_sync(0xffffffffu, own, 1);
+        return __uint_as_float((c & 1) ? __byte_perm(other, own, 0x7632) : __byte_perm(own, other, 0x5410));
+    } else {
+        return to_out<OutT>((sizeof(OutT) == 4 && M_ == 2) ? round_tf32(s) : s);
+    }
+}
+
 // One thread per (tile, padded channel); channel is the fastest index so that every load and
-// store of a warp covers 32 consecutive channels.  V[(xi*A+nu)][t][cp].
-// SPLIT (Cp % 32 == 0): a block of 32 words holds its 32 elements as bf16 hi = rn(v), then lo = rn(v - hi), the operand of the
-// compensated GEMM; neighbouring lanes swap halves, so that each stores one word.
+// store of a warp covers 32 consecutive channels: for layers with tiles enough to fill the GPU that way.
 template <int M_, typename OutT, bool SPLIT>
 __global__ void __launch_bounds__(128)
 wino_input_kernel(const float* __restrict__ x, OutT* __restrict__ V, int C, int Cp, int H, int W, int pad, int TH,
@@ -216,8 +242,7 @@ wino_input_kernel(const float* __restrict__ x, OutT* __restrict__ V, int C, int 
                 if (WinoBA<M_>::bt(i, l) != 0.f) s += WinoBA<M_>::bt(i, l) * d[l][j];
             tmp[i][j] = s;
         }
-    const int word = SPLIT ? (c & ~31) + ((c & 1) << 4) + ((c & 31) >> 1) : c;
-    OutT* out = V + (long long)t * Cp + word;
+    OutT* out = V + (long long)t * Cp + wino_word<SPLIT>(c);
 #pragma unroll
     for (int i = 0; i < A; ++i)
 #pragma unroll
@@ -226,30 +251,70 @@ wino_input_kernel(const float* __restrict__ x, OutT* __restrict__ V, int C, int 
 #pragma unroll
             for (int l = 0; l < A; ++l)
                 if (WinoBA<M_>::bt(j, l) != 0.f) s += tmp[i][l] * WinoBA<M_>::bt(j, l);
-            if constexpr (SPLIT) {
-                const __nv_bfloat16 hi = __float2bfloat16_rn(s), lo = __float2bfloat16_rn(s - __bfloat162float(hi));
-                const uint32_t own = (uint32_t)__bfloat16_as_ushort(hi) | (uint32_t)__bfloat16_as_ushort(lo) << 16;
-                const uint32_t other = __shfl_xor_sync(0xffffffffu, own, 1);
-                out[(long long)(i * A + j) * T * Cp] = __uint_as_float((c & 1) ? __byte_perm(other, own, 0x7632) : __byte_perm(own, other, 0x5410));
-            } else {
-                out[(long long)(i * A + j) * T * Cp] = to_out<OutT>((sizeof(OutT) == 4 && M_ == 2) ? round_tf32(s) : s);
-            }
+            out[(long long)(i * A + j) * T * Cp] = wino_operand<M_, OutT, SPLIT>(s, c);
         }
+}
+
+// A block takes one tile and 32 channels.
+template <int M_, typename OutT, bool SPLIT>
+__global__ void __launch_bounds__(32 * WinoBA<M_>::A)
+wino_input_tile_kernel(const float* __restrict__ x, OutT* __restrict__ V, int C, int Cp, int H, int W, int pad, int TH,
+                  int TW) {
+    constexpr int A = WinoBA<M_>::A;
+    __shared__ float tmp[A][A][32];                              // B^T d
+    const int lane = threadIdx.x & 31, col = threadIdx.x >> 5;
+    const int t = blockIdx.x, c = blockIdx.y * 32 + lane;
+    const int th = t / TW, tw = t - th * TW;
+    const int h0 = th * M_ - pad, w = tw * M_ - pad + col;
+    const bool inside = c < C && w >= 0 && w < W;
+    const float* src = x + ((long long)h0 * W + w) * C + c;
+    const long long plane = (long long)TH * TW * Cp;
+    OutT* out = V + (long long)(col * A) * plane + (long long)t * Cp + wino_word<SPLIT>(c);
+    pdl_enter();
+    float d[A];
+#pragma unroll
+    for (int l = 0; l < A; ++l) d[l] = inside && h0 + l >= 0 && h0 + l < H ? __ldg(src + (long long)l * W * C) : 0.f;
+#pragma unroll
+    for (int i = 0; i < A; ++i) {
+        float s = 0.f;
+#pragma unroll
+        for (int l = 0; l < A; ++l)
+            if (WinoBA<M_>::bt(i, l) != 0.f) s += WinoBA<M_>::bt(i, l) * d[l];
+        tmp[i][col][lane] = s;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int l = 0; l < A; ++l) d[l] = tmp[col][l][lane];        // the warp's row
+#pragma unroll
+    for (int j = 0; j < A; ++j) {                                // V = tmp B
+        float s = 0.f;
+#pragma unroll
+        for (int l = 0; l < A; ++l)
+            if (WinoBA<M_>::bt(j, l) != 0.f) s += d[l] * WinoBA<M_>::bt(j, l);
+        const OutT v = wino_operand<M_, OutT, SPLIT>(s, c);      // (a shuffle: by all lanes)
+        if (c < Cp) out[j * plane] = v;
+    }
 }
 
 nnv_status_t launch_wino_input(int m, bool bf16, bool split, const float* x, void* V, int C, int Cp, int H, int W, int pad,
                                int TH, int TW, cudaStream_t st) {
     const long long n = (long long)TH * TW * Cp;
-    const unsigned grid = (unsigned)((n + 127) / 128);
-#define NNV_WI(MM)                                                                                              \
-    if (bf16) NNV_LAUNCH((wino_input_kernel<MM, __nv_bfloat16, false>), grid, 128, 0, st, x, (__nv_bfloat16*)V, C, Cp, H, W, pad, TH, TW); \
-    else NNV_LAUNCH((wino_input_kernel<MM, float, false>), grid, 128, 0, st, x, (float*)V, C, Cp, H, W, pad, TH, TW);
-    if (split && m == 4) NNV_LAUNCH((wino_input_kernel<4, float, true>), grid, 128, 0, st, x, (float*)V, C, Cp, H, W, pad, TH, TW);
-    else if (split && m == 6) NNV_LAUNCH((wino_input_kernel<6, float, true>), grid, 128, 0, st, x, (float*)V, C, Cp, H, W, pad, TH, TW);
-    else if (m == 2) { NNV_WI(2) } else if (m == 4) { NNV_WI(4) } else if (m == 6) { NNV_WI(6) }
+    auto go = [&](auto mm, auto zero, auto pre) {
+        constexpr int M_ = decltype(mm)::value;
+        using OutT = decltype(zero);
+        constexpr bool S = decltype(pre)::value;
+        if (wino_tile_blocks<M_>(TH, TW, Cp))
+            return launch_pdl(wino_input_tile_kernel<M_, OutT, S>, dim3(TH * TW, ceil_div(Cp, 32)), dim3(32 * (M_ + 2)), 0, st, x, (OutT*)V, C, Cp, H, W, pad, TH, TW);
+        return launch_pdl(wino_input_kernel<M_, OutT, S>, dim3((unsigned)((n + 127) / 128)), dim3(128), 0, st, x, (OutT*)V, C, Cp, H, W, pad, TH, TW);
+    };
+    const std::integral_constant<int, 2> m2;
+    const std::integral_constant<int, 4> m4;
+    const std::integral_constant<int, 6> m6;
+    const __nv_bfloat16 b{};
+    if (m == 2) NNV_CUDA(bf16 ? go(m2, b, std::false_type()) : go(m2, 0.f, std::false_type()));
+    else if (m == 4) NNV_CUDA(bf16 ? go(m4, b, std::false_type()) : split ? go(m4, 0.f, std::true_type()) : go(m4, 0.f, std::false_type()));
+    else if (m == 6) NNV_CUDA(bf16 ? go(m6, b, std::false_type()) : split ? go(m6, 0.f, std::true_type()) : go(m6, 0.f, std::false_type()));
     else return fail(NNV_ERR_INVALID_ARG, "no Winograd tile size %d", m);
-#undef NNV_WI
-    NNV_CUDA(cudaGetLastError());
     return NNV_OK;
 }
 
@@ -317,15 +382,71 @@ wino_output_kernel(const float* __restrict__ Mt, float* __restrict__ y, const fl
     }
 }
 
+// A block takes one tile and 32 output channels; its first M_ warps write a row of the output tile each.
+template <int M_>
+__global__ void __launch_bounds__(32 * WinoBA<M_>::A)
+wino_output_tile_kernel(const float* __restrict__ Mt, float* __restrict__ y, const float* __restrict__ bias,
+                   const float* __restrict__ add, int act, int K, int OH, int OW, int TH, int TW) {
+    constexpr int A = WinoBA<M_>::A;
+    __shared__ float tmp[M_][A][32];                             // A^T M
+    const int lane = threadIdx.x & 31, col = threadIdx.x >> 5;
+    const int t = blockIdx.x, k = blockIdx.y * 32 + lane;
+    const int th = t / TW, tw = t - th * TW;
+    const bool live = k < K;
+    const long long plane = (long long)TH * TW * K;
+    const float* src = Mt + (long long)col * plane + (long long)t * K + k;
+    const int oh = th * M_ + col, ow = tw * M_;                  // the warp's row of the output tile (the last warps have none)
+    const bool writes = live && col < M_ && oh < OH;
+    const long long at = ((long long)oh * OW + ow) * K + k;
+    pdl_enter();
+    float v[A];
+#pragma unroll
+    for (int l = 0; l < A; ++l) v[l] = live ? __ldg(src + (long long)(l * A) * plane) : 0.f;
+    float av[M_];                                                // the residual's loads leave with the others
+    if (add) {
+#pragma unroll
+        for (int j = 0; j < M_; ++j) av[j] = writes && ow + j < OW ? __ldg(add + at + (long long)j * K) : 0.f;
+    }
+    const float b = bias && live ? __ldg(bias + k) : 0.f;
+#pragma unroll
+    for (int i = 0; i < M_; ++i) {
+        float s = 0.f;
+#pragma unroll
+        for (int l = 0; l < A; ++l)
+            if (WinoBA<M_>::at(i, l) != 0.f) s += WinoBA<M_>::at(i, l) * v[l];
+        tmp[i][col][lane] = s;
+    }
+    __syncthreads();
+    if (!writes) return;
+#pragma unroll
+    for (int l = 0; l < A; ++l) v[l] = tmp[col][l][lane];
+#pragma unroll
+    for (int j = 0; j < M_; ++j) {
+        float s = 0.f;
+#pragma unroll
+        for (int l = 0; l < A; ++l)
+            if (WinoBA<M_>::at(j, l) != 0.f) s += v[l] * WinoBA<M_>::at(j, l);
+        if (ow + j < OW) {
+            s += b;
+            if (add) s += av[j];
+            y[at + (long long)j * K] = apply_act(s, act);
+        }
+    }
+}
+
 nnv_status_t launch_wino_output(int m, const float* Mt, float* y, const float* bias, const float* add, int act,
                                 int K, int OH, int OW, int TH, int TW, cudaStream_t st) {
     const long long n = (long long)TH * TW * K;
-    const unsigned grid = (unsigned)((n + 127) / 128);
-    if (m == 2) NNV_LAUNCH((wino_output_kernel<2>), grid, 128, 0, st, Mt, y, bias, add, act, K, OH, OW, TH, TW);
-    else if (m == 4) NNV_LAUNCH((wino_output_kernel<4>), grid, 128, 0, st, Mt, y, bias, add, act, K, OH, OW, TH, TW);
-    else if (m == 6) NNV_LAUNCH((wino_output_kernel<6>), grid, 128, 0, st, Mt, y, bias, add, act, K, OH, OW, TH, TW);
+    auto go = [&](auto mm) {
+        constexpr int M_ = decltype(mm)::value;
+        if (wino_tile_blocks<M_>(TH, TW, K))
+            return launch_pdl(wino_output_tile_kernel<M_>, dim3(TH * TW, ceil_div(K, 32)), dim3(32 * (M_ + 2)), 0, st, Mt, y, bias, add, act, K, OH, OW, TH, TW);
+        return launch_pdl(wino_output_kernel<M_>, dim3((unsigned)((n + 127) / 128)), dim3(128), 0, st, Mt, y, bias, add, act, K, OH, OW, TH, TW);
+    };
+    if (m == 2) NNV_CUDA(go(std::integral_constant<int, 2>()));
+    else if (m == 4) NNV_CUDA(go(std::integral_constant<int, 4>()));
+    else if (m == 6) NNV_CUDA(go(std::integral_constant<int, 6>()));
     else return fail(NNV_ERR_INVALID_ARG, "no Winograd tile size %d", m);
-    NNV_CUDA(cudaGetLastError());
     return NNV_OK;
 }
 

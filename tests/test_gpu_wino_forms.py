@@ -1,0 +1,34 @@
+"""GPU parity of the Winograd layers on both sides of the rule that picks the form of their data transforms (a block per tile or a thread
+per tile and channel), with operands split ahead of the GEMM (channels in whole blocks of 32) and in it."""
+import numpy as np
+import pytest
+
+from oracle import model as omodel
+from paper_2206_07446_b200 import binding as nb
+from gpu_util import TOL, assert_conv_close, run_conv
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("variant,C,K,H,W", [
+    (nb.VAR_WINO_F4, 33, 40, 9, 14),       # 12 tiles, channels of a second block mostly absent; operands split in the GEMM
+    (nb.VAR_WINO_F4, 31, 7, 30, 11),       # a block of 32 with one channel of padding: split ahead
+    (nb.VAR_WINO_F6, 64, 33, 13, 25),      # split ahead, output channels end inside a block
+    (nb.VAR_WINO_F6, 20, 64, 19, 6),
+    (nb.VAR_WINO_F2, 40, 36, 61, 65),      # 1023 tiles: a block per tile on the input side (2046 blocks are too many), and on the output side
+    (nb.VAR_WINO_F2, 32, 70, 90, 92),      # 2070 tiles: a thread per tile and channel on both
+    (nb.VAR_WINO_F4, 32, 96, 128, 126),    # 1024 tiles: a block per tile on the input side, a thread on the output side (3072 blocks)
+    (nb.VAR_WINO_F6, 64, 24, 200, 190),    # 1088 tiles: thread, split ahead / block
+])
+def test_both_forms(variant, C, K, H, W):
+    L = dict(op=nb.OP_CONV, C=C, K=K, R=3, S=3, stride=1, pad=1, groups=1, H=H, W=W, in0=-1, in1=-1, act=1, has_bias=1)
+    rng = np.random.default_rng([17, C, K, H, W])
+    x = rng.uniform(-1, 1, (C, H, W)).astype(np.float32)
+    w = (rng.standard_normal((K, C, 3, 3)) * np.sqrt(2.0 / (9 * C))).astype(np.float32)
+    b = rng.uniform(-1, 1, K).astype(np.float32)
+    add = rng.uniform(-1, 1, (K, H, W)).astype(np.float32)
+    ref = omodel.run_layer(L, x, w, b, add)
+    for math in (nb.MATH_TF32, nb.MATH_BF16) if variant == nb.VAR_WINO_F2 else (nb.MATH_TF32,):
+        y = run_conv(nb.Plan([L], [0], [0]), 0, L, variant, math, x, w, b, add)
+        # F(4,3) and F(6,3) multiply error-compensated operands: 2^-16 a product, amplified by the transforms (measured 5e-5 / 9e-5)
+        assert_conv_close(y, ref, TOL[math] if variant == nb.VAR_WINO_F2 else 3e-4, (variant, math))
