@@ -54,9 +54,10 @@ __device__ __forceinline__ void pdl_enter() { pdl_wait(); pdl_trigger(); }
 // Every launch also asks for the largest shared-memory share of the L1.  Left to themselves the kernels that use little get another
 // share than those that use much, and an SM changes it only when nothing runs on it, which keeps a kernel from starting under its
 // predecessor's tail: 256 -> 256 F(2,3) @30, whose GEMM takes 199 KB between two transforms that take none, 12.7 -> 10.1 us; resident
-// ResNet-18-shaped inference with F(4,3) 258 -> 252, VGG-16-shaped @110 with F(6,3) 388 -> 373.
+// ResNet-18-shaped inference with F(4,3) 258 -> 252, VGG-16-shaped @110 with F(6,3) 388 -> 373.  (Not the weight transforms, which stream
+// through the L1 from a stream of their own: all of a ResNet-50-shaped model 64.8 us without, 67.4 with.)
 template <typename... Params, typename... Args>
-inline cudaError_t launch_pdl(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
+inline cudaError_t launch_pdl_carveout(int carveout, void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
@@ -66,10 +67,14 @@ inline cudaError_t launch_pdl(void (*kernel)(Params...), dim3 grid, dim3 block, 
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     attr[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
-    attr[1].val.sharedMemCarveout = cudaSharedmemCarveoutMaxShared;
+    attr[1].val.sharedMemCarveout = carveout;
     cfg.attrs = attr;
-    cfg.numAttrs = 2;
+    cfg.numAttrs = carveout >= 0 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+template <typename... Params, typename... Args>
+inline cudaError_t launch_pdl(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
+    return launch_pdl_carveout(cudaSharedmemCarveoutMaxShared, kernel, grid, block, smem, st, args...);
 }
 // Same, as thread-block clusters of `cluster_z` consecutive CTAs along grid z (1 = no cluster).
 template <typename... Params, typename... Args>

@@ -8,6 +8,9 @@
 
 #include "nnv_internal.h"
 
+// (without a preference for the L1's split: see launch_pdl)
+#define XF_LAUNCH(kernel, grid, block, st, ...) (void)launch_pdl_carveout(-1, kernel, dim3(grid), dim3(block), 0, st, __VA_ARGS__)
+
 namespace nnv {
 
 // G matrices of the Cook-Toom construction with points {0, +-1, +-2, +-1/2, inf} (the published
@@ -223,7 +226,7 @@ static nnv_status_t launch_ft(const float* g, void* U, int K, int C, int Cp, cud
     const unsigned grid = (unsigned)((F + ft_filters(M_) - 1) / ft_filters(M_));
     unsigned long long* stamp = next_stamp();
     next_stamp() = nullptr;
-    NNV_LAUNCH((filter_transform_kernel<M_, OutT>), grid, ft_threads(M_), 0, st, g, reinterpret_cast<OutT*>(U), K, C, Cp, stamp,
+    XF_LAUNCH((filter_transform_kernel<M_, OutT>), grid, ft_threads(M_), st, g, reinterpret_cast<OutT*>(U), K, C, Cp, stamp,
                host_src ? 1 : 0);
     NNV_CUDA(cudaGetLastError());
     return NNV_OK;
@@ -505,12 +508,12 @@ nnv_status_t launch_transform_batch(XformDesc* descs, int n, cudaStream_t st) {
             auto launch = [&](auto group) {
                 constexpr int G = decltype(group)::value;
                 if (b.n > XF_BATCH_SMALL) {
-                    NNV_LAUNCH((multi_transform_kernel<G, XF_BATCH_MAX>), blocks, xform_threads(G), 0, st, b);
+                    XF_LAUNCH((multi_transform_kernel<G, XF_BATCH_MAX>), blocks, xform_threads(G), st, b);
                 } else {
                     XformBatch<XF_BATCH_SMALL> small;
                     small.stamp = b.stamp; small.n = b.n; small.host_src = b.host_src; small.follows = b.follows;
                     std::copy(b.d, b.d + b.n, small.d);
-                    NNV_LAUNCH((multi_transform_kernel<G, XF_BATCH_SMALL>), blocks, xform_threads(G), 0, st, small);
+                    XF_LAUNCH((multi_transform_kernel<G, XF_BATCH_SMALL>), blocks, xform_threads(G), st, small);
                 }
             };
             if (grp == XG_PACK) launch(std::integral_constant<int, XG_PACK>{});
@@ -543,13 +546,13 @@ nnv_status_t launch_pack(bool bf16, const float* w, void* P, int K, int C, int R
     if (RS == 1) {
         const long long n = (long long)K * Qp;
         const unsigned grid = (unsigned)((n + PACK1X1_PER_BLOCK - 1) / PACK1X1_PER_BLOCK);
-        if (bf16) NNV_LAUNCH((pack1x1_kernel<__nv_bfloat16>), grid, PACK_THREADS, 0, st, w, (__nv_bfloat16*)P, K, C, Qp, stamp, hs);
-        else NNV_LAUNCH((pack1x1_kernel<float>), grid, PACK_THREADS, 0, st, w, (float*)P, K, C, Qp, stamp, hs);
+        if (bf16) XF_LAUNCH((pack1x1_kernel<__nv_bfloat16>), grid, PACK_THREADS, st, w, (__nv_bfloat16*)P, K, C, Qp, stamp, hs);
+        else XF_LAUNCH((pack1x1_kernel<float>), grid, PACK_THREADS, st, w, (float*)P, K, C, Qp, stamp, hs);
     } else {
         NNV_REQUIRE(8 * RS <= PACK_SLICE, NNV_ERR_UNSUPPORTED, "filter window of %d taps is too large to repack", RS);
         const unsigned grid = (unsigned)pack_blocks(K, C, RS);
-        if (bf16) NNV_LAUNCH((pack_kernel<__nv_bfloat16>), grid, PACK_THREADS, 0, st, w, (__nv_bfloat16*)P, K, C, RS, Qp, stamp, hs);
-        else NNV_LAUNCH((pack_kernel<float>), grid, PACK_THREADS, 0, st, w, (float*)P, K, C, RS, Qp, stamp, hs);
+        if (bf16) XF_LAUNCH((pack_kernel<__nv_bfloat16>), grid, PACK_THREADS, st, w, (__nv_bfloat16*)P, K, C, RS, Qp, stamp, hs);
+        else XF_LAUNCH((pack_kernel<float>), grid, PACK_THREADS, st, w, (float*)P, K, C, RS, Qp, stamp, hs);
     }
     NNV_CUDA(cudaGetLastError());
     return NNV_OK;
