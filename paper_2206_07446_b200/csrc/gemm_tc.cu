@@ -1045,6 +1045,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 #include "conv3x3_bf16.cuh"
 #include "gemm_sp.cuh"
 #include "wino_fused.cuh"
+#include "inverted_bottleneck.cuh"
 
 // ---- host side --------------------------------------------------------------------------------
 PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
@@ -1378,6 +1379,10 @@ constexpr decltype(&gemm_tc_kernel<0, false>) gemm_kernels[10][2] = {
     {gemm_tc_kernel<4, false>, gemm_tc_kernel<4, true>}, {gemm_tc_kernel<5, false>, gemm_tc_kernel<5, true>},
     {gemm_tc_kernel<6, false>, gemm_tc_kernel<6, true>}, {gemm_tc_kernel<7, false>, gemm_tc_kernel<7, true>},
     {gemm_tc_kernel<ROUNDED, false>, gemm_tc_kernel<ROUNDED, true>}, {gemm_tc_kernel<SPLIT_A, false>, gemm_tc_kernel<SPLIT_A, true>}};
+// [BF16 math][patches shared by a cluster]
+constexpr decltype(&inverted_bottleneck_kernel<false, false>) ib_kernels[2][2] = {
+    {inverted_bottleneck_kernel<false, false>, inverted_bottleneck_kernel<false, true>},
+    {inverted_bottleneck_kernel<true, false>, inverted_bottleneck_kernel<true, true>}};
 static_assert(GEMM_TF32 == 0 && GEMM_BF16 == 1 && GEMM_X3 == 2 && GEMM_BF16_CVT == 3, "the table's order");
 
 }  // namespace
@@ -1397,6 +1402,11 @@ nnv_status_t gemm_tc_init() {
         cudaFuncSetAttribute(conv3x3_tc_persistent_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
         cudaFuncSetAttribute(wino_f2_fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
         cudaFuncSetAttribute(conv3x3_tc_ws_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
+        for (auto& forms : ib_kernels)
+            for (auto* kernel : forms) {
+                cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
+                cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+            }
     });
     return NNV_OK;
 }
@@ -1824,6 +1834,197 @@ nnv_status_t launch_gemm_tc(const GemmArgs& a, cudaStream_t st) {
     return NNV_OK;
 }
 
+// ---- inverted bottleneck: shape of a launch -----------------------------------------------------
+namespace {
+
+struct IbShape {
+    int ph, pw, hw, rows, px, tiles_h, tiles_w;
+    int ranks, splits, both, step, nb_most, BN2, issuers, tmem_cols;
+    uint16_t first[IB_MAX_RANKS];
+    uint8_t count[IB_MAX_RANKS];
+    uint32_t pairs;                   // bit k: split k has two ranks
+    uint32_t w1_off, conv_off, d_off, w2_off, bar_off, par_off;
+    size_t smem_bytes;
+    double t;                         // estimated time, us
+};
+
+// The channel blocks of every CTA that shares a patch, in the order of the projection's own launch: its `splits` ranges of the n blocks,
+// whole (`both`: two accumulators, or with one issuer one) or an accumulator's blocks each.
+bool ib_ranks(int n, int splits, int issuers, bool unit, IbShape* s) {
+    s->ranks = 0; s->pairs = 0; s->nb_most = 0; s->splits = splits;
+    s->both = issuers == 2 && !unit;
+    s->step = issuers == 2 && unit ? 2 : 1;
+    for (int sp = 0; sp < splits; ++sp) {
+        const int k0 = n * sp / splits, k1 = n * (sp + 1) / splits;
+        for (int par = 0; par < s->step; ++par) {
+            const int count = ceil_div(k1 - k0 - par, s->step);
+            if (count <= 0) continue;
+            if (s->ranks == IB_MAX_RANKS || count > IB_MAX_NB) return false;
+            if (par == 1) s->pairs |= 1u << sp;
+            s->first[s->ranks] = (uint16_t)(k0 + par);
+            s->count[s->ranks] = (uint8_t)count;
+            s->nb_most = std::max(s->nb_most, count);
+            ++s->ranks;
+        }
+    }
+    return true;
+}
+
+// Shared memory of a launch; false where it does not fit.
+bool ib_layout(bool bf16, int nkb1, IbShape* s) {
+    const size_t xs = a_stage_of(s->rows), ds = bf16 ? (size_t)pad8(s->px) * 64 : a_stage_of(s->px);
+    const size_t conv = bf16 ? (size_t)nkb1 * pad8(s->rows) * 64 : 0;
+    const size_t w1 = (size_t)nkb1 * s->nb_most * (bf16 ? 2048 : 4096), w2 = (size_t)s->nb_most * s->BN2 * (bf16 ? 64 : 128);
+    const size_t recv = s->ranks > 1 ? (size_t)s->ranks * ceil_div(s->px, s->ranks) * s->BN2 * 4 : 0;
+    s->w1_off = (uint32_t)(nkb1 * xs);
+    s->conv_off = (uint32_t)align_up(s->w1_off + w1, 1024);
+    // first the operands of the expansion, then its output, then the rows received; behind them those of the projection, then its rows
+    const size_t r0 = align_up(std::max({(size_t)s->conv_off + conv, (size_t)s->nb_most * s->rows * IB_PITCH, recv}), 1024);
+    s->d_off = (uint32_t)r0;
+    s->w2_off = (uint32_t)align_up(r0 + s->nb_most * ds, 1024);
+    const size_t r1 = std::max((size_t)s->w2_off + w2, r0 + (size_t)s->px * s->BN2 * 4);
+    s->bar_off = (uint32_t)align_up(r1, 128);
+    s->par_off = (uint32_t)align_up(s->bar_off + IB_BAR_BYTES, 16);
+    s->smem_bytes = 1024 + s->par_off + 4 * ((size_t)s->nb_most * (64 + 288) + s->BN2);
+    // an MMA reads 128 rows of A, the last block's included
+    s->smem_bytes = std::max({s->smem_bytes, (size_t)1024 + (nkb1 - 1) * xs + A_STAGE_BYTES, (size_t)1024 + s->d_off + (s->nb_most - 1) * ds + A_STAGE_BYTES,
+                              (size_t)1024 + s->conv_off + conv + A_STAGE_BYTES / 2});
+    s->tmem_cols = 32;
+    while (s->tmem_cols < std::max(s->issuers * s->nb_most * 32, (s->both ? 2 : 1) * s->BN2)) s->tmem_cols *= 2;
+    if (s->ranks > 1) s->smem_bytes = std::max(s->smem_bytes, std::min((size_t)226 * 1024, tmem_share_bytes(s->tmem_cols)));   // (226 KB: an SM of its own)
+    return s->smem_bytes <= 226u * 1024u && s->tmem_cols <= 512;
+}
+
+// Clusters that find SMs of their own.
+int ib_lone(int ranks) {
+    static constexpr int lone[10] = {148, 148, 74, 48, 33, 24, 24, 15, 15, 14};
+    return ranks < 10 ? lone[ranks] : 7;
+}
+// Estimated time of a launch, us: waves of clusters x (start and phases of fixed length, the pixels' loads, the passes over accumulators
+// and pixels), plus the bytes from L2 over all CTAs.  A cluster of more than nine CTAs finds one place in a GPC; a second CTA on an SM adds half.
+// Fitted to 1867 launches of 78 blocks (TF32, 96 - 224 pixels): the chosen shapes are 1.1 % above the best measured ones on average (BF16,
+// 67 blocks: 1.5 %).
+int ib_occupancy(const IbShape& s) { return std::max(1, std::min({(int)(227u * 1024u / (s.smem_bytes + 1024)), 512 / s.tmem_cols, 2})); }
+double ib_us(const IbShape& s, bool bf16, int nkb1, int stride, int occ) {
+    const int one = ib_lone(s.ranks), clusters = s.tiles_h * s.tiles_w;
+    const int waves = ceil_div(clusters, one * occ), resident = std::min(occ, ceil_div(clusters, one));
+    const double weights = (bf16 ? 0.5 : 1.0) * s.nb_most * (nkb1 * 4096.0 + s.BN2 * 128.0), pixels = nkb1 * s.rows * 128.0;
+    const double phases = 8.4e-5 * pixels + 0.5 * s.nb_most + (stride == 2 ? 0.69 : 0.5) * ceil_div(s.nb_most * s.px, IB_THREADS / 16) +
+                          0.06 * ceil_div(ceil_div(s.px, s.ranks) * s.BN2, IB_THREADS);
+    return waves * (1.69 + phases * (0.5 + 0.5 * resident)) + 3.85e-8 * (weights + pixels) * clusters * s.ranks + (occ == 1 ? 0.29 : 0.0);
+}
+
+IbShape search_ib(bool bf16, int C, int E, int K, int OH, int OW, int stride, int splits, int issuers) {
+    const int nkb1 = ceil_div(C, 32);
+    IbShape best{};
+    best.t = 1e30;
+    for (int unit = 0; unit < (issuers == 2 ? 2 : 1); ++unit) {
+        IbShape s{};
+        s.BN2 = ceil_div(K, 16) * 16;
+        s.issuers = issuers;
+        if (!ib_ranks(ceil_div(E, 32), splits, issuers, unit != 0, &s)) continue;
+        if (s.BN2 > (s.both ? 256 : 512)) continue;
+        // Patches of the least height and width for their numbers of rows and columns, no more than four times as long as wide unless as long as the
+        // image.
+        for (int th = 1; th <= OH; ++th) {
+            const int ph = ceil_div(OH, th), hh = (ph - 1) * stride + 3;
+            if (hh * 3 > BM) continue;
+            if (th > 1 && ph == ceil_div(OH, th - 1)) continue;
+            for (int tw = 1; tw <= OW; ++tw) {
+                const int pw = ceil_div(OW, tw), hw = (pw - 1) * stride + 3;
+                if (hh * hw > BM || (tw > 1 && pw == ceil_div(OW, tw - 1))) continue;
+                if ((ph > 4 * pw && th > 1) || (pw > 4 * ph && tw > 1)) continue;
+                s.ph = ph; s.pw = pw; s.hw = hw; s.rows = hh * hw; s.px = ph * pw;
+                s.tiles_h = ceil_div(OH, ph); s.tiles_w = ceil_div(OW, pw);
+                if (ib_us(s, bf16, nkb1, stride, 2) >= best.t || !ib_layout(bf16, nkb1, &s)) continue;
+                s.t = ib_us(s, bf16, nkb1, stride, ib_occupancy(s));
+                if (s.t < best.t - 1e-9) best = s;
+            }
+        }
+    }
+    return best;
+}
+
+}  // namespace
+
+// The block's launch, if it is to be one: 1x1 expansion (TF32 or BF16 GEMM), 3x3 depthwise and 1x1 projection of the same math, whose
+// activations the GEMMs read in place.
+static bool ib_shape(const nnv_layer_desc_t& a, const nnv_layer_desc_t& d, const nnv_layer_desc_t& p, int math, IbShape* out) {
+    const int mode = math == NNV_MATH_BF16 ? GEMM_BF16_CVT : GEMM_TF32, align = math == NNV_MATH_BF16 ? 8 : 4;
+    const Tuning& tn = tuning();
+    if (tn.gemm_bn || tn.gemm_ring || tn.smallp_splits || (math == NNV_MATH_BF16 && !tn.bf16cvt)) return false;   // overrides of the GEMMs' launches
+    if (a.R != 1 || a.S != 1 || a.stride != 1 || a.pad != 0 || a.groups != 1 || p.R != 1 || p.S != 1 || p.stride != 1 || p.pad != 0 || p.groups != 1) return false;
+    if (d.R != 3 || d.S != 3 || d.pad != 1 || (d.stride != 1 && d.stride != 2) || d.groups != d.C || d.K != d.C || d.C != a.K || p.C != d.K) return false;
+    if (a.act == 0 || d.act == 0) return false;                // (a clamp would turn the NaNs of a linear layer into numbers)
+    if (a.C % align || a.K % align || p.K % 4 || a.C > 32 * IB_MAX_KB || a.K > 32 * 255 || p.K > 512) return false;
+    const int OH = (a.H - 1) / d.stride + 1, OW = (a.W - 1) / d.stride + 1, nkb1 = ceil_div(a.C, 32), nkb2 = ceil_div(a.K, 32);
+    if ((double)a.H * a.W * a.K >= 2.0e9 || (double)OH * OW * p.K >= 2.0e9) return false;         // 32-bit places in the outputs
+    const GemmTiling t1 = pick_gemm_tiling(mode, a.H * a.W, a.K, 1, nkb1), t2 = pick_gemm_tiling(mode, OH * OW, p.K, 1, nkb2);
+    if (t1.splits != 1) return false;
+    GemmShape g1, g2;
+    if (gemm_shape(mode, t1, a.H * a.W, a.K, 1, nkb1, true, false, &g1) != NNV_OK) return false;
+    if (gemm_shape(mode, t2, OH * OW, p.K, 1, nkb2, true, p.in1 >= 0, &g2) != NNV_OK) return false;
+    if (g1.issuers != g2.issuers) return false;
+    *out = search_ib(math == NNV_MATH_BF16, a.C, a.K, p.K, OH, OW, d.stride, g2.splits, g2.issuers);
+    return out->t < 1e29;
+}
+
+// The shape for a block, remembered by the calling thread (the search takes longer than a launch).
+static const IbShape* pick_ib(const nnv_layer_desc_t& a, const nnv_layer_desc_t& d, const nnv_layer_desc_t& p, int math) {
+    struct Entry { nnv_layer_desc_t a{}, d{}, p{}; int math = -1; uint64_t tuning = 0; bool use = false; IbShape s; };
+    static thread_local Entry table[64];
+    const uint32_t h = ((uint32_t)a.H * 2654435761u) ^ ((uint32_t)a.K * 40503u) ^ ((uint32_t)p.K * 9176u) ^ (uint32_t)(a.C * 131 + d.stride * 7 + math);
+    Entry& e = table[(h ^ (h >> 15)) & 63u];
+    auto same = [](const nnv_layer_desc_t& x, const nnv_layer_desc_t& y) {
+        return x.C == y.C && x.K == y.K && x.R == y.R && x.S == y.S && x.stride == y.stride && x.pad == y.pad && x.groups == y.groups && x.H == y.H && x.W == y.W && (x.in1 < 0) == (y.in1 < 0) && (x.act == 0) == (y.act == 0);
+    };
+    const Tuning& tn = tuning();
+    if (e.math != math || e.tuning != tn.generation || !same(e.a, a) || !same(e.d, d) || !same(e.p, p)) {
+        e.a = a; e.d = d; e.p = p; e.math = math; e.tuning = tn.generation;
+        e.use = ib_shape(a, d, p, math, &e.s);
+    }
+    return e.use ? &e.s : nullptr;
+}
+
+bool inverted_bottleneck_applies(const nnv_layer_desc_t& a, const nnv_layer_desc_t& d, const nnv_layer_desc_t& p, int math) {
+    return pick_ib(a, d, p, math) != nullptr;
+}
+
+nnv_status_t launch_inverted_bottleneck(const nnv_layer_desc_t& a, const nnv_layer_desc_t& d, const nnv_layer_desc_t& p, int math, const IbBuffers& io,
+                                        cudaStream_t st) {
+    NNV_TRY(gemm_tc_init());
+    const IbShape* s = pick_ib(a, d, p, math);
+    NNV_REQUIRE(s, NNV_ERR_UNSUPPORTED, "the three layers do not run as one launch");
+    const bool bf16 = math == NNV_MATH_BF16;
+    const int Qp1 = (a.C + 7) / 8 * 8, Qp2 = (p.C + 7) / 8 * 8;
+    CUtensorMap tmX, tmW1, tmW2;
+    const int w2_boxes = s->BN2 > 256 ? 2 : 1;
+    NNV_TRY(encode_halo_operand(&tmX, io.x, a.C, a.H, a.W, s->rows / s->hw, s->hw));
+    if (bf16) {
+        NNV_TRY(encode_bf16_weights(&tmW1, io.w1, Qp1, Qp1, a.K, 32));
+        NNV_TRY(encode_bf16_weights(&tmW2, io.w2, Qp2, Qp2, p.K, s->BN2 / w2_boxes));
+    } else {
+        NNV_TRY(encode_operand(&tmW1, io.w1, false, a.C, a.K, 1, Qp1, (int64_t)a.K * Qp1, 32));
+        NNV_TRY(encode_operand(&tmW2, io.w2, false, p.C, p.K, 1, Qp2, (int64_t)p.K * Qp2, s->BN2 / w2_boxes));
+    }
+    IbDev g{};
+    g.e = io.e; g.d = io.d; g.y = io.y; g.b1 = io.b1; g.b2 = io.b2; g.b3 = io.b3; g.addend = io.addend; g.wd = io.wd;
+    g.E = a.K; g.K = p.K; g.H = a.H; g.W = a.W; g.OH = p.H; g.OW = p.W; g.stride = d.stride;
+    g.most1 = a.act == 2 ? 6.f : INFINITY; g.most2 = d.act == 2 ? 6.f : INFINITY; g.act3 = p.act;
+    g.ph = s->ph; g.pw = s->pw; g.hw = s->hw; g.rows = s->rows; g.px = s->px; g.tiles_w = s->tiles_w;
+    g.nkb1 = ceil_div(a.C, 32); g.nb_most = s->nb_most; g.step = s->step; g.both = s->both; g.ranks = s->ranks; g.splits = s->splits; g.BN2 = s->BN2;
+    g.w2_boxes = w2_boxes; g.issuers = s->issuers; g.tmem_cols = s->tmem_cols;
+    g.magic_hw = 0xFFFFFFFFu / (uint32_t)s->hw + 1u; g.magic_pw = 0xFFFFFFFFu / (uint32_t)s->pw + 1u;
+    g.magic_nch = 0xFFFFFFFFu / (uint32_t)(s->BN2 / 4) + 1u; g.magic_n = 0xFFFFFFFFu / (uint32_t)s->BN2 + 1u; g.magic_px = 0xFFFFFFFFu / (uint32_t)s->px + 1u;
+    g.w1_off = s->w1_off; g.conv_off = s->conv_off; g.d_off = s->d_off; g.w2_off = s->w2_off; g.bar_off = s->bar_off; g.par_off = s->par_off;
+    std::copy(std::begin(s->first), std::end(s->first), g.first);
+    std::copy(std::begin(s->count), std::end(s->count), g.count);
+    g.pairs = s->pairs;
+    const dim3 grid(s->tiles_h * s->tiles_w, 1, s->ranks);
+    NNV_CUDA(launch_pdl_cluster(ib_kernels[bf16][s->ranks > 1], grid, dim3(IB_THREADS), s->smem_bytes, st, s->ranks, tmX, tmW1, tmW2, g));
+    return NNV_OK;
+}
+
 }  // namespace nnv
 
 // Host-side launch shape of gemm_tc_kernel for the tests (kernel mode, K blocks of 128 bytes).
@@ -1836,6 +2037,25 @@ extern "C" int nnv_internal_gemm_shape(int mode, int M, int N, int batch, int nk
                          (int32_t)s.stage_off, (int32_t)s.smem_bytes, (int32_t)gemm_stage_bytes(mode, s.BN, s.rows), gemm_tc_threads(mode)};
     std::copy(std::begin(v), std::end(v), out);
     return NNV_OK;
+}
+
+// The launch shape of an inverted-residual block C -> E -> K on an H x W image, for the tests; 1: the layers run as launches of their own.
+extern "C" int nnv_internal_ib_shape(int bf16, int C, int E, int K, int H, int W, int stride, int residual, int32_t* out) {
+    using namespace nnv;
+    nnv_layer_desc_t a{}, d{}, p{};
+    a.op = d.op = p.op = NNV_OP_CONV;
+    a.act = d.act = 1;
+    a.C = C; a.K = E; a.R = a.S = 1; a.stride = 1; a.groups = 1; a.H = H; a.W = W; a.in1 = -1;
+    d.C = d.K = d.groups = E; d.R = d.S = 3; d.stride = stride; d.pad = 1; d.H = H; d.W = W; d.in1 = -1;
+    p.C = E; p.K = K; p.R = p.S = 1; p.stride = 1; p.groups = 1; p.H = (H - 1) / stride + 1; p.W = (W - 1) / stride + 1; p.in1 = residual ? 0 : -1;
+    const IbShape* s = pick_ib(a, d, p, bf16 ? NNV_MATH_BF16 : NNV_MATH_TF32);
+    if (!s) return 1;
+    const int32_t v[] = {s->ph, s->pw, s->hw, s->rows, s->px, s->tiles_h, s->tiles_w, s->ranks, s->both, s->step, s->nb_most, s->BN2, s->issuers,
+                         s->tmem_cols, (int32_t)s->w1_off, (int32_t)s->conv_off, (int32_t)s->d_off, (int32_t)s->w2_off, (int32_t)s->bar_off,
+                         (int32_t)s->par_off, (int32_t)s->smem_bytes, (int32_t)s->pairs};
+    std::copy(std::begin(v), std::end(v), out);
+    for (int r = 0; r < IB_MAX_RANKS; ++r) { out[24 + 2 * r] = r < s->ranks ? s->first[r] : -1; out[25 + 2 * r] = r < s->ranks ? s->count[r] : 0; }
+    return 0;
 }
 
 extern "C" int nnv_internal_gemm_loaders(int mode, int nkb, int ring) { return nnv::gemm_loaders(mode, nkb, ring); }

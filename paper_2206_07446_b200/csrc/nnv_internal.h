@@ -357,6 +357,16 @@ nnv_status_t launch_gemm_tc(const GemmArgs& a, cudaStream_t st);
 // Convolution of a layer with few pixels by the weights-on-rows kernel: x NHWC [H*W][C], wt packed P[K][Qp].
 nnv_status_t launch_gemm_sp(const nnv_layer_desc_t& L, const LayerGeom& g, const SmallPPlan& sp, const float* x, const float* wt,
                             const float* bias, const float* addend, float* y, void* ws, cudaStream_t st);
+// An inverted-residual block -- 1x1 expansion, 3x3 depthwise, 1x1 projection, the GEMMs in `math` -- as one launch
+// (inverted_bottleneck.cuh); every output gets the bits that the three layers' own launches give it.
+struct IbBuffers {
+    const float* x; const void* w1; const float* wd; const void* w2;      // input, packed weights, raw depthwise weights
+    const float* b1; const float* b2; const float* b3; const float* addend;
+    float* e; float* d; float* y;                                          // the three layers' outputs
+};
+bool inverted_bottleneck_applies(const nnv_layer_desc_t& expand, const nnv_layer_desc_t& depthwise, const nnv_layer_desc_t& project, int math);
+nnv_status_t launch_inverted_bottleneck(const nnv_layer_desc_t& expand, const nnv_layer_desc_t& depthwise, const nnv_layer_desc_t& project,
+                                        int math, const IbBuffers& io, cudaStream_t st);
 // One-time host set-up of the GEMM (driver entry point, shared-memory attributes); call before
 // stream capture.
 nnv_status_t gemm_tc_init();
