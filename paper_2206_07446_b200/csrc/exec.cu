@@ -69,8 +69,13 @@ nnv_status_t do_exec(const nnv_plan& p, int layer, int v, int math, const void* 
         // F(2,3) runs as one TF32 / BF16 pass; F(4,3) and F(6,3) amplify operand rounding too much for
         // that, so their tile GEMM multiplies fp32 operands with the compensated bf16 scheme.
         if (m != 2) a.mode = GEMM_X3;
-        a.split_a = m != 2 && (g.Cp % 32) == 0;
+        const bool small = wino_small_applies(m, T, g.Cp, L.K);
+        a.split_a = m != 2 && (g.Cp % 32) == 0 && !small;
         NNV_TRY(launch_wino_input(m, bf16, a.split_a, x, V, L.C, g.Cp, L.H, L.W, L.pad, TH, TW, st));
+        if (small) {
+            NNV_TRY(launch_wino_small(m, (const float*)V, (const float*)d_wt, Mt, T, L.K, g.Cp, st));
+            return launch_wino_output(m, Mt, y, bias, add, L.act, L.K, g.OH, g.OW, TH, TW, st);
+        }
         a.A = V; a.B = d_wt; a.D = Mt;
         a.M = T; a.Kd = g.Cp; a.batch = a2;
         a.lda = g.Cp; a.ldb = g.Cp; a.ldd = L.K;

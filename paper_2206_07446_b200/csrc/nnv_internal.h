@@ -297,6 +297,9 @@ nnv_status_t launch_wino_input(int m, bool bf16, bool split, const float* d_x, v
 // Winograd output transform Y = A^T M A with the layer epilogue.
 nnv_status_t launch_wino_output(int m, const float* d_M, float* d_y, const float* d_bias, const float* d_add,
                                 int act, int K, int OH, int OW, int TH, int TW, cudaStream_t st);
+// The tile GEMM of F(4,3) / F(6,3) on a few tiles, in fp32: V[a2][T][Cp] and U[a2][K][Cp] fp32 -> M[a2][T][K].
+bool wino_small_applies(int m, int T, int Cp, int K);
+nnv_status_t launch_wino_small(int m, const float* d_V, const float* d_U, float* d_M, int T, int K, int Cp, cudaStream_t st);
 // fp32 direct convolution from raw OIHW weights (groups == 1).
 nnv_status_t launch_direct(const float* d_x, const float* d_w, const float* d_bias, const float* d_add,
                            float* d_y, int act, int C, int H, int W, int K, int R, int S, int stride, int pad,
