@@ -637,15 +637,19 @@ def nnv_device_status():
     return int(c.value)
 
 
-# The calls a program makes once per layer go through the extension module (the functions above, without ctypes' cost per
+# The calls a program makes once per layer or per inference go through the extension module (the functions above, without ctypes' cost per
 # argument); what it does not convert itself it hands back to them.
 try:
     from . import _nnvcall
 except ImportError as e:
     raise ImportError("_nnvcall.so is not built (%s). Run `python -m paper_2206_07446_b200.build`." % e)
-_nnvcall.set_fallbacks(nnv_conv_exec, nnv_transform_weights, nnv_transform_all, _check, ctypes.Array, Choice)
+_nnvcall.set_fallbacks(nnv_conv_exec, nnv_transform_weights, nnv_transform_all, nnv_cold_run, nnv_resident_run, nnv_warm_run, _check,
+                       ctypes.Array, Choice)
 nnv_conv_exec = _nnvcall.nnv_conv_exec
 nnv_transform_weights = _nnvcall.nnv_transform_weights
 nnv_transform_all = _nnvcall.nnv_transform_all
+nnv_cold_run = _nnvcall.nnv_cold_run
+nnv_resident_run = _nnvcall.nnv_resident_run
+nnv_warm_run = _nnvcall.nnv_warm_run
 
 EXPORTED_SYMBOLS = sorted(list(_SIGS.keys()) + ["nnv_last_error", "nnv_version"])

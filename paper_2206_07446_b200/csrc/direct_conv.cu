@@ -491,7 +491,8 @@ nnv_status_t launch_dt(const DirectDev& g, cudaStream_t st) {
     NNV_CUDA(attr);
     const dim3 grid(ceil_div(g.OH * g.OW, T), ceil_div(g.K, T), g.splits);
     NNV_REQUIRE(grid.y <= 65535, NNV_ERR_UNSUPPORTED, "too many output channels for the direct kernel");
-    NNV_CUDA(launch_pdl_cluster(direct_tile_kernel<TAPS, T>, grid, dim3(DT_THREADS), smem, st, g.splits, g));
+    const dim3 outputs(ceil_div(g.OH * g.OW, DC_T), ceil_div(g.K, DC_T));     // (as for direct_conv_kernel; 260 layers take the same either way)
+    NNV_CUDA(launch_pdl_attrs(stream_carveout(STREAM_LONE, outputs, dim3(DT_THREADS)), g.splits, direct_tile_kernel<TAPS, T>, grid, dim3(DT_THREADS), smem, st, g));
     return NNV_OK;
 }
 

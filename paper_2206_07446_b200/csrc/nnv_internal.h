@@ -206,10 +206,11 @@ struct GraphKey {
     int depth = 0;
     bool resident = false;
     bool host_io = false;
+    bool in_place[2] = {false, false};    // input, output: host memory that kernels address
     std::vector<int32_t> queues;          // preparation queue per layer (scheduled runs), else empty
     bool operator==(const GraphKey& o) const {
         if (tuning_gen != o.tuning_gen || ptrs != o.ptrs || w_bytes != o.w_bytes || depth != o.depth || resident != o.resident || host_io != o.host_io ||
-            queues != o.queues || choices.size() != o.choices.size())
+            in_place[0] != o.in_place[0] || in_place[1] != o.in_place[1] || queues != o.queues || choices.size() != o.choices.size())
             return false;
         for (size_t i = 0; i < choices.size(); ++i)
             if (choices[i].variant != o.choices[i].variant || choices[i].math != o.choices[i].math ||
@@ -221,6 +222,13 @@ struct GraphKey {
 struct CachedGraph {
     GraphKey key;
     cudaGraphExec_t exec = nullptr;       // null: recording failed, this argument set runs eagerly
+    // What a later call is compared with before anything is planned: a warm run's choices as the caller gives them (else the key's), and what
+    // the sizes that are no part of the key have to reach.
+    bool warm = false;
+    std::vector<nnv_choice_t> warm_choices;
+    uint64_t need_cached = 0, need_warm = 0;
+    bool zero_copy = false;               // kernels read the host weights in place
+    ArenaLayout layout;
 };
 }  // namespace nnv
 

@@ -1,4 +1,4 @@
-// Argument marshalling of the per-layer entry points for Python, as a CPython extension module.
+// Argument marshalling of the per-layer entry points and of the whole-model runs for Python, as a CPython extension module.
 //
 // A single layer's kernel runs for 3 - 6 us; the same call through ctypes spends ~2.5 us of host time converting a dozen
 // arguments one Python object at a time, about as much as everything below it, and calls issued back to back are then
@@ -9,6 +9,7 @@
 #include <Python.h>
 
 #include <stdint.h>
+#include <string.h>
 
 #include "nnv.h"
 
@@ -76,7 +77,7 @@ Arg choices(PyObject* o, PyObject* plan) {
     return a;
 }
 
-PyObject* g_fallback[3];                                      // the Python functions: conv_exec, transform_weights, transform_all
+PyObject* g_fallback[6];                                      // the Python functions: conv_exec, transform_weights, transform_all, the three runs
 PyObject* g_check;                                            // raises for a status that is not OK
 
 PyObject* finish(nnv_status_t st) {
@@ -143,15 +144,66 @@ PyObject* transform_all(PyObject*, PyObject* const* args, Py_ssize_t n, PyObject
     return finish(st);
 }
 
+// The whole-model runs: plan, choices as a ctypes array, then `kinds`.  Calls that ask for timings are Python's.
+bool convert_run(const char* kinds, PyObject* const* args, Py_ssize_t n, PyObject* kw, const nnv_choice_t** ch, uint64_t* v) {
+    const Py_ssize_t m = (Py_ssize_t)strlen(kinds) + 1;
+    if (n < m || n > m + 1 || (kw && PyTuple_GET_SIZE(kw) != 0) || (n == m + 1 && args[m] != Py_False)) return false;
+    const Arg c = choices(args[1], args[0]);
+    PyObject* rest[16];
+    rest[0] = args[0];
+    for (Py_ssize_t i = 2; i < m; ++i) rest[i - 1] = args[i];
+    if (!c.ok || !convert(kinds, rest, m - 1, nullptr, v)) return false;
+    *ch = (const nnv_choice_t*)P(c.v);
+    return true;
+}
+
+// nnv_cold_run(plan, choices, h_weights, w_bytes, h_cached, c_bytes, h_input, h_output, d_arena, arena_bytes, s_copy, s_xform, s_exec, depth)
+PyObject* cold_run(PyObject*, PyObject* const* args, Py_ssize_t n, PyObject* kw) {
+    uint64_t v[13];
+    const nnv_choice_t* ch;
+    if (!convert_run("paiaiaaaisssi", args, n, kw, &ch, v)) return PyObject_Vectorcall(g_fallback[3], args, n, kw);
+    nnv_status_t st;
+    Py_BEGIN_ALLOW_THREADS
+    st = nnv_cold_run((nnv_plan_t*)P(v[0]), ch, P(v[1]), v[2], P(v[3]), v[4], (const float*)P(v[5]), (float*)P(v[6]), P(v[7]), v[8], P(v[9]), P(v[10]),
+                      P(v[11]), (int32_t)v[12], nullptr);
+    Py_END_ALLOW_THREADS
+    return finish(st);
+}
+
+// nnv_resident_run(plan, choices, d_weights, w_bytes, d_cached, c_bytes, d_input, d_output, d_arena, arena_bytes, s_xform, s_exec, depth)
+PyObject* resident_run(PyObject*, PyObject* const* args, Py_ssize_t n, PyObject* kw) {
+    uint64_t v[12];
+    const nnv_choice_t* ch;
+    if (!convert_run("paiaiaaaissi", args, n, kw, &ch, v)) return PyObject_Vectorcall(g_fallback[4], args, n, kw);
+    nnv_status_t st;
+    Py_BEGIN_ALLOW_THREADS
+    st = nnv_resident_run((nnv_plan_t*)P(v[0]), ch, P(v[1]), v[2], P(v[3]), v[4], (const float*)P(v[5]), (float*)P(v[6]), P(v[7]), v[8], P(v[9]),
+                          P(v[10]), (int32_t)v[11], nullptr);
+    Py_END_ALLOW_THREADS
+    return finish(st);
+}
+
+// nnv_warm_run(plan, warm, d_warm, warm_bytes, w_bytes, h_input, h_output, d_arena, arena_bytes, s_xform, s_exec)
+PyObject* warm_run(PyObject*, PyObject* const* args, Py_ssize_t n, PyObject* kw) {
+    uint64_t v[10];
+    const nnv_choice_t* ch;
+    if (!convert_run("paiiaaaiss", args, n, kw, &ch, v)) return PyObject_Vectorcall(g_fallback[5], args, n, kw);
+    nnv_status_t st;
+    Py_BEGIN_ALLOW_THREADS
+    st = nnv_warm_run((nnv_plan_t*)P(v[0]), ch, P(v[1]), v[2], v[3], (const float*)P(v[4]), (float*)P(v[5]), P(v[6]), v[7], P(v[8]), P(v[9]), nullptr);
+    Py_END_ALLOW_THREADS
+    return finish(st);
+}
+
 PyObject* set_fallbacks(PyObject*, PyObject* const* args, Py_ssize_t n) {
-    if (n != 6) {
-        PyErr_SetString(PyExc_TypeError, "four functions and two classes expected");
+    if (n != 9) {
+        PyErr_SetString(PyExc_TypeError, "seven functions and two classes expected");
         return nullptr;
     }
-    for (int i = 0; i < 3; ++i) Py_XSETREF(g_fallback[i], Py_NewRef(args[i]));
-    Py_XSETREF(g_check, Py_NewRef(args[3]));
-    Py_XSETREF(g_array, Py_NewRef(args[4]));
-    Py_XSETREF(g_choice, Py_NewRef(args[5]));
+    for (int i = 0; i < 6; ++i) Py_XSETREF(g_fallback[i], Py_NewRef(args[i]));
+    Py_XSETREF(g_check, Py_NewRef(args[6]));
+    Py_XSETREF(g_array, Py_NewRef(args[7]));
+    Py_XSETREF(g_choice, Py_NewRef(args[8]));
     Py_RETURN_NONE;
 }
 
@@ -159,6 +211,9 @@ PyMethodDef g_methods[] = {
     {"nnv_conv_exec", (PyCFunction)(void (*)(void))conv_exec, METH_FASTCALL | METH_KEYWORDS, nullptr},
     {"nnv_transform_weights", (PyCFunction)(void (*)(void))transform_weights, METH_FASTCALL | METH_KEYWORDS, nullptr},
     {"nnv_transform_all", (PyCFunction)(void (*)(void))transform_all, METH_FASTCALL | METH_KEYWORDS, nullptr},
+    {"nnv_cold_run", (PyCFunction)(void (*)(void))cold_run, METH_FASTCALL | METH_KEYWORDS, nullptr},
+    {"nnv_resident_run", (PyCFunction)(void (*)(void))resident_run, METH_FASTCALL | METH_KEYWORDS, nullptr},
+    {"nnv_warm_run", (PyCFunction)(void (*)(void))warm_run, METH_FASTCALL | METH_KEYWORDS, nullptr},
     {"set_fallbacks", (PyCFunction)(void (*)(void))set_fallbacks, METH_FASTCALL, nullptr},
     {nullptr, nullptr, 0, nullptr}};
 
