@@ -2008,6 +2008,7 @@ nnv_status_t launch_inverted_bottleneck(const nnv_layer_desc_t& a, const nnv_lay
         NNV_TRY(encode_operand(&tmW2, io.w2, false, p.C, p.K, 1, Qp2, (int64_t)p.K * Qp2, s->BN2 / w2_boxes));
     }
     IbDev g{};
+    g.early = io.early;
     g.e = io.e; g.d = io.d; g.y = io.y; g.b1 = io.b1; g.b2 = io.b2; g.b3 = io.b3; g.addend = io.addend; g.wd = io.wd;
     g.E = a.K; g.K = p.K; g.H = a.H; g.W = a.W; g.OH = p.H; g.OW = p.W; g.stride = d.stride;
     g.most1 = a.act == 2 ? 6.f : INFINITY; g.most2 = d.act == 2 ? 6.f : INFINITY; g.act3 = p.act;

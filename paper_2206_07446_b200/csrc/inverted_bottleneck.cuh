@@ -30,7 +30,7 @@ struct IbDev {
     float* e; float* d; float* y;                             // outputs: expansion, depthwise, projection
     const float* b1; const float* b2; const float* b3;        // biases or null
     const float* addend; const float* wd;                     // residual of the projection or null; raw depthwise weights [E][9]
-    int E, K, H, W, OH, OW, stride, act3;
+    int E, K, H, W, OH, OW, stride, act3, early;
     float most1, most2;                                       // upper bounds of the first two activations
     int ph, pw, hw, rows, px, tiles_w;                        // patch, width and pixels of its halo, pixels of the patch
     int nkb1, nb_most, step, both, ranks, splits, BN2, w2_boxes, issuers, tmem_cols;
@@ -130,50 +130,57 @@ inverted_bottleneck_kernel(const __grid_constant__ CUtensorMap tmX, const __grid
     }
     const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t*>(sm + (holder - sbase));
     const uint32_t tacc = tmem_base + ((uint32_t)(quarter * 32) << 16);
-    pdl_wait();
-    pdl_trigger();
-
-    // Loads, dealt to the warps (each costs its thread ~165 cycles): the pixels by warps 0 and 7, what later phases need behind them, the
-    // expansion's weights by warps 2 - 5 and 8 - 15.
-    bool ok = true;
-    if (warp == 0 || warp == 7) {
-        if (elect_one()) {
-            for (int kb = warp == 0 ? 0 : 1; kb < g.nkb1; kb += 2) {
-                mbar_expect_tx(full_bar(kb), (uint32_t)g.rows * 128u);
-                tma_load_3d(sbase + kb * x_stage, &tmX, kb * 32, iw0, ih0, full_bar(kb));
+    // Loads, dealt to the warps (each costs its thread ~165 cycles): the pixels by warps 0 and 7, what later phases need by them as well, the
+    // expansion's weights by warps 2 - 5 and 8 - 15.  Weights that nothing before this launch in its stream still writes are fetched before the wait for
+    // the previous kernel.
+    auto load_weights = [&]() {
+        if (warp == 0) {
+            // a block's biases and raw depthwise taps [channel][9], as far as its channels exist
+            uint32_t bytes = g.b3 ? (uint32_t)g.K * 4u : 0u;
+            for (int j = 0; j < nb; ++j)
+                bytes += (uint32_t)min(32, g.E - (first + j * g.step) * 32) * (36u + (g.b1 ? 4u : 0u) + (g.b2 ? 4u : 0u));
+            mbar_expect_tx(par_bar, bytes);
+            for (int j = 0; j < nb; ++j) {
+                const int c = (first + j * g.step) * 32;
+                const uint32_t n = (uint32_t)min(32, g.E - c);
+                if (g.b1) bulk_load(smem_u32(sb1 + j * 32), g.b1 + c, n * 4u, par_bar);
+                bulk_load(smem_u32(swd + j * 288), g.wd + (long long)c * 9, n * 36u, par_bar);
+                if (g.b2) bulk_load(smem_u32(sb2 + j * 32), g.b2 + c, n * 4u, par_bar);
             }
-            if (warp == 0) {
-                // a block's biases and raw depthwise taps [channel][9], as far as its channels exist
-                uint32_t bytes = g.b3 ? (uint32_t)g.K * 4u : 0u;
-                for (int j = 0; j < nb; ++j)
-                    bytes += (uint32_t)min(32, g.E - (first + j * g.step) * 32) * (36u + (g.b1 ? 4u : 0u) + (g.b2 ? 4u : 0u));
-                mbar_expect_tx(par_bar, bytes);
-                for (int j = 0; j < nb; ++j) {
-                    const int c = (first + j * g.step) * 32;
-                    const uint32_t n = (uint32_t)min(32, g.E - c);
-                    if (g.b1) bulk_load(smem_u32(sb1 + j * 32), g.b1 + c, n * 4u, par_bar);
-                    bulk_load(smem_u32(swd + j * 288), g.wd + (long long)c * 9, n * 36u, par_bar);
-                    if (g.b2) bulk_load(smem_u32(sb2 + j * 32), g.b2 + c, n * 4u, par_bar);
-                }
-                if (g.b3) bulk_load(smem_u32(sb3), g.b3, (uint32_t)g.K * 4u, par_bar);
-            } else {
-                mbar_expect_tx(w2_bar, (uint32_t)nb * w2_stage);
-                const int box = g.BN2 / g.w2_boxes;
-                for (int j = 0; j < nb; ++j)
-                    for (int h = 0; h < g.w2_boxes; ++h)
-                        tma_load_3d(sbase + g.w2_off + j * w2_stage + (uint32_t)(h * box) * W_ROW, &tmW2, (first + j * g.step) * 32, h * box, 0, w2_bar);
-            }
-        }
-        __syncwarp();
-    } else if (warp != 1 && warp != 6) {
-        if (elect_one()) {
+            if (g.b3) bulk_load(smem_u32(sb3), g.b3, (uint32_t)g.K * 4u, par_bar);
+        } else if (warp == 7) {
+            mbar_expect_tx(w2_bar, (uint32_t)nb * w2_stage);
+            const int box = g.BN2 / g.w2_boxes;
+            for (int j = 0; j < nb; ++j)
+                for (int h = 0; h < g.w2_boxes; ++h)
+                    tma_load_3d(sbase + g.w2_off + j * w2_stage + (uint32_t)(h * box) * W_ROW, &tmW2, (first + j * g.step) * 32, h * box, 0, w2_bar);
+        } else if (warp != 1 && warp != 6) {
             for (int i = warp < 8 ? warp - 2 : warp - 4; i < g.nkb1 * nb; i += 12) {
                 const int kb = i / nb, j = i - kb * nb;
                 mbar_expect_tx(full_bar(kb), W1_BOX);
                 tma_load_3d(sbase + g.w1_off + (uint32_t)i * W1_BOX, &tmW1, kb * 32, (first + j * g.step) * 32, 0, full_bar(kb));
             }
         }
+    };
+    if (g.early) {
+        if (elect_one()) load_weights();
         __syncwarp();
+    }
+    pdl_wait();
+    pdl_trigger();
+    bool ok = true;
+    if ((warp == 0 || warp == 7) && elect_one()) {
+        for (int kb = warp == 0 ? 0 : 1; kb < g.nkb1; kb += 2) {
+            mbar_expect_tx(full_bar(kb), (uint32_t)g.rows * 128u);
+            tma_load_3d(sbase + kb * x_stage, &tmX, kb * 32, iw0, ih0, full_bar(kb));
+        }
+    }
+    __syncwarp();
+    if (!g.early && elect_one()) load_weights();
+    __syncwarp();
+    if (warp == 0 || warp == 7) {
+        // (through with their loads)
+    } else if (warp != 1 && warp != 6) {
         if constexpr (BF16) {
             // the pixels, rounded to bf16 (a row a thread; warps 8 - 11 and 12 - 15 take the blocks in turn): what the MMAs read
             if (warp >= 8)

@@ -374,6 +374,7 @@ struct IbBuffers {
     const float* x; const void* w1; const float* wd; const void* w2;      // input, packed weights, raw depthwise weights
     const float* b1; const float* b2; const float* b3; const float* addend;
     float* e; float* d; float* y;                                          // the three layers' outputs
+    bool early;                                                            // the weights are complete before anything in the launch's stream that it may overtake
 };
 bool inverted_bottleneck_applies(const nnv_layer_desc_t& expand, const nnv_layer_desc_t& depthwise, const nnv_layer_desc_t& project, int math);
 nnv_status_t launch_inverted_bottleneck(const nnv_layer_desc_t& expand, const nnv_layer_desc_t& depthwise, const nnv_layer_desc_t& project,

@@ -551,6 +551,7 @@ static nnv_status_t run_model(nnv_plan* p, const nnv_choice_t* choices, const vo
         const void* add = L.in1 >= 0 ? base + A.act_off[L.in1] : nullptr;
         if (fused[i]) {
             block = IbBuffers{};
+            block.early = !queued;                            // (events order the weights before this stream; a queue's preparations may run in it)
             block.x = (const float*)in; block.w1 = xf; block.b1 = L.has_bias ? (const float*)bias : nullptr; block.e = (float*)out;
             continue;
         }
