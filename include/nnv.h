@@ -608,8 +608,9 @@ nnv_status_t nnv_last_enqueue_ns(const nnv_plan_t* plan, uint64_t* ns);
  * last block's end of layer i's weight-transform launch (a grouped launch is booked on the first
  * layer of its group, the others get 0), exec_ns[i] = the same for the layer's tensor-core GEMM
  * kernel (0 for layers executed by other kernels).  Unlike event pairs around a kernel, which add
- * microseconds of their own and serialise the streams, the stamps do not disturb the run they
- * measure.  Both arrays hold one entry per layer; either may be NULL.  Synchronises the device. */
+ * microseconds of their own and serialise the streams, the stamps do not disturb the kernels they
+ * measure.  Runs with stamps or timings execute every layer by its own launches: blocks and layers
+ * that other runs fuse into one launch (with the same result bits) are apart in them.  Both arrays hold one entry per layer; either may be NULL.  Synchronises the device. */
 nnv_status_t nnv_kernel_times(const nnv_plan_t* plan, uint64_t* xform_ns, uint64_t* exec_ns);
 
 /* The same stamps as a timeline: xform_span[2i], xform_span[2i+1] = start and end of layer i's

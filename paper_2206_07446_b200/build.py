@@ -10,7 +10,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libnnv.so")
 PYCALL = os.path.join(HERE, "_nnvcall.so")
-SOURCES = ["plan.cpp", "scheduler.cpp", "cachefile.cpp", "transform.cu", "exec_kernels.cu", "direct_conv.cu", "wino_small.cu", "gemm_tc.cu", "exec.cu", "pipeline.cu", "noalloc.cu"]
+SOURCES = ["plan.cpp", "scheduler.cpp", "cachefile.cpp", "transform.cu", "exec_kernels.cu", "direct_conv.cu", "wino_small.cu", "wino_layer.cu", "gemm_tc.cu", "exec.cu", "pipeline.cu", "noalloc.cu"]
 
 
 def sources():

@@ -73,7 +73,7 @@ nnv_status_t do_exec(const nnv_plan& p, int layer, int v, int math, const void* 
         a.split_a = m != 2 && (g.Cp % 32) == 0 && !small;
         NNV_TRY(launch_wino_input(m, bf16, a.split_a, x, V, L.C, g.Cp, L.H, L.W, L.pad, TH, TW, st));
         if (small) {
-            NNV_TRY(launch_wino_small(m, (const float*)V, (const float*)d_wt, Mt, T, L.K, g.Cp, st));
+            NNV_TRY(launch_wino_small(m, (const float*)V, (const float*)d_wt, Mt, T, L.K, L.C, g.Cp, st));
             return launch_wino_output(m, Mt, y, bias, add, L.act, L.K, g.OH, g.OW, TH, TW, st);
         }
         a.A = V; a.B = d_wt; a.D = Mt;

@@ -6,6 +6,7 @@
 #include <type_traits>
 
 #include "nnv_internal.h"
+#include "wino_tables.cuh"
 
 namespace nnv {
 
@@ -131,56 +132,6 @@ nnv_status_t launch_im2col(bool bf16, const float* x, void* col, int C, int H, i
 }
 
 // ---- Winograd data transforms ---------------------------------------------------------------
-// B^T (alpha x alpha) and A^T (m x alpha) of the same Cook-Toom construction as the filter
-// transform's G: finite points {0, 1, -1, 2, -2, 1/2, -1/2} in that order, then infinity.
-template <int M_> struct WinoBA;
-template <> struct WinoBA<2> {
-    static constexpr int A = 4;
-    __host__ __device__ static constexpr float bt(int r, int c) {
-        constexpr float t[4][4] = {{1, 0, -1, 0}, {0, 1, 1, 0}, {0, -1, 1, 0}, {0, -1, 0, 1}};
-        return t[r][c];
-    }
-    __host__ __device__ static constexpr float at(int r, int c) {
-        constexpr float t[2][4] = {{1, 1, 1, 0}, {0, 1, -1, 1}};
-        return t[r][c];
-    }
-};
-template <> struct WinoBA<4> {
-    static constexpr int A = 6;
-    __host__ __device__ static constexpr float bt(int r, int c) {
-        constexpr float t[6][6] = {{4, 0, -5, 0, 1, 0},  {0, -4, -4, 1, 1, 0}, {0, 4, -4, -1, 1, 0},
-                                   {0, -2, -1, 2, 1, 0}, {0, 2, -1, -2, 1, 0}, {0, 4, 0, -5, 0, 1}};
-        return t[r][c];
-    }
-    __host__ __device__ static constexpr float at(int r, int c) {
-        constexpr float t[4][6] = {{1, 1, 1, 1, 1, 0}, {0, 1, -1, 2, -2, 0}, {0, 1, 1, 4, 4, 0}, {0, 1, -1, 8, -8, 1}};
-        return t[r][c];
-    }
-};
-template <> struct WinoBA<6> {
-    static constexpr int A = 8;
-    __host__ __device__ static constexpr float bt(int r, int c) {
-        constexpr float t[8][8] = {{1, 0, -5.25f, 0, 5.25f, 0, -1, 0},
-                                   {0, 1, 1, -4.25f, -4.25f, 1, 1, 0},
-                                   {0, -1, 1, 4.25f, -4.25f, -1, 1, 0},
-                                   {0, .5f, .25f, -2.5f, -1.25f, 2, 1, 0},
-                                   {0, -.5f, .25f, 2.5f, -1.25f, -2, 1, 0},
-                                   {0, 2, 4, -2.5f, -5, .5f, 1, 0},
-                                   {0, -2, 4, 2.5f, -5, -.5f, 1, 0},
-                                   {0, -1, 0, 5.25f, 0, -5.25f, 0, 1}};
-        return t[r][c];
-    }
-    __host__ __device__ static constexpr float at(int r, int c) {
-        constexpr float t[6][8] = {{1, 1, 1, 1, 1, 1, 1, 0},
-                                   {0, 1, -1, 2, -2, .5f, -.5f, 0},
-                                   {0, 1, 1, 4, 4, .25f, .25f, 0},
-                                   {0, 1, -1, 8, -8, .125f, -.125f, 0},
-                                   {0, 1, 1, 16, 16, .0625f, .0625f, 0},
-                                   {0, 1, -1, 32, -32, .03125f, -.03125f, 1}};
-        return t[r][c];
-    }
-};
-
 // Two forms of each data transform.  A thread per (tile, channel) loads A*A values, works through ~2 A*A*A multiply-adds and stores as
 // many: on a layer of a few thousand of them (512 -> 512 @7, F(4,3): 16 blocks) a handful of warps do everything one after the other.
 // So up to WT_BLOCKS blocks the work of a tile is dealt to A warps: a warp for every column of the tile and then, through shared memory,
@@ -231,28 +182,23 @@ wino_input_kernel(const float* __restrict__ x, OutT* __restrict__ V, int C, int 
             d[i][j] = (c < C && h >= 0 && h < H && w >= 0 && w < W) ? __ldg(x + ((long long)h * W + w) * C + c) : 0.f;
         }
     }
-    float tmp[A][A];                                             // tmp = B^T d
 #pragma unroll
-    for (int i = 0; i < A; ++i)
+    for (int j = 0; j < A; ++j) {                                // B^T d
+        float col[A], v[A];
 #pragma unroll
-        for (int j = 0; j < A; ++j) {
-            float s = 0.f;
+        for (int i = 0; i < A; ++i) col[i] = d[i][j];
+        wino_input(col, v);
 #pragma unroll
-            for (int l = 0; l < A; ++l)
-                if (WinoBA<M_>::bt(i, l) != 0.f) s += WinoBA<M_>::bt(i, l) * d[l][j];
-            tmp[i][j] = s;
-        }
+        for (int i = 0; i < A; ++i) d[i][j] = v[i];
+    }
     OutT* out = V + (long long)t * Cp + wino_word<SPLIT>(c);
 #pragma unroll
-    for (int i = 0; i < A; ++i)
+    for (int i = 0; i < A; ++i) {                                // (B^T d) B
+        float v[A];
+        wino_input(d[i], v);
 #pragma unroll
-        for (int j = 0; j < A; ++j) {                            // V = tmp B
-            float s = 0.f;
-#pragma unroll
-            for (int l = 0; l < A; ++l)
-                if (WinoBA<M_>::bt(j, l) != 0.f) s += tmp[i][l] * WinoBA<M_>::bt(j, l);
-            out[(long long)(i * A + j) * T * Cp] = wino_operand<M_, OutT, SPLIT>(s, c);
-        }
+        for (int j = 0; j < A; ++j) out[(long long)(i * A + j) * T * Cp] = wino_operand<M_, OutT, SPLIT>(v[j], c);
+    }
 }
 
 // A block takes one tile and 32 channels.
@@ -274,24 +220,17 @@ wino_input_tile_kernel(const float* __restrict__ x, OutT* __restrict__ V, int C,
     float d[A];
 #pragma unroll
     for (int l = 0; l < A; ++l) d[l] = inside && h0 + l >= 0 && h0 + l < H ? __ldg(src + (long long)l * W * C) : 0.f;
+    float s[A];
+    wino_input(d, s);
 #pragma unroll
-    for (int i = 0; i < A; ++i) {
-        float s = 0.f;
-#pragma unroll
-        for (int l = 0; l < A; ++l)
-            if (WinoBA<M_>::bt(i, l) != 0.f) s += WinoBA<M_>::bt(i, l) * d[l];
-        tmp[i][col][lane] = s;
-    }
+    for (int i = 0; i < A; ++i) tmp[i][col][lane] = s[i];
     __syncthreads();
 #pragma unroll
     for (int l = 0; l < A; ++l) d[l] = tmp[col][l][lane];        // the warp's row
+    wino_input(d, s);                                            // V = tmp B
 #pragma unroll
-    for (int j = 0; j < A; ++j) {                                // V = tmp B
-        float s = 0.f;
-#pragma unroll
-        for (int l = 0; l < A; ++l)
-            if (WinoBA<M_>::bt(j, l) != 0.f) s += d[l] * WinoBA<M_>::bt(j, l);
-        const OutT v = wino_operand<M_, OutT, SPLIT>(s, c);      // (a shuffle: by all lanes)
+    for (int j = 0; j < A; ++j) {
+        const OutT v = wino_operand<M_, OutT, SPLIT>(s[j], c);   // (a shuffle: by all lanes)
         if (c < Cp) out[j * plane] = v;
     }
 }

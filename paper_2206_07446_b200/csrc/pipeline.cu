@@ -299,6 +299,18 @@ static nnv_status_t run_model(nnv_plan* p, const nnv_choice_t* choices, const vo
         }
     }
 
+    // Winograd layers that run as one launch from their raw weights: neither transformed weights nor the data transforms' results are written.
+    // Not where the stages are to be timed each, nor in a pass that prepares the weights for later ones.
+    std::vector<char> from_raw(n, 0);
+    if (!tm && !stamp_base && !wc) {
+        for (int i = 0; i < n; ++i) {
+            const nnv_layer_desc_t& L = p->layers[i];
+            if (L.op != NNV_OP_CONV || on_side[i] || choices[i].cached == NNV_ARM_CACHED || (choices[i].cached == NNV_ARM_ZERO_COPY && !resident)) continue;
+            const int m = wino_m(choices[i].variant);
+            from_raw[i] = m > 2 && wino_layer_applies(m, L.C, L.K, ceil_div(p->geom[i].OH, m) * ceil_div(p->geom[i].OW, m));
+        }
+    }
+
     // Everything the pass puts on the streams: fork from s_exec, the per-layer operations, join back.
     auto enqueue = [&]() -> nnv_status_t {
     if (stamp_base) NNV_CUDA(cudaMemsetAsync(stamp_base, 0, sizeof(unsigned long long) * 2 * STAMP_SLOTS_PER_LAYER * n, s_exec));
@@ -360,7 +372,7 @@ static nnv_status_t run_model(nnv_plan* p, const nnv_choice_t* choices, const vo
             const nnv_layer_desc_t& L = p->layers[i];
             if (L.op != NNV_OP_CONV) continue;
             const nnv_choice_t ch = choices[i];
-            if (!variant_has_transform(ch.variant) || ch.cached == NNV_ARM_CACHED) continue;
+            if (!variant_has_transform(ch.variant) || ch.cached == NNV_ARM_CACHED || from_raw[i]) continue;
             const XformDesc d = make_xform_desc(*p, i, ch, (const uint8_t*)weights + L.w_off, base + A.xf_off[i]);
             const int g = first_bytes < (1u << 20) ? 0 : first_bytes < (9u << 20) ? 1 : 2;
             first_bytes += raw_weight_bytes(L);
@@ -405,7 +417,7 @@ static nnv_status_t run_model(nnv_plan* p, const nnv_choice_t* choices, const vo
         const uint8_t* raw = depth ? base + A.raw_slot0 + (uint64_t)slot * A.raw_slot_bytes : base + A.raw_off[i];
         const uint8_t* bias = depth ? raw + A.raw_bias_off : base + A.bias_off[i];
         const uint8_t* xf = depth ? base + A.xf_slot0 + (uint64_t)slot * A.xf_slot_bytes : base + A.xf_off[i];
-        const bool has_xf = variant_has_transform(ch.variant);
+        const bool has_xf = variant_has_transform(ch.variant) && !from_raw[i];
         const bool cached = has_xf && ch.cached == NNV_ARM_CACHED;
         // zero-copy arm: no copy, the transform kernel reads the host blob itself (with the weights already on the
         // device, or when the raw copy has to stay for warm runs, it is the raw arm)
@@ -481,7 +493,7 @@ static nnv_status_t run_model(nnv_plan* p, const nnv_choice_t* choices, const vo
                     std::vector<XformDesc> descs;
                     for (int k = c.first; k <= c.last; ++k) {
                         const nnv_layer_desc_t& Lk = p->layers[k];
-                        if (Lk.op != NNV_OP_CONV || !variant_has_transform(choices[k].variant) || choices[k].cached == NNV_ARM_CACHED) continue;
+                        if (Lk.op != NNV_OP_CONV || !variant_has_transform(choices[k].variant) || choices[k].cached == NNV_ARM_CACHED || from_raw[k]) continue;
                         if ((choices[k].cached == NNV_ARM_ZERO_COPY) != c.zero_copy) continue;
                         XformDesc d = make_xform_desc(*p, k, choices[k], c.zero_copy ? (const void*)((const uint8_t*)weights + Lk.w_off)
                                                                                    : (const void*)(base + A.raw_off[k]), base + A.xf_off[k]);
@@ -564,6 +576,12 @@ static nnv_status_t run_model(nnv_plan* p, const nnv_choice_t* choices, const vo
             NNV_TRY(launch_inverted_bottleneck(p->layers[i - 2], p->layers[i - 1], L, ch.math, block, se));
             for (int k = i - 2; k <= i; ++k)
                 if (need_done[k]) NNV_CUDA(cudaEventRecord(EV(k, 2), se));
+            continue;
+        }
+        if (from_raw[i]) {
+            NNV_TRY(launch_wino_layer(wino_m(ch.variant), (const float*)in, (const float*)raw, L.has_bias ? (const float*)bias : nullptr,
+                                      (const float*)add, (float*)out, L.act, L.C, L.H, L.W, L.K, L.pad, p->geom[i].OH, p->geom[i].OW, !queued, se));
+            if (need_done[i]) NNV_CUDA(cudaEventRecord(EV(i, 2), se));
             continue;
         }
         stamp_for(i, 1);

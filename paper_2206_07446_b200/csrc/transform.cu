@@ -7,48 +7,12 @@
 #include <type_traits>
 
 #include "nnv_internal.h"
+#include "wino_tables.cuh"
 
 // (without a preference for the L1's split: see launch_pdl_attrs)
 #define XF_LAUNCH(kernel, grid, block, st, ...) (void)launch_pdl_attrs(NO_CARVEOUT, 1, kernel, dim3(grid), dim3(block), 0, st, __VA_ARGS__)
 
 namespace nnv {
-
-// G matrices of the Cook-Toom construction with points {0, +-1, +-2, +-1/2, inf} (the published
-// F(m,3) minimal-filtering matrices); row j belongs to point j, the last row to infinity.
-template <int M_> struct WinoG;
-template <> struct WinoG<2> {
-    static constexpr int A = 4;
-    __host__ __device__ static constexpr float g(int r, int c) {
-        constexpr float t[4][3] = {{1.f, 0.f, 0.f}, {.5f, .5f, .5f}, {.5f, -.5f, .5f}, {0.f, 0.f, 1.f}};
-        return t[r][c];
-    }
-};
-template <> struct WinoG<4> {
-    static constexpr int A = 6;
-    __host__ __device__ static constexpr float g(int r, int c) {
-        constexpr float t[6][3] = {{1.f / 4.f, 0.f, 0.f},
-                                   {-1.f / 6.f, -1.f / 6.f, -1.f / 6.f},
-                                   {-1.f / 6.f, 1.f / 6.f, -1.f / 6.f},
-                                   {1.f / 24.f, 1.f / 12.f, 1.f / 6.f},
-                                   {1.f / 24.f, -1.f / 12.f, 1.f / 6.f},
-                                   {0.f, 0.f, 1.f}};
-        return t[r][c];
-    }
-};
-template <> struct WinoG<6> {
-    static constexpr int A = 8;
-    __host__ __device__ static constexpr float g(int r, int c) {
-        constexpr float t[8][3] = {{1.f, 0.f, 0.f},
-                                   {-2.f / 9.f, -2.f / 9.f, -2.f / 9.f},
-                                   {-2.f / 9.f, 2.f / 9.f, -2.f / 9.f},
-                                   {1.f / 90.f, 1.f / 45.f, 2.f / 45.f},
-                                   {1.f / 90.f, -1.f / 45.f, 2.f / 45.f},
-                                   {32.f / 45.f, 16.f / 45.f, 8.f / 45.f},
-                                   {32.f / 45.f, -16.f / 45.f, 8.f / 45.f},
-                                   {0.f, 0.f, 1.f}};
-        return t[r][c];
-    }
-};
 
 // Four consecutive values of a plane: 16 bytes of fp32, 8 of bf16.
 __device__ __forceinline__ void store_plane4(float* p, const float* v) { *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]); }
@@ -158,13 +122,12 @@ __device__ __forceinline__ void filter_transform_block(const float* __restrict__
         for (int j = 0; j < NF; ++j)
 #pragma unroll
             for (int i = 0; i < 3; ++i)
-                t[j][i] = w[j][i * 3 + 0] * WinoG<M_>::g(nu, 0) + w[j][i * 3 + 1] * WinoG<M_>::g(nu, 1) +
-                          w[j][i * 3 + 2] * WinoG<M_>::g(nu, 2);
+                t[j][i] = wino_filter<M_>(nu, w[j][i * 3], w[j][i * 3 + 1], w[j][i * 3 + 2]);
     };
     auto plane_values = [&](int xi, const float (&t)[NF][3], float* v) {
 #pragma unroll
         for (int j = 0; j < NF; ++j) {
-            v[j] = WinoG<M_>::g(xi, 0) * t[j][0] + WinoG<M_>::g(xi, 1) * t[j][1] + WinoG<M_>::g(xi, 2) * t[j][2];
+            v[j] = wino_filter<M_>(xi, t[j][0], t[j][1], t[j][2]);
             if (pad[j]) v[j] = 0.f;                              // padded channels hold +0, never -0
         }
     };

@@ -6,7 +6,9 @@
 //   - A block owns 64 output channels of one plane b; V's plane lies in shared memory.  Eight warps: four groups of 16 channels x two halves of the
 //     input channels.  Eight lanes read 128 contiguous bytes of a channel's row, a warp four rows at a time, sixteen in all, so that a word of V
 //     read from shared memory serves four rows of a lane.
-//   - The lanes' sums are reduced by exchanging halves (3.5 T shuffles), the halves of the input channels through shared memory; the order is fixed.
+//   - The lanes' sums are reduced by exchanging halves (3.5 T shuffles), the halves of the input channels through shared memory; the order is fixed,
+//     and wino_layer.cu's is the same: a layer has the same bits whether its weights come transformed or raw.  (Where that kernel deals the channels to eight
+//     blocks, a half is summed as two quarters.)
 // 512 -> 512 F(4,3) @7 in a model, U in the L2: 7.4 us against 11.3 on the tensor cores.
 #include <algorithm>
 #include <type_traits>
@@ -22,13 +24,14 @@ constexpr int WS_K = 64, WS_THREADS = 256;
 template <int T, int UN>
 __global__ void __launch_bounds__(WS_THREADS, 2)
 wino_small_kernel(const float* __restrict__ V, const float* __restrict__ U, float* __restrict__ M, int tiles, int K, int Cp,
-                  unsigned long long* stamp) {
+                  int quarters, unsigned long long* stamp) {
     extern __shared__ __align__(16) float sv[];                // V's plane [T][pitch], later the partial sums [2][64][T + 1]
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int cl = lane & 7, rl = lane >> 3, rg = warp & 3, half = warp >> 2;
     const int b = blockIdx.y, k0 = blockIdx.x * WS_K;
     const int pitch = ((Cp + 31) & ~31) + 4;                   // (eight lanes read 128 bytes of a row: any pitch will do)
     const int blocks = (Cp + 31) / 32, i0 = blocks * half / 2, i1 = blocks * (half + 1) / 2;
+    const int middle = T <= 4 && quarters ? blocks * (2 * half + 1) / 4 : -1;    // where a sum of its own begins
     const float* const u = U + ((long long)b * K + k0 + rg * 16 + rl) * Cp + 4 * cl;
     const int rows = K - k0 - rg * 16 - rl;                    // rows 4 r of this lane that exist: 4 r < rows
     float acc[4][T];
@@ -36,6 +39,11 @@ wino_small_kernel(const float* __restrict__ V, const float* __restrict__ U, floa
     for (int r = 0; r < 4; ++r)
 #pragma unroll
         for (int t = 0; t < T; ++t) acc[r][t] = 0.f;
+    float first[4][T <= 4 ? T : 1];
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int t = 0; t < (T <= 4 ? T : 1); ++t) first[r][t] = 0.f;
     float4 w[UN][4];
     auto fetch = [&](int i, float4 (&f)[4]) {
         const bool in = i < i1 && 32 * i + 4 * cl < Cp;
@@ -63,16 +71,30 @@ wino_small_kernel(const float* __restrict__ V, const float* __restrict__ U, floa
             for (int r = 0; r < 4; ++r) x[r] = w[n][r];
             fetch(i + UN + n, w[n]);
             // (a block beyond the half multiplies zeros with whatever V holds there: with V's own numbers, which may be infinite)
+            if constexpr (T <= 4) {
+                if (i + n == middle) {
+#pragma unroll
+                    for (int r = 0; r < 4; ++r)
+#pragma unroll
+                        for (int t = 0; t < T; ++t) { first[r][t] = acc[r][t]; acc[r][t] = 0.f; }
+                }
+            }
             if (i + n < i1) {
                 const float* row = sv + 32 * (i + n) + 4 * cl;
 #pragma unroll
                 for (int t = 0; t < T; ++t) {
                     const float4 y = *reinterpret_cast<const float4*>(row + t * pitch);
 #pragma unroll
-                    for (int r = 0; r < 4; ++r) acc[r][t] = fmaf(x[r].x, y.x, fmaf(x[r].y, y.y, fmaf(x[r].z, y.z, fmaf(x[r].w, y.w, acc[r][t]))));
+                    for (int r = 0; r < 4; ++r) acc[r][t] = fmaf(x[r].w, y.w, fmaf(x[r].z, y.z, fmaf(x[r].y, y.y, fmaf(x[r].x, y.x, acc[r][t]))));
                 }
             }
         }
+    }
+    if constexpr (T <= 4) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int t = 0; t < T; ++t) acc[r][t] = first[r][t] + acc[r][t];
     }
     // Eight lanes' sums: each exchange halves what a lane holds.  It ends up with row 2 (cl >> 2) + (cl >> 1 & 1) and half of the tiles.
     auto trade = [&](float keep_low, float keep_high, int bit) {
@@ -116,15 +138,16 @@ bool wino_small_applies(int m, int T, int Cp, int K) {
     return m != 2 && Cp <= 2048 && (T <= 8 ? bytes <= 40e6 : T <= 12 && bytes <= 5e6);
 }
 
-nnv_status_t launch_wino_small(int m, const float* V, const float* U, float* M, int T, int K, int Cp, cudaStream_t st) {
+nnv_status_t launch_wino_small(int m, const float* V, const float* U, float* M, int T, int K, int C, int Cp, cudaStream_t st) {
     unsigned long long* const stamp = next_stamp();
     next_stamp() = nullptr;
+    const int quarters = wino_layer_quarters(m, C, K, T);
     auto go = [&](auto tt, auto kernel) -> cudaError_t {
         constexpr int TT = decltype(tt)::value;
         const size_t smem = sizeof(float) * std::max((size_t)TT * (align_up(Cp, 32) + 4), (size_t)2 * WS_K * (TT + 1));
         static const cudaError_t attr = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(float) * TT * (2048 + 4)));
         if (attr != cudaSuccess) return attr;
-        return launch_pdl(kernel, dim3(ceil_div(K, WS_K), (m + 2) * (m + 2)), dim3(WS_THREADS), smem, st, V, U, M, T, K, Cp, stamp);
+        return launch_pdl(kernel, dim3(ceil_div(K, WS_K), (m + 2) * (m + 2)), dim3(WS_THREADS), smem, st, V, U, M, T, K, Cp, quarters, stamp);
     };
     const std::integral_constant<int, 4> t4;
     const std::integral_constant<int, 8> t8;
