@@ -31,7 +31,7 @@ def _model(C, K, H, W, pad, act, bias):
     (nb.VAR_WINO_F4, 256, 256, 14, 14, 1, 2, 1),       # sixteen tiles: the tensor cores'
     (nb.VAR_WINO_F4, 128, 128, 10, 11, 1, 0, 1),       # nine tiles, five groups
     (nb.VAR_WINO_F4, 4, 3, 2, 3, 1, 0, 0),             # less than a tile, a slice, a block of outputs; the second layer's three channels are another kernel's
-    (nb.VAR_WINO_F4, 36, 40, 5, 18, 1, 1, 1),          # channels and outputs that end inside their blocks, an odd number of tiles
+    (nb.VAR_WINO_F4, 36, 40, 5, 18, 1, 1, 1),          # channels and outputs that end inside their blocks
     (nb.VAR_WINO_F4, 64, 64, 23, 21, 1, 1, 1),         # more tiles still
     (nb.VAR_WINO_F4, 100, 132, 11, 8, 0, 2, 1),         # no padding
     (nb.VAR_WINO_F4, 72, 200, 6, 5, 2, 1, 0),          # an output larger than the input
