@@ -162,6 +162,10 @@ nnv_status_t nnv_plan_destroy(nnv_plan_t* plan);
  *   bf16cvt=0|1           BF16-math GEMMs read the fp32 activation and round it inside the kernel (1, default) or
  *                         from an explicit bf16 im2col matrix (0)
  *   winofused=auto|0|1    F(2x2,3x3) with TF32 math as one kernel (input transform, tile GEMMs, output transform)
+ *   winosmall=0|1         F(4,3) / F(6,3) layers of a few tiles on the fp32 tile GEMM (1, default; an override of the GEMM's
+ *                         tiling takes them to the tensor cores, which it is for)
+ *   winolayer=0|1         whole-model runs execute such layers from their raw weights as one launch (1, default)
+ *   block=0|1             whole-model runs execute inverted-residual blocks as one launch (1, default)
  *   smallp=0|1|N          the weights-on-rows kernel for layers of at most 256 pixels: off, on, on with N K splits
  *   side=0|1  merge=0|1  group=0|1   side stream for residual branches, merged reads, grouped transforms
  *   copies_first=0|1      merged reads are all put on the copy stream before the first kernel (1, default) or layer by layer

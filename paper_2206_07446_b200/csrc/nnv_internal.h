@@ -191,6 +191,8 @@ struct Tuning {
     int copies_first = 1;                     // merged reads all enqueued before the first kernel
     int chunk_first_kb = 1024, chunk_max_kb = 32768;   // merged reads: size target of the first chunk, doubling up to the maximum
     int winofused = -1;                       // the one-kernel F(2x2,3x3) path: -1 the library decides, 0 off, 1 on where it applies
+    int winosmall = 1, winolayer = 1;         // F(4,3) / F(6,3) on a few tiles: the fp32 tile GEMM, whole layers from raw weights as one launch
+    int block = 1;                            // inverted-residual blocks as one launch
     int bf16cvt = 1;                          // BF16 math straight from the fp32 activation (rounded inside the GEMM); 0: explicit bf16 im2col
     int smallp = 1;                           // the weights-on-rows kernel for layers with few pixels
     int smallp_splits = 0;                    // 0 = the cost model decides

@@ -284,7 +284,7 @@ static nnv_status_t run_model(nnv_plan* p, const nnv_choice_t* choices, const vo
     // same bit for bit.  Not where the layers are to be timed each, where fewer staging slots than layers hold their weights, or where
     // the weights arrive in different copies (the first layers would wait for the last one's).
     std::vector<char> fused(n, 0);
-    if (!tm && !stamp_base && (depth == 0 || depth >= 3)) {
+    if (tn.block && !tm && !stamp_base && (depth == 0 || depth >= 3)) {
         for (int i = 0; i + 2 < n; ++i) {
             const nnv_layer_desc_t &a = p->layers[i], &d = p->layers[i + 1], &q = p->layers[i + 2];
             if (a.op != NNV_OP_CONV || d.op != NNV_OP_CONV || q.op != NNV_OP_CONV) continue;
@@ -302,7 +302,7 @@ static nnv_status_t run_model(nnv_plan* p, const nnv_choice_t* choices, const vo
     // Winograd layers that run as one launch from their raw weights: neither transformed weights nor the data transforms' results are written.
     // Not where the stages are to be timed each, nor in a pass that prepares the weights for later ones.
     std::vector<char> from_raw(n, 0);
-    if (!tm && !stamp_base && !wc) {
+    if (tn.winolayer && !tm && !stamp_base && !wc) {
         for (int i = 0; i < n; ++i) {
             const nnv_layer_desc_t& L = p->layers[i];
             if (L.op != NNV_OP_CONV || on_side[i] || choices[i].cached == NNV_ARM_CACHED || (choices[i].cached == NNV_ARM_ZERO_COPY && !resident)) continue;

@@ -88,6 +88,12 @@ static const char* parse_tuning(const char* spec, Tuning* t, char* item, size_t 
         } else if (!std::strcmp(key, "winofused")) {
             if (!std::strcmp(val, "auto")) { t->winofused = -1; ok = true; }
             else ok = flag(&t->winofused);
+        } else if (!std::strcmp(key, "winosmall")) {
+            ok = flag(&t->winosmall);
+        } else if (!std::strcmp(key, "winolayer")) {
+            ok = flag(&t->winolayer);
+        } else if (!std::strcmp(key, "block")) {
+            ok = flag(&t->block);
         } else if (!std::strcmp(key, "bf16cvt")) {
             ok = flag(&t->bf16cvt);
         } else if (!std::strcmp(key, "smallp")) {

@@ -351,3 +351,11 @@ nnv_status_t launch_wino_layer(int m, const float* x, const float* w, const floa
 }
 
 }  // namespace nnv
+
+// Which kernels run an F(m,3) layer of `tiles` tiles, for the tests: the fp32 tile GEMM, a whole layer in one launch, that launch's tiles a block, slices
+// and quads of input channels.
+extern "C" void nnv_internal_wino_rule(int m, int C, int K, int tiles, int32_t* out) {
+    const nnv::WlPlan p = nnv::wl_plan(m, C, K, tiles);
+    const int32_t v[] = {nnv::wino_small_applies(m, tiles, (int)nnv::align_up(C, 8), K), p.use, p.T, p.slices, p.quads};
+    std::copy(std::begin(v), std::end(v), out);
+}

@@ -134,6 +134,8 @@ wino_small_kernel(const float* __restrict__ V, const float* __restrict__ U, floa
 // 512 -> 512 @7 16.4 / 15.3, F(6,3) 128 -> 128 @11 7.3 / 5.7, 256 -> 256 @11 11.7 / 9.5; with U of 67 MB (F(6,3) 512 -> 512 @11 21.9 / 23.0, F(4,3) 1024 -> 512
 // @7 23.4 / 23.4) and beyond eight tiles (F(4,3) 128 -> 128 @11 6.8 / 6.7, 512 -> 512 @11 16.0 / 18.2) the other has caught up.
 bool wino_small_applies(int m, int T, int Cp, int K) {
+    const Tuning& tn = tuning();
+    if (!tn.winosmall || tn.gemm_bn || tn.gemm_ring) return false;     // (overrides of the tensor cores' tile GEMM)
     const double bytes = 4.0 * (m + 2) * (m + 2) * K * Cp;
     return m != 2 && Cp <= 2048 && (T <= 8 ? bytes <= 40e6 : T <= 12 && bytes <= 5e6);
 }

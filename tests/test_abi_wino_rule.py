@@ -1,0 +1,31 @@
+"""Which kernels F(4,3) and F(6,3) layers of a few tiles run on (host arithmetic, no GPU)."""
+import ctypes
+
+import pytest
+
+from paper_2206_07446_b200 import binding as nb
+
+
+def rule(m, C, K, tiles):
+    out = (ctypes.c_int32 * 5)()
+    nb._lib.nnv_internal_wino_rule(m, C, K, tiles, out)
+    return dict(zip(("small", "layer", "T", "slices", "quads"), out))
+
+
+@pytest.mark.parametrize("m,C,K,tiles", [(4, 512, 512, 4), (4, 64, 64, 1), (6, 256, 256, 1), (6, 64, 96, 9)])
+def test_overrides_reach_layers_of_few_tiles(m, C, K, tiles):
+    """An override of the GEMM's tiling is for the tensor cores' tile GEMM, in every path that a layer takes."""
+    try:
+        nb.nnv_tuning_set("")
+        assert rule(m, C, K, tiles)["small"]
+        for spec in ("gemm_tile=64,2", "gemm_ring=4", "winosmall=0"):
+            nb.nnv_tuning_set(spec)
+            r = rule(m, C, K, tiles)
+            assert not r["small"] and not r["layer"], (spec, r)
+        nb.nnv_tuning_set("winosmall=1;winolayer=0;block=0")
+        assert rule(m, C, K, tiles)["small"]
+        for bad in ("winosmall=2", "winolayer=on", "block=-1"):
+            with pytest.raises(nb.NnvError):
+                nb.nnv_tuning_set(bad)
+    finally:
+        nb.nnv_tuning_set(None)
