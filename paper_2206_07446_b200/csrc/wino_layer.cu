@@ -297,18 +297,33 @@ wino_layer_kernel(const WlDev g) {
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// Tiles a block, slices and whether the layer is to run here: within one wave at two blocks an SM (more pays the filter transform too often:
-// F(4,3) 512 -> 512 @14 23.7 us without, 38 with, 384 -> 384 @14 15.3 / 25), where wino_small.cu runs the tile GEMM for transformed weights, whose sums it
-// follows.  Two tiles a block (four: as fast alone, but then only eight SMs of a wave have a second block, which sets the time: 512 -> 512 @7
-// 13.4 us against 12.5), F(6,3) one where that fits the wave.
-// Against the filter transform on its own stream and the three kernels after it, us a layer in a row of such layers, without / with: F(4,3)
-// 64 -> 64 @7 5.0 / 4.7, @10 5.5 / 4.8, 128 -> 128 @10 7.7 / 6.9, 256 -> 256 @7 8.3 / 6.9, 512 -> 512 @7 23.4 / 13.3, @4 22.4 / 9.6, F(6,3) 64 -> 64 @16 6.2 / 5.4,
-// 192 -> 192 @7 8.4 / 7.4, 256 -> 256 @5 9.3 / 7.3, 384 -> 384 @12 22.5 / 16.3.  Behind with F(6,3) on one tile of few channels (32 -> 32 @5 4.9 / 5.4) and on
-// more than four of more than 64 (128 -> 128 @16 7.5 / 8.1).
-struct WlPlan { bool use; int T, slices, quads; };
+// Estimated us of a layer inside a pass: here, and as the filter transform on its own stream with the three kernels for transformed weights.  Here: a base,
+// the slice's quads one after the other, dearer as blocks begin to share an SM (clusters of four and eight: from about 56 blocks on, all of
+// them from 80) and fill the wave; F(6,3) pays for a second tile a block.  There: the bytes of U beyond the ~6 MB that the transform's own
+// launches hide, channels and outputs.  Fitted to 1483 layers of 16 - 1024 channels on 1 - 12 tiles in rows of eight (5 - 8 % off).
+double wl_us(int m, int T, int slices, int quads, long long blocks) {
+    const double q = std::max(quads, 4), shared = std::min(1.0, std::max(0.0, (blocks - 56) / 24.0)), full = std::max(0.0, (blocks - 80) / 184.0);
+    return (m == 6 ? 3.5 : 2.7) + (slices == 8 ? 0.45 : 0.0) + 0.194 * q * (1 + shared) + full * (1.7 + 0.08 * q) + (m == 6 && T == 2 ? 3.3 : 0.0);
+}
+double wl_separate_us(int m, int C, int K, int tiles) {
+    const double mb = 4e-6 * (m + 2) * (m + 2) * C * K, hidden = m == 6 ? 6.0 : 5.0;
+    return (m == 6 ? 3.86 : 3.35) + 0.005 * C + (m == 6 ? 0.0058 : 0.0035) * K + 0.6 * std::min(10.0, std::max(0.0, mb - hidden)) +
+           0.37 * std::max(0.0, mb - 16) + 0.11 * std::max(0, tiles - 8) + (m == 6 ? 0.0005 : 0.0008) * tiles * C;
+}
+
+// Tiles a block, slices and whether the layer is to run here: where it fits one wave at two blocks an SM (more pays the filter transform too often:
+// F(4,3) 512 -> 512 @14 23.7 us without, 38 with, 384 -> 384 @14 15.3 / 25), wino_small.cu runs the tile GEMM for transformed weights, whose sums it
+// follows, and the estimate is lower.  Two tiles a block (four: as fast alone, but then only eight SMs of a wave have a second block, which sets the time:
+// 512 -> 512 @7 13.4 us against 12.5), F(6,3) one where that fits the wave.
+// us a layer in a row of such layers, separate / here: F(4,3) 64 -> 64 @8 4.2 / 3.6, 128 -> 128 4.8 / 4.3, 256 -> 256 8.6 / 6.1, 512 -> 512 23.0 / 12.9, @4
+// 20.8 / 8.8, F(6,3) 64 -> 64 @12 4.8 / 4.4, 384 -> 384 23.7 / 16.1, 192 -> 192 @6 7.8 / 6.0, 256 -> 256 12.9 / 6.8.  What the estimate leaves to the separate
+// kernels: F(6,3) 16 -> 192 @12x24 4.9 / 6.4, 64 -> 128 @18 5.5 / 6.4, 192 -> 32 @12 5.1 / 6.0, F(4,3) 192 -> 192 @8x16 6.5 / 7.5, 256 -> 160 @8x16 7.1 / 8.6.
+// Of the 1483 layers 203 would be more than 3 % slower here without it, 12 - 17 are with it.  Cold passes, where the link hides the filter transform, gain less:
+// a ResNet-18-shaped model @224 with F(4,3) 902 / 892 us, staged three deep 991 / 979.
+struct WlPlan { bool fits, use; int T, slices, quads; };
 WlPlan wl_plan(int m, int C, int K, int tiles) {
     constexpr long long WAVE = 264;                            // clusters of eight, two blocks an SM
-    WlPlan p{false, m == 4 ? 2 : 1, 4, 0};
+    WlPlan p{false, false, m == 4 ? 2 : 1, 4, 0};
     if (C % 4 != 0 || C > 512 || (m == 6 && (tiles == 1 ? C < 128 : tiles > 4 && C > 64)) || !wino_small_applies(m, tiles, align_up(C, 8), K)) return p;
     if (C > 256) {
         if (tiles > 4) return p;                               // (the GEMM for transformed weights would need more registers to follow)
@@ -316,8 +331,9 @@ WlPlan wl_plan(int m, int C, int K, int tiles) {
     }
     auto blocks = [&]() { return (long long)ceil_div(K, WL_K) * ceil_div(tiles, p.T) * p.slices; };
     if (m == 6 && tiles <= 4 && blocks() > WAVE) p.T = 2;
-    p.use = blocks() <= WAVE;
+    p.fits = blocks() <= WAVE;
     p.quads = ceil_div(C, 32) * 8 / p.slices;
+    p.use = p.fits && wl_us(m, p.T, p.slices, p.quads, blocks()) < 0.98 * wl_separate_us(m, C, K, tiles);
     return p;
 }
 
@@ -336,14 +352,14 @@ nnv_status_t launch_wl(WlDev g, cudaStream_t st) {
 bool wino_layer_applies(int m, int C, int K, int tiles) { return wl_plan(m, C, K, tiles).use; }
 int wino_layer_quarters(int m, int C, int K, int tiles) {
     const WlPlan p = wl_plan(m, C, K, tiles);
-    return p.use && p.slices == 8;
+    return p.fits && p.slices == 8;
 }
 
 nnv_status_t launch_wino_layer(int m, const float* x, const float* w, const float* bias, const float* add, float* y, int act, int C, int H, int W,
                                int K, int pad, int OH, int OW, bool early, cudaStream_t st) {
     const int TW = ceil_div(OW, m), tiles = ceil_div(OH, m) * TW;
     const WlPlan p = wl_plan(m, C, K, tiles);
-    NNV_REQUIRE(p.use, NNV_ERR_UNSUPPORTED, "no one-launch Winograd layer for this shape");
+    NNV_REQUIRE(p.fits, NNV_ERR_UNSUPPORTED, "no one-launch Winograd layer for this shape");
     const int* status = nullptr;
     NNV_TRY(device_status_address(&status));
     WlDev g{x, w, bias, add, y, C, H, W, K, pad, OH, OW, TW, tiles, act, p.slices, p.quads, early ? 1 : 0, const_cast<int*>(status)};

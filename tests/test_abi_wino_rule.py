@@ -29,3 +29,14 @@ def test_overrides_reach_layers_of_few_tiles(m, C, K, tiles):
                 nb.nnv_tuning_set(bad)
     finally:
         nb.nnv_tuning_set(None)
+
+
+@pytest.mark.parametrize("m,C,K,tiles,layer", [
+    # separate kernels / one launch, us a layer in a row of them: 4.9 / 6.4, 5.2 / 6.4, 5.5 / 6.4, 5.1 / 6.0, 6.5 / 7.5, 7.1 / 8.6
+    (6, 16, 192, 8, 0), (6, 32, 256, 6, 0), (6, 64, 128, 9, 0), (6, 192, 32, 4, 0), (4, 192, 192, 8, 0), (4, 256, 160, 8, 0),
+    # 23.0 / 12.9, 8.6 / 6.1, 4.6 / 3.8, 23.7 / 16.1, 7.8 / 6.0, 12.7 / 6.5
+    (4, 512, 512, 4, 1), (4, 256, 256, 4, 1), (4, 64, 64, 9, 1), (6, 384, 384, 4, 1), (6, 192, 192, 1, 1), (4, 96, 1024, 4, 1),
+    (4, 512, 512, 5, 0), (4, 6, 64, 1, 0), (6, 64, 64, 1, 0)])         # outside what the kernel does
+def test_one_launch_where_it_is_the_faster(m, C, K, tiles, layer):
+    nb.nnv_tuning_set(None)
+    assert rule(m, C, K, tiles)["layer"] == layer
