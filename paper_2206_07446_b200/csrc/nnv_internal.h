@@ -309,11 +309,12 @@ nnv_status_t launch_wino_output(int m, const float* d_M, float* d_y, const float
                                 int act, int K, int OH, int OW, int TH, int TW, cudaStream_t st);
 // The tile GEMM of F(4,3) / F(6,3) on a few tiles, in fp32: V[a2][T][Cp] and U[a2][K][Cp] fp32 -> M[a2][T][K].
 bool wino_small_applies(int m, int T, int Cp, int K);
+int wino_small_groups(int m, int C, int K, int T);
 nnv_status_t launch_wino_small(int m, const float* d_V, const float* d_U, float* d_M, int T, int K, int C, int Cp, cudaStream_t st);
 // A whole F(4,3) / F(6,3) layer on a small image from raw OIHW weights as one launch, in fp32 (wino_layer.cu).  early: the weights are complete
 // before anything in the launch's stream that it may overtake.
 bool wino_layer_applies(int m, int C, int K, int tiles);
-int wino_layer_quarters(int m, int C, int K, int tiles);      // its sums are of quarters of the input channels (else of halves)
+int wino_layer_parts(int m, int C, int K, int tiles);         // its sums are of so many parts of the input channels (2 or 4; 0: it never runs the layer)
 nnv_status_t launch_wino_layer(int m, const float* d_x, const float* d_w, const float* d_bias, const float* d_add, float* d_y, int act, int C, int H,
                                int W, int K, int pad, int OH, int OW, bool early, cudaStream_t st);
 // fp32 direct convolution from raw OIHW weights (groups == 1).

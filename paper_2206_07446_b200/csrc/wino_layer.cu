@@ -350,9 +350,9 @@ nnv_status_t launch_wl(WlDev g, cudaStream_t st) {
 }  // namespace
 
 bool wino_layer_applies(int m, int C, int K, int tiles) { return wl_plan(m, C, K, tiles).use; }
-int wino_layer_quarters(int m, int C, int K, int tiles) {
+int wino_layer_parts(int m, int C, int K, int tiles) {
     const WlPlan p = wl_plan(m, C, K, tiles);
-    return p.fits && p.slices == 8;
+    return !p.fits ? 0 : p.slices == 8 ? 4 : 2;
 }
 
 nnv_status_t launch_wino_layer(int m, const float* x, const float* w, const float* bias, const float* add, float* y, int act, int C, int H, int W,
@@ -369,9 +369,9 @@ nnv_status_t launch_wino_layer(int m, const float* x, const float* w, const floa
 }  // namespace nnv
 
 // Which kernels run an F(m,3) layer of `tiles` tiles, for the tests: the fp32 tile GEMM, a whole layer in one launch, that launch's tiles a block, slices
-// and quads of input channels.
+// and quads of input channels, and the tile GEMM's groups of output channels.
 extern "C" void nnv_internal_wino_rule(int m, int C, int K, int tiles, int32_t* out) {
     const nnv::WlPlan p = nnv::wl_plan(m, C, K, tiles);
-    const int32_t v[] = {nnv::wino_small_applies(m, tiles, (int)nnv::align_up(C, 8), K), p.use, p.T, p.slices, p.quads};
+    const int32_t v[] = {nnv::wino_small_applies(m, tiles, (int)nnv::align_up(C, 8), K), p.use, p.T, p.slices, p.quads, nnv::wino_small_groups(m, C, K, tiles)};
     std::copy(std::begin(v), std::end(v), out);
 }

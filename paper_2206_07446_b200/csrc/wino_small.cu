@@ -4,7 +4,7 @@
 // fills 128 rows whatever T is and splits every word of U into bf16 parts on its way through shared memory; here a word goes from memory
 // into a register and is multiplied T times, in fp32.
 //   - A block owns 64 output channels of one plane b; V's plane lies in shared memory.  Eight warps: four groups of 16 channels x two halves of the
-//     input channels.  Eight lanes read 128 contiguous bytes of a channel's row, a warp four rows at a time, sixteen in all, so that a word of V
+//     input channels, or, where that leaves SMs idle and lone warps with long sums, two groups x quarters or one x eighths (below).  Eight lanes read 128 contiguous bytes of a channel's row, a warp four rows at a time, sixteen in all, so that a word of V
 //     read from shared memory serves four rows of a lane.
 //   - The lanes' sums are reduced by exchanging halves (3.5 T shuffles), the halves of the input channels through shared memory; the order is fixed,
 //     and wino_layer.cu's is the same: a layer has the same bits whether its weights come transformed or raw.  (Where that kernel deals the channels to eight
@@ -18,20 +18,22 @@
 namespace nnv {
 namespace {
 
-constexpr int WS_K = 64, WS_THREADS = 256;
+constexpr int WS_THREADS = 256;
 
-// T: tiles, rounded up (tiles that do not exist have zeros in shared memory); UN: 32-channel blocks in flight.
-template <int T, int UN>
+// T: tiles, rounded up (tiles that do not exist have zeros in shared memory); UN: 32-channel blocks in flight; GROUPS: warps side by side, 16 output channels
+// each, the others share out the input channels.
+template <int T, int UN, int GROUPS>
 __global__ void __launch_bounds__(WS_THREADS, 2)
 wino_small_kernel(const float* __restrict__ V, const float* __restrict__ U, float* __restrict__ M, int tiles, int K, int Cp,
                   int quarters, unsigned long long* stamp) {
-    extern __shared__ __align__(16) float sv[];                // V's plane [T][pitch], later the partial sums [2][64][T + 1]
+    constexpr int WS_K = 16 * GROUPS, PARTS = 8 / GROUPS;
+    extern __shared__ __align__(16) float sv[];                // V's plane [T][pitch], later the partial sums [PARTS][WS_K][T + 1]
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int cl = lane & 7, rl = lane >> 3, rg = warp & 3, half = warp >> 2;
+    const int cl = lane & 7, rl = lane >> 3, rg = warp % GROUPS, part = warp / GROUPS;
     const int b = blockIdx.y, k0 = blockIdx.x * WS_K;
     const int pitch = ((Cp + 31) & ~31) + 4;                   // (eight lanes read 128 bytes of a row: any pitch will do)
-    const int blocks = (Cp + 31) / 32, i0 = blocks * half / 2, i1 = blocks * (half + 1) / 2;
-    const int middle = T <= 4 && quarters ? blocks * (2 * half + 1) / 4 : -1;    // where a sum of its own begins
+    const int blocks = (Cp + 31) / 32, i0 = blocks * part / PARTS, i1 = blocks * (part + 1) / PARTS;
+    const int middle = T <= 4 && PARTS == 2 && quarters ? blocks * (2 * part + 1) / 4 : -1;    // where a sum of its own begins
     const float* const u = U + ((long long)b * K + k0 + rg * 16 + rl) * Cp + 4 * cl;
     const int rows = K - k0 - rg * 16 - rl;                    // rows 4 r of this lane that exist: 4 r < rows
     float acc[4][T];
@@ -113,14 +115,18 @@ wino_small_kernel(const float* __restrict__ V, const float* __restrict__ U, floa
     __syncthreads();                                           // V is read no more
     {
         const int row = rg * 16 + rl + 4 * (2 * (cl >> 2) + (cl >> 1 & 1));
-        float* dst = sv + (half * WS_K + row) * (T + 1) + (cl & 1) * (T / 2);
+        float* dst = sv + (part * WS_K + row) * (T + 1) + (cl & 1) * (T / 2);
 #pragma unroll
         for (int t = 0; t < T / 2; ++t) dst[t] = s[t];
     }
     __syncthreads();
     for (int i = tid; i < T * WS_K; i += WS_THREADS) {
         const int t = i / WS_K, k = i % WS_K;
-        if (t < tiles && k0 + k < K) M[((long long)b * tiles + t) * K + k0 + k] = sv[k * (T + 1) + t] + sv[(WS_K + k) * (T + 1) + t];
+        if (t >= tiles || k0 + k >= K) continue;
+        float sum = sv[k * (T + 1) + t];
+#pragma unroll
+        for (int q = 1; q < PARTS; ++q) sum += sv[(q * WS_K + k) * (T + 1) + t];
+        M[((long long)b * tiles + t) * K + k0 + k] = sum;
     }
     if (stamp) {
         __syncthreads();
@@ -140,21 +146,37 @@ bool wino_small_applies(int m, int T, int Cp, int K) {
     return m != 2 && Cp <= 2048 && (T <= 8 ? bytes <= 40e6 : T <= 12 && bytes <= 5e6);
 }
 
+// Groups of 16 output channels a block: the fewest that leave at most two blocks an SM and no part of the input channels empty; four where wino_layer.cu
+// sums the layer too.  us of a layer, tensor cores / four groups / as chosen: F(4,3) 960 -> 16 @12x16 10.6 / 16.1 / 10.4, 640 -> 48 @12 10.2 / 12.4 / 9.0, 1024 -> 256 @8x12
+// 15.6 / 17.0 / 13.7, F(6,3) 448 -> 32 @18 9.6 / 13.2 / 8.8; over 563 layers of 16 - 1024 channels 0.904 of the time that four groups take everywhere (the best of
+// the three forms 0.901), 7 of them more than 3 % behind the tensor cores (1024 outputs of up to 32 inputs on nine tiles or more).
+int wino_small_groups(int m, int C, int K, int T) {
+    if (wino_layer_parts(m, C, K, T)) return 4;
+    for (int g = 1; g < 4; g *= 2)
+        if (ceil_div(K, 16 * g) * (m + 2) * (m + 2) <= 2 * 148 && 8 / g <= ceil_div(C, 32)) return g;
+    return 4;
+}
+
 nnv_status_t launch_wino_small(int m, const float* V, const float* U, float* M, int T, int K, int C, int Cp, cudaStream_t st) {
     unsigned long long* const stamp = next_stamp();
     next_stamp() = nullptr;
-    const int quarters = wino_layer_quarters(m, C, K, T);
-    auto go = [&](auto tt, auto kernel) -> cudaError_t {
-        constexpr int TT = decltype(tt)::value;
-        const size_t smem = sizeof(float) * std::max((size_t)TT * (align_up(Cp, 32) + 4), (size_t)2 * WS_K * (TT + 1));
+    const int quarters = wino_layer_parts(m, C, K, T) == 4;
+    auto go = [&](auto tt, auto gg, auto kernel) -> cudaError_t {
+        constexpr int TT = decltype(tt)::value, WS_K = 16 * decltype(gg)::value;
+        const size_t smem = sizeof(float) * std::max((size_t)TT * (align_up(Cp, 32) + 4), (size_t)128 * (TT + 1));
         static const cudaError_t attr = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(float) * TT * (2048 + 4)));
         if (attr != cudaSuccess) return attr;
         return launch_pdl(kernel, dim3(ceil_div(K, WS_K), (m + 2) * (m + 2)), dim3(WS_THREADS), smem, st, V, U, M, T, K, Cp, quarters, stamp);
     };
-    const std::integral_constant<int, 4> t4;
-    const std::integral_constant<int, 8> t8;
-    const std::integral_constant<int, 12> t12;
-    NNV_CUDA(T <= 4 ? go(t4, wino_small_kernel<4, 3>) : T <= 8 ? go(t8, wino_small_kernel<8, 2>) : go(t12, wino_small_kernel<12, 2>));
+    auto pick = [&](auto gg) {
+        constexpr int GG = decltype(gg)::value;
+        const std::integral_constant<int, 4> t4;
+        const std::integral_constant<int, 8> t8;
+        const std::integral_constant<int, 12> t12;
+        return T <= 4 ? go(t4, gg, wino_small_kernel<4, 3, GG>) : T <= 8 ? go(t8, gg, wino_small_kernel<8, 2, GG>) : go(t12, gg, wino_small_kernel<12, 2, GG>);
+    };
+    const int groups = wino_small_groups(m, C, K, T);
+    NNV_CUDA(groups == 1 ? pick(std::integral_constant<int, 1>()) : groups == 2 ? pick(std::integral_constant<int, 2>()) : pick(std::integral_constant<int, 4>()));
     return NNV_OK;
 }
 

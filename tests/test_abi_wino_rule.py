@@ -7,9 +7,9 @@ from paper_2206_07446_b200 import binding as nb
 
 
 def rule(m, C, K, tiles):
-    out = (ctypes.c_int32 * 5)()
+    out = (ctypes.c_int32 * 6)()
     nb._lib.nnv_internal_wino_rule(m, C, K, tiles, out)
-    return dict(zip(("small", "layer", "T", "slices", "quads"), out))
+    return dict(zip(("small", "layer", "T", "slices", "quads", "groups"), out))
 
 
 @pytest.mark.parametrize("m,C,K,tiles", [(4, 512, 512, 4), (4, 64, 64, 1), (6, 256, 256, 1), (6, 64, 96, 9)])
@@ -40,3 +40,11 @@ def test_overrides_reach_layers_of_few_tiles(m, C, K, tiles):
 def test_one_launch_where_it_is_the_faster(m, C, K, tiles, layer):
     nb.nnv_tuning_set(None)
     assert rule(m, C, K, tiles)["layer"] == layer
+
+
+@pytest.mark.parametrize("m,C,K,tiles,groups", [
+    (4, 960, 16, 12, 1), (4, 640, 48, 9, 1), (6, 448, 32, 9, 1), (4, 1024, 256, 6, 2), (6, 1024, 96, 1, 2),     # lone warps with long sums otherwise
+    (4, 96, 64, 9, 4), (4, 512, 512, 4, 4), (4, 300, 512, 8, 4), (4, 40, 800, 12, 4)])                        # summed by the one-launch layer too, or enough blocks
+def test_groups_of_output_channels(m, C, K, tiles, groups):
+    nb.nnv_tuning_set(None)
+    assert rule(m, C, K, tiles)["small"] and rule(m, C, K, tiles)["groups"] == groups
