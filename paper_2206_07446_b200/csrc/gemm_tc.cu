@@ -26,6 +26,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <mutex>
@@ -1837,17 +1838,6 @@ nnv_status_t launch_gemm_tc(const GemmArgs& a, cudaStream_t st) {
 // ---- inverted bottleneck: shape of a launch -----------------------------------------------------
 namespace {
 
-struct IbShape {
-    int ph, pw, hw, rows, px, tiles_h, tiles_w;
-    int ranks, splits, both, step, nb_most, BN2, issuers, tmem_cols;
-    uint16_t first[IB_MAX_RANKS];
-    uint8_t count[IB_MAX_RANKS];
-    uint32_t pairs;                   // bit k: split k has two ranks
-    uint32_t w1_off, conv_off, d_off, w2_off, bar_off, par_off;
-    size_t smem_bytes;
-    double t;                         // estimated time, us
-};
-
 // The channel blocks of every CTA that shares a patch, in the order of the projection's own launch: its `splits` ranges of the n blocks,
 // whole (`both`: two accumulators, or with one issuer one) or an accumulator's blocks each.
 bool ib_ranks(int n, int splits, int issuers, bool unit, IbShape* s) {
@@ -1918,6 +1908,15 @@ IbShape search_ib(bool bf16, int C, int E, int K, int OH, int OW, int stride, in
     const int nkb1 = ceil_div(C, 32);
     IbShape best{};
     best.t = 1e30;
+    // The patch heights and widths there are: the least of every number of rows, while a halo of three columns fits the rows of an MMA.
+    int heights[BM], widths[BM];
+    auto sizes = [&](int n, int* out) {
+        int count = 0;
+        for (int v = std::min(n, (BM / 3 - 3) / stride + 1); v >= 1; --v)
+            if (ceil_div(n, ceil_div(n, v)) == v) out[count++] = v;
+        return count;
+    };
+    const int nh = sizes(OH, heights), nw = sizes(OW, widths);
     for (int unit = 0; unit < (issuers == 2 ? 2 : 1); ++unit) {
         IbShape s{};
         s.BN2 = ceil_div(K, 16) * 16;
@@ -1926,14 +1925,12 @@ IbShape search_ib(bool bf16, int C, int E, int K, int OH, int OW, int stride, in
         if (s.BN2 > (s.both ? 256 : 512)) continue;
         // Patches of the least height and width for their numbers of rows and columns, no more than four times as long as wide unless as long as the
         // image.
-        for (int th = 1; th <= OH; ++th) {
-            const int ph = ceil_div(OH, th), hh = (ph - 1) * stride + 3;
-            if (hh * 3 > BM) continue;
-            if (th > 1 && ph == ceil_div(OH, th - 1)) continue;
-            for (int tw = 1; tw <= OW; ++tw) {
-                const int pw = ceil_div(OW, tw), hw = (pw - 1) * stride + 3;
-                if (hh * hw > BM || (tw > 1 && pw == ceil_div(OW, tw - 1))) continue;
-                if ((ph > 4 * pw && th > 1) || (pw > 4 * ph && tw > 1)) continue;
+        for (int h = 0; h < nh; ++h) {
+            const int ph = heights[h], hh = (ph - 1) * stride + 3;
+            for (int w = 0; w < nw; ++w) {
+                const int pw = widths[w], hw = (pw - 1) * stride + 3;
+                if (hh * hw > BM) continue;
+                if ((ph > 4 * pw && ph < OH) || (pw > 4 * ph && pw < OW)) continue;
                 s.ph = ph; s.pw = pw; s.hw = hw; s.rows = hh * hw; s.px = ph * pw;
                 s.tiles_h = ceil_div(OH, ph); s.tiles_w = ceil_div(OW, pw);
                 if (ib_us(s, bf16, nkb1, stride, 2) >= best.t || !ib_layout(bf16, nkb1, &s)) continue;
@@ -1969,32 +1966,24 @@ static bool ib_shape(const nnv_layer_desc_t& a, const nnv_layer_desc_t& d, const
     return out->t < 1e29;
 }
 
-// The shape for a block, remembered by the calling thread (the search takes longer than a launch).
-static const IbShape* pick_ib(const nnv_layer_desc_t& a, const nnv_layer_desc_t& d, const nnv_layer_desc_t& p, int math) {
-    struct Entry { nnv_layer_desc_t a{}, d{}, p{}; int math = -1; uint64_t tuning = 0; bool use = false; IbShape s; };
-    static thread_local Entry table[64];
-    const uint32_t h = ((uint32_t)a.H * 2654435761u) ^ ((uint32_t)a.K * 40503u) ^ ((uint32_t)p.K * 9176u) ^ (uint32_t)(a.C * 131 + d.stride * 7 + math);
-    Entry& e = table[(h ^ (h >> 15)) & 63u];
-    auto same = [](const nnv_layer_desc_t& x, const nnv_layer_desc_t& y) {
-        return x.C == y.C && x.K == y.K && x.R == y.R && x.S == y.S && x.stride == y.stride && x.pad == y.pad && x.groups == y.groups && x.H == y.H && x.W == y.W && (x.in1 < 0) == (y.in1 < 0) && (x.act == 0) == (y.act == 0);
-    };
+// Searches for the shape of a block so far, for the tests.
+static std::atomic<uint64_t> g_ib_searches{0};
+
+const IbShape* inverted_bottleneck_shape(const nnv_layer_desc_t& a, const nnv_layer_desc_t& d, const nnv_layer_desc_t& p, int math, IbEntry* e) {
     const Tuning& tn = tuning();
-    if (e.math != math || e.tuning != tn.generation || !same(e.a, a) || !same(e.d, d) || !same(e.p, p)) {
-        e.a = a; e.d = d; e.p = p; e.math = math; e.tuning = tn.generation;
-        e.use = ib_shape(a, d, p, math, &e.s);
+    if (!e->known || e->tuning != tn.generation) {
+        g_ib_searches.fetch_add(1, std::memory_order_relaxed);
+        e->use = ib_shape(a, d, p, math, &e->shape);
+        e->tuning = tn.generation;
+        e->known = true;
     }
-    return e.use ? &e.s : nullptr;
+    return e->use ? &e->shape : nullptr;
 }
 
-bool inverted_bottleneck_applies(const nnv_layer_desc_t& a, const nnv_layer_desc_t& d, const nnv_layer_desc_t& p, int math) {
-    return pick_ib(a, d, p, math) != nullptr;
-}
-
-nnv_status_t launch_inverted_bottleneck(const nnv_layer_desc_t& a, const nnv_layer_desc_t& d, const nnv_layer_desc_t& p, int math, const IbBuffers& io,
-                                        cudaStream_t st) {
+nnv_status_t launch_inverted_bottleneck(const nnv_layer_desc_t& a, const nnv_layer_desc_t& d, const nnv_layer_desc_t& p, int math, const IbShape& shape,
+                                        const IbBuffers& io, cudaStream_t st) {
     NNV_TRY(gemm_tc_init());
-    const IbShape* s = pick_ib(a, d, p, math);
-    NNV_REQUIRE(s, NNV_ERR_UNSUPPORTED, "the three layers do not run as one launch");
+    const IbShape* const s = &shape;
     const bool bf16 = math == NNV_MATH_BF16;
     const int Qp1 = (a.C + 7) / 8 * 8, Qp2 = (p.C + 7) / 8 * 8;
     CUtensorMap tmX, tmW1, tmW2;
@@ -2049,7 +2038,8 @@ extern "C" int nnv_internal_ib_shape(int bf16, int C, int E, int K, int H, int W
     a.C = C; a.K = E; a.R = a.S = 1; a.stride = 1; a.groups = 1; a.H = H; a.W = W; a.in1 = -1;
     d.C = d.K = d.groups = E; d.R = d.S = 3; d.stride = stride; d.pad = 1; d.H = H; d.W = W; d.in1 = -1;
     p.C = E; p.K = K; p.R = p.S = 1; p.stride = 1; p.groups = 1; p.H = (H - 1) / stride + 1; p.W = (W - 1) / stride + 1; p.in1 = residual ? 0 : -1;
-    const IbShape* s = pick_ib(a, d, p, bf16 ? NNV_MATH_BF16 : NNV_MATH_TF32);
+    IbEntry entry;
+    const IbShape* s = inverted_bottleneck_shape(a, d, p, bf16 ? NNV_MATH_BF16 : NNV_MATH_TF32, &entry);
     if (!s) return 1;
     const int32_t v[] = {s->ph, s->pw, s->hw, s->rows, s->px, s->tiles_h, s->tiles_w, s->ranks, s->both, s->step, s->nb_most, s->BN2, s->issuers,
                          s->tmem_cols, (int32_t)s->w1_off, (int32_t)s->conv_off, (int32_t)s->d_off, (int32_t)s->w2_off, (int32_t)s->bar_off,
@@ -2058,6 +2048,8 @@ extern "C" int nnv_internal_ib_shape(int bf16, int C, int E, int K, int H, int W
     for (int r = 0; r < IB_MAX_RANKS; ++r) { out[24 + 2 * r] = r < s->ranks ? s->first[r] : -1; out[25 + 2 * r] = r < s->ranks ? s->count[r] : 0; }
     return 0;
 }
+
+extern "C" uint64_t nnv_internal_ib_searches() { return nnv::g_ib_searches.load(std::memory_order_relaxed); }
 
 extern "C" int nnv_internal_gemm_loaders(int mode, int nkb, int ring) { return nnv::gemm_loaders(mode, nkb, ring); }
 

@@ -21,7 +21,6 @@
 // @7 8.2 / 7.3; of 145 blocks of 96 - 224 pixel images (BF16 too) every one was faster.  Warm MobileNetV2-shaped inference @160 168.6 -> 131.0.
 constexpr int IB_MAX_KB = 8;             // 32-channel blocks of the block's input
 constexpr int IB_MAX_NB = 8;             // 32-channel blocks of the expansion in one CTA
-constexpr int IB_MAX_RANKS = 16;
 constexpr int IB_THREADS = 512;
 constexpr int IB_PITCH = 144;            // bytes from a pixel to the next in the expansion's tiles
 constexpr int IB_BAR_BYTES = 8 * (2 * IB_MAX_KB + 8);

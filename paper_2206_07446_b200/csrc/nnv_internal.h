@@ -232,6 +232,24 @@ struct CachedGraph {
     bool zero_copy = false;               // kernels read the host weights in place
     ArenaLayout layout;
 };
+// How an inverted-residual block runs as one launch (inverted_bottleneck.cuh).
+constexpr int IB_MAX_RANKS = 16;
+struct IbShape {
+    int ph, pw, hw, rows, px, tiles_h, tiles_w;
+    int ranks, splits, both, step, nb_most, BN2, issuers, tmem_cols;
+    uint16_t first[IB_MAX_RANKS];
+    uint8_t count[IB_MAX_RANKS];
+    uint32_t pairs;                   // bit k: split k has two ranks
+    uint32_t w1_off, conv_off, d_off, w2_off, bar_off, par_off;
+    size_t smem_bytes;
+    double t;                         // estimated time, us
+};
+// What the search found for the three layers from one on, in one math; found once by a plan (the search costs the host as much as a launch or two).
+struct IbEntry {
+    bool known = false, use = false;
+    uint64_t tuning = 0;
+    IbShape shape;
+};
 }  // namespace nnv
 
 struct nnv_plan {
@@ -250,6 +268,7 @@ struct nnv_plan {
     int stamped_layers = 0;               // layers whose kernels stamped the device clock in the last run (opts.kernel_stamps)
     uint64_t last_enqueue_ns = 0;         // host time the last run spent putting its work on the streams
     bool warm_pending = false;            // warm preparations may still be running (first warm run waits)
+    std::vector<nnv::IbEntry> blocks;     // of the block that starts at layer i, TF32 at 2 i, BF16 at 2 i + 1
 };
 
 namespace nnv {
@@ -385,9 +404,11 @@ struct IbBuffers {
     float* e; float* d; float* y;                                          // the three layers' outputs
     bool early;                                                            // the weights are complete before anything in the launch's stream that it may overtake
 };
-bool inverted_bottleneck_applies(const nnv_layer_desc_t& expand, const nnv_layer_desc_t& depthwise, const nnv_layer_desc_t& project, int math);
+// The block's shape, or null where its layers run as launches of their own; `entry` remembers it.
+const IbShape* inverted_bottleneck_shape(const nnv_layer_desc_t& expand, const nnv_layer_desc_t& depthwise, const nnv_layer_desc_t& project, int math,
+                                         IbEntry* entry);
 nnv_status_t launch_inverted_bottleneck(const nnv_layer_desc_t& expand, const nnv_layer_desc_t& depthwise, const nnv_layer_desc_t& project,
-                                        int math, const IbBuffers& io, cudaStream_t st);
+                                        int math, const IbShape& shape, const IbBuffers& io, cudaStream_t st);
 // One-time host set-up of the GEMM (driver entry point, shared-memory attributes); call before
 // stream capture.
 nnv_status_t gemm_tc_init();

@@ -280,10 +280,11 @@ static nnv_status_t run_model(nnv_plan* p, const nnv_choice_t* choices, const vo
     };
     p->stamped_layers = stamp_base ? n : 0;
 
-    // Inverted-residual blocks that run as one launch, with the third layer's (fused[i]: the block starts at layer i); the result is the
+    // Inverted-residual blocks that may run as one launch, with the third layer's (may_fuse[i]: the block starts at layer i); the result is the
     // same bit for bit.  Not where the layers are to be timed each, where fewer staging slots than layers hold their weights, or where
-    // the weights arrive in different copies (the first layers would wait for the last one's).
-    std::vector<char> fused(n, 0);
+    // the weights arrive in different copies (the first layers would wait for the last one's).  Which of them do is decided when the pass has come to
+    // them: the search for a block's shape, once a plan, then costs the host nothing before the weights are on their way.
+    std::vector<char> may_fuse(n, 0);
     if (tn.block && !tm && !stamp_base && (depth == 0 || depth >= 3)) {
         for (int i = 0; i + 2 < n; ++i) {
             const nnv_layer_desc_t &a = p->layers[i], &d = p->layers[i + 1], &q = p->layers[i + 2];
@@ -293,9 +294,7 @@ static nnv_status_t run_model(nnv_plan* p, const nnv_choice_t* choices, const vo
                 continue;
             if (d.in0 != i || q.in0 != i + 1 || a.in1 >= 0 || d.in1 >= 0 || q.in1 >= i || on_side[i] || on_side[i + 1] || on_side[i + 2]) continue;
             if (merge && (chunk_of[i] != chunk_of[i + 1] || chunk_of[i] != chunk_of[i + 2])) continue;
-            if (!inverted_bottleneck_applies(a, d, q, choices[i].math)) continue;
-            fused[i] = 1;
-            i += 2;
+            may_fuse[i] = 1;
         }
     }
 
@@ -392,7 +391,9 @@ static nnv_status_t run_model(nnv_plan* p, const nnv_choice_t* choices, const vo
     }
 
     std::vector<int> conv_ids;
-    IbBuffers block{};                                        // of the fused block that the loop is in
+    int block_from = -3;                                      // the latest block that runs as one launch
+    const IbShape* block_shape = nullptr;
+    IbBuffers block{};
     cudaEvent_t waited[2] = {nullptr, nullptr};               // the latest event s_exec / s_side waited for
     for (int i = 0; i < n; ++i) {
         const nnv_layer_desc_t& L = p->layers[i];
@@ -561,19 +562,24 @@ static nnv_status_t run_model(nnv_plan* p, const nnv_choice_t* choices, const vo
         if (wait_warm && i < (int)p->warm_ev.size() && p->warm_ev[i]) NNV_CUDA(cudaStreamWaitEvent(se, p->warm_ev[i], 0));
         if (tm) NNV_CUDA(cudaEventRecord(TEV(i, 4), se));
         const void* add = L.in1 >= 0 ? base + A.act_off[L.in1] : nullptr;
-        if (fused[i]) {
-            block = IbBuffers{};
-            block.early = !queued;                            // (events order the weights before this stream; a queue's preparations may run in it)
-            block.x = (const float*)in; block.w1 = xf; block.b1 = L.has_bias ? (const float*)bias : nullptr; block.e = (float*)out;
-            continue;
+        if (may_fuse[i] && i > block_from + 2) {
+            if (p->blocks.empty()) p->blocks.resize(2 * (size_t)n);
+            block_shape = inverted_bottleneck_shape(L, p->layers[i + 1], p->layers[i + 2], ch.math, &p->blocks[2 * i + (ch.math == NNV_MATH_BF16)]);
+            if (block_shape) {
+                block_from = i;
+                block = IbBuffers{};
+                block.early = !queued;                        // (events order the weights before this stream; a queue's preparations may run in it)
+                block.x = (const float*)in; block.w1 = xf; block.b1 = L.has_bias ? (const float*)bias : nullptr; block.e = (float*)out;
+                continue;
+            }
         }
-        if (i >= 1 && fused[i - 1]) {
+        if (i == block_from + 1) {
             block.wd = (const float*)raw; block.b2 = L.has_bias ? (const float*)bias : nullptr; block.d = (float*)out;
             continue;
         }
-        if (i >= 2 && fused[i - 2]) {
+        if (i == block_from + 2) {
             block.w2 = xf; block.b3 = L.has_bias ? (const float*)bias : nullptr; block.addend = (const float*)add; block.y = (float*)out;
-            NNV_TRY(launch_inverted_bottleneck(p->layers[i - 2], p->layers[i - 1], L, ch.math, block, se));
+            NNV_TRY(launch_inverted_bottleneck(p->layers[i - 2], p->layers[i - 1], L, ch.math, *block_shape, block, se));
             for (int k = i - 2; k <= i; ++k)
                 if (need_done[k]) NNV_CUDA(cudaEventRecord(EV(k, 2), se));
             continue;
