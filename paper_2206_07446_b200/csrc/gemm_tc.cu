@@ -1966,8 +1966,8 @@ static bool ib_shape(const nnv_layer_desc_t& a, const nnv_layer_desc_t& d, const
     return out->t < 1e29;
 }
 
-// Searches for the shape of a block so far, for the tests.
-static std::atomic<uint64_t> g_ib_searches{0};
+// Searches for the shape of a block and launches of one so far, for the tests.
+static std::atomic<uint64_t> g_ib_searches{0}, g_ib_launches{0};
 
 const IbShape* inverted_bottleneck_shape(const nnv_layer_desc_t& a, const nnv_layer_desc_t& d, const nnv_layer_desc_t& p, int math, IbEntry* e) {
     const Tuning& tn = tuning();
@@ -2011,6 +2011,7 @@ nnv_status_t launch_inverted_bottleneck(const nnv_layer_desc_t& a, const nnv_lay
     std::copy(std::begin(s->count), std::end(s->count), g.count);
     g.pairs = s->pairs;
     const dim3 grid(s->tiles_h * s->tiles_w, 1, s->ranks);
+    g_ib_launches.fetch_add(1, std::memory_order_relaxed);
     NNV_CUDA(launch_pdl_cluster(ib_kernels[bf16][s->ranks > 1], grid, dim3(IB_THREADS), s->smem_bytes, st, s->ranks, tmX, tmW1, tmW2, g));
     return NNV_OK;
 }
@@ -2049,6 +2050,7 @@ extern "C" int nnv_internal_ib_shape(int bf16, int C, int E, int K, int H, int W
     return 0;
 }
 
+extern "C" uint64_t nnv_internal_ib_launches() { return nnv::g_ib_launches.load(std::memory_order_relaxed); }
 extern "C" uint64_t nnv_internal_ib_searches() { return nnv::g_ib_searches.load(std::memory_order_relaxed); }
 
 extern "C" int nnv_internal_gemm_loaders(int mode, int nkb, int ring) { return nnv::gemm_loaders(mode, nkb, ring); }

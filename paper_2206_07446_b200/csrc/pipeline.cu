@@ -281,11 +281,18 @@ static nnv_status_t run_model(nnv_plan* p, const nnv_choice_t* choices, const vo
     p->stamped_layers = stamp_base ? n : 0;
 
     // Inverted-residual blocks that may run as one launch, with the third layer's (may_fuse[i]: the block starts at layer i); the result is the
-    // same bit for bit.  Not where the layers are to be timed each, where fewer staging slots than layers hold their weights, or where
-    // the weights arrive in different copies (the first layers would wait for the last one's).  Which of them do is decided when the pass has come to
-    // them: the search for a block's shape, once a plan, then costs the host nothing before the weights are on their way.
+    // same bit for bit.  Not where the layers are to be timed each.  A block's launch waits for the weights of all three layers and holds their staging
+    // slots until its end, which must not stand in the way of the next block's preparation (MobileNetV2-shaped @224, us, separate / one launch):
+    //   - weights resident, from four slots on: 3 157 / 185, in BF16 170 / 179, 4 158 / 158, 173 / 160, 6 158 / 121, unstaged 158 / 119;
+    //   - copied into the slots, recorded, from four as well: 3 560 / 721, 4 558 / 536, 5 558 / 496, 6 559 / 445;
+    //   - eager, where the host gets through the calls no sooner, from six, two blocks' worth: 3 500 / 688, 4 492 / 539, 5 504 / 534, 6 495 / 444;
+    //   - layer by layer into places of their own the later start costs less than the launches: a continuous cold run 513 / 460, without merged
+    //     copies 491 / 450, three preparation queues 562 / 492, two 574 / 516; a single queue 680 / 691;
+    //   - with merged copies the three layers have to be in one: another would be waited for from the first layer on.
+    // Which of them do is decided when the pass has come to them: the search for a block's shape, once a plan, then costs the host nothing before the
+    // weights are on their way.
     std::vector<char> may_fuse(n, 0);
-    if (tn.block && !tm && !stamp_base && (depth == 0 || depth >= 3)) {
+    if (tn.block && !tm && !stamp_base && (depth == 0 || depth >= (resident || recorded ? 4 : 6)) && !(queued && n_little < 2)) {
         for (int i = 0; i + 2 < n; ++i) {
             const nnv_layer_desc_t &a = p->layers[i], &d = p->layers[i + 1], &q = p->layers[i + 2];
             if (a.op != NNV_OP_CONV || d.op != NNV_OP_CONV || q.op != NNV_OP_CONV) continue;
