@@ -577,3 +577,16 @@ nnv_status_t launch_direct(const float* x, const float* w, const float* bias, co
 }
 
 }  // namespace nnv
+
+// Which kernel runs a direct layer of P pixels on channels in fours (9 or 1 taps), for the tests: the tile of direct_tile_kernel (0: the other one), the split.
+extern "C" void nnv_internal_direct_rule(int P, int C, int K, int taps, int32_t* out) {
+    using namespace nnv;
+    const int jc = taps == 9 ? 288 : 64;
+    int tile = 0, splits = 0;
+    if (!pick_tile(P, C, K, taps, &tile, &splits)) {
+        tile = 0;
+        splits = pick_split(P, C, K, jc, ceil_div(C * taps, jc), taps).splits;
+    }
+    out[0] = tile;
+    out[1] = splits;
+}
