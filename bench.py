@@ -12,7 +12,8 @@ switched OFF, and every call is enqueued eagerly (no recorded graph: a cold infe
   e2e     the same step through nnv_cold_run with HOST input and output (their copies inside too)
   arms    beside them: the bypass arm (selection may take cached post-transform weights), the
           graph-replayed variant of the headline, and the device-resident pass (no read stage)
-  roofline*  kernel durations come from the per-layer events of the TIMED headline steps
+  roofline*  kernel durations come from the kernels' own clock stamps in further steps of the same kind, on a plan
+          whose runs launch every layer by itself (stamps keep layers apart that a plain plan's runs fuse)
 
 `python bench.py` (1 GPU) or under torch.distributed.run with --gpus N (independent replicas; the path
 does not shard).  One JSON line on standard output; the whole report goes to --report FILE or standard error.
@@ -20,6 +21,7 @@ does not shard).  One JSON line on standard output; the whole report goes to --r
 (or a sweep of shapes) through the C ABI instead of a whole step.
 """
 import argparse
+import ctypes
 import json
 import os
 import statistics
@@ -256,23 +258,11 @@ class ClockSampler:
         return out
 
 
-def count_launches(layers, choices, plan, nb, transforms):
-    """Kernels of this library launched by one pass: layout conversion in and out, `transforms` weight transforms (layers of one
-    copy share a launch), and the layers' own kernels."""
-    n = 2 + transforms
-    for i, L in enumerate(layers):
-        if L["op"] != wl.OP_CONV:
-            n += 1
-            continue
-        v, m, _ = choices[i]
-        if v in (nb.VAR_DIRECT, nb.VAR_DEPTHWISE):
-            n += 1
-            continue
-        if v in (nb.VAR_WINO_F2, nb.VAR_WINO_F4, nb.VAR_WINO_F6):
-            n += 3
-        else:
-            n += 1 + (1 if nb.nnv_exec_workspace_bytes(plan, i, v, m) else 0)
-    return n
+def launches_made(nb):
+    """Kernels of this library that this thread has launched so far (those of replayed graphs are not among them)."""
+    f = nb._lib.nnv_internal_launches
+    f.restype = ctypes.c_uint64
+    return f()
 
 
 def raw_bytes(L):
@@ -407,9 +397,11 @@ def measure(args, config, steps, warmup, minimal, rank, world, local, ranks):
     layers = wl.CONFIGS[args.config]()
     ws, bs = wl.make_weights(layers)
     x = wl.make_input(layers)
-    # the headline is eager; a second plan over the same blob replays recorded graphs for the side arms
-    model = harness.model_from_workload(layers, ws, bs, wl.weight_blob, use_graphs=0, kernel_stamps=1)
+    # the headline is eager; a second plan over the same blob replays recorded graphs for the side arms, a third one's kernels
+    # stamp the device clock (and its runs launch every layer by itself, also those that a plain plan's runs fuse)
+    model = harness.model_from_workload(layers, ws, bs, wl.weight_blob, use_graphs=0)
     plan_g = model.second_plan(use_graphs=1)
+    plan_s = model.second_plan(use_graphs=0, kernel_stamps=1)
     math = nb.MATH_BF16 if args.math == "bf16" else nb.MATH_TF32
 
     # offline decision stage: profile every candidate kernel, select per layer by cold cost
@@ -443,12 +435,16 @@ def measure(args, config, steps, warmup, minimal, rank, world, local, ranks):
 
     last_ms = []                                              # per-step times of the most recent timed region
 
+    launched = [0]                                            # kernels launched inside the most recent timed region
+
     def timed_region(step_fn, steps, warmup):
         """W untimed + K timed steps between barriers; mean ms per step (max over ranks)."""
         for k in range(warmup):
             step_fn(k, False)
         barrier()
+        launched[0] = launches_made(nb)
         out = [step_fn(k, True) for k in range(steps)]
+        launched[0] = launches_made(nb) - launched[0]
         barrier()
         ms = [ev0[k].elapsed_time(ev1[k]) for k in range(steps)]
         last_ms[:] = ms
@@ -483,12 +479,12 @@ def measure(args, config, steps, warmup, minimal, rank, world, local, ranks):
                             model.arena, model.arena.numel(), s_copy, s_xform, s_exec, args.cold_depth)
         if timed:
             ev1[k].record(s_exec)
-            return nb.nnv_kernel_times(model.plan)            # the kernels' own device-clock stamps of this step
 
     sampler.start()
     torch.cuda.cudart().cudaProfilerStart()                  # a profiler attached with "profile from start off" sees the timed steps only
-    value, step_timings = timed_region(step_value, args.steps, args.warmup)
+    value, _ = timed_region(step_value, args.steps, args.warmup)
     value_median = reduce_max(statistics.median(last_ms))
+    gpu_launches = launched[0]
     y_gpu = model.d_output.cpu().numpy()
 
     # ---- e2e: the same step through nnv_cold_run, input and output in pinned host memory ---------------------
@@ -506,9 +502,21 @@ def measure(args, config, steps, warmup, minimal, rank, world, local, ranks):
             enq.append(nb.nnv_last_enqueue_ns(model.plan))
 
     e2e, _ = timed_region(step_e2e, args.steps, args.warmup)
+    gpu_launches += launched[0]
     torch.cuda.cudart().cudaProfilerStop()
     y_e2e = model.h_output.numpy().copy()
     e2e_wall = reduce_max(1e3 * sum(wall) / len(wall))
+
+    # ---- the headline's step with stamping kernels, for their durations: the same kernels, choices and overlap, each layer by launches of its own ----
+    def step_stamped(k, timed):
+        begin(k, timed, (s_copy, s_xform))
+        nb.nnv_cold_run_dio(plan_s, ch_raw_c, model.h_weights, model.w_bytes, None, 0, model.d_input, model.d_output,
+                            model.arena, model.arena.numel(), s_copy, s_xform, s_exec, args.cold_depth)
+        if timed:
+            ev1[k].record(s_exec)
+            return nb.nnv_kernel_times(plan_s)
+
+    stamped_ms, step_timings = timed_region(step_stamped, min(args.steps, args.arm_steps), 2)
 
     # ---- the same step at every pipeline depth (staging slots; 1 = read, transform, execute one layer after the other) ----
     depth_ms = {}
@@ -733,9 +741,9 @@ def measure(args, config, steps, warmup, minimal, rank, world, local, ranks):
     peaks = load_peaks()
 
     # ---- rooflines: kernel durations are the kernels' own device-clock stamps (first block in, last block
-    # out) taken INSIDE the timed headline steps; event pairs around 5 us kernels add microseconds of their own
+    # out) taken INSIDE steps like the headline's (step_stamped); event pairs around 5 us kernels add microseconds of their own
     # and serialise the streams (the same step with per-layer events takes 1.8x as long)
-    xf, ex = {}, {}                                              # layer -> [ns] over the timed steps
+    xf, ex = {}, {}                                              # layer -> [ns] over the stamped steps
     for xs, es in step_timings:
         for i in range(len(layers)):
             if xs[i]:
@@ -767,7 +775,7 @@ def measure(args, config, steps, warmup, minimal, rank, world, local, ranks):
         roof = dict(hbm if t_hbm >= t_tensor else tens)           # the binding roofline of these launches
         roof.update({"kernel": "gemm_tc_kernel / gemm_sp_kernel (+ splitk_reduce_kernel) / conv3x3_tc_kernel: the tcgen05 GEMM of every im2col / 1x1 layer",
                      "traffic": NCU_GEMM_TRAFFIC_BYTES.get((args.config, args.math)),
-                     "durations": "device-clock stamps written by the kernels themselves inside the timed steps (CUDA events time the step)",
+                     "durations": "device-clock stamps written by the kernels themselves in %d further steps that launch each layer by itself (CUDA events time the headline)" % len(step_timings),
                      "peak_source": peaks["source"] + (" HBM copy" if t_hbm >= t_tensor else " bf16 burst" + ("" if math == nb.MATH_BF16 else " x 0.5 (tf32:bf16 nominal ratio)")),
                      "other_roofline": tens if t_hbm >= t_tensor else hbm,
                      "launches_per_step": len(single), "flops_per_step": gfl, "bytes_per_step": gby,
@@ -780,12 +788,12 @@ def measure(args, config, steps, warmup, minimal, rank, world, local, ranks):
         xbytes = sum(raw_bytes(layers[i]) + nb.nnv_transformed_bytes(model.plan, i, c[0], c[1]) for i, c in enumerate(choices_raw)
                      if c is not None and c[0] not in (nb.VAR_DIRECT, nb.VAR_DEPTHWISE))
         tns = sum(avg(v) for v in xf.values())
-        xroof = {"kernel": "multi_transform_kernel (filter transform + repack), the grouped launches of the timed headline steps",
+        xroof = {"kernel": "multi_transform_kernel (filter transform + repack), the grouped launches of the stamped steps",
                  "bound": "hbm", "achieved": xbytes / tns, "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": xbytes / tns / peaks["hbm_gbs"],
                  "traffic": None, "peak_source": peaks["source"], "launches_per_step": len(xf), "bytes_per_step": xbytes,
                  "sum_us_per_step": tns / 1e3, "avg_launch_us": tns / len(xf) / 1e3,
-                 "durations": "device-clock stamps written by the kernels themselves inside the timed steps"}
-    # per layer: the tensor-core kernel's duration inside the timed steps against the layer's own roofline
+                 "durations": "device-clock stamps written by the kernels themselves in the stamped steps"}
+    # per layer: the tensor-core kernel's duration inside the stamped steps against the layer's own roofline
     per_layer = []
     for i in sorted(ex):
         L = layers[i]
@@ -803,7 +811,6 @@ def measure(args, config, steps, warmup, minimal, rank, world, local, ranks):
     exec_ns = sum(avg(v) for v in ex.values())
     xform_ns = sum(avg(v) for v in xf.values())
     n_xf = len(xf)                                               # a grouped launch stamps its first layer
-    per_step_launches = count_launches(layers, choices_raw, model.plan, nb, n_xf)
 
     h2d_value = h2d_bytes(layers, choices_raw, model.plan, nb, 0)
     h2d_e2e = h2d_bytes(layers, choices_raw, model.plan, nb, x.nbytes)
@@ -814,7 +821,9 @@ def measure(args, config, steps, warmup, minimal, rank, world, local, ranks):
         "config": config_dict(args),
         "run": {"what": "nnv_cold_run_dio: raw weights H2D + transform + execution, eager (no CUDA graph), selection with allow_cached = 0",
                 "pipeline_depth": args.cold_depth, "replicas": world, "weights_bytes": int(model.w_bytes),
-                "h2d_bytes_per_step": h2d_value, "transform_launches_per_step": n_xf,
+                "h2d_bytes_per_step": h2d_value, "kernel_launches_per_step": gpu_launches // (2 * args.steps),
+                "stamped": {"ms": stamped_ms, "transform_launches_per_step": n_xf,
+                            "what": "the same step with kernels that stamp the device clock and no layers fused; rooflines, per_layer and breakdown are of it"},
                 "cached_layers": sum(1 for c in choices_raw if c is not None and c[2])},
         "e2e": {"value": e2e, "unit": UNIT, "h2d_bytes_per_step": h2d_e2e,
                 "d2h_bytes_per_step": int(model.h_output.numel() * 4), "host_wall_ms": e2e_wall,
@@ -822,7 +831,7 @@ def measure(args, config, steps, warmup, minimal, rank, world, local, ranks):
                 "what": "nnv_cold_run: as `value`, plus the input image from and the output to pinned host memory",
                 "host_link": {"bound": "pcie", "bulk_copy_gbs": link_gbs, "floor_ms": h2d_e2e / link_gbs / 1e6,
                               "frac_of_floor": (h2d_e2e / link_gbs / 1e6) / e2e if e2e > 0 else None}},
-        "gpu_launches": 2 * per_step_launches * args.steps,
+        "gpu_launches": gpu_launches,
         "clocks": clocks,
         "roofline": roof,
         "roofline_transform": xroof,

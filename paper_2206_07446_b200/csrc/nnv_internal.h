@@ -38,6 +38,8 @@ nnv_status_t fail(nnv_status_t code, const char* fmt, ...);
         if (s__ != NNV_OK) return s__;        \
     } while (0)
 
+uint64_t& launches_made();                                    // kernels that the calling thread has launched or recorded
+
 // ---- programmatic dependent launch ----------------------------------------------------------
 // Every kernel is launched with the programmatic-stream-serialization attribute and starts with
 // pdl_enter(): it waits until the previous grid has completed and its writes are visible, then lets the
@@ -89,6 +91,7 @@ inline cudaError_t launch_pdl_attrs(int carveout, int cluster_z, void (*kernel)(
         attr[cfg.numAttrs].val.clusterDim.y = 1;
         attr[cfg.numAttrs++].val.clusterDim.z = (unsigned)cluster_z;
     }
+    ++launches_made();
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
 }
 template <typename... Params, typename... Args>

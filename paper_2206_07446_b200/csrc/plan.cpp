@@ -27,6 +27,11 @@ static Tuning g_tuning;
 static std::atomic<uint64_t> g_tuning_generation{0};
 
 // (asked several times a launch: a thread takes the lock and the copy only when something has been set since)
+uint64_t& launches_made() {
+    static thread_local uint64_t n = 0;
+    return n;
+}
+
 const Tuning& tuning() {
     static thread_local Tuning seen;
     if (seen.generation != g_tuning_generation.load(std::memory_order_acquire)) {
@@ -613,3 +618,6 @@ nnv_status_t nnv_switch_set(const nnv_plan_t* p, const nnv_choice_t* cold, const
 }
 
 }  // extern "C"
+
+// Kernels that the calling thread has launched so far (a replayed graph's are not among them), for the benchmark.
+extern "C" uint64_t nnv_internal_launches() { return nnv::launches_made(); }

@@ -47,10 +47,10 @@ class Model:
         self.h_cached = None
         self.c_bytes = 0
 
-    def second_plan(self, use_graphs):
+    def second_plan(self, use_graphs, kernel_stamps=0):
         """Another plan over the same layers and weight blob (e.g. one that replays recorded graphs beside an eager one)."""
         return nb.Plan(self.layers, self.w_off, self.b_off, opts=dict(default_math=nb.MATH_TF32, allow_cached=1, max_depth=4,
-                                                                      kernel_stamps=0, use_graphs=use_graphs))
+                                                                      kernel_stamps=kernel_stamps, use_graphs=use_graphs))
 
     def out_hw(self, i):
         L = self.layers[i]
