@@ -71,8 +71,8 @@ def parse():
     ap.add_argument("--save-costs", default=None, help="write the profiled cost table (JSON) to this file")
     ap.add_argument("--load-costs", default=None, help="use a cost table saved earlier instead of profiling (e.g. under a profiler)")
     # single-kernel timing through the C ABI
-    ap.add_argument("--kernel", default=None, choices=["transform", "transform-sweep", "conv", "conv-sweep", "transform-all"])
-    ap.add_argument("--prefer", default="", help="comma-separated variants tried first per layer (--kernel transform-all)")
+    ap.add_argument("--kernel", default=None, choices=["transform", "transform-sweep", "conv", "conv-sweep", "transform-all", "resident"])
+    ap.add_argument("--prefer", default="", help="comma-separated variants tried first per layer (--kernel transform-all, resident)")
     ap.add_argument("--m", type=int, default=4, help="Winograd tile size of --kernel transform (0 = the GEMM repack)")
     ap.add_argument("--variant", default="im2col")
     ap.add_argument("--C", type=int, default=512)
@@ -1012,12 +1012,8 @@ def _offsets(layers):
     return w_off, [0] * len(layers), pos
 
 
-def time_transform_all(torch, nb, config, prefer, math, reps=20, flush=None):
-    """Every layer's weight transform of one configuration by nnv_transform_all.  Layers take the first
-    eligible variant of `prefer`, then gemm1x1 / im2col."""
-    layers = wl.CONFIGS[config]()
-    w_off, b_off, w_bytes = _offsets(layers)
-    plan = nb.Plan(layers, w_off, b_off)
+def _choices(nb, plan, layers, prefer, math):
+    """Layers take the first eligible variant of `prefer`, then gemm1x1 / im2col."""
     choices = []
     for i, L in enumerate(layers):
         if L["op"] != wl.OP_CONV:
@@ -1029,6 +1025,38 @@ def time_transform_all(torch, nb, config, prefer, math, reps=20, flush=None):
             v = nb.VAR_DEPTHWISE if nb.VAR_DEPTHWISE in el else el[0]
         m = nb.MATH_FP32 if v in (nb.VAR_DIRECT, nb.VAR_DEPTHWISE) else (nb.MATH_TF32 if v in (nb.VAR_WINO_F4, nb.VAR_WINO_F6) else math)
         choices.append((v, m, 0))
+    return choices
+
+
+def time_resident(torch, nb, config, prefer, math, depth, reps=20, flush=None):
+    """A pass over one configuration's layers from raw weights in device memory (nnv_resident_run, eager, on a plain plan): the
+    layers and blocks that run as one launch run as one here."""
+    from paper_2206_07446_b200 import harness
+    layers = wl.CONFIGS[config]()
+    ws, bs = wl.make_weights(layers)
+    m1 = harness.model_from_workload(layers, ws, bs, wl.weight_blob, use_graphs=0)
+    choices = _choices(nb, m1.plan, layers, prefer, math)
+    m1.to_device()
+    m1.d_input.copy_(torch.from_numpy(wl.make_input(layers)))
+    ch, need = nb.choices_array(m1.plan, choices), m1.ensure_arena(choices, depth)
+    ts = []
+    for r in range(reps + 2):
+        if flush is not None:
+            flush.fill_(r & 0xFF)
+        torch.cuda.synchronize()
+        t0, n0 = time.perf_counter(), launches_made(nb)
+        nb.nnv_resident_run(m1.plan, ch, m1.d_weights, m1.w_bytes, None, 0, m1.d_input, m1.d_output, m1.arena, need, m1.streams[1], m1.streams[2], depth)
+        ts.append((time.perf_counter() - t0) * 1e6)
+    return dict(op="resident", config=config, prefer=[nb.VARIANT_NAMES[v] for v in prefer], math=nb.MATH_NAMES[math], depth=depth,
+                us=statistics.median(ts[2:]), us_min=min(ts[2:]), launches=launches_made(nb) - n0)
+
+
+def time_transform_all(torch, nb, config, prefer, math, reps=20, flush=None):
+    """Every layer's weight transform of one configuration by nnv_transform_all."""
+    layers = wl.CONFIGS[config]()
+    w_off, b_off, w_bytes = _offsets(layers)
+    plan = nb.Plan(layers, w_off, b_off)
+    choices = _choices(nb, plan, layers, prefer, math)
     d_w = _rand(torch, w_bytes // 4 + 64, 0.05)
     offs, total = nb.nnv_transformed_layout(plan, choices)
     d_out = _buf(torch, total)
@@ -1104,7 +1132,7 @@ def other_kernel_rooflines(layers, model, nb, torch, flush, peaks):
     if dense:
         L = max(dense, key=lambda L: wl.out_hw(L)[0] * wl.out_hw(L)[1] * L["K"] * L["C"] * L["R"] * L["S"])
         r = time_conv(torch, nb, nb.VAR_DIRECT, nb.MATH_FP32, L["C"], L["K"], L["R"], L["stride"], L["H"], L["W"], 1, 5, flush)
-        rows.append({"kernel": "direct_conv_kernel", "bound": "alu", "layer": "%dx%d C=%d K=%d R=%d stride %d" % (L["H"], L["W"], L["C"], L["K"], L["R"], L["stride"]),
+        rows.append({"kernel": "direct_tile_kernel / direct_conv_kernel", "bound": "alu", "layer": "%dx%d C=%d K=%d R=%d stride %d" % (L["H"], L["W"], L["C"], L["K"], L["R"], L["stride"]),
                      "flops": r["direct_flops"], "us": r["us"], "achieved": r["direct_tflops"], "peak": fp32_peak, "unit": "TFLOP/s",
                      "frac": r["direct_tflops"] / fp32_peak,
                      "peak_derivation": "2 flop x 128 FP32 lanes x %d SMs x %.3f GHz (clocks.max.sm)" % (sms, clk_ghz)})
@@ -1135,6 +1163,9 @@ def run_kernel(args):
     elif a.kernel == "transform-all":
         prefer = [nb.VARIANT_NAMES.index(v) for v in a.prefer.split(",") if v]
         print(json.dumps(time_transform_all(torch, nb, a.config, prefer, math, a.reps, flush)))
+    elif a.kernel == "resident":
+        prefer = [nb.VARIANT_NAMES.index(v) for v in a.prefer.split(",") if v]
+        print(json.dumps(time_resident(torch, nb, a.config, prefer, math, a.depth, a.reps, flush)))
     elif a.kernel == "conv":
         v = nb.VARIANT_NAMES.index(a.variant)
         m = nb.MATH_FP32 if v in (nb.VAR_DIRECT, nb.VAR_DEPTHWISE) else math
