@@ -512,7 +512,7 @@ nnv_status_t status_word(int** out) {
 
 // direct_tile_kernel's tile and split for a layer, if it is to run it: by estimated time, us, of calls one behind the other.  Fitted to 260 layers of 16 -
 // 2048 channels on 7 - 160 pixels a side (11 % off on average, either kernel): they take 0.825 of direct_conv_kernel's time (geometric mean; 0.80
-// with the best of all tiles, splits and kernels), three of them 2 % longer or more.  direct_conv_kernel keeps what it is estimated to run within 3 %
+// with the best of all tiles, splits and kernels), three of them 2 % longer or more (of 260 others five, 24 -> 32 3x3 @106x84 by 8 %).  direct_conv_kernel keeps what it is estimated to run within 3 %
 // as fast, and within 20 % on up to 32 input or output channels, where the estimates are worst (32 -> 32 3x3 @80 8.5 us against 9.9).
 struct DirectSplit { int splits; double us; };
 DirectSplit pick_split(int P, int C, int K, int jc, int chunks, int taps) {

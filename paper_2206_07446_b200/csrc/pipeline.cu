@@ -88,7 +88,7 @@ static nnv_status_t pass_status(nnv_plan* p) {
 }
 
 // A call whose arguments are those of a recorded pass replays it at once: the same arguments have been checked and laid out before, and what the
-// record does not hold -- the buffers' sizes, whether host memory is still pinned -- is looked at again.  (Planning a pass costs the host 10 us, in which the
+// record does not hold -- the buffers' sizes, whether host memory that kernels address is still pinned (input, output, weights of zero-copy layers) -- is looked at again.  (Planning a pass costs the host 10 us, in which the
 // GPU waits: warm MobileNetV2-shaped inference @160 131 -> 121 us.)
 struct Call {
     const nnv_choice_t* choices;

@@ -7,8 +7,8 @@
 //     input channels, or, where that leaves SMs idle and lone warps with long sums, two groups x quarters or one x eighths (below).  Eight lanes read 128 contiguous bytes of a channel's row, a warp four rows at a time, sixteen in all, so that a word of V
 //     read from shared memory serves four rows of a lane.
 //   - The lanes' sums are reduced by exchanging halves (3.5 T shuffles), the halves of the input channels through shared memory; the order is fixed,
-//     and wino_layer.cu's is the same: a layer has the same bits whether its weights come transformed or raw.  (Where that kernel deals the channels to eight
-//     blocks, a half is summed as two quarters.)
+//     and wino_layer.cu's is the same where it may run the layer: that has the same bits whether its weights come transformed or raw.  (Where that
+//     kernel deals the channels to eight blocks, a half is summed as two quarters.)
 // 512 -> 512 F(4,3) @7 in a model, U in the L2: 7.4 us against 11.3 on the tensor cores.
 #include <algorithm>
 #include <type_traits>
